@@ -74,8 +74,8 @@ enum {
   GEDWALK_GAINS_ALL = 1,  /* maximize: evaluate every vertex's exact gain at every step (no pruning) */
   GEDWALK_STOCHASTIC = 2, /* maximize: stochastic greedy (Appendix D), see gedwalk_maximize */
   GEDWALK_ADAPTIVE_L = 4, /* maximize: lazy greedy with l-doubling (Algorithm 2), see gedwalk_maximize */
-  GEDWALK_DEVICE_LOOP = 8 /* maximize: with the lookahead on, run the k steps as one device-resident
-                           * CUDA graph instead of the host loop; same kernels, same result */
+  GEDWALK_DEVICE_LOOP = 8 /* maximize: accepted; the one greedy loop reads back once per run of several
+                           * steps, so there is no second, device-resident one to choose */
 };
 
 /* gedwalk_graph_upload flags */
@@ -310,17 +310,14 @@ GEDWALK_API gedwalk_status gedwalk_gains(gedwalk_graph_t g, const int32_t* S, in
  * where splitmix64(x) is the first output of that generator started from state x;
  * an empty sample falls back to all of V \ S. The argmax within the sample is exact.
  * It cannot be combined with GEDWALK_GAINS_ALL or an init group.
- * Without a flag, on an undirected graph, each run of sweeps also computes the
- * next steps' phi^miss vectors and exact gains for guessed winners (lookahead):
- * a step whose winner was guessed needs no sweep. Every pick is still certified
- * against the bounds of the actual group, so the results do not depend on it.
- * params->lookahead (1 = off, 3; 7 in FP32) sets the number of steps per run
- * (0: 7 in FP32, 3 in FP64); params->spec_cols the width of the one-step fused
- * sweep when the lookahead is off. Other values return INVALID.
- * The host drives the steps: one synchronisation per bound pass, to read the
- * selection. With the lookahead on, GEDWALK_DEVICE_LOOP runs the k steps as one
- * device-resident CUDA graph instead (conditional nodes: the certification loop
- * never returns to the host). The picks and gains do not depend on it.
+ * On an undirected graph each run of sweeps also computes the next steps' bounds
+ * and exact gains for guessed winners (lookahead): a step whose winner was
+ * guessed needs no sweep. Every pick is still certified against the bounds of
+ * the actual group, so the results do not depend on it. params->lookahead
+ * (1 = off, 3; 7 in FP32; read without a flag) sets the number of steps per run
+ * (0: 7 in FP32, 3 in FP64); params->spec_cols the width of the one-step run
+ * when the lookahead is off. Other values return INVALID. The host drives the
+ * steps with one synchronisation per run.
  * GEDWALK_ADAPTIVE_L runs the lazy greedy of Algorithm 2 (Section 3.2.3): the
  * walk length l starts at 1 and only doubles. At each step u, the vertex with the
  * largest L_l(S, u) = GED_{<=l}(S, u), is taken when it is separated from v, the

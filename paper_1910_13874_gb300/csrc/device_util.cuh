@@ -1,0 +1,140 @@
+// Device helpers shared by the kernels: per-lane column sums, the best-16 lists of the selection
+// passes, stochastic greedy's draw.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <climits>
+#include <cstdint>
+
+namespace gw {
+
+// Per-lane column sums over the rows of one unit. FP64 vectors sum in FP64. FP32 vectors sum with
+// compensated FP32 additions (Kahan: the error is at most 2u * sum |y| + O(m u^2), u = 2^-24, over
+// m <= 128 rows) and convert once per unit to FP64, in which every later sum (over lanes, units and
+// sweeps) is taken. On a GB300 an FP64 addition costs about 64 FP32 ones, and one conversion and
+// one FP64 addition per row and column cost more than the rest of the epilogue.
+template <typename T, int N>
+struct ColAcc {
+  double s[N];
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int k = 0; k < N; ++k) s[k] = 0.0;
+  }
+  __device__ __forceinline__ void add(int k, double y) { s[k] += y; }
+  __device__ __forceinline__ double get(int k) const { return s[k]; }
+};
+template <int N>
+struct ColAcc<float, N> {
+  float s[N], c[N];
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int k = 0; k < N; ++k) s[k] = c[k] = 0.0f;
+  }
+  __device__ __forceinline__ void add(int k, float y) {
+    const float t1 = __fsub_rn(y, c[k]);
+    const float t = __fadd_rn(s[k], t1);
+    c[k] = __fsub_rn(__fsub_rn(t, s[k]), t1);
+    s[k] = t;
+  }
+  __device__ __forceinline__ double get(int k) const { return static_cast<double>(s[k]) - static_cast<double>(c[k]); }
+};
+
+// ---------------------------------------------------------------- selection
+constexpr int kTopK = 16;
+
+struct Stale {
+  float ub;      // last exact gain rounded up (an upper bound for every later step)
+  int32_t step;  // step in which it was evaluated, -1 if never
+};
+
+constexpr unsigned long long kNoZero = ~0ull;
+__host__ __device__ inline int32_t zero_caller(unsigned long long z) {
+  return z == kNoZero ? INT_MAX : static_cast<int32_t>(z >> 32);
+}
+__host__ __device__ inline int32_t zero_internal(unsigned long long z) {
+  return static_cast<int32_t>(z & 0xffffffffull);
+}
+
+__device__ __forceinline__ bool better(float a, int ia, float b, int ib) { return a > b || (a == b && ia < ib); }
+
+// Stochastic greedy's counter-based draw: the first output of splitmix64 (Steele, Lea & Flood,
+// 2014) started from state seed ^ (step << 32) ^ v, v a caller id.
+__device__ __forceinline__ uint64_t sample_hash(uint64_t seed, uint32_t step, uint32_t v) {
+  uint64_t z = (seed ^ (static_cast<uint64_t>(step) << 32) ^ static_cast<uint64_t>(v)) + 0x9e3779b97f4a7c15ULL;
+  z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ULL;
+  z = (z ^ (z >> 27)) * 0x94d049bb133111ebULL;
+  return z ^ (z >> 31);
+}
+
+constexpr unsigned kFullMask = 0xffffffffu;
+
+// A warp's sorted list of its kTopK best (value, id) pairs in the order of `better`: lane i <
+// kTopK holds the i-th entry (value -1, id INT_MAX: empty); `tag` travels with its entry.
+struct WarpList {
+  float v = -1.0f;
+  int id = INT_MAX;
+  int tag = 0;
+};
+
+// Offers every lane's (x, ix, tag) where `want` holds. Only the lanes that beat the list's last
+// entry are inserted, one at a time (lowest lane first); after each insertion the others are
+// checked again against the new last entry. Ids must be distinct. All 32 lanes take part.
+__device__ __forceinline__ void warp_list_offer(WarpList& w, bool want, float x, int ix, int tag) {
+  const int lane = threadIdx.x & 31;
+  float tv = __shfl_sync(kFullMask, w.v, kTopK - 1);
+  int ti = __shfl_sync(kFullMask, w.id, kTopK - 1);
+  unsigned m = __ballot_sync(kFullMask, want && better(x, ix, tv, ti));
+  while (m) {
+    const int src = __ffs(m) - 1;
+    const float cv = __shfl_sync(kFullMask, x, src);
+    const int ci = __shfl_sync(kFullMask, ix, src);
+    const int ct = __shfl_sync(kFullMask, tag, src);
+    // the entries ahead of the new one form a prefix of the sorted list
+    const int pos = __popc(__ballot_sync(kFullMask, lane < kTopK && better(w.v, w.id, cv, ci)));
+    const float uv = __shfl_up_sync(kFullMask, w.v, 1);
+    const int ui = __shfl_up_sync(kFullMask, w.id, 1);
+    const int ut = __shfl_up_sync(kFullMask, w.tag, 1);
+    if (lane == pos) {
+      w.v = cv;
+      w.id = ci;
+      w.tag = ct;
+    } else if (lane > pos && lane < kTopK) {
+      w.v = uv;
+      w.id = ui;
+      w.tag = ut;
+    }
+    tv = __shfl_sync(kFullMask, w.v, kTopK - 1);
+    ti = __shfl_sync(kFullMask, w.id, kTopK - 1);
+    m &= m - 1;
+    m &= __ballot_sync(kFullMask, want && better(x, ix, tv, ti));
+  }
+}
+
+// Merges the NW warp lists of a block into warp 0's list (staged through shared memory sv/si/st,
+// NW * kTopK entries each). Every thread of the block calls it.
+template <int NW>
+__device__ void block_list_merge(WarpList& w, float* sv, int* si, int* st) {
+  static_assert(kTopK == 16, "two warp lists per 32-lane offer");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane < kTopK) {
+    sv[warp * kTopK + lane] = w.v;
+    si[warp * kTopK + lane] = w.id;
+    st[warp * kTopK + lane] = w.tag;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    for (int j = 1; j < NW; j += 2) {  // lists j and j + 1 on lanes 0-15 and 16-31
+      const int src = j + (lane >> 4);
+      const bool ok = src < NW;
+      const int e = src * kTopK + (lane & 15);
+      const float x = ok ? sv[e] : -1.0f;
+      const int ix = ok ? si[e] : INT_MAX;
+      const int t = ok ? st[e] : 0;
+      warp_list_offer(w, ix != INT_MAX, x, ix, t);
+    }
+  }
+  __syncthreads();
+}
+
+}  // namespace gw

@@ -111,9 +111,8 @@ void profile_end(cudaStream_t s, cudaEvent_t a, double bytes, int key) {
 double sweep_bytes(int mode, bool fp64, int cols, int32_t n, int64_t nnz, bool weighted) {
   const double es = mode == MODE_TOTALS ? 8.0 : (fp64 ? 8.0 : 4.0);
   double b = 4.0 * double(nnz) + 4.0 * (double(n) + 1.0) + 2.0 * cols * es * double(n);
-  if (mode == MODE_SCORE || mode == MODE_FUSED || mode == MODE_CAND || mode == MODE_LOOK) b += double(n) / 8.0;
+  if (mode != MODE_TOTALS && mode != MODE_PLAIN) b += double(n) / 8.0;
   if (mode == MODE_FUSED) b += es * double(n);
-  if (mode == MODE_LOOK) b += es * double(n) * (cols - 1);  // one phi^miss row per level
   if (weighted) b += es * double(n);  // the vertex scales
   return b;
 }
@@ -179,25 +178,24 @@ void SweepGraph::reset() {
 int64_t Workspace::device_bytes() const {
   int64_t b = 0;
   for (const DevBuf* d : {&x0, &x1, &mtab, &ztab, &pvec, &partial, &counters, &slots, &parts, &mask, &stale, &sel,
-                          &small, &members, &ctl})
+                          &small, &members, &xs, &cnt, &tail, &bound})
     b += static_cast<int64_t>(d->bytes);
   return b;
 }
 
 void Workspace::release_device() {
   for (SweepGraph& sg : graphs) sg.reset();
-  greedy_loop.reset();
   for (DevBuf* d : {&x0, &x1, &mtab, &ztab, &pvec, &partial, &counters, &slots, &parts, &mask, &stale, &sel, &small,
-                    &members, &ctl})
+                    &members, &xs, &cnt, &tail, &bound})
     d->release();
 }
 
 Workspace::~Workspace() {
   for (SweepGraph& sg : graphs) sg.reset();
-  greedy_loop.reset();
   if (order_ev) cudaEventDestroy(order_ev);
   if (own_stream) cudaStreamDestroy(own_stream);
   if (pinned) cudaFreeHost(pinned);
+  if (run_io) cudaFreeHost(run_io);
 }
 
 gedwalk_status Workspace::ensure_pinned(size_t need) {
@@ -963,6 +961,28 @@ gedwalk_status ensure_totals(Graph& g, double alpha, int32_t rows, cudaStream_t 
   g.Wa.resize(rows);
   for (int32_t r = r0; r < rows; ++r) g.Wa[r] = tmp[r];
   g.tt_rows = rows;
+  return GEDWALK_OK;
+}
+
+gedwalk_status totals_into(Graph& g, Workspace& ws, double* T, double alpha, int32_t rows, cudaStream_t s) {
+  const size_t n = static_cast<size_t>(g.n);
+  GW_TRY(ensure_sweep_scratch(g, ws, 1, true, s));
+  if (g.weighted) {
+    GW_CUDA(cudaMemcpyAsync(T, g.rs_d.p, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
+  } else {
+    fill_f64_kernel<<<grid_for(g.n), 256, 0, s>>>(T, g.n, 1.0);
+    GW_KCHECK();
+  }
+  SweepArgs a = base_args(g, ws);
+  a.alpha = alpha;
+  for (int32_t r = 1; r < rows; ++r) {
+    a.X = T + static_cast<size_t>(r - 1) * n;
+    a.Y = T + static_cast<size_t>(r) * n;
+    if (g.n_active < g.n)
+      GW_CUDA(cudaMemsetAsync(T + static_cast<size_t>(r) * n + g.n_active, 0,
+                              sizeof(double) * (n - static_cast<size_t>(g.n_active)), s));
+    GW_TRY(launch_sweep(MODE_TOTALS, true, 1, a, s));
+  }
   return GEDWALK_OK;
 }
 

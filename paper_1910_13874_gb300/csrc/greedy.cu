@@ -1,20 +1,21 @@
 // Greedy GED-Walk maximisation (problem (ii), Def. ged-max; Prop. greedy_approx) and
 // all-vertex exact marginal gains.
 //
-// A step with current group S:
-//  1. L fused sweeps compute phi^miss_1..L under S (column 0, stored in a table) and,
-//     in the same pass, the exact gains of up to kSpec "speculative" candidates
-//     (columns 1..), chosen before S was known from bounds that stay valid when S
-//     grows: the last exact gain (submodularity, Prop. ged_submod) and the previous
-//     step's Lemma-initialize bound (P_i is non-increasing in S).
-//  2. One pass over all vertices forms the Lemma-initialize bound
-//       ub(x) = sum_{i=1..L} alpha^i P_i(S, x) = sum_{1 <= a+b <= L} y_a(x) y_b(x),
-//     y_a = alpha^a phi^miss_a (psi^miss = phi^miss on an undirected graph), takes
-//     min(ub, last exact gain), and selects the best-bounded unevaluated vertices.
-//  3. The best evaluated candidate wins once no unevaluated bound (inflated by the
-//     rounding tolerance) reaches its gain; otherwise the next batch of candidates
-//     is evaluated exactly and step 2 repeats. A vertex whose bound is exactly 0
-//     has gain exactly 0. Among equal gains the lowest caller id wins.
+// Undirected graphs: runs of half the walk length (run.cu). A chain run carries the next steps'
+// guessed winners c_1..c_D, each under S and the earlier ones, and brings for every level the best
+// upper bounds of the unevaluated vertices and the exact gain of its guess. A step takes the guess
+// once no bound (inflated by the rounding tolerance) reaches its gain; otherwise the best-bounded
+// vertices are evaluated exactly, side by side under S, until the best exact gain is beyond every
+// bound. No result depends on the guesses. A vertex whose bound is exactly 0 has gain exactly 0.
+// Among equal gains the lowest caller id wins.
+//
+// Directed graphs (maximize_directed): a step with current group S runs L fused sweeps (phi^miss_1..L
+// under S in column 0, stored in a table, and the exact gains of speculative candidates), the psi^miss
+// sweeps of the other orientation on the reverse CSR, and one pass over all vertices with the
+// Lemma-initialize bound
+//       ub(x) = sum_{i=1..L} alpha^i P_i(S, x) = sum_{1 <= a+b <= L} y_a(x) z_b(x),
+// y_a = alpha^a phi^miss_a, z_b = alpha^b psi^miss_b, min'd with the last exact gain; then the same
+// certification.
 // The gain of candidate c counts walks of length 1..L in G[V\S] through c
 // (proof of Prop. ged_submod): h_0 = e_c, h_t = alpha 1_{V\S} . A h_{t-1} except
 // h_t(c) = phi^miss_t(c); gain = sum_t sum_v h_t(v) in FP64.
@@ -25,20 +26,14 @@
 #include <cmath>
 #include <cstdlib>
 
-#include "internal.h"
+#include "run.h"
 
 namespace gw {
 namespace {
 
-constexpr int kTopK = 16;
 constexpr int kSelPerSM = 4;               // resident blocks of the bound pass per SM
 constexpr int kSelU = 2;                   // vertices per lane and iteration of the bound pass
 constexpr int kSelBlocks = 152 * kSelPerSM;
-
-struct Stale {
-  float ub;      // last exact gain rounded up (an upper bound for every later step)
-  int32_t step;  // step in which it was evaluated, -1 if never
-};
 
 struct SelOut {  // device -> host after each selection pass
   float val[kTopK];
@@ -51,25 +46,6 @@ struct SelOut {  // device -> host after each selection pass
   double gains[16];  // exact gains of the last candidate batch
 };
 
-constexpr unsigned long long kNoZero = ~0ull;
-__host__ __device__ inline int32_t zero_caller(unsigned long long z) {
-  return z == kNoZero ? INT_MAX : static_cast<int32_t>(z >> 32);
-}
-__host__ __device__ inline int32_t zero_internal(unsigned long long z) {
-  return static_cast<int32_t>(z & 0xffffffffull);
-}
-
-__device__ __forceinline__ bool better(float a, int ia, float b, int ib) { return a > b || (a == b && ia < ib); }
-
-// Stochastic greedy's counter-based draw: the first output of splitmix64 (Steele, Lea & Flood,
-// 2014) started from state seed ^ (step << 32) ^ v, v a caller id.
-__device__ __forceinline__ uint64_t sample_hash(uint64_t seed, uint32_t step, uint32_t v) {
-  uint64_t z = (seed ^ (static_cast<uint64_t>(step) << 32) ^ static_cast<uint64_t>(v)) + 0x9e3779b97f4a7c15ULL;
-  z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ULL;
-  z = (z ^ (z >> 27)) * 0x94d049bb133111ebULL;
-  return z ^ (z >> 31);
-}
-
 // Sampling of one selection pass; thr == UINT64_MAX means every vertex takes part.
 struct Sampling {
   uint64_t thr;
@@ -77,166 +53,21 @@ struct Sampling {
   uint32_t step;
 };
 
-constexpr unsigned kFullMask = 0xffffffffu;
-
-// A warp's sorted list of its kTopK best (value, id) pairs in the order of `better`: lane i <
-// kTopK holds the i-th entry (value -1, id INT_MAX: empty); `tag` travels with its entry.
-struct WarpList {
-  float v = -1.0f;
-  int id = INT_MAX;
-  int tag = 0;
-};
-
-// Offers every lane's (x, ix, tag) where `want` holds. Only the lanes that beat the list's last
-// entry are inserted, one at a time (lowest lane first); after each insertion the others are
-// checked again against the new last entry. Ids must be distinct. All 32 lanes take part.
-__device__ __forceinline__ void warp_list_offer(WarpList& w, bool want, float x, int ix, int tag) {
-  const int lane = threadIdx.x & 31;
-  float tv = __shfl_sync(kFullMask, w.v, kTopK - 1);
-  int ti = __shfl_sync(kFullMask, w.id, kTopK - 1);
-  unsigned m = __ballot_sync(kFullMask, want && better(x, ix, tv, ti));
-  while (m) {
-    const int src = __ffs(m) - 1;
-    const float cv = __shfl_sync(kFullMask, x, src);
-    const int ci = __shfl_sync(kFullMask, ix, src);
-    const int ct = __shfl_sync(kFullMask, tag, src);
-    // the entries ahead of the new one form a prefix of the sorted list
-    const int pos = __popc(__ballot_sync(kFullMask, lane < kTopK && better(w.v, w.id, cv, ci)));
-    const float uv = __shfl_up_sync(kFullMask, w.v, 1);
-    const int ui = __shfl_up_sync(kFullMask, w.id, 1);
-    const int ut = __shfl_up_sync(kFullMask, w.tag, 1);
-    if (lane == pos) {
-      w.v = cv;
-      w.id = ci;
-      w.tag = ct;
-    } else if (lane > pos && lane < kTopK) {
-      w.v = uv;
-      w.id = ui;
-      w.tag = ut;
-    }
-    tv = __shfl_sync(kFullMask, w.v, kTopK - 1);
-    ti = __shfl_sync(kFullMask, w.id, kTopK - 1);
-    m &= m - 1;
-    m &= __ballot_sync(kFullMask, want && better(x, ix, tv, ti));
-  }
-}
-
-// Merges the NW warp lists of a block into warp 0's list (staged through shared memory sv/si/st,
-// NW * kTopK entries each). Every thread of the block calls it.
-template <int NW>
-__device__ void block_list_merge(WarpList& w, float* sv, int* si, int* st) {
-  static_assert(kTopK == 16, "two warp lists per 32-lane offer");
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane < kTopK) {
-    sv[warp * kTopK + lane] = w.v;
-    si[warp * kTopK + lane] = w.id;
-    st[warp * kTopK + lane] = w.tag;
-  }
-  __syncthreads();
-  if (warp == 0) {
-    for (int j = 1; j < NW; j += 2) {  // lists j and j + 1 on lanes 0-15 and 16-31
-      const int src = j + (lane >> 4);
-      const bool ok = src < NW;
-      const int e = src * kTopK + (lane & 15);
-      const float x = ok ? sv[e] : -1.0f;
-      const int ix = ok ? si[e] : INT_MAX;
-      const int t = ok ? st[e] : 0;
-      warp_list_offer(w, ix != INT_MAX, x, ix, t);
-    }
-  }
-  __syncthreads();
-}
-
 // mtab row 0 = phi^miss_0 = 1_{V\S}; X column 0 (fused) = the same; candidate columns = e_c.
-// On a weighted graph X holds the scaled vectors (times s_v, rs); the table the true values.
 template <typename T>
 __global__ void greedy_init(T* __restrict__ m0, T* __restrict__ X, int cols, int first_cand_col,
-                            const int32_t* __restrict__ cand, const uint32_t* __restrict__ mask, int32_t n,
-                            const T* __restrict__ rs) {
+                            const int32_t* __restrict__ cand, const uint32_t* __restrict__ mask, int32_t n) {
   __shared__ int sc[16];
   if (threadIdx.x < 16) sc[threadIdx.x] = threadIdx.x < cols - first_cand_col ? cand[threadIdx.x] : -1;
   __syncthreads();
   for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
     const bool inS = (mask[v >> 5] >> (v & 31)) & 1u;
     const T m = inS ? T(0) : T(1);
-    const T sv = rs ? rs[v] : T(1);
     if (m0) m0[v] = m;
     T* row = X + static_cast<size_t>(v) * cols;
-    if (first_cand_col == 1) row[0] = m * sv;
-    for (int j = first_cand_col; j < cols; ++j) row[j] = (sc[j - first_cand_col] == v) ? sv : T(0);
+    if (first_cand_col == 1) row[0] = m;
+    for (int j = first_cand_col; j < cols; ++j) row[j] = (sc[j - first_cand_col] == v) ? T(1) : T(0);
   }
-}
-
-// MODE_LOOK initialisation for a run of C - 1 levels with guesses c_1..c_{C-1}: column 0 is
-// phi^miss_0 under S, column j >= 1 the unit vector of c_j (0 without one); table d, row 0, is
-// phi^miss_0 under S + {c_1..c_d}. The walk vectors are written 16 bytes per thread (consecutive
-// threads, consecutive chunks).
-template <typename T>
-struct Vec16;
-template <>
-struct Vec16<float> {
-  using type = float4;
-  __device__ static float4 make(const float* e) { return make_float4(e[0], e[1], e[2], e[3]); }
-};
-template <>
-struct Vec16<double> {
-  using type = double2;
-  __device__ static double2 make(const double* e) { return make_double2(e[0], e[1]); }
-};
-
-template <typename T, int C>
-__global__ void look_init(T* __restrict__ tab, int64_t tab_stride, T* __restrict__ X,
-                          const int32_t* __restrict__ cand, const uint32_t* __restrict__ mask, int32_t n,
-                          const T* __restrict__ rs) {
-  constexpr int LV = C - 1;                               // levels
-  constexpr int per = 16 / static_cast<int>(sizeof(T));  // elements per 16-byte chunk
-  static_assert(C % per == 0, "a row is whole 16-byte chunks");
-  constexpr int cpr = C / per;                            // chunks per row
-  __shared__ int sc[LV];
-  if (threadIdx.x < LV) sc[threadIdx.x] = cand[threadIdx.x];
-  __syncthreads();
-  const int64_t chunks = static_cast<int64_t>(n) * cpr;
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  using V = typename Vec16<T>::type;
-  for (int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; q < chunks; q += stride) {
-    const int32_t v = static_cast<int32_t>(q / cpr);
-    const int part = static_cast<int>(q % cpr);
-    const bool inS = (__ldg(mask + (v >> 5)) >> (v & 31)) & 1u;
-    const T sv = rs ? rs[v] : T(1);
-    T e[per];
-#pragma unroll
-    for (int j = 0; j < per; ++j) {
-      const int col = part * per + j;
-      if (col == 0) e[j] = inS ? T(0) : sv;
-      else e[j] = sc[col - 1] == v ? sv : T(0);
-    }
-    reinterpret_cast<V*>(X)[q] = Vec16<T>::make(e);
-  }
-  for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-    bool out = (__ldg(mask + (v >> 5)) >> (v & 31)) & 1u;
-#pragma unroll
-    for (int d = 0; d < LV; ++d) {
-      if (d > 0 && sc[d - 1] == v) out = true;
-      tab[tab_stride * d + v] = out ? T(0) : T(1);
-    }
-  }
-}
-
-// cols = levels + 1: 4 or (FP32) 8, the only shapes greedy_shape admits
-template <typename T>
-void launch_look_init(int cols, int blocks, cudaStream_t s, T* tab, int64_t tab_stride, T* X, const int32_t* cand,
-                      const uint32_t* mask, int32_t n, const T* rs) {
-  if (cols == 4 || sizeof(T) == 8) look_init<T, 4><<<blocks, 256, 0, s>>>(tab, tab_stride, X, cand, mask, n, rs);
-  else look_init<T, 8><<<blocks, 256, 0, s>>>(tab, tab_stride, X, cand, mask, n, rs);
-}
-
-// Records one exact gain known on the host (a lookahead level's candidate) for this step.
-__global__ void set_stale(Stale* __restrict__ stale, int32_t v, double gain, int32_t step, double* __restrict__ out) {
-  Stale st;
-  st.ub = __double2float_ru(gain);
-  st.step = step;
-  stale[v] = st;
-  out[0] = gain;
 }
 
 __global__ void update_stale(Stale* __restrict__ stale, const int32_t* __restrict__ cand,
@@ -325,17 +156,10 @@ __global__ void __launch_bounds__(kThreads, kSelPerSM) ub_select(const T* __rest
                                                      const Stale* __restrict__ stale, int32_t step,
                                                      const int32_t* __restrict__ perm, float* __restrict__ sel_v,
                                                      int* __restrict__ sel_id, SelOut* __restrict__ out,
-                                                     const Sampling smp, const int32_t* level_ptr,
-                                                     int64_t level_stride, const int32_t* step_ptr) {
+                                                     const Sampling smp) {
   constexpr int NW = kThreads / 32;
   static_assert(2 * NW >= kTopK, "the final merge gives each warp two block lists");
   constexpr int U = kSelU;
-  if (level_ptr) {  // the table (lookahead level) the device-resident loop chose for this step
-    const int64_t off = level_stride * __ldg(level_ptr);
-    mtab += off;
-    ztab += off;
-  }
-  if (step_ptr) step = __ldg(step_ptr);  // the device-resident loop's step
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int nsampled = 0;
   WarpList w;
@@ -429,20 +253,18 @@ template <typename T>
 cudaError_t launch_ub_select(int nb, cudaStream_t s, const T* mtab, const T* ztab, int32_t L, int32_t n,
                              int32_t n_scan, const uint32_t* mask,
                              const Stale* stale, int32_t step, const int32_t* perm, float* sel_v, int* sel_id,
-                             SelOut* out, const Sampling& smp,
-                             const int32_t* level_ptr = nullptr, int64_t level_stride = 0,
-                             const int32_t* step_ptr = nullptr) {
+                             SelOut* out, const Sampling& smp) {
 #define GW_UB(LL)                                                                                          \
   case LL:                                                                                                 \
     ub_select<T, LL><<<nb, kThreads, 0, s>>>(mtab, ztab, L, n, n_scan, mask, stale, step, perm, sel_v, sel_id, \
-                                             out, smp, level_ptr, level_stride, step_ptr);                 \
+                                             out, smp);                 \
     break;
   switch (L) {
     GW_UB(1) GW_UB(2) GW_UB(3) GW_UB(4) GW_UB(5) GW_UB(6) GW_UB(7) GW_UB(8)
     GW_UB(9) GW_UB(10) GW_UB(11) GW_UB(12) GW_UB(13) GW_UB(14) GW_UB(15) GW_UB(16)
     default:
       ub_select<T, 0><<<nb, kThreads, 0, s>>>(mtab, ztab, L, n, n_scan, mask, stale, step, perm, sel_v, sel_id,
-                                              out, smp, level_ptr, level_stride, step_ptr);
+                                              out, smp);
   }
 #undef GW_UB
   return cudaGetLastError();
@@ -492,29 +314,11 @@ struct GreedyCtx {
   double* d_gains;
   SelOut* h_out;
   int64_t sweeps = 0;
-  size_t tab_off = 0;  // elements: the phi^miss table in use (lookahead level) within ws.mtab
-  // device-resident loop: candidate rows read the table level the device chose (nullptr: none)
-  const int32_t* level_ptr = nullptr;
-  int64_t level_stride = 0;
-  // device-resident loop: a kernel stamps the device clock around the sweeps (stamp >= 0)
-  void* stamp_ctl = nullptr;
-  int stamp_end = 0;
 };
 
-// Stamps the device clock (%globaltimer, nanoseconds) into the controller: kind 0 opens an
-// interval, kind 1 adds it to the lookahead runs' time, kind 2 to the candidate batches'.
-__global__ void ctl_stamp(unsigned long long* __restrict__ t, int kind) {
-  if (threadIdx.x != 0) return;
-  unsigned long long now;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-  if (kind == 0) t[0] = now;
-  else t[kind] += now - t[0];
-}
-
-// Issues init + L sweeps + column-sum reduction on c.s. ev (optional): two external events
-// around each sweep (graph capture).
-// rev (directed graphs, MODE_FUSED with one column): the sweeps run on the reverse CSR and fill
-// the psi^miss table instead.
+// Issues init + L sweeps + column-sum reduction on c.s. ev (optional): two external events around
+// the run of sweeps (graph capture; event nodes between kernel nodes cost a few microseconds each).
+// rev (MODE_FUSED with one column): the sweeps run on the reverse CSR and fill the psi^miss table.
 gedwalk_status issue_sweeps(GreedyCtx& c, int mode, int cols, bool profile, const std::vector<cudaEvent_t>* ev,
                             bool rev) {
   Graph& g = c.g;
@@ -522,71 +326,37 @@ gedwalk_status issue_sweeps(GreedyCtx& c, int mode, int cols, bool profile, cons
   const bool fp64 = c.r.fp64;
   const int first = mode == MODE_FUSED ? 1 : 0;
   DevBuf& tab = rev ? ws.ztab : ws.mtab;
-  const size_t off = rev ? 0 : c.tab_off;  // elements
-  const int64_t look_stride = static_cast<int64_t>(c.L + 1) * g.n;  // elements between level tables
-  void* m0 = mode == MODE_FUSED ? tab.as<char>() + off * c.es : nullptr;
-  if (mode == MODE_LOOK) {
-    // cols - 1 lookahead levels: 3 or (FP32) 7 (the shape admits no other)
-    const int64_t chunks = static_cast<int64_t>(g.n) * cols * static_cast<int64_t>(c.es) / 16;
-    if (fp64)
-      launch_look_init<double>(cols, blocks_for(chunks), c.s, ws.mtab.as<double>(), look_stride, ws.x0.as<double>(),
-                               c.d_cand, ws.mask.as<uint32_t>(), g.n, g.weighted ? g.rs_d.as<double>() : nullptr);
-    else
-      launch_look_init<float>(cols, blocks_for(chunks), c.s, ws.mtab.as<float>(), look_stride, ws.x0.as<float>(),
-                              c.d_cand, ws.mask.as<uint32_t>(), g.n, g.weighted ? g.rs_f.as<float>() : nullptr);
-  } else if (fp64)
+  void* m0 = mode == MODE_FUSED ? tab.p : nullptr;
+  if (fp64)
     greedy_init<double><<<blocks_for(g.n), 256, 0, c.s>>>(static_cast<double*>(m0), ws.x0.as<double>(), cols, first,
-                                                           c.d_cand, ws.mask.as<uint32_t>(), g.n,
-                                                           g.weighted ? g.rs_d.as<double>() : nullptr);
+                                                           c.d_cand, ws.mask.as<uint32_t>(), g.n);
   else
     greedy_init<float><<<blocks_for(g.n), 256, 0, c.s>>>(static_cast<float*>(m0), ws.x0.as<float>(), cols, first,
-                                                          c.d_cand, ws.mask.as<uint32_t>(), g.n,
-                                                          g.weighted ? g.rs_f.as<float>() : nullptr);
+                                                          c.d_cand, ws.mask.as<uint32_t>(), g.n);
   GW_KCHECK();
   SweepArgs a = rev ? base_args_rev(g, ws) : base_args(g, ws);
   a.alpha = c.r.alpha;
   a.cand = c.d_cand;
   void* cur = ws.x0.p;
   void* nxt = ws.x1.p;
+  if (ev) GW_CUDA(cudaEventRecordWithFlags((*ev)[0], c.s, cudaEventRecordExternal));
   for (int32_t t = 1; t <= c.L; ++t) {
     a.X = cur;
     a.Y = nxt;
     a.accumulate = t > 1;
-    char* row = tab.as<char>() + (off + static_cast<size_t>(t) * g.n) * c.es;
+    char* row = tab.as<char>() + static_cast<size_t>(t) * g.n * c.es;
     if (mode == MODE_FUSED) a.Mout = row;
-    else if (mode == MODE_LOOK) a.Mout = tab.as<char>() + static_cast<size_t>(t) * g.n * c.es;
     else a.Min = row;
-    a.mout_stride = look_stride;
-    a.level_ptr = c.level_ptr;
-    a.level_stride = c.level_stride;
-    // external events bracket the whole run of sweeps (event nodes between kernel nodes cost
-    // a few microseconds each)
-    if (ev && t == 1) GW_CUDA(cudaEventRecordWithFlags((*ev)[0], c.s, cudaEventRecordExternal));
-    if (c.stamp_ctl && t == 1) {
-      ctl_stamp<<<1, 32, 0, c.s>>>(static_cast<unsigned long long*>(c.stamp_ctl), 0);
-      GW_KCHECK();
-    }
     GW_TRY(launch_sweep(mode, fp64, cols, a, c.s, profile));
-    if (ev && t == c.L) GW_CUDA(cudaEventRecordWithFlags((*ev)[1], c.s, cudaEventRecordExternal));
-    if (c.stamp_ctl && t == c.L) {
-      ctl_stamp<<<1, 32, 0, c.s>>>(static_cast<unsigned long long*>(c.stamp_ctl), c.stamp_end);
-      GW_KCHECK();
-    }
     std::swap(cur, nxt);
   }
+  if (ev) GW_CUDA(cudaEventRecordWithFlags((*ev)[1], c.s, cudaEventRecordExternal));
   const int nsum = sweep_sums(mode, cols);
   if (nsum > 0) GW_TRY(reduce_slots(g, ws, nsum, c.d_gains, c.s, rev));
   return GEDWALK_OK;
 }
 
-uint64_t mix_key(uint64_t h, uint64_t v) {
-  h ^= v + 0x9e3779b97f4a7c15ULL + (h << 6) + (h >> 2);
-  return h;
-}
-
-// Runs L sweeps. mode MODE_FUSED (column 0 = phi^miss, table rows written) or MODE_CAND. On a
-// capturable stream the sequence is captured once per configuration (on its second use) and
-// replayed as a CUDA graph.
+// Runs L sweeps. mode MODE_FUSED (column 0 = phi^miss, table rows written) or MODE_CAND.
 gedwalk_status run_sweeps(GreedyCtx& c, int mode, int cols, const std::vector<int32_t>& cand, bool rev = false) {
   Graph& g = c.g;
   Workspace& ws = c.ws;
@@ -599,86 +369,22 @@ gedwalk_status run_sweeps(GreedyCtx& c, int mode, int cols, const std::vector<in
   GW_TRY(ws.x1.ensure(vbytes, c.s));
   GW_TRY(ensure_sweep_scratch(g, ws, cols, fp64, c.s));
   c.sweeps += c.L;
-  if (c.s == nullptr || g.plan.num_units == 0) return issue_sweeps(c, mode, cols, true, nullptr, rev);
-  uint64_t key = 0;
-  for (uint64_t v : {uint64_t(mode), uint64_t(cols), uint64_t(fp64), uint64_t(c.L), uint64_t(g.n), uint64_t(rev),
-                     uint64_t(c.tab_off),
-                     reinterpret_cast<uint64_t>(ws.ztab.p),
-                     reinterpret_cast<uint64_t>(&g), reinterpret_cast<uint64_t>(c.s),
-                     reinterpret_cast<uint64_t>(ws.x0.p), reinterpret_cast<uint64_t>(ws.x1.p),
-                     reinterpret_cast<uint64_t>(ws.mtab.p), reinterpret_cast<uint64_t>(ws.slots.p),
-                     reinterpret_cast<uint64_t>(ws.parts.p), reinterpret_cast<uint64_t>(ws.partial.p),
-                     reinterpret_cast<uint64_t>(ws.counters.p), reinterpret_cast<uint64_t>(ws.mask.p),
-                     reinterpret_cast<uint64_t>(c.d_cand), reinterpret_cast<uint64_t>(c.d_gains)}) {
-    key = mix_key(key, v);
-  }
+  if (g.plan.num_units == 0) return issue_sweeps(c, mode, cols, true, nullptr, rev);
   uint64_t abits;
   memcpy(&abits, &c.r.alpha, 8);
-  key = mix_key(key, abits);
-  if (key == 0) key = 1;  // 0 marks a free cache entry
-  // the workspace's entry for this configuration, else the least recently used one
-  SweepGraph* hit = nullptr;
-  SweepGraph* lru = &ws.graphs[0];
-  for (SweepGraph& e : ws.graphs) {
-    if (e.key == key) hit = &e;
-    if (e.last_use < lru->last_use) lru = &e;
-  }
-  if (!hit) {
-    lru->reset();
-    lru->key = key;
-    hit = lru;
-  }
-  SweepGraph& sg = *hit;
-  sg.last_use = ++ws.graph_clock;
-  if (!sg.exec) {
-    if (sg.uses++ < 1) return issue_sweeps(c, mode, cols, true, nullptr, rev);  // set-up happens outside capture
-    sg.ev.assign(2, nullptr);
-    for (cudaEvent_t& e : sg.ev) GW_CUDA(cudaEventCreate(&e));
-    GW_CUDA(cudaStreamBeginCapture(c.s, cudaStreamCaptureModeThreadLocal));
-    set_capturing(true);
-    const gedwalk_status st = issue_sweeps(c, mode, cols, false, &sg.ev, rev);
-    set_capturing(false);
-    cudaGraph_t graph = nullptr;
-    const cudaError_t ce = cudaStreamEndCapture(c.s, &graph);
-    if (st != GEDWALK_OK || ce != cudaSuccess || !graph) {
-      // Nothing captured has run. Another thread can invalidate a capture (a call that waits for
-      // the whole device, such as cudaFree); the sequence then runs directly, and a genuine error
-      // shows up again there.
-      if (graph) cudaGraphDestroy(graph);
-      cudaGetLastError();
-      sg.reset();
-      return issue_sweeps(c, mode, cols, true, nullptr, rev);
-    }
-    const cudaError_t ie = cudaGraphInstantiate(&sg.exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (ie != cudaSuccess) {
-      sg.exec = nullptr;
-      sg.reset();
-      return fail(GEDWALK_ERR_DEVICE, "graph instantiation failed: %s", cudaGetErrorString(ie));
-    }
-    sg.kernels = 1 + c.L + (sweep_sums(mode, cols) > 0 ? 2 : 0);
-    sg.sweeps = c.L;
-    sg.bytes = sweep_bytes(mode, fp64, cols, g.n, g.nnz, g.weighted);
-    sg.prof_key = (mode * 1000 + cols) * 2 + (fp64 ? 1 : 0);
-  }
-  GW_CUDA(cudaGraphLaunch(sg.exec, c.s));
-  count_launches(sg.kernels);
-  sg.timing_pending = profiling();
-  return GEDWALK_OK;
-}
-
-// After a synchronisation: hands the sweep timings of graph replays to the profiler.
-void read_graph_timing(Workspace& ws) {
-  for (SweepGraph& sg : ws.graphs) {
-    if (!sg.timing_pending) continue;
-    sg.timing_pending = false;
-    float ms = 0.0f;  // the run of sweeps, shared evenly among them
-    if (sg.ev.size() == 2 && cudaEventElapsedTime(&ms, sg.ev[0], sg.ev[1]) == cudaSuccess) {
-      for (int t = 0; t < sg.sweeps; ++t) profile_add(ms / sg.sweeps, sg.bytes, sg.prof_key);
-    } else {
-      cudaGetLastError();
-    }
-  }
+  auto bits = [](const void* p) { return static_cast<uint64_t>(reinterpret_cast<uintptr_t>(p)); };
+  Sequence q;
+  q.key = mix_all({uint64_t(mode), uint64_t(cols), uint64_t(fp64), uint64_t(c.L), uint64_t(g.n), uint64_t(rev), abits,
+                   bits(ws.ztab.p), bits(&g), bits(c.s), bits(ws.x0.p), bits(ws.x1.p), bits(ws.mtab.p), bits(ws.slots.p),
+                   bits(ws.parts.p), bits(ws.partial.p), bits(ws.counters.p), bits(ws.mask.p), bits(c.d_cand),
+                   bits(c.d_gains)});
+  q.kernels = 1 + c.L + (sweep_sums(mode, cols) > 0 ? 2 : 0);
+  q.sweeps = c.L;
+  q.bytes = sweep_bytes(mode, fp64, cols, g.n, g.nnz);
+  q.prof_key = (mode * 1000 + cols) * 2 + (fp64 ? 1 : 0);
+  return run_sequence(ws, c.s, q, [&](bool profile, const std::vector<cudaEvent_t>* ev) {
+    return issue_sweeps(c, mode, cols, profile, ev, rev);
+  });
 }
 
 // The stream a greedy run uses: the caller's, or (for the legacy default stream, which cannot
@@ -696,299 +402,38 @@ gedwalk_status greedy_stream(Workspace& ws, cudaStream_t caller, cudaStream_t* o
   return GEDWALK_OK;
 }
 
-// ---------------------------------------------------------------- device-resident greedy loop
-// The plain greedy with lookahead runs as one CUDA graph: an outer WHILE node over the k steps; in
-// each, a controller kernel either takes the next lookahead level (its table and its candidate's
-// exact gain are already there) or starts a new run (IF node: the L lookahead sweeps), then an
-// inner WHILE node repeats bound pass -> merge -> certification, with a candidate batch (IF node)
-// whenever the best exact value does not beat every unevaluated bound. The decisions the host loop
-// takes (certification, the next candidates, the speculative guesses, the lookahead level) are
-// taken by single-thread kernels on the same data, in the same order and with the same ties, so
-// the picks and gains are those of the host loop. A step that needs more than `max_batches`
-// candidate batches stops the loop with an error flag instead of running on.
-constexpr int kMaxEval = 64;  // exact values one step keeps (the largest, if more)
-
-struct DevCtl {
-  int32_t step, k, levels, L;
-  int32_t look_lvl, tab_level;  // the level the next step may take; the table this step reads
-  int32_t run_look, looping, run_cand, n_last;
-  int32_t first_batch, guessed, e_n, spec_n;
-  int32_t iso_next, batches_step, err, cols_cand;
-  int32_t look_c[8];
-  int32_t spec_v[8];
-  int32_t e_v[kMaxEval];
-  double look_g[8];
-  double spec_g[8];
-  double e_g[kMaxEval];
-  long long evals, batches, spec_miss, runs, cand_batches, iters;
-  unsigned long long t[3];  // device clock: interval start, lookahead-run sweeps, candidate-batch sweeps
-};
-
-__device__ __forceinline__ bool dev_in(const uint32_t* mask, int32_t v) { return (mask[v >> 5] >> (v & 31)) & 1u; }
-
-// Opens a step: the next lookahead level, or a new run whose guesses are the best remaining values
-// (at the first step without any, the highest-degree vertices outside S).
-__global__ void ctl_begin(DevCtl* __restrict__ c, Stale* __restrict__ stale, const uint32_t* __restrict__ mask,
-                          int32_t n, int32_t* __restrict__ cand, cudaGraphConditionalHandle h_run,
-                          cudaGraphConditionalHandle h_loop) {
-  if (threadIdx.x != 0) return;
-  c->e_n = 0;
-  c->first_batch = 1;
-  c->guessed = 0;
-  c->batches_step = 0;
-  c->n_last = 0;
-  c->looping = 1;
-  const int lvl = c->look_lvl;
-  if (lvl > 0 && lvl < c->levels && c->look_c[lvl] >= 0) {
-    const int32_t v = c->look_c[lvl];
-    c->tab_level = lvl;
-    Stale st;
-    st.ub = __double2float_ru(c->look_g[lvl]);
-    st.step = c->step;
-    stale[v] = st;
-    c->e_v[0] = v;
-    c->e_g[0] = c->look_g[lvl];
-    c->e_n = 1;
-    c->guessed = 1;
-    c->run_look = 0;
-  } else {
-    int m = 0;
-    for (int j = 0; j < c->spec_n && m < c->levels; ++j) cand[m++] = c->spec_v[j];
-    if (m == 0 && c->step == 0)
-      for (int32_t v = 0; v < n && m < c->levels; ++v)
-        if (!dev_in(mask, v)) cand[m++] = v;
-    for (int j = m; j < 16; ++j) cand[j] = -1;
-    for (int j = 0; j < c->levels; ++j) c->look_c[j] = cand[j];
-    c->look_lvl = 0;
-    c->tab_level = 0;
-    c->guessed = m > 0;
-    c->n_last = m > 0 ? 1 : 0;  // level 0's guess has its exact gain once the run is done
-    c->evals += m;
-    c->batches += m > 0;
-    c->runs += 1;
-    c->run_look = 1;
-  }
-  cudaGraphSetConditional(h_run, c->run_look ? 1u : 0u);
-  cudaGraphSetConditional(h_loop, 1u);
-}
-
-// After a run: the exact gains of every level's guess (each under S + the earlier guesses).
-__global__ void ctl_after_run(DevCtl* __restrict__ c, const double* __restrict__ gains) {
-  if (threadIdx.x < c->levels) c->look_g[threadIdx.x] = gains[threadIdx.x];
-}
-
-// Records the exact gains of the last evaluated candidates (as the stale bounds of this step and
-// in the step's list of exact values, which keeps the kMaxEval largest).
-__global__ void ctl_record(DevCtl* __restrict__ c, Stale* __restrict__ stale, const int32_t* __restrict__ cand,
-                           const double* __restrict__ gains, const int32_t* __restrict__ perm) {
-  if (threadIdx.x != 0) return;
-  for (int j = 0; j < c->n_last; ++j) {
-    const int32_t v = cand[j];
-    if (v < 0) continue;
-    Stale st;
-    st.ub = __double2float_ru(gains[j]);
-    st.step = c->step;
-    stale[v] = st;
-    if (c->e_n < kMaxEval) {
-      c->e_v[c->e_n] = v;
-      c->e_g[c->e_n] = gains[j];
-      ++c->e_n;
-    } else {  // replace the smallest exact value (never the best: certification needs only that)
-      int w = 0;
-      for (int i = 1; i < kMaxEval; ++i)
-        if (c->e_g[i] < c->e_g[w] || (c->e_g[i] == c->e_g[w] && perm[c->e_v[i]] > perm[c->e_v[w]])) w = i;
-      if (gains[j] > c->e_g[w]) {
-        c->e_v[w] = v;
-        c->e_g[w] = gains[j];
-      }
-    }
-  }
-  c->n_last = 0;
-}
-
-__device__ __forceinline__ bool cand_first(double ga, int32_t ca, double gb, int32_t cb) {
-  return ga > gb || (ga == gb && ca < cb);
-}
-
-// Certification after a bound pass: the best exact value wins once it beats every unevaluated
-// bound (inflated by tol); then the step's outputs, the vertex joins S, the next step's guesses and
-// lookahead level are set. Otherwise the best-bounded unevaluated vertices become a candidate batch.
-__global__ void ctl_certify(DevCtl* __restrict__ c, const SelOut* __restrict__ sel, uint32_t* __restrict__ mask,
-                            const int32_t* __restrict__ perm, int32_t n, int32_t* __restrict__ cand,
-                            int32_t* __restrict__ out_group, double* __restrict__ out_gains, double tol,
-                            int32_t max_batches, cudaGraphConditionalHandle h_loop,
-                            cudaGraphConditionalHandle h_cand) {
-  if (threadIdx.x != 0) return;
-  ++c->iters;
-  // the zero-gain candidate: the bound pass's, or the smallest isolated row outside S
-  unsigned long long z = sel->zero_min;
-  while (c->iso_next < n && dev_in(mask, c->iso_next)) ++c->iso_next;
-  if (c->iso_next < n) {
-    const unsigned long long iso =
-        (static_cast<unsigned long long>(perm[c->iso_next]) << 32) | static_cast<uint32_t>(c->iso_next);
-    if (iso < z) z = iso;
-  }
-  // the best exact value (larger gain first, then the lower caller id)
-  int32_t bv = -1, bc = INT_MAX;
-  double bg = -1.0;
-  for (int j = 0; j < c->e_n; ++j) {
-    const int32_t cc = perm[c->e_v[j]];
-    if (bv < 0 || cand_first(c->e_g[j], cc, bg, bc)) {
-      bv = c->e_v[j];
-      bc = cc;
-      bg = c->e_g[j];
-    }
-  }
-  if (z != kNoZero && (bv < 0 || cand_first(0.0, zero_caller(z), bg, bc))) {
-    bv = zero_internal(z);
-    bc = zero_caller(z);
-    bg = 0.0;
-  }
-  const bool top_empty = sel->id[0] == INT_MAX;
-  const double ub0 = top_empty ? -1.0 : static_cast<double>(sel->val[0]) * (1.0 + tol);
-  const bool certified = top_empty || (bv >= 0 && ub0 < bg);
-  if (certified) {
-    if (bv < 0) {  // no vertex left to add
-      c->err = 2;
-      c->looping = 0;
-      c->run_cand = 0;
-    } else {
-      out_group[c->step] = bc;
-      out_gains[c->step] = bg;
-      mask[bv >> 5] |= 1u << (bv & 31);
-      // the next run's guesses: the best remaining values, exact or bounds, positive only
-      int32_t pv[kMaxEval + kTopK];
-      double pg[kMaxEval + kTopK];
-      int np = 0;
-      for (int j = 0; j < c->e_n; ++j)
-        if (c->e_v[j] != bv) {
-          pv[np] = c->e_v[j];
-          pg[np++] = c->e_g[j];
-        }
-      for (int j = 0; j < kTopK; ++j)
-        if (sel->id[j] != INT_MAX && sel->id[j] != bv) {
-          pv[np] = sel->id[j];
-          pg[np++] = static_cast<double>(sel->val[j]);
-        }
-      int ns = 0;
-      while (ns < c->levels) {
-        int w = -1;
-        for (int j = 0; j < np; ++j) {
-          if (pv[j] < 0 || !(pg[j] > 0.0)) continue;
-          if (w < 0 || cand_first(pg[j], perm[pv[j]], pg[w], perm[pv[w]])) w = j;
-        }
-        if (w < 0) break;
-        c->spec_v[ns] = pv[w];
-        c->spec_g[ns++] = pg[w];
-        pv[w] = -1;
-      }
-      c->spec_n = ns;
-      const int lvl = c->look_lvl;
-      if (lvl >= 0 && bv == c->look_c[lvl] && lvl + 1 < c->levels && c->look_c[lvl + 1] >= 0) c->look_lvl = lvl + 1;
-      else c->look_lvl = -1;
-      ++c->step;
-      c->looping = 0;
-      c->run_cand = 0;
-    }
-  } else {
-    if (c->first_batch && c->guessed) ++c->spec_miss;
-    c->first_batch = 0;
-    int m = 0;
-    for (int j = 0; j < kTopK && m < c->cols_cand; ++j)
-      if (sel->id[j] != INT_MAX) cand[m++] = sel->id[j];
-    for (int j = m; j < 16; ++j) cand[j] = -1;
-    c->n_last = m;
-    c->evals += m;
-    c->batches += 1;
-    c->cand_batches += 1;
-    if (++c->batches_step > max_batches) {
-      c->err = 1;
-      c->looping = 0;
-      c->run_cand = 0;
-    } else {
-      c->looping = 1;
-      c->run_cand = 1;
-    }
-  }
-  cudaGraphSetConditional(h_loop, c->looping ? 1u : 0u);
-  cudaGraphSetConditional(h_cand, c->run_cand ? 1u : 0u);
-}
-
-__global__ void ctl_end(const DevCtl* __restrict__ c, cudaGraphConditionalHandle h_step) {
-  if (threadIdx.x == 0) cudaGraphSetConditional(h_step, (c->step < c->k && c->err == 0) ? 1u : 0u);
-}
-
-// Adds a conditional node (IF or WHILE, one body) at the current point of a capture on s.
-gedwalk_status add_conditional(cudaStream_t s, cudaGraphConditionalHandle h, cudaGraphConditionalNodeType type,
-                               cudaGraph_t* body) {
-  cudaStreamCaptureStatus st;
-  cudaGraph_t graph = nullptr;
-  const cudaGraphNode_t* deps = nullptr;
-  size_t nd = 0;
-  GW_CUDA(cudaStreamGetCaptureInfo(s, &st, nullptr, &graph, &deps, nullptr, &nd));
-  if (st != cudaStreamCaptureStatusActive) return fail(GEDWALK_ERR_DEVICE, "stream is not capturing");
-  cudaGraphNodeParams p{};
-  p.type = cudaGraphNodeTypeConditional;
-  p.conditional.handle = h;
-  p.conditional.type = type;
-  p.conditional.size = 1;
-  cudaGraphNode_t node;
-  GW_CUDA(cudaGraphAddNode(&node, graph, deps, nullptr, nd, &p));
-  GW_CUDA(cudaStreamUpdateCaptureDependencies(s, &node, nullptr, 1, cudaStreamSetCaptureDependencies));
-  *body = p.conditional.phGraph_out[0];
-  return GEDWALK_OK;
-}
-
-// Captures `fill` into `graph` on s (BeginCaptureToGraph); the capture ends whatever fill returns.
-template <class F>
-gedwalk_status capture_into(cudaStream_t s, cudaGraph_t graph, F&& fill) {
-  GW_CUDA(cudaStreamBeginCaptureToGraph(s, graph, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-  set_capturing(true);
-  const gedwalk_status st = fill();
-  set_capturing(false);
-  cudaGraph_t out = nullptr;
-  const cudaError_t ce = cudaStreamEndCapture(s, &out);
-  if (st != GEDWALK_OK) {
-    cudaGetLastError();
-    return st;
-  }
-  if (ce != cudaSuccess) return fail(GEDWALK_ERR_DEVICE, "capture of the greedy loop failed: %s", cudaGetErrorString(ce));
-  return GEDWALK_OK;
-}
-
 }  // namespace
 
 gedwalk_status greedy_shape(const Graph& g, const Resolved& r, int32_t flags, GreedyShape* out) {
   GreedyShape sh{};
   const bool adaptive = (flags & GEDWALK_ADAPTIVE_L) != 0;
-  // phi^miss + speculative candidates. Every gather costs one L2 sector whatever the row width,
-  // so narrow rows are cheapest; one speculative candidate certifies most steps (a miss costs one
-  // extra candidate batch). The adaptive variant certifies the best two exact gains (u and v of
-  // its separation test), so it speculates on three candidates.
-  sh.cols_fused = adaptive ? 4 : 2;
+  // One-step runs (directed graphs, lookahead off, spec_cols): phi^miss and the candidates likely to
+  // win. One certifies most steps (a miss costs one candidate batch); on a directed graph the
+  // adaptive variant certifies the best two exact gains, so it speculates on three.
+  sh.cols_fused = adaptive && g.directed ? 4 : 2;
   if (r.spec_cols != 0) {
     if (!(r.spec_cols == 2 || r.spec_cols == 4 || (r.spec_cols == 8 && !r.fp64)))
       return fail(GEDWALK_ERR_INVALID, "spec_cols must be 0, 2, 4 or (FP32) 8");
     sh.cols_fused = r.spec_cols;
   }
-  // Lookahead (plain greedy on an undirected graph): one run of sweeps carries `levels` steps,
-  // level d under S + {c_1..c_d} with the guessed winners c_d; a step whose winner was guessed
-  // needs no sweep of its own. The run's rows hold levels + 1 columns (phi^miss under S and one
-  // column per guess; every level's phi^miss is a difference of them). A gather costs one L2
-  // sector request whatever the row width up to 32 bytes, so 7 FP32 levels (3 FP64) cost little
-  // more per sweep than one.
+  // Lookahead (undirected graphs): one run carries `levels` steps, level d under S + {c_1..c_d} with
+  // the guessed winners c_d; a step whose winner was guessed needs no run of its own. The run's rows
+  // hold levels + 1 columns. A gather costs one L2 sector request whatever the row width up to 32
+  // bytes, so 7 FP32 levels (3 FP64) cost little more per sweep than one.
+  const bool plain = (flags & (GEDWALK_ADAPTIVE_L | GEDWALK_STOCHASTIC | GEDWALK_GAINS_ALL)) == 0;
   sh.levels = 1;
-  if (!(flags & (GEDWALK_ADAPTIVE_L | GEDWALK_STOCHASTIC | GEDWALK_GAINS_ALL)) && !g.directed) {
+  if (!g.directed && !(flags & GEDWALK_GAINS_ALL)) {
     sh.levels = r.fp64 ? 3 : 7;
-    if (r.lookahead != 0) {
+    if (plain && r.lookahead != 0) {
       if (!(r.lookahead == 1 || r.lookahead == 3 || (!r.fp64 && r.lookahead == 7)))
         return fail(GEDWALK_ERR_INVALID, "lookahead must be 0, 1, 3 or (FP32) 7");
       sh.levels = r.lookahead;
     }
+    if (!plain && r.spec_cols != 0) sh.levels = 1;  // the caller fixed the one-step width
   }
-  // Candidate batches run when the evaluated guess is not certified; the winner is nearly always
-  // among the best few bounds, and a narrower batch is a cheaper sweep.
-  sh.cols_cand = 4;
+  // Candidate batches run when the evaluated guess is not certified: as wide as one sector carries
+  // (undirected; directed batches hold no phi^miss column).
+  sh.cols_cand = g.directed || r.fp64 ? 4 : 8;
   sh.cols_all = r.fp64 ? 8 : 16;
   sh.ell_max = 1;
   while (adaptive && sh.ell_max < r.L) sh.ell_max *= 2;
@@ -999,302 +444,278 @@ gedwalk_status greedy_shape(const Graph& g, const Resolved& r, int32_t flags, Gr
   return GEDWALK_OK;
 }
 
-namespace {
-// GEDWALK_DEVICE_LOOP: the plain greedy with lookahead runs its k steps as one CUDA graph.
-bool uses_device_loop(const Graph& g, const GreedyShape& sh, int32_t flags, int32_t k) {
-  return (flags & GEDWALK_DEVICE_LOOP) && sh.levels > 1 &&
-         (flags & (GEDWALK_GAINS_ALL | GEDWALK_STOCHASTIC | GEDWALK_ADAPTIVE_L)) == 0 && !g.directed && k > 0 &&
-         g.plan.num_units > 0;
-}
-// Its controller block: the state, then the group and the gains of up to kcap steps.
-int32_t loop_kcap(int32_t k) {
-  int32_t kcap = 64;
-  while (kcap < k) kcap *= 2;
-  return kcap;
-}
-size_t loop_ctl_bytes(int32_t k) {
-  return (sizeof(DevCtl) + 255) / 256 * 256 + static_cast<size_t>(loop_kcap(k)) * (sizeof(double) + sizeof(int32_t)) +
-         256;
-}
-}  // namespace
-
 int64_t maximize_footprint(const Graph& g, const Resolved& r, int32_t flags, int32_t k) {
+  (void)k;
   GreedyShape sh{};
   if (greedy_shape(g, r, flags, &sh) != GEDWALK_OK) return 0;
   const int64_t n = g.n, es = r.fp64 ? 8 : 4;
-  const int64_t slices = std::max(std::max(g.plan.num_slices, g.directed ? g.plan_r.num_slices : 0), 1);
-  const int64_t heavy = std::max(std::max(g.plan.num_heavy, g.directed ? g.plan_r.num_heavy : 0), 1);
-  const int64_t slots = std::max(std::max(g.plan.num_slots, g.directed ? g.plan_r.num_slots : 0), 1);
+  if (!g.directed) {
+    int64_t b = run_bytes(g, sh.tab_L, sh.cols_max, r.fp64, (flags & GEDWALK_GAINS_ALL) == 0);
+    if (flags & GEDWALK_ADAPTIVE_L)  // the final group is scored at the full length
+      b += 2 * n * 2 * es + static_cast<int64_t>(std::max(g.plan.num_slots, 1)) * 2 * 8;
+    return b;
+  }
+  const int64_t slices = std::max(std::max(g.plan.num_slices, g.plan_r.num_slices), 1);
+  const int64_t heavy = std::max(std::max(g.plan.num_heavy, g.plan_r.num_heavy), 1);
+  const int64_t slots = std::max(std::max(g.plan.num_slots, g.plan_r.num_slots), 1);
   int64_t b = 0;
-  b += static_cast<int64_t>(sh.tab_L + 1) * n * es * sh.levels;  // phi^miss tables
-  if (g.directed) b += static_cast<int64_t>(sh.tab_L + 1) * n * es;  // psi^miss table
-  b += 2 * n * sh.cols_max * es;                                    // walk vectors x0, x1
+  b += 2 * static_cast<int64_t>(sh.tab_L + 1) * n * es;  // phi^miss and psi^miss tables
+  b += 2 * n * sh.cols_max * es;                         // walk vectors x0, x1
   b += slices * sh.cols_max * es + heavy * 4 + slots * sh.cols_max * 8 + sh.cols_max * kReduceParts * 8;
-  b += (n + 31) / 32 * 4;                                           // S bitmask
+  b += (n + 31) / 32 * 4;                                // S bitmask
   b += n * static_cast<int64_t>(sizeof(Stale)) + static_cast<int64_t>(kSelBlocks) * kTopK * 8;
   b += static_cast<int64_t>(sizeof(SelOut)) + 16 * 4 + 16 * 8 + 256;
-  if (uses_device_loop(g, sh, flags, k)) b += static_cast<int64_t>(loop_ctl_bytes(k));
   return b;
 }
 
 namespace {
+// What both loops need to know of a maximisation.
+struct GreedyRun {
+  int32_t k;
+  int32_t flags;
+  GreedyShape shape;
+  double tol;       // relative inflation of bounds against rounding
+  double eps_sep;   // adaptive: the separation
+  double coef;      // adaptive: B_l = coef * Wa[l] (Eq. comb-bound, or Lemma spectral-bound)
+  std::vector<double> Wa;
+  double sample_m;  // stochastic: about this many vertices outside S are sampled per step (Appendix D)
+  bool adaptive() const { return (flags & GEDWALK_ADAPTIVE_L) != 0; }
+  bool stochastic() const { return (flags & GEDWALK_STOCHASTIC) != 0; }
+  bool gains_all() const { return (flags & GEDWALK_GAINS_ALL) != 0; }
+  double bound_at(int32_t l) const { return coef * Wa[l]; }
+  // Step st's sample: vertex v (caller id) is drawn when hash(seed, st, v) < threshold, i.e. with
+  // probability p = m / |V \ S|; UINT64_MAX: all of V \ S.
+  uint64_t threshold(const Graph& g, int32_t st) const {
+    if (stochastic() && st < g.n) {
+      const double p = sample_m / static_cast<double>(g.n - st);
+      const double scaled = p * 18446744073709551616.0;
+      if (p < 1.0 && scaled < 18446744073709551615.0) return static_cast<uint64_t>(scaled);
+    }
+    return ~0ull;
+  }
+};
 
-uint64_t mix_all(std::initializer_list<uint64_t> vs) {
-  uint64_t key = 0;
-  for (uint64_t v : vs) key ^= v + 0x9e3779b97f4a7c15ULL + (key << 6) + (key >> 2);
-  return key;
-}
+// Isolated vertices (rows [n_active, n)) start and end no walk: their bound and gain are exactly
+// 0. The selections skip them, and the smallest caller id among those outside S stands for them
+// among the zero gains. Stochastic greedy scans them all: they belong to its samples. The
+// relabelling is a stable sort by degree, so the isolated rows hold increasing caller ids.
+struct Isolated {
+  int32_t next;
+  unsigned long long zero(const Graph& g, const std::vector<char>& inS, unsigned long long z) {
+    while (next < g.n && inS[next]) ++next;
+    if (next < g.n)
+      z = std::min(z, (static_cast<unsigned long long>(g.perm[next]) << 32) | static_cast<uint32_t>(next));
+    return z;
+  }
+};
 
-// Runs the k steps of the plain greedy with lookahead as one CUDA graph launch (the loop's graph is
-// built once per configuration of the workspace) and reads back the group and the gains.
-gedwalk_status run_device_loop(GreedyCtx& c, int32_t k, int levels, int cols_cand, int cols_max, size_t tab_elems,
-                               int nb_sel, int32_t n_scan, double tol, Stale* stale, float* sel_v, int* sel_id,
-                               int32_t* group, double* gains, bool* launched) {
-  *launched = false;
-  Graph& g = c.g;
-  Workspace& ws = c.ws;
-  const cudaStream_t s = c.s;
-  const bool fp64 = c.r.fp64;
-  const int32_t L = c.L;
-  // controller state, then the outputs for up to kcap steps
-  const int32_t kcap = loop_kcap(k);
-  const size_t ctl_bytes = (sizeof(DevCtl) + 255) / 256 * 256;
-  GW_TRY(ws.ctl.ensure(loop_ctl_bytes(k), s));
-  char* base = ws.ctl.as<char>();
-  DevCtl* dctl = reinterpret_cast<DevCtl*>(base);
-  double* d_ogains = reinterpret_cast<double*>(base + ctl_bytes);
-  int32_t* d_ogroup = reinterpret_cast<int32_t*>(d_ogains + kcap);
-  const int32_t* d_level = reinterpret_cast<const int32_t*>(base + offsetof(DevCtl, tab_level));
-  const int32_t* d_step = reinterpret_cast<const int32_t*>(base + offsetof(DevCtl, step));
-  void* d_stamp = base + offsetof(DevCtl, t);
-  // buffers the captured sweeps use, sized before the capture
-  const size_t es = fp64 ? 8 : 4;
-  GW_TRY(ws.x0.ensure(static_cast<size_t>(g.n) * cols_max * es, s));
-  GW_TRY(ws.x1.ensure(static_cast<size_t>(g.n) * cols_max * es, s));
-  GW_TRY(ensure_sweep_scratch(g, ws, cols_max, fp64, s));
-  GW_TRY(configure_sweep(MODE_LOOK, fp64, levels + 1));
-  GW_TRY(configure_sweep(MODE_CAND, fp64, cols_cand));
-  DevCtl h{};
-  h.k = k;
-  h.levels = levels;
-  h.L = L;
-  h.look_lvl = -1;
-  h.iso_next = n_scan;
-  h.cols_cand = cols_cand;
-  for (int j = 0; j < 8; ++j) h.look_c[j] = -1;
-  GW_CUDA(cudaMemcpyAsync(dctl, &h, sizeof h, cudaMemcpyHostToDevice, s));
-  const int32_t max_batches = n_scan / std::max(cols_cand, 1) + 64;
-  uint64_t abits;
-  memcpy(&abits, &c.r.alpha, 8);
-  uint64_t tbits;
-  memcpy(&tbits, &tol, 8);
-  const uint64_t key = mix_all(
-      {uint64_t(levels), uint64_t(cols_cand), uint64_t(fp64), uint64_t(L), uint64_t(g.n), uint64_t(kcap),
-       uint64_t(nb_sel), uint64_t(n_scan), abits, tbits, reinterpret_cast<uint64_t>(&g), reinterpret_cast<uint64_t>(s),
-       reinterpret_cast<uint64_t>(ws.x0.p), reinterpret_cast<uint64_t>(ws.x1.p), reinterpret_cast<uint64_t>(ws.mtab.p),
-       reinterpret_cast<uint64_t>(ws.slots.p), reinterpret_cast<uint64_t>(ws.parts.p),
-       reinterpret_cast<uint64_t>(ws.partial.p), reinterpret_cast<uint64_t>(ws.counters.p),
-       reinterpret_cast<uint64_t>(ws.mask.p), reinterpret_cast<uint64_t>(ws.stale.p),
-       reinterpret_cast<uint64_t>(ws.sel.p), reinterpret_cast<uint64_t>(ws.small.p),
-       reinterpret_cast<uint64_t>(ws.ctl.p)});
-  SweepGraph& sg = ws.greedy_loop;
-  if (sg.key != key || !sg.exec) {
-    sg.reset();
-    cudaGraph_t root = nullptr;
-    GW_CUDA(cudaGraphCreate(&root, 0));
-    struct Owner {
-      cudaGraph_t g;
-      ~Owner() {
-        if (g) cudaGraphDestroy(g);
+// The greedy loop of an undirected graph, on runs of half the walk length (run.cu).
+gedwalk_status maximize_runs(Graph& g, Workspace& ws, const Resolved& r, const GreedyRun& p,
+                             const std::vector<int32_t>& init, int32_t* group, double* gains,
+                             std::vector<int32_t>* S_all) {
+  const GreedyShape& sh = p.shape;
+  const bool chain = sh.levels > 1;
+  const int n_spec = chain ? sh.levels : sh.cols_fused - 1;
+  const bool select = !p.gains_all();
+  RunEngine eng(g, ws, r, r.stream);
+  eng.n_scan = p.stochastic() ? g.n : g.n_active;
+  GW_TRY(eng.setup(sh.tab_L, sh.cols_max, select, init));
+  GW_TRY(eng.set_length(p.adaptive() ? 1 : r.L, select));
+  std::vector<char> inS(g.n, 0);
+  for (int32_t v : init) inS[v] = 1;
+  *S_all = init;
+  Isolated iso{eng.n_scan};
+  auto draws = [&](int32_t step) {
+    eng.in->step = step;
+    eng.in->seed = r.seed;
+    for (int l = 0; l < kRunLevels; ++l) eng.in->thr[l] = p.threshold(g, step + l);
+  };
+  // Guesses from stored bounds: the best outside S, or per coming step the best of its sample.
+  auto guess = [&](int32_t step, std::vector<int32_t>* to) -> gedwalk_status {
+    draws(step);
+    GW_TRY(eng.guess(p.stochastic() ? n_spec : 1));
+    to->clear();
+    for (int l = 0; l < n_spec; ++l) {
+      const LevelSel& sel = eng.out->lv[p.stochastic() ? l : 0];
+      int32_t pick = -1;
+      for (int j = 0; j < kTopK && pick < 0; ++j)
+        if (sel.id[j] != INT_MAX && std::find(to->begin(), to->end(), sel.id[j]) == to->end()) pick = sel.id[j];
+      if (pick < 0) break;
+      to->push_back(pick);
+    }
+    return GEDWALK_OK;
+  };
+  std::vector<int32_t> spec;
+  if (select && p.k > 0) GW_TRY(guess(0, &spec));
+  RunOut look{};                // the last run's answers, and
+  std::vector<int32_t> look_c;  // its guesses
+  int lvl = -1;                 // its level that stands under the current S (-1: none)
+
+  for (int32_t step = 0; step < p.k; ++step) {
+    Cand best{-1.0, -1, INT_MAX};
+    if (p.gains_all()) {
+      const unsigned long long z = iso.zero(g, inS, kNoZero);  // isolated vertices gain nothing
+      if (z != kNoZero) best = Cand{0.0, zero_internal(z), zero_caller(z)};
+      std::vector<int32_t> batch;
+      for (int32_t v = 0; v <= g.n_active; ++v) {
+        if (v < g.n_active && !inS[v]) batch.push_back(v);
+        if (static_cast<int>(batch.size()) < sh.cols_all - 1 && !(v == g.n_active && !batch.empty())) continue;
+        GW_TRY(eng.run(false, sh.cols_all, false, batch));
+        for (size_t j = 0; j < batch.size(); ++j) {
+          Cand e{eng.out->gains[j], batch[j], g.perm[batch[j]]};
+          if (best.v < 0 || cand_before(e, best)) best = e;
+        }
+        ws.st_evals += static_cast<int64_t>(batch.size());
+        ++ws.st_batches;
+        batch.clear();
       }
-    } owner{root};
-    cudaGraphConditionalHandle h_step, h_run, h_loop, h_cand;
-    GW_CUDA(cudaGraphConditionalHandleCreate(&h_step, root, 1, cudaGraphCondAssignDefault));
-    cudaGraphNodeParams p{};
-    p.type = cudaGraphNodeTypeConditional;
-    p.conditional.handle = h_step;
-    p.conditional.type = cudaGraphCondTypeWhile;
-    p.conditional.size = 1;
-    cudaGraphNode_t n_step;
-    GW_CUDA(cudaGraphAddNode(&n_step, root, nullptr, nullptr, 0, &p));
-    cudaGraph_t body_step = p.conditional.phGraph_out[0];
-    GW_CUDA(cudaGraphConditionalHandleCreate(&h_run, body_step, 0, 0));
-    GW_CUDA(cudaGraphConditionalHandleCreate(&h_loop, body_step, 0, 0));
-    cudaGraph_t body_run = nullptr, body_loop = nullptr, body_cand = nullptr;
-    uint32_t* mask = ws.mask.as<uint32_t>();
-    const int32_t* perm = g.perm_d.as<int32_t>();
-    // step: open (level or run), the run, the certification loop, close
-    GW_TRY(capture_into(s, body_step, [&]() -> gedwalk_status {
-      ctl_begin<<<1, 32, 0, s>>>(dctl, stale, mask, g.n, c.d_cand, h_run, h_loop);
-      GW_CUDA(cudaGetLastError());
-      GW_TRY(add_conditional(s, h_run, cudaGraphCondTypeIf, &body_run));
-      GW_TRY(add_conditional(s, h_loop, cudaGraphCondTypeWhile, &body_loop));
-      ctl_end<<<1, 32, 0, s>>>(dctl, h_step);
-      GW_CUDA(cudaGetLastError());
-      return GEDWALK_OK;
-    }));
-    // the lookahead run: init, L sweeps (device-clock stamps around them), column sums, the gains
-    GW_TRY(capture_into(s, body_run, [&]() -> gedwalk_status {
-      c.tab_off = 0;
-      c.stamp_ctl = d_stamp;
-      c.stamp_end = 1;
-      const gedwalk_status st = issue_sweeps(c, MODE_LOOK, levels + 1, false, nullptr, false);
-      c.stamp_ctl = nullptr;
-      GW_TRY(st);
-      ctl_after_run<<<1, 32, 0, s>>>(dctl, c.d_gains);
-      GW_CUDA(cudaGetLastError());
-      return GEDWALK_OK;
-    }));
-    // one certification round: record the last gains, bound pass, merge, certify, maybe a batch
-    GW_CUDA(cudaGraphConditionalHandleCreate(&h_cand, body_loop, 0, 0));
-    GW_TRY(capture_into(s, body_loop, [&]() -> gedwalk_status {
-      ctl_record<<<1, 32, 0, s>>>(dctl, stale, c.d_cand, c.d_gains, perm);
-      GW_CUDA(cudaGetLastError());
-      reset_selection<<<1, 1, 0, s>>>(c.d_out);
-      GW_CUDA(cudaGetLastError());
-      const Sampling all{~0ull, 0, 0};
-      if (fp64)
-        GW_CUDA(launch_ub_select<double>(nb_sel, s, ws.mtab.as<double>(), ws.mtab.as<double>(), L, g.n, n_scan, mask,
-                                         stale, 0, perm, sel_v, sel_id, c.d_out, all, d_level,
-                                         static_cast<int64_t>(tab_elems), d_step));
-      else
-        GW_CUDA(launch_ub_select<float>(nb_sel, s, ws.mtab.as<float>(), ws.mtab.as<float>(), L, g.n, n_scan, mask,
-                                        stale, 0, perm, sel_v, sel_id, c.d_out, all, d_level,
-                                        static_cast<int64_t>(tab_elems), d_step));
-      ctl_certify<<<1, 32, 0, s>>>(dctl, c.d_out, mask, perm, g.n, c.d_cand, d_ogroup, d_ogains, tol, max_batches,
-                                   h_loop, h_cand);
-      GW_CUDA(cudaGetLastError());
-      return add_conditional(s, h_cand, cudaGraphCondTypeIf, &body_cand);
-    }));
-    // the candidate batch: candidate rows read the table of the step's level
-    GW_TRY(capture_into(s, body_cand, [&]() -> gedwalk_status {
-      c.tab_off = 0;
-      c.level_ptr = d_level;
-      c.level_stride = static_cast<int64_t>(tab_elems);
-      c.stamp_ctl = d_stamp;
-      c.stamp_end = 2;
-      const gedwalk_status st = issue_sweeps(c, MODE_CAND, cols_cand, false, nullptr, false);
-      c.stamp_ctl = nullptr;
-      c.level_ptr = nullptr;
-      c.level_stride = 0;
-      return st;
-    }));
-    GW_CUDA(cudaGraphInstantiate(&sg.exec, root, 0));
-    sg.key = key;
+    } else {
+      for (;;) {  // one attempt per walk length (a single attempt unless adaptive)
+        std::vector<Cand> E;  // evaluated with the current S
+        if (lvl < 0) {
+          look_c = spec;
+          look_c.resize(n_spec, -1);
+          draws(step);
+          GW_TRY(eng.run(chain, n_spec + 1, true, look_c));
+          look = *eng.out;
+          lvl = 0;
+          for (int32_t v : look_c) ws.st_evals += v >= 0;
+          ++ws.st_batches;
+        }
+        LevelSel sel = look.lv[lvl];
+        for (int j = chain ? lvl : 0; j < (chain ? lvl + 1 : n_spec); ++j)
+          if (look_c[j] >= 0) E.push_back(Cand{look.gains[j], look_c[j], g.perm[look_c[j]]});
+        const bool guessed = !E.empty();
+        bool everyone = false;  // an empty sample: all of V \ S competes
+        if (p.threshold(g, step) != ~0ull && sel.sampled == 0) {
+          everyone = true;
+          draws(step);
+          eng.in->thr[0] = ~0ull;
+          for (const Cand& e : E) eng.stale(e.v, e.g, step);
+          GW_TRY(eng.run(false, sh.cols_cand, true, {}));
+          sel = eng.out->lv[0];
+        }
+        bool first_batch = true, separated = true;
+        std::vector<Cand> X;  // exact values for the current S, best first
+        std::vector<int32_t> top;
+        const int32_t left = g.n - static_cast<int32_t>(S_all->size());
+        for (;;) {
+          // certify: the best exact value beats every bound not yet evaluated (a zero bound is an
+          // exact zero gain; the lowest such caller id stands for all of them)
+          top.clear();
+          for (int j = 0; j < kTopK; ++j)
+            if (sel.id[j] != INT_MAX) top.push_back(sel.id[j]);
+          X = E;
+          const unsigned long long z = iso.zero(g, inS, sel.zero_min);
+          if (z != kNoZero) X.push_back(Cand{0.0, zero_internal(z), zero_caller(z)});
+          std::sort(X.begin(), X.end(), cand_before);
+          const double ub0 = top.empty() ? -1.0 : static_cast<double>(sel.val[0]) * (1.0 + p.tol);
+          const bool u_ok = top.empty() || (!X.empty() && ub0 < X[0].g);
+          bool decided = u_ok;
+          if (p.adaptive()) {
+            // Separation test (Algorithm 2): u, the best, is taken when L(u) > L(v) + B_l - eps_sep,
+            // v the best of the rest (a zero gain where nothing else is left to evaluate). The test
+            // is monotone in L(u) and L(v), so bounds of them decide it wherever both of its
+            // outcomes agree; the last vertex outside S needs no v.
+            const double B = p.bound_at(eng.L);
+            auto test = [&](double gu, double gv) { return gu > (gv + B) - p.eps_sep; };
+            const double gu = X.empty() ? -1.0 : X[0].g;
+            const double v_lo = X.size() >= 2 ? X[1].g : 0.0, v_hi = std::max(v_lo, ub0);
+            if (left <= 1) {
+              separated = true;
+            } else if (!test(std::max(gu, ub0), 0.0)) {
+              separated = false;  // even the best possible gain is not separated
+              decided = true;
+            } else if (u_ok) {
+              separated = test(gu, v_hi);
+              decided = separated || !test(gu, v_lo);
+            }
+          }
+          if (decided) break;
+          if (first_batch) {
+            ws.st_spec_miss += guessed;
+            for (const Cand& e : E) eng.stale(e.v, e.g, step);
+          }
+          first_batch = false;
+          std::vector<int32_t> last(top.begin(), top.begin() + std::min<size_t>(top.size(), sh.cols_cand - 1));
+          draws(step);
+          if (everyone) eng.in->thr[0] = ~0ull;
+          GW_TRY(eng.run(false, sh.cols_cand, true, last));
+          for (size_t j = 0; j < last.size(); ++j) E.push_back(Cand{eng.out->gains[j], last[j], g.perm[last[j]]});
+          ws.st_evals += static_cast<int64_t>(last.size());
+          ++ws.st_batches;
+          sel = eng.out->lv[0];
+        }
+        best = X.empty() ? Cand{-1.0, -1, INT_MAX} : X[0];
+        // guesses for the next run: best remaining values, exact or not (a retry keeps the best too)
+        std::vector<Cand> pool(X.begin() + (X.empty() || !separated ? 0 : 1), X.end());
+        for (size_t j = 0; j < top.size(); ++j)
+          pool.push_back(Cand{static_cast<double>(sel.val[j]), top[j], g.perm[top[j]]});
+        std::sort(pool.begin(), pool.end(), cand_before);
+        spec.clear();
+        for (const Cand& e : pool)
+          if (static_cast<int>(spec.size()) < n_spec && e.g > 0.0) spec.push_back(e.v);
+        if (separated) break;
+        ++ws.st_sep_fail;
+        if (2 * eng.L > sh.ell_max)
+          return fail(GEDWALK_ERR_DEVICE, "walk length passed %d without separation", sh.ell_max);
+        // the bounds of the shorter length are no upper bounds for the longer one: reset them
+        GW_TRY(eng.set_length(2 * eng.L, true));
+        GW_CUDA(cudaMemsetAsync(ws.stale.p, 0xff, static_cast<size_t>(g.n) * sizeof(Stale), r.stream));
+        lvl = -1;
+      }
+      // the next level is valid only when this step took the vertex it assumed
+      if (chain && best.v == look_c[lvl] && lvl + 1 < sh.levels && look_c[lvl + 1] >= 0) ++lvl;
+      else lvl = -1;
+    }
+    if (best.v < 0) return fail(GEDWALK_ERR_INVALID, "no vertex left to add");
+    ws.st_ell.push_back(eng.L);
+    group[step] = best.caller;
+    gains[step] = best.g;
+    inS[best.v] = 1;
+    S_all->push_back(best.v);
+    eng.added.push_back(best.v);
+    if (best.g == 0.0 && !p.stochastic() && !p.adaptive()) {
+      // every remaining gain is 0 (submodularity): the lowest caller ids follow
+      int32_t caller = 0;
+      while (++step < p.k) {
+        while (inS[g.inv[caller]]) ++caller;
+        const int32_t v = g.inv[caller];
+        inS[v] = 1;
+        S_all->push_back(v);
+        ws.st_ell.push_back(eng.L);
+        group[step] = caller;
+        gains[step] = 0.0;
+      }
+      break;
+    }
+    if (p.stochastic() && lvl < 0 && step + 1 < p.k) GW_TRY(guess(step + 1, &spec));
   }
-  *launched = true;
-  GW_CUDA(cudaGraphLaunch(sg.exec, s));
-  DevCtl out{};
-  std::vector<double> og(k);
-  std::vector<int32_t> ogr(k);
-  GW_CUDA(cudaMemcpyAsync(&out, dctl, sizeof out, cudaMemcpyDeviceToHost, s));
-  GW_CUDA(cudaMemcpyAsync(og.data(), d_ogains, sizeof(double) * k, cudaMemcpyDeviceToHost, s));
-  GW_CUDA(cudaMemcpyAsync(ogr.data(), d_ogroup, sizeof(int32_t) * k, cudaMemcpyDeviceToHost, s));
-  GW_CUDA(cudaStreamSynchronize(s));
-  if (out.err == 2) return fail(GEDWALK_ERR_INVALID, "no vertex left to add");
-  if (out.err != 0 || out.step != k)
-    return fail(GEDWALK_ERR_DEVICE, "the greedy loop stopped at step %d of %d (certification exceeded %d batches)",
-                out.step, k, max_batches);
-  for (int32_t j = 0; j < k; ++j) {
-    group[j] = ogr[j];
-    if (gains) gains[j] = og[j];
-  }
-  ws.st_evals = out.evals;
-  ws.st_batches = out.batches;
-  ws.st_spec_miss = out.spec_miss;
-  ws.st_sweeps = (out.runs + out.cand_batches) * L;
-  ws.st_ell.assign(k, L);
-  // launches the graph ran: per step open/close, per run init + L sweeps + 2 stamps + 2 reduce +
-  // after_run, per certification round 4 kernels, per batch init + L sweeps + 2 stamps + 2 reduce
-  count_launches(static_cast<int>(2 * k + out.runs * (L + 6) + out.iters * 4 + out.cand_batches * (L + 5)));
-  if (profiling()) {  // the sweeps' device time, from the device-clock stamps around each run / batch
-    const double b_look = sweep_bytes(MODE_LOOK, fp64, levels + 1, g.n, g.nnz, g.weighted);
-    const double b_cand = sweep_bytes(MODE_CAND, fp64, cols_cand, g.n, g.nnz, g.weighted);
-    const int64_t n_look = out.runs * L, n_cand = out.cand_batches * L;
-    for (int64_t i = 0; i < n_look; ++i)
-      profile_add(static_cast<double>(out.t[1]) / 1e6 / n_look, b_look, (MODE_LOOK * 1000 + levels + 1) * 2 + fp64);
-    for (int64_t i = 0; i < n_cand; ++i)
-      profile_add(static_cast<double>(out.t[2]) / 1e6 / n_cand, b_cand, (MODE_CAND * 1000 + cols_cand) * 2 + fp64);
-  }
+  ws.st_sweeps = eng.sweeps;
   return GEDWALK_OK;
 }
 
-}  // namespace
-
-namespace {
-// Waits for a stream when a call leaves early with an error, so that nothing it launched still
-// runs when its buffers are reused or freed.
-struct SyncOnError {
-  cudaStream_t s = nullptr;
-  bool ok = false;
-  ~SyncOnError() {
-    if (!ok && s) {
-      cudaStreamSynchronize(s);
-      cudaGetLastError();
-    }
-  }
-};
-}  // namespace
-
-gedwalk_status maximize_impl(Graph& g, Workspace& ws, int32_t k, const Resolved& r_in, int32_t flags,
-                             const std::vector<int32_t>& init_int, int32_t* group, double* gains, double* score) {
-  Resolved r = r_in;
-  GW_TRY(greedy_stream(ws, r_in.stream, &r.stream));
-  SyncOnError guard{r.stream};
+// The greedy loop of a directed graph: one-step fused runs of the full length.
+gedwalk_status maximize_directed(Graph& g, Workspace& ws, const Resolved& r, const GreedyRun& p,
+                                 const std::vector<int32_t>& init_int, int32_t* group, double* gains,
+                                 std::vector<int32_t>* S_out) {
+  const int32_t k = p.k;
   cudaStream_t s = r.stream;
   const size_t es = r.fp64 ? 8 : 4;
-  const bool adaptive = (flags & GEDWALK_ADAPTIVE_L) != 0;
-  GreedyShape shape{};
-  GW_TRY(greedy_shape(g, r, flags, &shape));
-  const int cols_fused = shape.cols_fused;
-  const int levels = shape.levels;
-  const bool look = levels > 1;
-  const int n_spec = look ? levels : cols_fused - 1;
-  const int cols_cand = shape.cols_cand;
-  const int cols_all = shape.cols_all;
-  const double tol = r.fp64 ? 1e-11 : 1e-5;  // relative inflation of bounds against rounding
-  const bool gains_all = (flags & GEDWALK_GAINS_ALL) != 0;
-  const bool stochastic = (flags & GEDWALK_STOCHASTIC) != 0;
-  if (stochastic && (gains_all || !init_int.empty()))
-    return fail(GEDWALK_ERR_INVALID, "stochastic greedy cannot be combined with GEDWALK_GAINS_ALL or an init group");
-  if (stochastic && !(r.eta > 0.0 && r.eta < 1.0)) return fail(GEDWALK_ERR_INVALID, "eta must lie in (0, 1)");
-  if (adaptive && (gains_all || stochastic || !init_int.empty()))
-    return fail(GEDWALK_ERR_INVALID,
-                "GEDWALK_ADAPTIVE_L cannot be combined with GEDWALK_GAINS_ALL, GEDWALK_STOCHASTIC or an init group");
-  if (adaptive && !(r.eps > 0.0)) return fail(GEDWALK_ERR_INVALID, "GEDWALK_ADAPTIVE_L needs epsilon (L must be 0)");
-  // stochastic greedy: about m vertices outside S are sampled per step (Appendix D)
-  const double sample_m = std::ceil(static_cast<double>(g.n) / std::max(k, 1) * std::log(1.0 / (stochastic ? r.eta : 0.5)));
-  // adaptive: l runs through the powers of two from 1; B_l < eps_sep separates any pair, and r.L
-  // (the first l with B_l < eps_sep) bounds the largest power reached.
-  const double eps_sep = r.eps;
-  const int32_t ell_max = shape.ell_max;
-  const int32_t L = shape.tab_L;  // rows of the miss table
-  double coef = 0.0;  // B_l = coef * Wa_l (Eq. comb-bound, or Lemma spectral-bound)
-  std::vector<double> Wa;  // the walk totals this run needs, copied under the table's lock
-  if (adaptive) {
-    GW_TRY(bound_coef(g, r.alpha, r.bound_kind, s, &coef));
-    GW_TRY(ensure_totals(g, r.alpha, ell_max + 1, s));
-    std::shared_lock<std::shared_mutex> rl(g.tt_lock);
-    if (g.tt_alpha != r.alpha || g.tt_rows < ell_max + 1)
-      return fail(GEDWALK_ERR_INVALID, "the walk-total table was replaced for another alpha during the call");
-    Wa.assign(g.Wa.begin(), g.Wa.begin() + ell_max + 1);
-  }
-  auto bound_at = [&](int32_t l) { return coef * Wa[l]; };
-  ws.st_evals = ws.st_batches = ws.st_sweeps = ws.st_spec_miss = ws.st_sep_fail = 0;
-  ws.st_ell.clear();
-
-  const size_t tab_elems = static_cast<size_t>(L + 1) * g.n;  // one phi^miss table
-  GW_TRY(ws.mtab.ensure(tab_elems * levels * es, s));
-  for (int d = 0; d < levels; ++d) GW_TRY(zero_isolated_tail(g, ws.mtab.as<char>() + d * tab_elems * es, es, L, s));
-  if (g.directed) {
-    GW_TRY(ws.ztab.ensure(static_cast<size_t>(L + 1) * g.n * es, s));
-    GW_TRY(zero_isolated_tail(g, ws.ztab.p, es, L, s));
-  }
+  const bool adaptive = p.adaptive(), gains_all = p.gains_all(), stochastic = p.stochastic();
+  const int cols_fused = p.shape.cols_fused, cols_cand = p.shape.cols_cand, cols_all = p.shape.cols_all;
+  const int n_spec = cols_fused - 1;
+  const double tol = p.tol;
+  const int32_t ell_max = p.shape.ell_max;
+  const int32_t L = p.shape.tab_L;  // rows of the miss table
+  GW_TRY(ws.mtab.ensure(static_cast<size_t>(L + 1) * g.n * es, s));
+  GW_TRY(zero_isolated_tail(g, ws.mtab.p, es, L, s));
+  GW_TRY(ws.ztab.ensure(static_cast<size_t>(L + 1) * g.n * es, s));
+  GW_TRY(zero_isolated_tail(g, ws.ztab.p, es, L, s));
   GW_TRY(ws.stale.ensure(static_cast<size_t>(g.n) * sizeof(Stale), s));
   GW_TRY(ws.sel.ensure(static_cast<size_t>(kSelBlocks) * kTopK * 8, s));
   GW_TRY(ws.small.ensure(sizeof(SelOut) + 16 * sizeof(int32_t) + 16 * sizeof(double) + 256, s));
-  GW_TRY(ws.ensure_pinned(sizeof(SelOut) + 64 + 8 * sizeof(double)));
-  double* h_look = reinterpret_cast<double*>(static_cast<char*>(ws.pinned) + sizeof(SelOut) + 64);
+  GW_TRY(ws.ensure_pinned(sizeof(SelOut) + 64));
   GW_TRY(upload_mask(g, ws, init_int, s));
   GW_CUDA(cudaMemsetAsync(ws.stale.p, 0xff, static_cast<size_t>(g.n) * sizeof(Stale), s));  // step -1, ub NaN
 
@@ -1314,93 +735,32 @@ gedwalk_status maximize_impl(Graph& g, Workspace& ws, int32_t k, const Resolved&
     hmask[v >> 5] |= 1u << (v & 31);
     inS[v] = 1;
   }
-  std::vector<int32_t> S_all = init_int;
+  std::vector<int32_t>& S_all = *S_out;
+  S_all = init_int;
   std::vector<Cand> spec;  // next step's speculative candidates (internal ids)
-  int look_lvl = -1;                  // lookahead level of the next step (-1: none valid)
-  std::vector<int32_t> look_c;        // guessed winners c_1..c_levels of the last lookahead run
-  double look_g[8] = {0};             // their exact gains, each under S + {c_1..c_d}
-  // The step's sample: vertex v (caller id) is drawn when hash(seed, step, v) < thr, i.e. with
-  // probability p = m / |V \ S| (all of V \ S when p >= 1).
-  auto sampling_for = [&](int32_t st) {
-    Sampling smp{~0ull, r.seed, static_cast<uint32_t>(st)};
-    if (stochastic) {
-      const double p = sample_m / static_cast<double>(g.n - st);
-      const double scaled = p * 18446744073709551616.0;
-      if (p < 1.0 && scaled < 18446744073709551615.0) smp.thr = static_cast<uint64_t>(scaled);
-    }
-    return smp;
-  };
-  // Isolated vertices (rows [n_active, n)) start and end no walk: their bound and gain are exactly
-  // 0. The bound pass skips them, and the smallest caller id among those outside S stands for
-  // them among the zero gains. Stochastic greedy scans them all: they belong to its samples.
-  // The relabelling is a stable sort by degree, so the isolated rows hold increasing caller ids.
+  auto sampling_for = [&](int32_t st) { return Sampling{p.threshold(g, st), r.seed, static_cast<uint32_t>(st)}; };
   const int32_t n_scan = stochastic ? g.n : g.n_active;
-  int32_t iso_next = stochastic ? g.n : g.n_active;  // first isolated row not in S
+  Isolated iso{n_scan};
   const int nb_sel = sel_blocks(n_scan);
   // One bound + selection pass into c.d_out / c.h_out; `step` decides which stale gains are exact.
   auto select_pass = [&](int32_t st, const Sampling& smp) -> gedwalk_status {
     reset_selection<<<1, 1, 0, s>>>(c.d_out);
     GW_KCHECK();
     if (r.fp64)
-      GW_CUDA(launch_ub_select<double>(nb_sel, s, ws.mtab.as<double>() + c.tab_off,
-                                       g.directed ? ws.ztab.as<double>() : ws.mtab.as<double>() + c.tab_off, c.L, g.n,
-                                       n_scan, ws.mask.as<uint32_t>(), stale, st, g.perm_d.as<int32_t>(), sel_v,
-                                       sel_id, c.d_out, smp));
+      GW_CUDA(launch_ub_select<double>(nb_sel, s, ws.mtab.as<double>(), ws.ztab.as<double>(), c.L, g.n, n_scan,
+                                       ws.mask.as<uint32_t>(), stale, st, g.perm_d.as<int32_t>(), sel_v, sel_id, c.d_out,
+                                       smp));
     else
-      GW_CUDA(launch_ub_select<float>(nb_sel, s, ws.mtab.as<float>() + c.tab_off,
-                                      g.directed ? ws.ztab.as<float>() : ws.mtab.as<float>() + c.tab_off, c.L, g.n,
-                                      n_scan, ws.mask.as<uint32_t>(), stale, st, g.perm_d.as<int32_t>(), sel_v,
-                                      sel_id, c.d_out, smp));
+      GW_CUDA(launch_ub_select<float>(nb_sel, s, ws.mtab.as<float>(), ws.ztab.as<float>(), c.L, g.n, n_scan,
+                                      ws.mask.as<uint32_t>(), stale, st, g.perm_d.as<int32_t>(), sel_v, sel_id, c.d_out,
+                                      smp));
     count_launch();
     GW_CUDA(cudaMemcpyAsync(c.h_out, c.d_out, sizeof(SelOut), cudaMemcpyDeviceToHost, s));
     GW_CUDA(cudaStreamSynchronize(s));
     read_graph_timing(ws);
-    while (iso_next < g.n && inS[iso_next]) ++iso_next;
-    if (iso_next < g.n) {
-      const unsigned long long iso =
-          (static_cast<unsigned long long>(g.perm[iso_next]) << 32) | static_cast<uint32_t>(iso_next);
-      c.h_out->zero_min = std::min(c.h_out->zero_min, iso);
-    }
+    c.h_out->zero_min = iso.zero(g, inS, c.h_out->zero_min);
     return GEDWALK_OK;
   };
-
-  // The plain greedy with lookahead runs as one CUDA graph (device-resident loop); the others keep
-  // the host loop below.
-  // GED_{<=L} of the final group. From an empty start it is the sum of the picks' exact gains
-  // g_L(S_j, c_j) = GED_{<=L}(S_j + c_j) - GED_{<=L}(S_j), telescoping from GED_{<=L}(empty) = 0;
-  // otherwise (an init group, or gains at shorter walk lengths) two-state sweeps over the group.
-  auto group_score = [&](const std::vector<int32_t>& S_fin) -> gedwalk_status {
-    if (init_int.empty() && !adaptive && gains) {
-      double v = 0.0;
-      for (int32_t j = 0; j < k; ++j) v += gains[j];
-      *score = v;
-      return GEDWALK_OK;
-    }
-    double v = 0;
-    GW_TRY(score_one(g, ws, S_fin, r, &v));
-    *score = v;
-    return GEDWALK_OK;
-  };
-  bool device_loop = uses_device_loop(g, shape, flags, k);
-  if (device_loop) {
-    bool launched = false;
-    const gedwalk_status st = run_device_loop(c, k, levels, cols_cand, shape.cols_max, tab_elems, nb_sel, n_scan, tol,
-                                              stale, sel_v, sel_id, group, gains, &launched);
-    if (st != GEDWALK_OK && launched) return st;
-    if (st != GEDWALK_OK) {  // the loop's graph could not be built: the host loop below runs instead
-      cudaGetLastError();
-      ws.greedy_loop.reset();
-      device_loop = false;
-    }
-  }
-  if (device_loop) {
-    std::vector<int32_t> S_dev = init_int;
-    for (int32_t j = 0; j < k; ++j) S_dev.push_back(g.inv[group[j]]);
-    if (score) GW_TRY(group_score(S_dev));
-    GW_CUDA(cudaStreamSynchronize(s));
-    guard.ok = true;
-    return GEDWALK_OK;
-  }
 
   for (int32_t step = 0; step < k; ++step) {
     std::vector<Cand> E;  // evaluated with the current S
@@ -1428,48 +788,14 @@ gedwalk_status maximize_impl(Graph& g, Workspace& ws, int32_t k, const Resolved&
     } else {
       Sampling smp = sampling_for(step);
       for (;;) {  // one attempt per walk length (a single attempt unless adaptive)
-        // 1. fused sweeps: phi^miss under S plus the speculative candidates (on a directed graph
-        // first psi^miss, the walks of the other orientation, on the reverse CSR)
+        // 1. psi^miss on the reverse CSR, then fused sweeps: phi^miss under S plus the speculative
+        // candidates
         std::vector<int32_t> sc, last;
         E.clear();
-        bool look_run = false;
-        if (look && look_lvl > 0 && look_lvl < levels && look_c[look_lvl] >= 0) {
-          // the last winner was this level's predecessor: its table and its candidate's exact gain
-          // were computed with the current S
-          const int32_t cl = look_c[look_lvl];
-          c.tab_off = static_cast<size_t>(look_lvl) * tab_elems;
-          set_stale<<<1, 1, 0, s>>>(stale, cl, look_g[look_lvl], step, c.d_out->gains);
-          GW_KCHECK();
-          E.push_back(Cand{look_g[look_lvl], cl, g.perm[cl]});
-          sc.push_back(cl);
-        } else if (look && (!spec.empty() || step == 0)) {
-          if (spec.empty()) {
-            // the first step has no bounds yet: guess the highest-degree vertices outside S (new
-            // ids run by decreasing degree), GED-Walk's leading order for small alpha
-            for (int32_t v = 0; v < g.n && static_cast<int>(spec.size()) < levels; ++v)
-              if (!inS[v]) spec.push_back(Cand{0.0, v, g.perm[v]});
-          }
-          sc.assign(levels, -1);
-          for (size_t j = 0; j < spec.size() && j < static_cast<size_t>(levels); ++j) sc[j] = spec[j].v;
-          c.tab_off = 0;
-          GW_TRY(run_sweeps(c, MODE_LOOK, levels + 1, sc));
-          GW_CUDA(cudaMemcpyAsync(h_look, c.d_gains, sizeof(double) * levels, cudaMemcpyDeviceToHost, s));
-          look_lvl = 0;
-          look_c = sc;
-          look_run = true;
-          last.push_back(sc[0]);  // level 0's candidate is exact now; deeper levels wait for theirs
-          for (int32_t v : sc) ws.st_evals += v >= 0;
-          ++ws.st_batches;
-          sc.resize(1);
-        } else {
-          if (g.directed) GW_TRY(run_sweeps(c, MODE_FUSED, 1, {}, true));
-          for (const Cand& e : spec) sc.push_back(e.v);
-          const int cf = sc.empty() ? 1 : cols_fused;
-          c.tab_off = 0;
-          look_lvl = -1;
-          GW_TRY(run_sweeps(c, MODE_FUSED, cf, sc));
-          last = sc;
-        }
+        GW_TRY(run_sweeps(c, MODE_FUSED, 1, {}, true));
+        for (const Cand& e : spec) sc.push_back(e.v);
+        GW_TRY(run_sweeps(c, MODE_FUSED, sc.empty() ? 1 : cols_fused, sc));
+        last = sc;
         bool first_batch = true;
         std::vector<Cand> X;  // exact values for the current S, best first
         std::vector<int32_t> top;
@@ -1485,15 +811,9 @@ gedwalk_status maximize_impl(Graph& g, Workspace& ws, int32_t k, const Resolved&
             smp.thr = ~0ull;
             continue;
           }
-          if (look_run) {  // the gains of every level arrived with the first synchronisation
-            for (int d = 0; d < levels; ++d) look_g[d] = h_look[d];
-            look_run = false;
-            for (size_t j = 0; j < last.size(); ++j) E.push_back(Cand{c.h_out->gains[j], last[j], g.perm[last[j]]});
-          } else {
-            for (size_t j = 0; j < last.size(); ++j) E.push_back(Cand{c.h_out->gains[j], last[j], g.perm[last[j]]});
-            ws.st_evals += static_cast<int64_t>(last.size());
-            if (!last.empty()) ++ws.st_batches;
-          }
+          for (size_t j = 0; j < last.size(); ++j) E.push_back(Cand{c.h_out->gains[j], last[j], g.perm[last[j]]});
+          ws.st_evals += static_cast<int64_t>(last.size());
+          if (!last.empty()) ++ws.st_batches;
           // 3. certify: the first `need` exact values beat every bound not yet evaluated (a zero
           // bound is an exact zero gain; the lowest such caller id stands for all of them)
           top.clear();
@@ -1529,7 +849,7 @@ gedwalk_status maximize_impl(Graph& g, Workspace& ws, int32_t k, const Resolved&
         // zero gains; with u the last vertex outside S there is no v.
         const int32_t left = g.n - static_cast<int32_t>(S_all.size());
         const double gv = X.size() >= 2 ? X[1].g : 0.0;
-        if (left <= 1 || best.g > (gv + bound_at(c.L)) - eps_sep) break;
+        if (left <= 1 || best.g > (gv + p.bound_at(c.L)) - p.eps_sep) break;
         ++ws.st_sep_fail;
         if (2 * c.L > ell_max) return fail(GEDWALK_ERR_DEVICE, "walk length passed %d without separation", ell_max);
         c.L *= 2;
@@ -1543,15 +863,9 @@ gedwalk_status maximize_impl(Graph& g, Workspace& ws, int32_t k, const Resolved&
       }
     }
     ws.st_ell.push_back(c.L);
-    if (look) {  // the next level is valid only when this step took the vertex it assumed
-      if (look_lvl >= 0 && best.v == look_c[look_lvl] && look_lvl + 1 < levels && look_c[look_lvl + 1] >= 0)
-        ++look_lvl;
-      else
-        look_lvl = -1;
-    }
     if (best.v < 0) return fail(GEDWALK_ERR_INVALID, "no vertex left to add");
     group[step] = best.caller;
-    if (gains) gains[step] = best.g;
+    gains[step] = best.g;
     const int32_t w = best.v;
     inS[w] = 1;
     S_all.push_back(w);
@@ -1573,8 +887,73 @@ gedwalk_status maximize_impl(Graph& g, Workspace& ws, int32_t k, const Resolved&
     }
   }
   ws.st_sweeps = c.sweeps;
-  if (score) GW_TRY(group_score(S_all));
-  GW_CUDA(cudaStreamSynchronize(s));
+  return GEDWALK_OK;
+}
+
+// Waits for a stream when a call leaves early with an error, so that nothing it launched still
+// runs when its buffers are reused or freed.
+struct SyncOnError {
+  cudaStream_t s = nullptr;
+  bool ok = false;
+  ~SyncOnError() {
+    if (!ok && s) {
+      cudaStreamSynchronize(s);
+      cudaGetLastError();
+    }
+  }
+};
+}  // namespace
+
+gedwalk_status maximize_impl(Graph& g, Workspace& ws, int32_t k, const Resolved& r_in, int32_t flags,
+                             const std::vector<int32_t>& init_int, int32_t* group, double* gains, double* score) {
+  Resolved r = r_in;
+  GW_TRY(greedy_stream(ws, r_in.stream, &r.stream));
+  SyncOnError guard{r.stream};
+  GreedyRun p{};
+  p.k = k;
+  p.flags = flags;
+  GW_TRY(greedy_shape(g, r, flags, &p.shape));
+  // Rounding of the values a certification compares, beyond what the bounds themselves allow for. A
+  // run's first vector is exact counts and its sums are rounded a few times each (about 2e-7 in all,
+  // measured against 64 bits); the full-length sweeps of a directed graph round more often.
+  p.tol = r.fp64 ? 1e-11 : g.directed ? 1e-5 : 1e-6;
+  if (p.stochastic() && (p.gains_all() || !init_int.empty()))
+    return fail(GEDWALK_ERR_INVALID, "stochastic greedy cannot be combined with GEDWALK_GAINS_ALL or an init group");
+  if (p.stochastic() && !(r.eta > 0.0 && r.eta < 1.0)) return fail(GEDWALK_ERR_INVALID, "eta must lie in (0, 1)");
+  if (p.adaptive() && (p.gains_all() || p.stochastic() || !init_int.empty()))
+    return fail(GEDWALK_ERR_INVALID,
+                "GEDWALK_ADAPTIVE_L cannot be combined with GEDWALK_GAINS_ALL, GEDWALK_STOCHASTIC or an init group");
+  if (p.adaptive() && !(r.eps > 0.0)) return fail(GEDWALK_ERR_INVALID, "GEDWALK_ADAPTIVE_L needs epsilon (L must be 0)");
+  p.sample_m = std::ceil(static_cast<double>(g.n) / std::max(k, 1) * std::log(1.0 / (p.stochastic() ? r.eta : 0.5)));
+  // adaptive: l runs through the powers of two from 1; B_l < eps_sep separates any pair, and r.L
+  // (the first l with B_l < eps_sep) bounds the largest power reached.
+  p.eps_sep = r.eps;
+  if (p.adaptive()) {
+    GW_TRY(bound_coef(g, r.alpha, r.bound_kind, r.stream, &p.coef));
+    GW_TRY(ensure_totals(g, r.alpha, p.shape.ell_max + 1, r.stream));
+    std::shared_lock<std::shared_mutex> rl(g.tt_lock);
+    if (g.tt_alpha != r.alpha || g.tt_rows < p.shape.ell_max + 1)
+      return fail(GEDWALK_ERR_INVALID, "the walk-total table was replaced for another alpha during the call");
+    p.Wa.assign(g.Wa.begin(), g.Wa.begin() + p.shape.ell_max + 1);
+  }
+  ws.st_evals = ws.st_batches = ws.st_sweeps = ws.st_spec_miss = ws.st_sep_fail = 0;
+  ws.st_ell.clear();
+  std::vector<int32_t> S_all;
+  if (g.directed) GW_TRY(maximize_directed(g, ws, r, p, init_int, group, gains, &S_all));
+  else GW_TRY(maximize_runs(g, ws, r, p, init_int, group, gains, &S_all));
+  if (score) {
+    // GED_{<=L} of the final group. From an empty start it is the sum of the picks' exact gains
+    // g_L(S_j, c_j) = GED_{<=L}(S_j + c_j) - GED_{<=L}(S_j), telescoping from GED_{<=L}(empty) = 0;
+    // otherwise (an init group, or gains at shorter walk lengths) two-state sweeps over the group.
+    if (init_int.empty() && !p.adaptive()) {
+      double v = 0.0;
+      for (int32_t j = 0; j < k; ++j) v += gains[j];
+      *score = v;
+    } else {
+      GW_TRY(score_one(g, ws, S_all, r, score));
+    }
+  }
+  GW_CUDA(cudaStreamSynchronize(r.stream));
   guard.ok = true;
   return GEDWALK_OK;
 }
@@ -1587,6 +966,25 @@ gedwalk_status gains_impl(Graph& g, Workspace& ws, const std::vector<int32_t>& S
   cudaStream_t s = r.stream;
   const size_t es = r.fp64 ? 8 : 4;
   const int cols_all = r.fp64 ? 8 : 16;
+  std::vector<char> inS(g.n, 0);
+  for (int32_t v : S_int) inS[v] = 1;
+  for (int32_t v = 0; v < g.n; ++v) gains_caller[v] = 0.0;
+  std::vector<int32_t> batch;
+  if (!g.directed) {  // an isolated vertex gains nothing
+    RunEngine eng(g, ws, r, s);
+    GW_TRY(eng.setup(r.L, cols_all, false, S_int));
+    GW_TRY(eng.set_length(r.L, false));
+    for (int32_t v = 0; v <= g.n_active; ++v) {
+      if (v < g.n_active && !inS[v]) batch.push_back(v);
+      if (static_cast<int>(batch.size()) < cols_all - 1 && !(v == g.n_active && !batch.empty())) continue;
+      GW_TRY(eng.run(false, cols_all, false, batch));
+      for (size_t j = 0; j < batch.size(); ++j) gains_caller[g.perm[batch[j]]] = eng.out->gains[j];
+      batch.clear();
+    }
+    GW_CUDA(cudaStreamSynchronize(s));
+    guard.ok = true;
+    return GEDWALK_OK;
+  }
   GW_TRY(ws.mtab.ensure(static_cast<size_t>(r.L + 1) * g.n * es, s));
   GW_TRY(zero_isolated_tail(g, ws.mtab.p, es, r.L, s));
   GW_TRY(ws.small.ensure(sizeof(SelOut) + 16 * sizeof(int32_t) + 16 * sizeof(double) + 256, s));
@@ -1595,11 +993,7 @@ gedwalk_status gains_impl(Graph& g, Workspace& ws, const std::vector<int32_t>& S
   c.d_out = ws.small.as<SelOut>();
   c.d_cand = reinterpret_cast<int32_t*>(c.d_out + 1);
   c.d_gains = reinterpret_cast<double*>(c.d_cand + 16);
-  std::vector<char> inS(g.n, 0);
-  for (int32_t v : S_int) inS[v] = 1;
-  for (int32_t v = 0; v < g.n; ++v) gains_caller[v] = 0.0;
   GW_TRY(run_sweeps(c, MODE_FUSED, 1, {}));
-  std::vector<int32_t> batch;
   for (int32_t v = 0; v <= g.n; ++v) {
     if (v < g.n && !inS[v]) batch.push_back(v);
     if (static_cast<int>(batch.size()) == cols_all || (v == g.n && !batch.empty())) {

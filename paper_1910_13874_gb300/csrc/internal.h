@@ -135,7 +135,7 @@ struct SweepGraph {
 // creates one per concurrent request slot.
 struct Workspace {
   DevBuf x0, x1;     // walk vectors, [n][C]
-  DevBuf mtab;       // phi^miss table, [(L+1)][n]
+  DevBuf mtab;       // directed graphs: phi^miss table, [(L+1)][n]
   DevBuf ztab;       // directed graphs: psi^miss table (walks in the other orientation), [(L+1)][n]
   DevBuf pvec;       // power iteration: three FP64 vectors and the statistics
   DevBuf partial;    // heavy-slice partial sums, [num_slices][C]
@@ -147,7 +147,10 @@ struct Workspace {
   DevBuf sel;        // greedy: per-block candidate lists
   DevBuf small;      // small device-side results
   DevBuf members;    // batched scoring: member ids / group ids / accumulators
-  DevBuf pinned_dummy;
+  DevBuf xs;         // runs: the stored walk vectors x_1..x_H, each [n_active][C]
+  DevBuf cnt;        // runs: |N(v) cap S| per vertex
+  DevBuf tail;       // runs: bound of the walk pairs longer than the stored half, float[n]
+  DevBuf bound;      // runs: the last level's bounds, float[n]
   int64_t st_evals = 0, st_batches = 0, st_sweeps = 0, st_spec_miss = 0;  // last maximize
   std::vector<int32_t> st_ell;  // last maximize: the walk length of each step
   int64_t st_sep_fail = 0;      // last maximize: failed separation tests (l doublings)
@@ -156,11 +159,11 @@ struct Workspace {
   static constexpr int kGraphCache = 16;
   SweepGraph graphs[kGraphCache];
   uint64_t graph_clock = 0;
-  SweepGraph greedy_loop;  // the device-resident greedy loop of the last configuration
-  DevBuf ctl;              // its controller state and outputs
   cudaStream_t own_stream = nullptr;  // capturable stream used when the caller passes stream 0
   cudaEvent_t order_ev = nullptr;     // orders own_stream after the caller's stream
   std::vector<uint8_t> host_small;  // staging
+  void* run_io = nullptr;           // pinned block of the runs' copies: one size, kept while captured
+                                    // sequences refer to it
   void* pinned = nullptr;           // pinned host staging buffer
   size_t pinned_bytes = 0;
   ~Workspace();
@@ -237,10 +240,11 @@ struct Graph {
 enum SweepMode : int {
   MODE_TOTALS = 0,  // y = alpha A x, FP64, stores the column sum
   MODE_SCORE = 1,   // two-state hit/miss step, sums h
-  MODE_FUSED = 2,   // greedy: column 0 = phi^miss under S, columns 1.. candidate columns
-  MODE_CAND = 3,    // greedy: candidate columns only; candidate rows read phi^miss from a table
+  MODE_FUSED = 2,   // directed greedy: column 0 = phi^miss under S, columns 1.. candidate columns
+  MODE_CAND = 3,    // directed greedy: candidate columns only; candidate rows read phi^miss from a table
   MODE_PLAIN = 4,   // batched scoring: y = alpha A x, no mask
-  MODE_LOOK = 5     // greedy lookahead: phi^miss under S, then the walks through c_j avoiding S + {c_1..c_{j-1}}
+  MODE_LOOK = 5,    // run, chain: phi^miss under S, then the walks through c_j avoiding S + {c_1..c_{j-1}}
+  MODE_PAR = 6      // run: phi^miss under S, then the walks through each c_j avoiding S
 };
 
 struct SweepArgs {
@@ -260,19 +264,15 @@ struct SweepArgs {
   double* slots;
   int32_t accumulate;
   void* Mout;
-  int64_t mout_stride;  // MODE_LOOK: elements between the phi^miss tables of consecutive levels
   const void* Min;
   const int32_t* cand;
+  const int32_t* live;  // runs: whether candidate j has a neighbour outside its base set
   int32_t hub;  // rows [0, hub) of x are gathered with L1 retention priority (set by the launcher)
   // Vertex scales s of a weighted graph (nullptr: unweighted). Vectors are then gathered in the
   // scaled form x~ = s * x: (N x)(v) = s_v (A x~)(v) for N = diag(s) A diag(s), so the epilogue
   // computes the true value alpha s_v (A x~)(v), sums it, and stores it times s_v.
   const float* rs_f;
   const double* rs_d;
-  // MODE_CAND with the table chosen on the device: candidate rows read Min + level * level_stride
-  // (level read from level_ptr once per launch; nullptr: Min as given)
-  const int32_t* level_ptr;
-  int64_t level_stride;
 };
 
 // Profiling hooks around sweep launches (no-ops unless gedwalk_profile(1) was called).
@@ -289,9 +289,6 @@ void set_capturing(bool on);
 // and the phi^miss row where the mode reads or writes them.
 double sweep_bytes(int mode, bool fp64, int cols, int32_t n, int64_t nnz, bool weighted = false);
 
-// Sets a sweep instantiation's launch attributes on the current device (before a stream capture
-// that launches it; launch_sweep does it on first use otherwise).
-gedwalk_status configure_sweep(int mode, bool fp64, int cols);
 // Launches one sweep (instantiated for the supported (type, columns, mode) triples).
 gedwalk_status launch_sweep(int mode, bool fp64, int cols, const SweepArgs& a, cudaStream_t s, bool profile = true);
 // Column-sum count of a mode at width cols.
@@ -329,7 +326,7 @@ struct Resolved {
 struct GreedyShape {
   int32_t levels;     // lookahead levels per run of sweeps (1 = no lookahead)
   int32_t cols_fused; // columns of the fused sweep (phi^miss + speculative candidates)
-  int32_t cols_cand;  // columns of a candidate batch
+  int32_t cols_cand;  // columns of a candidate batch (undirected: phi^miss and the candidates)
   int32_t cols_all;   // columns per batch of GEDWALK_GAINS_ALL
   int32_t tab_L;      // rows 0..tab_L of every phi^miss table
   int32_t ell_max;    // adaptive: the largest walk length it may reach (else L)
@@ -344,6 +341,9 @@ int64_t score_batch_footprint(const Graph& g, int64_t members, int32_t groups);
 gedwalk_status resolve(Graph& g, const gedwalk_params* p, double eps_override, Resolved* r);
 // Ensures the FP64 walk-total table holds rows 0..rows-1 for alpha.
 gedwalk_status ensure_totals(Graph& g, double alpha, int32_t rows, cudaStream_t s);
+// Walk totals t_0..t_{rows-1} (FP64, rows g.n apart) into a table of the caller's, with the caller's
+// workspace (undirected graphs).
+gedwalk_status totals_into(Graph& g, Workspace& ws, double* T, double alpha, int32_t rows, cudaStream_t s);
 // Truncation length from the chosen tail bound (device-side test).
 gedwalk_status truncation_length(Graph& g, double alpha, double eps, int32_t* L, double* bound, cudaStream_t s,
                                  int32_t kind = 0);

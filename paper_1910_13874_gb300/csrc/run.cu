@@ -1,0 +1,894 @@
+// Runs of the greedy maximisation on an undirected graph: sweeps of half the walk length and the
+// pass in which the halves meet.
+//
+// With M = alpha 1_{V\S} A symmetric on V \ S, a walk of length a + b that avoids S is a walk of
+// length a and one of length b that end at the same vertex v (its vertex number a). So with
+// phi_t(v) the S-avoiding walks of length t that end at v, and k_t(v) those among them that visit
+// c, the walks of length a + b through c number
+//     sum_v [ k_a(v) phi_b(v) + (phi_a(v) - k_a(v)) k_b(v) ]
+// (the first half visits c, or it does not and the second half does). All terms are >= 0. The gain
+// of c sums the lengths 1..L; with H = ceil(L/2), the lengths up to H are plain sums of k_t and
+// every length H + a, a = 1..L-H, pairs with b = H:
+//     gain(c) = sum_v [ K(v) + V(v) phi_H(v) + (P(v) - V(v)) k_H(v) ],
+//     K = sum_{t=1..H} k_t,  V = sum_{t=1..L-H} k_t,  P = sum_{t=1..L-H} phi_t.
+// Half the sweeps, one pass over the stored vectors. Weighted graphs (symmetric weights) alike.
+//
+// The first sweep is no sweep either: phi_1(v) = alpha |N(v) \ S| is a count kept per vertex, and
+// k_1 is alpha on the candidate's neighbours. (Weighted graphs sweep from the unit vectors.)
+//
+// Bounds. The gain pairs first visits with continuations, sum_{1<=p+q<=L} f_p phi_q at c, where
+// f_p <= phi_p counts the walks whose only visit to c is their end: f_p = phi_p - sum_m s_m phi_{p-m}
+// with s_m the closed walks from c that return first at step m. Any lower bounds of s_m give an
+// upper bound of f: s_2 = alpha^2 |N(c) \ S| exactly, s_4 >= alpha^2 phi_2 - alpha^3 phi_1 (c-u-v-u-c,
+// v != c). With p, q <= H all pairs but (0,0) (and, for odd L, (H,H)) belong to the sum, so it is
+// F + U + F U with U = sum phi_t, F = sum f_t: no convolution. The pairs with p or q above H are
+// bounded once per maximisation by their value without S (walks avoiding S only get fewer as S
+// grows), from the walk-total table.
+//
+// Measured on a GB300 (one maximisation, before: full-length sweeps that store every level's phi, a
+// bound pass per step and the visits-times-continuations bound): R-MAT scale 22, k = 100, FP32 143.2
+// -> 40.9 ms (60 + 8 sweeps of 495 us instead of 135 of 587 and 54 of 498); Erdos-Renyi n = 100,003,
+// degree 16, k = 27 19.4 -> 2.3 ms (the sharper bound leaves one candidate batch); Barabasi-Albert
+// n = 10^6, k = 25, FP64 38.1 -> 12.4 ms; Algorithm 2 on R-MAT scale 20, k = 50 94.1 -> 11.1 ms.
+#include <algorithm>
+#include <cmath>
+
+#include "run.h"
+
+namespace gw {
+
+uint64_t mix_all(std::initializer_list<uint64_t> vs) {
+  uint64_t key = 0;
+  for (uint64_t v : vs) key ^= v + 0x9e3779b97f4a7c15ULL + (key << 6) + (key >> 2);
+  return key ? key : 1;  // 0 marks a free cache entry
+}
+
+gedwalk_status run_sequence(Workspace& ws, cudaStream_t s, const Sequence& q,
+                            const std::function<gedwalk_status(bool, const std::vector<cudaEvent_t>*)>& issue) {
+  if (s == nullptr) return issue(true, nullptr);
+  // the workspace's entry for this configuration, else the least recently used one
+  SweepGraph* hit = nullptr;
+  SweepGraph* lru = &ws.graphs[0];
+  for (SweepGraph& e : ws.graphs) {
+    if (e.key == q.key) hit = &e;
+    if (e.last_use < lru->last_use) lru = &e;
+  }
+  if (!hit) {
+    lru->reset();
+    lru->key = q.key;
+    hit = lru;
+  }
+  SweepGraph& sg = *hit;
+  sg.last_use = ++ws.graph_clock;
+  if (!sg.exec) {
+    if (sg.uses++ < 1) return issue(true, nullptr);  // set-up happens outside capture
+    sg.ev.assign(2, nullptr);
+    for (cudaEvent_t& e : sg.ev) GW_CUDA(cudaEventCreate(&e));
+    GW_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+    set_capturing(true);
+    const gedwalk_status st = issue(false, &sg.ev);
+    set_capturing(false);
+    cudaGraph_t graph = nullptr;
+    const cudaError_t ce = cudaStreamEndCapture(s, &graph);
+    if (st != GEDWALK_OK || ce != cudaSuccess || !graph) {
+      // Nothing captured has run. Another thread can invalidate a capture (a call that waits for
+      // the whole device, such as cudaFree); the sequence then runs directly, and a genuine error
+      // shows up again there.
+      if (graph) cudaGraphDestroy(graph);
+      cudaGetLastError();
+      sg.reset();
+      return issue(true, nullptr);
+    }
+    const cudaError_t ie = cudaGraphInstantiate(&sg.exec, graph, 0);
+    cudaGraphDestroy(graph);
+    if (ie != cudaSuccess) {
+      sg.exec = nullptr;
+      sg.reset();
+      return fail(GEDWALK_ERR_DEVICE, "graph instantiation failed: %s", cudaGetErrorString(ie));
+    }
+    sg.kernels = q.kernels;
+    sg.sweeps = q.sweeps;
+    sg.bytes = q.bytes;
+    sg.prof_key = q.prof_key;
+  }
+  GW_CUDA(cudaGraphLaunch(sg.exec, s));
+  count_launches(sg.kernels);
+  sg.timing_pending = profiling();
+  return GEDWALK_OK;
+}
+
+void read_graph_timing(Workspace& ws) {
+  for (SweepGraph& sg : ws.graphs) {
+    if (!sg.timing_pending) continue;
+    sg.timing_pending = false;
+    float ms = 0.0f;  // the run of sweeps, shared evenly among them
+    if (sg.sweeps > 0 && sg.ev.size() == 2 && cudaEventElapsedTime(&ms, sg.ev[0], sg.ev[1]) == cudaSuccess) {
+      for (int t = 0; t < sg.sweeps; ++t) profile_add(ms / sg.sweeps, sg.bytes, sg.prof_key);
+    } else {
+      cudaGetLastError();
+    }
+  }
+}
+
+namespace {
+
+constexpr int kChunks = 32;  // blocks that share one vertex's neighbours (hubs have 10^5)
+
+__device__ __forceinline__ bool in_set(const uint32_t* __restrict__ mask, int32_t v) {
+  return (__ldg(mask + (v >> 5)) >> (v & 31)) & 1u;
+}
+
+// S grows by list[0..count): the mask bits, and cnt[u] = |N(u) cap S| of every neighbour u.
+__device__ __forceinline__ void join_set(const int32_t* __restrict__ list, int32_t count,
+                                         const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                                         uint32_t* __restrict__ mask, int32_t* __restrict__ cnt) {
+  for (int32_t i = blockIdx.y; i < count; i += gridDim.y) {
+    const int32_t v = list[i];
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(mask + (v >> 5), 1u << (v & 31));
+    const int64_t e1 = rp[v + 1];
+    for (int64_t j = rp[v] + static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; j < e1;
+         j += static_cast<int64_t>(gridDim.x) * blockDim.x)
+      atomicAdd(cnt + ci[j], 1);
+  }
+}
+
+__global__ void join_kernel(const int32_t* __restrict__ list, int32_t count, const int32_t* __restrict__ rp,
+                            const int32_t* __restrict__ ci, uint32_t* __restrict__ mask, int32_t* __restrict__ cnt) {
+  join_set(list, count, rp, ci, mask, cnt);
+}
+
+// Opens a run: the vertices that joined S, the exact gains known on the host, the pass's counters.
+__global__ void run_begin(RunDev* __restrict__ d, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                          uint32_t* __restrict__ mask, int32_t* __restrict__ cnt, Stale* __restrict__ stale) {
+  if (blockIdx.x == 0 && blockIdx.y == 0) {
+    const int t = threadIdx.x;
+    if (t < kRunCols) d->adj[t] = 0;
+    if (t < kRunLevels) {
+      d->out.lv[t].zero_min = kNoZero;
+      d->out.lv[t].sampled = 0;
+    }
+    if (t == 0) {
+      d->done = 0;
+      if (stale)
+        for (int j = 0; j < d->in.n_stale; ++j)  // in order: a vertex may come twice
+          stale[d->in.stale_id[j]] = Stale{__double2float_ru(d->in.stale_gain[j]), d->in.stale_step[j]};
+    }
+  }
+  join_set(d->in.added, d->in.n_added, rp, ci, mask, cnt);
+}
+
+template <typename T>
+struct Chunk16;
+template <>
+struct Chunk16<float> {
+  using type = float4;
+  __device__ static float4 make(const float* e) { return make_float4(e[0], e[1], e[2], e[3]); }
+};
+template <>
+struct Chunk16<double> {
+  using type = double2;
+  __device__ static double2 make(const double* e) { return make_double2(e[0], e[1]); }
+};
+
+// The first stored vector of a run, rows [0, n_active). Unweighted: x_1, column 0 = alpha |N(v) \ S|
+// (0 on S), the candidate columns 0 (run_scatter fills them). Weighted (rs): x_0 scaled by s, column
+// 0 = s on V \ S, candidate column j = s at the candidate. 16 bytes per thread, consecutive.
+template <typename T, int C>
+__global__ void run_init(T* __restrict__ X, const RunDev* __restrict__ d, const int32_t* __restrict__ rp,
+                         const int32_t* __restrict__ cnt, const uint32_t* __restrict__ mask, int32_t n_active, T alpha,
+                         const T* __restrict__ rs) {
+  constexpr int per = 16 / static_cast<int>(sizeof(T)) < C ? 16 / static_cast<int>(sizeof(T)) : C;
+  constexpr int cpr = C / per;  // chunks per row
+  const int64_t chunks = static_cast<int64_t>(n_active) * cpr;
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  for (int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; q < chunks; q += stride) {
+    const int32_t v = static_cast<int32_t>(q / cpr);
+    const int part = static_cast<int>(q % cpr);
+    T e[per];
+#pragma unroll
+    for (int j = 0; j < per; ++j) e[j] = T(0);
+    if (rs) {
+      const T sv = rs[v];
+      if (part == 0 && !in_set(mask, v)) e[0] = sv;
+#pragma unroll
+      for (int j = 0; j < per; ++j) {
+        const int col = part * per + j;
+        if (col > 0 && __ldg(&d->in.cand[col - 1]) == v) e[j] = sv;
+      }
+    } else if (part == 0 && !in_set(mask, v)) {
+      e[0] = alpha * static_cast<T>(rp[v + 1] - rp[v] - cnt[v]);
+    }
+    if constexpr (per * sizeof(T) == 16) {
+      reinterpret_cast<typename Chunk16<T>::type*>(X)[q] = Chunk16<T>::make(e);
+    } else {
+#pragma unroll
+      for (int j = 0; j < per; ++j) X[q * per + j] = e[j];
+    }
+  }
+}
+
+// Unweighted x_1 of the candidate columns: alpha on the neighbours outside the column's base set
+// (S, with the earlier candidates in a chain), and, for a chain, the number of earlier candidates
+// next to each candidate. Weighted graphs take only the counts.
+template <typename T, bool CHAIN>
+__global__ void run_scatter(T* __restrict__ X, int cols, RunDev* __restrict__ d, const int32_t* __restrict__ rp,
+                            const int32_t* __restrict__ ci, const uint32_t* __restrict__ mask, T alpha, int write) {
+  __shared__ int sc[kRunCols];
+  if (threadIdx.x < kRunCols) sc[threadIdx.x] = d->in.cand[threadIdx.x];
+  __syncthreads();
+  const int j = blockIdx.y;
+  const int32_t c = sc[j];
+  if (c < 0) return;
+  const int64_t e1 = rp[c + 1];
+  for (int64_t e = rp[c] + static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < e1;
+       e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+    const int32_t v = ci[e];
+    bool base = false;
+    if (CHAIN)
+      for (int i = 0; i < j; ++i) base |= sc[i] == v;
+    if (base) atomicAdd(&d->adj[j], 1);
+    else if (write && !in_set(mask, v)) X[static_cast<size_t>(v) * cols + j + 1] = alpha;
+  }
+}
+
+// The candidates' own rows: live[j] says whether c_j has a neighbour outside its base set; x_1 there
+// is phi_1 under that set.
+template <typename T, bool CHAIN>
+__global__ void run_own(T* __restrict__ X, int cols, RunDev* __restrict__ d, const int32_t* __restrict__ rp,
+                        const int32_t* __restrict__ cnt, T alpha, int write) {
+  const int j = threadIdx.x;
+  if (j >= kRunCols) return;
+  const int32_t c = j < cols - 1 ? d->in.cand[j] : -1;
+  int32_t dg = 0;
+  if (c >= 0) {
+    dg = rp[c + 1] - rp[c] - cnt[c] - (CHAIN ? d->adj[j] : 0);
+    if (write) X[static_cast<size_t>(c) * cols + j + 1] = alpha * static_cast<T>(dg);
+  }
+  d->live[j] = dg > 0;
+}
+
+// Tail bounds from the walk-total table t_0..t_L (FP64, rows n apart; times s on a weighted graph):
+//   tail(v) = sum over pairs p + q <= L with p or q above H of t_p t_q = 2 sum_{a>H} t_a Q_{L-a},
+//   Q_q = t_0 + ... + t_q,
+// rounded up; and (about) the bound of the empty group, F + U + F U + tail, for the first guesses.
+__global__ void tail_kernel(const double* __restrict__ T, int64_t n, int32_t n_active, int32_t L, int32_t H,
+                            const double* __restrict__ rs, double alpha, float* __restrict__ tail,
+                            float* __restrict__ bound) {
+  for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n_active; v += gridDim.x * blockDim.x) {
+    const double inv = rs ? 1.0 / rs[v] : 1.0;
+    double Q = 0.0, acc = 0.0;
+    for (int32_t q = 0; q < L - H; ++q) {
+      Q += T[static_cast<size_t>(q) * n + v] * inv;
+      acc += T[static_cast<size_t>(L - q) * n + v] * inv * Q;
+    }
+    double U = 0.0;
+    for (int32_t t = 1; t <= H; ++t) U += T[static_cast<size_t>(t) * n + v] * inv;
+    acc *= 2.0 * (1.0 + 1e-12);
+    tail[v] = __double2float_ru(acc);
+    const double f1 = T[n + v] * inv, f2 = H >= 2 ? T[2 * n + v] * inv : 0.0;
+    const double s2 = rs ? 0.0 : alpha * f1, s4 = rs || H < 4 ? 0.0 : alpha * alpha * f2 - alpha * alpha * alpha * f1;
+    const double F = U - (H >= 2 ? (s2 + s4) * (1.0 + U) : 0.0);
+    bound[v] = static_cast<float>(F + U + F * U + acc);
+  }
+}
+
+struct MeetArgs {
+  const void* xs;      // x_1 .. x_H, each [n_active][C]
+  int64_t stride;      // elements from x_t to x_{t+1}
+  int32_t L, H;
+  int32_t n_scan, n_active;
+  const int32_t* rp;
+  const int32_t* cnt;
+  const uint32_t* mask;
+  const int32_t* perm;
+  const float* tail;
+  float* bound;        // the last level's bounds
+  Stale* stale;
+  const float* rs_f;
+  const double* rs_d;
+  double alpha;
+  double* part;        // [block][C - 1] gain sums
+  float* sel_v;        // [level][block][kTopK]
+  int* sel_id;
+  RunDev* d;
+};
+
+template <typename T>
+__device__ __forceinline__ float f_up(T x) {
+  if constexpr (sizeof(T) == 8) return __double2float_ru(x);
+  else return x;
+}
+template <typename T>
+__device__ __forceinline__ float f_down(T x) {
+  if constexpr (sizeof(T) == 8) return __double2float_rd(x);
+  else return x;
+}
+template <typename T>
+__device__ __forceinline__ T pos(T x) {
+  return x > T(0) ? x : T(0);
+}
+
+// Merges the block lists of one level on one warp: the kTopK best heads, then the entries of their
+// blocks (any other block's head has kTopK better entries ahead of it).
+__device__ __forceinline__ void merge_level(const float* __restrict__ sel_v, const int* __restrict__ sel_id, int blocks,
+                                            LevelSel* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  WarpList h;
+  for (int b0 = 0; b0 < blocks; b0 += 32) {
+    const int blk = b0 + lane;
+    const bool ok = blk < blocks;
+    const float x = ok ? __ldcg(sel_v + static_cast<size_t>(blk) * kTopK) : -1.0f;
+    const int ix = ok ? __ldcg(sel_id + static_cast<size_t>(blk) * kTopK) : INT_MAX;
+    warp_list_offer(h, ix != INT_MAX, x, ix, blk);
+  }
+  WarpList f;
+#pragma unroll
+  for (int j = 0; j < kTopK; j += 2) {
+    const int src = j + (lane >> 4);
+    const int tag = __shfl_sync(kFullMask, h.tag, src);
+    const int hid = __shfl_sync(kFullMask, h.id, src);
+    const size_t e = static_cast<size_t>(hid != INT_MAX ? tag : 0) * kTopK + (lane & 15);
+    const float x = hid != INT_MAX ? __ldcg(sel_v + e) : -1.0f;
+    const int ix = hid != INT_MAX ? __ldcg(sel_id + e) : INT_MAX;
+    warp_list_offer(f, ix != INT_MAX, x, ix, 0);
+  }
+  if (lane < kTopK) {
+    out->val[lane] = f.v;
+    out->id[lane] = f.id;
+  }
+}
+
+// A block's lists (one per warp and level) to sel_v / sel_id: warp l merges level l.
+template <int NL>
+__device__ __forceinline__ void block_levels(WarpList (&w)[NL], float* sv, int* si, float* __restrict__ sel_v,
+                                             int* __restrict__ sel_id) {
+  constexpr int NW = kThreads / 32;
+  static_assert(NL <= NW, "one warp per level");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int l = 0; l < NL; ++l)
+    if (lane < kTopK) {
+      sv[(l * NW + warp) * kTopK + lane] = w[l].v;
+      si[(l * NW + warp) * kTopK + lane] = w[l].id;
+    }
+  __syncthreads();
+  if (warp < NL) {
+    WarpList f;
+#pragma unroll
+    for (int j = 0; j < NW; j += 2) {
+      const int e = (warp * NW + j + (lane >> 4)) * kTopK + (lane & 15);
+      warp_list_offer(f, si[e] != INT_MAX, sv[e], si[e], 0);
+    }
+    if (lane < kTopK) {
+      const size_t o = (static_cast<size_t>(warp) * gridDim.x + blockIdx.x) * kTopK + lane;
+      sel_v[o] = f.v;
+      sel_id[o] = f.id;
+    }
+  }
+}
+
+// The meeting pass: one thread per row adds up the row's stored vectors x_1..x_H (coalesced, each
+// read once) and forms the candidates' gain terms and, with SEL, every level's bound; the best
+// kTopK unevaluated vertices of each level go to out->lv. In a chain level d stands under
+// T_d = S + {c_1..c_d}, phi(T_d) = column 0 - columns 1..d (a walk that avoids S avoids c_1..c_d or
+// has a first c_j among them, counted in column j); differences are clamped at 0, and a vertex
+// without a neighbour outside T_d (an exact count) has bound exactly 0. The last block to finish
+// merges the lists and adds the gain sums in block order. Bound by the H rows it streams.
+template <typename T, int C, bool CHAIN, bool SEL>
+__global__ void __launch_bounds__(kThreads, 2) meet_kernel(const MeetArgs a) {
+  constexpr int D = C - 1;
+  constexpr int NL = CHAIN ? D : 1;
+  constexpr int NW = kThreads / 32;
+  __shared__ int s_cand[D];
+  __shared__ float sv[SEL ? NL * NW * kTopK : 1];
+  __shared__ int si[SEL ? NL * NW * kTopK : 1];
+  __shared__ double sg[NW][D];
+  __shared__ int is_last;
+  const RunIn& in = a.d->in;
+  if (threadIdx.x < D) s_cand[threadIdx.x] = in.cand[threadIdx.x];
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int H = a.H;
+  const bool odd = (a.L & 1) != 0;
+  const T* __restrict__ xs = static_cast<const T*>(a.xs);
+  const T* __restrict__ rs = sizeof(T) == 8 ? reinterpret_cast<const T*>(a.rs_d) : reinterpret_cast<const T*>(a.rs_f);
+  // directed rounding keeps a bound above that of the stored vectors; e covers the vectors' own
+  // rounding where differences of columns cancel, keep the returns' where they reduce f
+  constexpr float e = sizeof(T) == 8 ? 1e-15f : 2.5e-7f;
+  constexpr float keep = 1.0f - 2e-6f;
+  const float infl = __fadd_ru(1.0f, __fmul_ru(static_cast<float>(H), 1.2e-7f));
+  const float al2 = __double2float_rd(a.alpha * a.alpha), al3 = __double2float_ru(a.alpha * a.alpha * a.alpha);
+  const int step = in.step;
+  bool sampling = false;
+  if (SEL) {
+#pragma unroll
+    for (int l = 0; l < NL; ++l) sampling |= in.thr[l] != ~0ull;
+  }
+  ColAcc<T, D> acc;
+  acc.zero();
+  WarpList w[NL];
+  int nsampled[NL];
+#pragma unroll
+  for (int l = 0; l < NL; ++l) nsampled[l] = 0;
+  const int32_t stride = gridDim.x * kThreads;
+  for (int32_t base = blockIdx.x * kThreads + warp * 32; base < a.n_scan; base += stride) {
+    const int32_t v = base + lane;
+    const bool ok = v < a.n_scan;
+    const bool has = v < a.n_active;
+    // sums over t: B to H-1, A2 to H-2, A4 to H-4; x_1, x_2 and x_H
+    T B[C], A2[C], A4[C], f1[C], f2[C], xh[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) B[c] = A2[c] = A4[c] = f1[c] = f2[c] = xh[c] = T(0);
+    if (has) {
+      const T* p = xs + static_cast<size_t>(v) * C;
+#pragma unroll 2
+      for (int t = 1; t <= H; ++t, p += a.stride) {
+        T x[C];
+        if constexpr (sizeof(T) * C >= 16) {
+#pragma unroll
+          for (int k = 0; k < static_cast<int>(sizeof(T)) * C / 16; ++k) {
+            const float4 q = __ldcs(reinterpret_cast<const float4*>(p) + k);
+            memcpy(&x[k * (16 / static_cast<int>(sizeof(T)))], &q, 16);
+          }
+        } else {
+#pragma unroll
+          for (int c = 0; c < C; ++c) x[c] = __ldcs(p + c);
+        }
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          if (SEL) {
+            if (t <= H - 4) A4[c] += x[c];
+            if (t <= H - 2) A2[c] += x[c];
+            if (t == 1) f1[c] = x[c];
+            if (t == 2) f2[c] = x[c];
+          }
+          if (t < H) B[c] += x[c];
+          else xh[c] = x[c];
+        }
+      }
+      if (rs) {
+        const T inv = T(1) / rs[v];
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          B[c] *= inv;
+          xh[c] *= inv;
+          if (SEL) {
+            A2[c] *= inv;
+            A4[c] *= inv;
+            f1[c] *= inv;
+            f2[c] *= inv;
+          }
+        }
+      }
+    }
+    // running values of the level's phi: sums to H and to L - H, x_H, and what the bound needs
+    T rh = xh[0], rb = B[0];
+    T r2 = A2[0], r4 = A4[0], q1 = f1[0], q2 = f2[0];
+    bool out = false;
+    int dg = 0;
+    float tail = 0.0f;
+    Stale st{0.0f, -1};
+    uint32_t caller = 0;
+    if (SEL && ok) {
+      out = in_set(a.mask, v);
+      if (has) {
+        dg = a.rp[v + 1] - a.rp[v] - a.cnt[v];
+        tail = a.tail[v];
+      }
+      st = a.stale[v];
+      if (sampling) caller = static_cast<uint32_t>(__ldg(a.perm + v));
+    }
+    const float slack_u = __fmul_ru(e, f_up(B[0] + xh[0])), slack_2 = e * f_up(A2[0]), slack_4 = e * f_up(A4[0]);
+    const float slack_1 = e * f_up(f1[0]), slack_q = e * f_up(f2[0]), slack_h = e * f_up(xh[0]);
+    bool evaluated = false;
+    if (SEL && !CHAIN) {
+#pragma unroll
+      for (int j = 0; j < D; ++j) evaluated |= s_cand[j] == v;
+    }
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      if (SEL && d < NL) {
+        float ub = 0.0f;
+        if (dg > 0) {
+          const float U = __fmaf_ru(f_up(pos(rb + rh)), infl, slack_u);
+          const float p1lo = fmaxf(0.0f, __fsub_rd(f_down(pos(q1)), slack_1));
+          float s2, s4 = 0.0f;
+          if (rs) {  // Cauchy-Schwarz: sum of squared weights >= (their sum)^2 / their number
+            s2 = __fdiv_rd(__fmul_rd(p1lo, p1lo), static_cast<float>(dg));
+          } else {
+            s2 = __fmul_rd(al2, static_cast<float>(dg));
+            const float p2lo = fmaxf(0.0f, __fsub_rd(f_down(pos(q2)), slack_q));
+            const float p1up = __fadd_ru(f_up(pos(q1)), slack_1);
+            s4 = fmaxf(0.0f, __fsub_rd(__fmul_rd(al2, p2lo), __fmul_ru(al3, p1up)));
+          }
+          float corr = 0.0f;
+          if (H >= 2) corr = __fmul_rd(s2, __fadd_rd(1.0f, fmaxf(0.0f, __fsub_rd(f_down(pos(r2)), slack_2))));
+          if (H >= 4)
+            corr = __fadd_rd(corr, __fmul_rd(s4, __fadd_rd(1.0f, fmaxf(0.0f, __fsub_rd(f_down(pos(r4)), slack_4)))));
+          corr = __fmul_rd(corr, keep);
+          const float F = fmaxf(0.0f, __fsub_ru(U, corr));
+          ub = __fadd_ru(__fmaf_ru(F, U, __fadd_ru(F, U)), tail);
+          if (odd) {  // the pair (H, H) is longer than L
+            const float hlo = fmaxf(0.0f, __fsub_rd(f_down(pos(rh)), slack_h));
+            ub = __fsub_ru(ub, __fmul_rd(hlo, fmaxf(0.0f, __fsub_rd(hlo, corr))));
+          }
+          if (!(ub >= 0.0f)) ub = INFINITY;  // overflow: nothing is known
+          if (st.step >= 0 && st.ub < ub) ub = st.ub;
+        }
+        if (d == NL - 1 && ok && a.bound) a.bound[v] = ub;
+        bool want = ok && !out;
+        if (want && in.thr[d] != ~0ull) want = sample_hash(in.seed, static_cast<uint32_t>(step + d), caller) < in.thr[d];
+        nsampled[d] += want;
+        want = want && st.step != step + d && !(CHAIN ? s_cand[d] == v : evaluated);
+        if (want && ub == 0.0f)
+          atomicMin(&a.d->out.lv[d].zero_min,
+                    (static_cast<unsigned long long>(__ldg(a.perm + v)) << 32) | static_cast<uint32_t>(v));
+        warp_list_offer(w[d], want && ub != 0.0f, ub, v, 0);
+      }
+      // gain terms of candidate d + 1 under the level's set
+      const T k = B[d + 1] + xh[d + 1];
+      const T vv = odd ? B[d + 1] : k;
+      const T pp = odd ? pos(rb) : pos(rb + rh);
+      acc.add(d, k + vv * pos(rh) + pos(pp - vv) * xh[d + 1]);
+      if (CHAIN) {
+        rb -= B[d + 1];
+        rh -= xh[d + 1];
+        if (SEL) {
+          r2 -= A2[d + 1];
+          r4 -= A4[d + 1];
+          q1 -= f1[d + 1];
+          q2 -= f2[d + 1];
+          dg -= f1[d + 1] > T(0);
+          out |= s_cand[d] == v;
+        }
+      }
+    }
+  }
+  // gain sums of the block
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    double x = acc.get(d);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFullMask, x, o);
+    if (lane == 0) sg[warp][d] = x;
+  }
+  if (SEL) {
+    if (sampling) {
+#pragma unroll
+      for (int l = 0; l < NL; ++l) {
+        int x = nsampled[l];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFullMask, x, o);
+        if (lane == 0 && x) atomicAdd(&a.d->out.lv[l].sampled, x);
+      }
+    }
+    block_levels<NL>(w, sv, si, a.sel_v, a.sel_id);
+  }
+  __syncthreads();
+  if (threadIdx.x < D) {
+    double x = 0.0;
+    for (int i = 0; i < NW; ++i) x += sg[i][threadIdx.x];
+    a.part[static_cast<size_t>(blockIdx.x) * D + threadIdx.x] = x;
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) is_last = atomicAdd(&a.d->done, 1) == static_cast<int>(gridDim.x) - 1;
+  __syncthreads();
+  if (!is_last) return;
+  __threadfence();
+  const int blocks = static_cast<int>(gridDim.x);
+  if (SEL) {
+    if (warp < NL)
+      merge_level(a.sel_v + static_cast<size_t>(warp) * blocks * kTopK, a.sel_id + static_cast<size_t>(warp) * blocks * kTopK,
+                  blocks, &a.d->out.lv[warp]);
+  }
+  for (int d = warp; d < D; d += NW) {
+    double x = 0.0;
+    for (int b = lane; b < blocks; b += 32) x += __ldcg(a.part + static_cast<size_t>(b) * D + d);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFullMask, x, o);
+    if (lane == 0) {
+      a.d->out.gains[d] = x;
+      // exact under S (a chain's deeper levels stand under larger sets: no bound yet)
+      if (SEL && s_cand[d] >= 0 && (!CHAIN || d == 0)) a.stale[s_cand[d]] = Stale{__double2float_ru(x), step};
+    }
+  }
+}
+
+// Selections of kRunLevels steps' samples (or, without sampling, one of all) from stored bounds: a
+// choice of guesses, so the bounds may belong to an earlier set.
+__global__ void __launch_bounds__(kThreads) guess_kernel(const float* __restrict__ bound, int32_t n_scan, int32_t n_active,
+                                                         const uint32_t* __restrict__ mask,
+                                                         const int32_t* __restrict__ perm, int levels,
+                                                         float* __restrict__ sel_v, int* __restrict__ sel_id,
+                                                         RunDev* __restrict__ d) {
+  constexpr int NW = kThreads / 32;
+  __shared__ float sv[kRunLevels * NW * kTopK];
+  __shared__ int si[kRunLevels * NW * kTopK];
+  __shared__ int is_last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  WarpList w[kRunLevels];
+  const int32_t stride = gridDim.x * kThreads;
+  for (int32_t base = blockIdx.x * kThreads + warp * 32; base < n_scan; base += stride) {
+    const int32_t v = base + lane;
+    const bool live = v < n_scan && v < n_active && !in_set(mask, v);
+    const float b = live ? bound[v] : 0.0f;
+    const uint32_t caller = live ? static_cast<uint32_t>(__ldg(perm + v)) : 0u;
+#pragma unroll
+    for (int l = 0; l < kRunLevels; ++l) {
+      if (l >= levels) break;
+      bool want = live && b > 0.0f;
+      if (want && d->in.thr[l] != ~0ull)
+        want = sample_hash(d->in.seed, static_cast<uint32_t>(d->in.step + l), caller) < d->in.thr[l];
+      warp_list_offer(w[l], want, b, v, 0);
+    }
+  }
+  block_levels<kRunLevels>(w, sv, si, sel_v, sel_id);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) is_last = atomicAdd(&d->done, 1) == static_cast<int>(gridDim.x) - 1;
+  __syncthreads();
+  if (!is_last) return;
+  __threadfence();
+  const int blocks = static_cast<int>(gridDim.x);
+  if (warp < kRunLevels)
+    merge_level(sel_v + static_cast<size_t>(warp) * blocks * kTopK, sel_id + static_cast<size_t>(warp) * blocks * kTopK, blocks,
+                &d->out.lv[warp]);
+}
+
+int grid_of(int64_t n) { return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 16))); }
+int meet_grid(int32_t n_scan) {
+  return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(kMeetBlocks, (int64_t(n_scan) + kThreads - 1) / kThreads)));
+}
+
+template <typename T, int C>
+cudaError_t launch_init(cudaStream_t s, T* X, RunDev* d, const Graph& g, const Workspace& ws, bool chain, double alpha) {
+  const T* rs = !g.weighted ? nullptr : sizeof(T) == 8 ? static_cast<const T*>(g.rs_d.p) : static_cast<const T*>(g.rs_f.p);
+  const int32_t* rp = g.rp.as<int32_t>();
+  const int32_t* ci = g.ci.as<int32_t>();
+  const int32_t* cnt = ws.cnt.as<int32_t>();
+  const uint32_t* mask = ws.mask.as<uint32_t>();
+  const T al = static_cast<T>(alpha);
+  const int write = g.weighted ? 0 : 1;
+  run_init<T, C><<<grid_of(static_cast<int64_t>(g.n_active) * C * sizeof(T) / 16), 256, 0, s>>>(X, d, rp, cnt, mask,
+                                                                                              g.n_active, al, rs);
+  if (chain) {
+    run_scatter<T, true><<<dim3(kChunks, C - 1), 256, 0, s>>>(X, C, d, rp, ci, mask, al, write);
+    run_own<T, true><<<1, 32, 0, s>>>(X, C, d, rp, cnt, al, write);
+  } else {
+    if (write) run_scatter<T, false><<<dim3(kChunks, C - 1), 256, 0, s>>>(X, C, d, rp, ci, mask, al, write);
+    run_own<T, false><<<1, 32, 0, s>>>(X, C, d, rp, cnt, al, write);
+  }
+  return cudaGetLastError();
+}
+
+template <typename T, int C, bool CHAIN, bool SEL>
+cudaError_t launch_meet(cudaStream_t s, const MeetArgs& a) {
+  meet_kernel<T, C, CHAIN, SEL><<<meet_grid(a.n_scan), kThreads, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+int64_t run_bytes(const Graph& g, int32_t L_max, int cols, bool fp64, bool select) {
+  const int64_t n = g.n, H = (L_max + 1) / 2, es = fp64 ? 8 : 4;
+  int64_t b = std::max<int64_t>(static_cast<int64_t>(g.n_active) * H * cols * es, 16);  // x_1 .. x_H (x_0: weighted)
+  if (g.weighted) b += static_cast<int64_t>(g.n_active) * cols * es;
+  b += n * 4 + (n + 31) / 32 * 4;                           // |N(v) cap S|, S bitmask
+  b += static_cast<int64_t>(kMeetBlocks) * (cols - 1) * 8;  // gain sums
+  b += static_cast<int64_t>(sizeof(RunDev)) + 256;
+  if (select) b += n * (4 + 4 + static_cast<int64_t>(sizeof(Stale))) + static_cast<int64_t>(kMeetBlocks) * kRunLevels * kTopK * 8;
+  const int64_t es_p = es;
+  b += static_cast<int64_t>(std::max(g.plan.num_slices, 1)) * cols * es_p + std::max(g.plan.num_heavy, 1) * 4;
+  return b;
+}
+
+gedwalk_status RunEngine::setup(int32_t L_max, int cols, bool select, const std::vector<int32_t>& init) {
+  const size_t n = static_cast<size_t>(g.n), H_max = static_cast<size_t>((L_max + 1) / 2), es = r.fp64 ? 8 : 4;
+  const size_t row = static_cast<size_t>(g.n_active) * cols * es;
+  GW_TRY(ws.xs.ensure(row * (H_max + (g.weighted ? 1 : 0)), s));
+  GW_TRY(ws.cnt.ensure(n * sizeof(int32_t), s));
+  const size_t words = (n + 31) / 32;
+  GW_TRY(ws.mask.ensure(words * 4, s));
+  GW_TRY(ws.parts.ensure(static_cast<size_t>(kMeetBlocks) * (cols - 1) * sizeof(double), s));
+  GW_TRY(ws.small.ensure(sizeof(RunDev) + 256, s));
+  // the captured sequences copy from and to this block: it must outlive them at one address (a
+  // pinned block freed and made again at the same address is another allocation to the driver)
+  if (!ws.run_io && cudaMallocHost(&ws.run_io, sizeof(RunOut) + sizeof(RunIn)) != cudaSuccess) {
+    cudaGetLastError();
+    ws.run_io = nullptr;
+    return fail(GEDWALK_ERR_OOM, "pinned host allocation of %zu bytes failed", sizeof(RunOut) + sizeof(RunIn));
+  }
+  out = static_cast<RunOut*>(ws.run_io);
+  in = reinterpret_cast<RunIn*>(out + 1);
+  memset(in, 0, sizeof *in);
+  for (uint64_t& t : in->thr) t = ~0ull;
+  GW_TRY(ws.partial.ensure(static_cast<size_t>(std::max(g.plan.num_slices, 1)) * cols * es, s));
+  const size_t cbytes = static_cast<size_t>(std::max(g.plan.num_heavy, 1)) * sizeof(unsigned);
+  if (ws.counters.bytes < cbytes || !ws.counters.p) GW_TRY(ws.counters.ensure(cbytes, s, /*zero=*/true));
+  if (select) {
+    GW_TRY(ws.stale.ensure(n * sizeof(Stale), s));
+    GW_TRY(ws.sel.ensure(static_cast<size_t>(kMeetBlocks) * kRunLevels * kTopK * 8, s));
+    GW_TRY(ws.tail.ensure(n * sizeof(float), s));
+    GW_TRY(ws.bound.ensure(n * sizeof(float), s));
+    GW_CUDA(cudaMemsetAsync(ws.stale.p, 0xff, n * sizeof(Stale), s));  // step -1
+  }
+  GW_CUDA(cudaMemsetAsync(ws.cnt.p, 0, n * sizeof(int32_t), s));
+  GW_CUDA(cudaMemsetAsync(ws.mask.p, 0, words * 4, s));
+  if (!init.empty()) {
+    DevBuf& list = ws.members;
+    GW_TRY(list.ensure(init.size() * sizeof(int32_t), s));
+    GW_TRY(ws.ensure_pinned(init.size() * sizeof(int32_t)));
+    int32_t* st = static_cast<int32_t*>(ws.pinned);
+    std::copy(init.begin(), init.end(), st);
+    GW_CUDA(cudaMemcpyAsync(list.p, st, init.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+    const int items = static_cast<int>(std::min<size_t>(init.size(), 4096));
+    join_kernel<<<dim3(kChunks, items), 256, 0, s>>>(list.as<int32_t>(), static_cast<int32_t>(init.size()),
+                                                     g.rp.as<int32_t>(), g.ci.as<int32_t>(), ws.mask.as<uint32_t>(),
+                                                     ws.cnt.as<int32_t>());
+    GW_KCHECK();
+  }
+  return GEDWALK_OK;
+}
+
+gedwalk_status RunEngine::set_length(int32_t length, bool select) {
+  L = length;
+  H = (L + 1) / 2;
+  if (!select || g.n_active == 0) return GEDWALK_OK;
+  // tail bounds from the walk totals; the table is read under its lock, to the end of the kernel
+  const double* rs = g.weighted ? g.rs_d.as<double>() : nullptr;
+  {
+    std::shared_lock<std::shared_mutex> rl(g.tt_lock);
+    if (g.tt_alpha == r.alpha && g.tt_rows >= L + 1) {
+      tail_kernel<<<grid_of(g.n_active), 256, 0, s>>>(g.ttab.as<double>(), g.n, g.n_active, L, H, rs, r.alpha, ws.tail.as<float>(),
+                                                      ws.bound.as<float>());
+      GW_KCHECK();
+      GW_CUDA(cudaStreamSynchronize(s));
+      return GEDWALK_OK;
+    }
+  }
+  // no table for this alpha (a forced L beyond the bound's reach): totals of this call's own
+  const size_t n = static_cast<size_t>(g.n);
+  GW_TRY(ws.ztab.ensure(static_cast<size_t>(L + 1) * n * sizeof(double), s));
+  GW_TRY(totals_into(g, ws, ws.ztab.as<double>(), r.alpha, L + 1, s));
+  tail_kernel<<<grid_of(g.n_active), 256, 0, s>>>(ws.ztab.as<double>(), g.n, g.n_active, L, H, rs, r.alpha, ws.tail.as<float>(),
+                                                  ws.bound.as<float>());
+  GW_KCHECK();
+  return GEDWALK_OK;
+}
+
+void RunEngine::stale(int32_t v, double gain, int32_t step) {
+  if (in->n_stale == kRunCols) return;  // a bound the passes then do without
+  in->stale_id[in->n_stale] = v;
+  in->stale_gain[in->n_stale] = gain;
+  in->stale_step[in->n_stale++] = step;
+}
+
+// More joined vertices than a run carries go ahead of it.
+gedwalk_status RunEngine::push_added() {
+  RunDev* d = ws.small.as<RunDev>();
+  while (added.size() > kRunCols) {
+    std::copy(added.end() - kRunCols, added.end(), in->added);
+    GW_CUDA(cudaMemcpyAsync(d->in.added, in->added, sizeof in->added, cudaMemcpyHostToDevice, s));
+    join_kernel<<<dim3(kChunks, kRunCols), 256, 0, s>>>(d->in.added, kRunCols, g.rp.as<int32_t>(), g.ci.as<int32_t>(),
+                                                        ws.mask.as<uint32_t>(), ws.cnt.as<int32_t>());
+    GW_KCHECK();
+    GW_CUDA(cudaStreamSynchronize(s));  // the pinned block is reused
+    added.resize(added.size() - kRunCols);
+  }
+  in->n_added = static_cast<int32_t>(added.size());
+  std::copy(added.begin(), added.end(), in->added);
+  added.clear();
+  return GEDWALK_OK;
+}
+
+gedwalk_status RunEngine::issue(bool chain, int cols, bool select, bool profile, const std::vector<cudaEvent_t>* ev) {
+  RunDev* d = ws.small.as<RunDev>();
+  const bool fp64 = r.fp64;
+  const size_t es = fp64 ? 8 : 4;
+  const size_t row = static_cast<size_t>(g.n_active) * cols;
+  GW_CUDA(cudaMemcpyAsync(&d->in, in, sizeof(RunIn), cudaMemcpyHostToDevice, s));
+  run_begin<<<dim3(kChunks, kRunCols), 256, 0, s>>>(d, g.rp.as<int32_t>(), g.ci.as<int32_t>(), ws.mask.as<uint32_t>(),
+                                                    ws.cnt.as<int32_t>(), select ? ws.stale.as<Stale>() : nullptr);
+  GW_KCHECK();
+  // x_1 .. x_H; a weighted graph starts one sweep earlier, from x_0 behind them
+  char* xs = ws.xs.as<char>();
+  char* x0 = g.weighted ? xs + row * es * H : xs;
+#define GW_RUN(T, C) \
+  if (fp64 == (sizeof(T) == 8) && cols == C) GW_CUDA((launch_init<T, C>(s, reinterpret_cast<T*>(x0), d, g, ws, chain, r.alpha)));
+  GW_RUN(float, 2) GW_RUN(float, 4) GW_RUN(float, 8) GW_RUN(float, 16) GW_RUN(double, 2) GW_RUN(double, 4) GW_RUN(double, 8)
+#undef GW_RUN
+  for (int i = 0; i < 3; ++i) count_launch();
+  SweepArgs a = base_args(g, ws);
+  a.alpha = r.alpha;
+  a.cand = d->in.cand;
+  a.live = d->live;
+  const int mode = chain ? MODE_LOOK : MODE_PAR;
+  if (ev) GW_CUDA(cudaEventRecordWithFlags((*ev)[0], s, cudaEventRecordExternal));
+  for (int32_t t = g.weighted ? 1 : 2; t <= H; ++t) {
+    a.X = t == 1 ? x0 : xs + row * es * (t - 2);
+    a.Y = xs + row * es * (t - 1);
+    GW_TRY(launch_sweep(mode, fp64, cols, a, s, profile));
+  }
+  if (ev) GW_CUDA(cudaEventRecordWithFlags((*ev)[1], s, cudaEventRecordExternal));
+  MeetArgs m{};
+  m.xs = xs;
+  m.stride = static_cast<int64_t>(row);
+  m.L = L;
+  m.H = H;
+  m.n_scan = select ? n_scan : g.n_active;
+  m.n_active = g.n_active;
+  m.rp = g.rp.as<int32_t>();
+  m.cnt = ws.cnt.as<int32_t>();
+  m.mask = ws.mask.as<uint32_t>();
+  m.perm = g.perm_d.as<int32_t>();
+  m.tail = ws.tail.as<float>();
+  m.bound = ws.bound.as<float>();
+  m.stale = ws.stale.as<Stale>();
+  m.rs_f = g.weighted ? g.rs_f.as<float>() : nullptr;
+  m.rs_d = g.weighted ? g.rs_d.as<double>() : nullptr;
+  m.alpha = r.alpha;
+  m.part = ws.parts.as<double>();
+  m.sel_v = ws.sel.as<float>();
+  m.sel_id = reinterpret_cast<int*>(m.sel_v + static_cast<size_t>(kMeetBlocks) * kRunLevels * kTopK);
+  m.d = d;
+#define GW_MEET(T, C, CH, SE) \
+  if (fp64 == (sizeof(T) == 8) && cols == C && chain == CH && select == SE) GW_CUDA((launch_meet<T, C, CH, SE>(s, m)));
+  GW_MEET(float, 4, true, true) GW_MEET(float, 8, true, true) GW_MEET(double, 4, true, true)
+  GW_MEET(float, 2, false, true) GW_MEET(float, 4, false, true) GW_MEET(float, 8, false, true)
+  GW_MEET(double, 2, false, true) GW_MEET(double, 4, false, true)
+  GW_MEET(float, 16, false, false) GW_MEET(double, 8, false, false)
+#undef GW_MEET
+  count_launch();
+  GW_CUDA(cudaMemcpyAsync(out, &d->out, sizeof(RunOut), cudaMemcpyDeviceToHost, s));
+  return GEDWALK_OK;
+}
+
+gedwalk_status RunEngine::run(bool chain, int cols, bool select, const std::vector<int32_t>& cand) {
+  for (int j = 0; j < kRunCols; ++j) in->cand[j] = j < static_cast<int>(cand.size()) && j < cols - 1 ? cand[j] : -1;
+  GW_TRY(push_added());
+  const int swept = g.weighted ? H : H - 1;
+  sweeps += swept;
+  const int mode = chain ? MODE_LOOK : MODE_PAR;
+  uint64_t abits;
+  memcpy(&abits, &r.alpha, 8);
+  auto bits = [](const void* p) { return static_cast<uint64_t>(reinterpret_cast<uintptr_t>(p)); };
+  Sequence q;
+  q.key = mix_all({uint64_t(mode), uint64_t(cols), uint64_t(r.fp64), uint64_t(L), uint64_t(select), uint64_t(n_scan), abits,
+                   bits(&g), bits(s), bits(ws.xs.p), bits(ws.cnt.p), bits(ws.mask.p), bits(ws.parts.p), bits(ws.small.p),
+                   bits(ws.partial.p), bits(ws.counters.p), bits(ws.stale.p), bits(ws.sel.p), bits(ws.tail.p),
+                   bits(ws.bound.p), bits(ws.run_io), bits(g.rp.p), bits(g.ci.p), bits(g.plan.units.p)});
+  q.kernels = 5 + swept;
+  q.sweeps = swept;
+  q.bytes = sweep_bytes(mode, r.fp64, cols, g.n_active, g.nnz, g.weighted);
+  q.prof_key = (mode * 1000 + cols) * 2 + (r.fp64 ? 1 : 0);
+  GW_TRY(run_sequence(ws, s, q, [&](bool profile, const std::vector<cudaEvent_t>* ev) {
+    return issue(chain, cols, select, profile, ev);
+  }));
+  GW_CUDA(cudaStreamSynchronize(s));
+  read_graph_timing(ws);
+  in->n_stale = 0;
+  in->n_added = 0;
+  return GEDWALK_OK;
+}
+
+gedwalk_status RunEngine::guess(int levels) {
+  RunDev* d = ws.small.as<RunDev>();
+  GW_TRY(push_added());
+  GW_CUDA(cudaMemcpyAsync(&d->in, in, sizeof(RunIn), cudaMemcpyHostToDevice, s));
+  run_begin<<<dim3(kChunks, kRunCols), 256, 0, s>>>(d, g.rp.as<int32_t>(), g.ci.as<int32_t>(), ws.mask.as<uint32_t>(),
+                                                    ws.cnt.as<int32_t>(), ws.stale.as<Stale>());
+  GW_KCHECK();
+  float* sel_v = ws.sel.as<float>();
+  guess_kernel<<<meet_grid(n_scan), kThreads, 0, s>>>(
+      ws.bound.as<float>(), n_scan, g.n_active, ws.mask.as<uint32_t>(), g.perm_d.as<int32_t>(), levels, sel_v,
+      reinterpret_cast<int*>(sel_v + static_cast<size_t>(kMeetBlocks) * kRunLevels * kTopK), d);
+  GW_KCHECK();
+  GW_CUDA(cudaMemcpyAsync(out, &d->out, sizeof(RunOut), cudaMemcpyDeviceToHost, s));
+  GW_CUDA(cudaStreamSynchronize(s));
+  in->n_stale = 0;
+  in->n_added = 0;
+  return GEDWALK_OK;
+}
+
+}  // namespace gw

@@ -1,0 +1,102 @@
+// Runs of sweeps of half the walk length, joined by the meeting pass (run.cu).
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <functional>
+
+#include "device_util.cuh"
+#include "internal.h"
+
+namespace gw {
+
+constexpr int kRunCols = 16;            // widest run: column 0 and 15 candidates
+constexpr int kRunCands = kRunCols - 1;
+constexpr int kRunLevels = 7;           // lookahead levels with a selection of their own
+constexpr int kMeetBlocks = 304;        // two resident blocks of the meeting pass per SM
+
+// What a run is told, copied to the device as its first operation.
+struct RunIn {
+  int32_t cand[kRunCols];      // candidate of column j + 1, -1: none
+  int32_t added[kRunCols];     // vertices that joined S since the last run
+  int32_t n_added;
+  int32_t n_stale;             // exact gains known on the host, to be recorded
+  int32_t stale_id[kRunCols];
+  int32_t stale_step[kRunCols];
+  double stale_gain[kRunCols];
+  int32_t step;                // greedy step of level 0
+  uint64_t seed;               // stochastic greedy: the draws of the levels' steps
+  uint64_t thr[kRunLevels];    // UINT64_MAX: every vertex takes part
+};
+
+// The best kTopK bounds among the vertices not evaluated, for one level.
+struct LevelSel {
+  float val[kTopK];
+  int32_t id[kTopK];
+  // the vertex with bound exactly 0 and the smallest caller id, (caller id << 32) | internal id
+  unsigned long long zero_min;
+  int32_t sampled;  // stochastic greedy: sampled vertices outside the level's set
+  int32_t pad;
+};
+
+struct RunOut {  // device -> host, one copy per run
+  LevelSel lv[kRunLevels];
+  double gains[kRunCols];
+};
+
+struct RunDev {  // device-side state of the runs of one workspace
+  RunIn in;
+  RunOut out;
+  int32_t live[kRunCols];  // whether candidate j has a neighbour outside its base set
+  int32_t adj[kRunCols];   // chain: earlier candidates that are neighbours of candidate j
+  int32_t done;            // blocks of the meeting (or guess) pass that have finished
+};
+
+// Runs a launch sequence, captured once per configuration (on its second use) and replayed as a
+// CUDA graph; directly on the legacy default stream. `issue` gets the two timing events of a
+// capture (or null).
+struct Sequence {
+  uint64_t key;
+  int kernels, sweeps;
+  double bytes;
+  int prof_key;
+};
+gedwalk_status run_sequence(Workspace& ws, cudaStream_t s, const Sequence& q,
+                            const std::function<gedwalk_status(bool profile, const std::vector<cudaEvent_t>* ev)>& issue);
+// After a synchronisation: hands the sweep timings of graph replays to the profiler.
+void read_graph_timing(Workspace& ws);
+uint64_t mix_all(std::initializer_list<uint64_t> vs);
+
+// The runs of one maximisation (or one gains call) on an undirected graph.
+struct RunEngine {
+  Graph& g;
+  Workspace& ws;
+  const Resolved& r;
+  cudaStream_t s;
+  int32_t L = 0, H = 0;
+  int32_t n_scan = 0;  // rows of the selections (stochastic greedy scans isolated vertices too)
+  int64_t sweeps = 0;
+  RunIn* in = nullptr;   // pinned; step, seed, thr and the stale list are the caller's to fill
+  RunOut* out = nullptr; // pinned; valid after run() or guess()
+  std::vector<int32_t> added;  // joined S on the host, not yet on the device
+
+  RunEngine(Graph& g_, Workspace& ws_, const Resolved& r_, cudaStream_t s_) : g(g_), ws(ws_), r(r_), s(s_) {}
+  // Buffers for runs of up to cols columns and walk length L_max; S = init.
+  gedwalk_status setup(int32_t L_max, int cols, bool select, const std::vector<int32_t>& init);
+  // Walk length of the following runs; with a selection, the tail bounds for it.
+  gedwalk_status set_length(int32_t length, bool select);
+  // One run: chain (candidate j under S + the earlier ones) or not (every candidate under S).
+  gedwalk_status run(bool chain, int cols, bool select, const std::vector<int32_t>& cand);
+  // Selections of `levels` steps' samples from the last pass's bounds (a choice of guesses only).
+  gedwalk_status guess(int levels);
+  void stale(int32_t v, double gain, int32_t step);
+
+ private:
+  gedwalk_status push_added();
+  gedwalk_status issue(bool chain, int cols, bool select, bool profile, const std::vector<cudaEvent_t>* ev);
+};
+
+// Device bytes of the buffers RunEngine::setup makes.
+int64_t run_bytes(const Graph& g, int32_t L_max, int cols, bool fp64, bool select);
+
+}  // namespace gw

@@ -31,6 +31,7 @@
 #include <atomic>
 #include <cstdint>
 
+#include "device_util.cuh"
 #include "internal.h"
 
 namespace gw {
@@ -210,10 +211,10 @@ struct Scatter {
 template <int MODE, int C>
 struct Sums {
   static constexpr int N = MODE == MODE_TOTALS ? 1 : MODE == MODE_SCORE ? 1
-                           : (MODE == MODE_FUSED || MODE == MODE_LOOK) ? C - 1 : MODE == MODE_CAND ? C : 0;
-  // the sum fed by column c, or -1 (MODE_FUSED and MODE_LOOK: columns 1.., the candidates)
+                           : MODE == MODE_FUSED ? C - 1 : MODE == MODE_CAND ? C : 0;
+  // the sum fed by column c, or -1 (MODE_FUSED: columns 1.., the candidates)
   __device__ __forceinline__ static int slot(int c) {
-    constexpr int first = (MODE == MODE_FUSED || MODE == MODE_LOOK) ? 1 : 0;
+    constexpr int first = MODE == MODE_FUSED ? 1 : 0;
     return c >= first && c - first < N ? c - first : -1;
   }
 };
@@ -221,45 +222,22 @@ struct Sums {
 // Number of candidate ids a mode reads (the only rows whose epilogue differs from y = alpha s).
 template <int MODE, int C>
 struct Cands {
-  static constexpr int N = (MODE == MODE_FUSED || MODE == MODE_LOOK) ? C - 1 : MODE == MODE_CAND ? C : 0;
-};
-
-// Per-lane column sums over the rows of one unit. FP64 vectors sum in FP64. FP32 vectors sum with
-// compensated FP32 additions (Kahan: the error is at most 2u * sum |y| + O(m u^2), u = 2^-24, over
-// m <= 128 rows) and convert once per unit to FP64, in which every later sum (over lanes, units and
-// sweeps) is taken. On a GB300 an FP64 addition costs about 64 FP32 ones, and one conversion and
-// one FP64 addition per row and column cost more than the rest of the epilogue.
-template <typename T, int N>
-struct ColAcc {
-  double s[N];
-  __device__ __forceinline__ void zero() {
-#pragma unroll
-    for (int k = 0; k < N; ++k) s[k] = 0.0;
-  }
-  __device__ __forceinline__ void add(int k, double y) { s[k] += y; }
-  __device__ __forceinline__ double get(int k) const { return s[k]; }
-};
-template <int N>
-struct ColAcc<float, N> {
-  float s[N], c[N];
-  __device__ __forceinline__ void zero() {
-#pragma unroll
-    for (int k = 0; k < N; ++k) s[k] = c[k] = 0.0f;
-  }
-  __device__ __forceinline__ void add(int k, float y) {
-    const float t1 = __fsub_rn(y, c[k]);
-    const float t = __fadd_rn(s[k], t1);
-    c[k] = __fsub_rn(__fsub_rn(t, s[k]), t1);
-    s[k] = t;
-  }
-  __device__ __forceinline__ double get(int k) const { return static_cast<double>(s[k]) - static_cast<double>(c[k]); }
+  static constexpr int N = (MODE == MODE_FUSED || MODE == MODE_LOOK || MODE == MODE_PAR) ? C - 1 : MODE == MODE_CAND ? C : 0;
 };
 
 // The epilogue of the rows whose warp holds a candidate row (at most kCandSlots rows of the graph;
 // every lane of the warp calls it, shuffles inside). y holds alpha * s, zeroed on S.
+// Runs (MODE_LOOK, MODE_PAR): column j >= 1 counts the walks through c_j that avoid its base set,
+// T_{j-1} = S + {c_1..c_{j-1}} (MODE_LOOK) or S (MODE_PAR). At c_j's own row these are all the walks
+// that avoid the base set (each visits c_j where it ends): column 0 there, less the columns 1..j-1 in
+// a chain (a walk that avoids S avoids c_1..c_{j-1} or has a first one among them), clamped at 0;
+// 0 for a candidate without a neighbour outside its base set. A chain's columns beyond j are 0 at
+// c_j, which their base sets hold. The lane holds columns c0..c0+CPL-1 of the row's group, whose
+// column blocks lie in natural order over its first lanes (duplicates beyond them).
 template <typename T, int C, int MODE, int CPL>
-__device__ __forceinline__ void candidate_rows(const SweepArgs& a, const int* __restrict__ s_cand, int r, bool valid,
-                                               int c0, int base, T (&y)[CPL]) {
+__device__ __forceinline__ void candidate_rows(const SweepArgs& a, const int* __restrict__ s_cand,
+                                               const int* __restrict__ s_live, int r, bool valid, int c0, int base,
+                                               T (&y)[CPL]) {
   if constexpr (MODE == MODE_FUSED) {
     // column 0 is phi^miss under S; candidate column j >= 1 takes it at the candidate's row
     // (every S-avoiding walk ending at c_j visits c_j)
@@ -270,70 +248,47 @@ __device__ __forceinline__ void candidate_rows(const SweepArgs& a, const int* __
       if (valid && c >= 1 && s_cand[c - 1] == r) y[k] = m;
     }
   } else if constexpr (MODE == MODE_CAND) {
-    const T* min = static_cast<const T*>(a.Min) + (a.level_ptr ? a.level_stride * __ldg(a.level_ptr) : 0);
+    const T* min = static_cast<const T*>(a.Min);
 #pragma unroll
     for (int k = 0; k < CPL; ++k)
       if (valid && s_cand[c0 + k] == r) y[k] = __ldg(min + r);
-  }
-}
-
-// MODE_LOOK epilogue for row r: D = C - 1 levels of one lookahead run, T_d = S + {c_1..c_d}.
-// Column 0 is phi^miss under S; column j >= 1 counts the walks through c_j that avoid T_{j-1}
-// (at c_j's own row: all of phi^miss(T_{j-1}), every such walk ending there visits c_j). A walk
-// that avoids S either avoids c_1..c_d or has a first c_j among them, so
-//   phi^miss(T_d) = column 0 - columns 1..d,
-// which gives every level's phi^miss (table d, d = 0..D-1) and c_j's own-row value without
-// columns of their own. The differences are clamped at 0 (their exact value is never negative).
-// The lane holds columns c0..c0+CPL-1 of the row's group, whose column blocks lie in natural
-// order over its first lanes (duplicates beyond them); every lane of the warp calls it.
-template <typename T, int C, int CPL>
-__device__ __forceinline__ void look_rows(const SweepArgs& a, const int* __restrict__ s_cand, int r, bool valid,
-                                          bool store, int c0, int base, T (&y)[CPL], bool maybe_cand) {
-  constexpr int NB = C / CPL;  // column blocks of a group
-  T y0 = y[0];                 // column 0 sits in block 0, on the group's first lane
-  T run = T(0);                // running sum of columns 1.. (starts with the blocks before this lane's)
-  if constexpr (NB > 1) {
-    const int blk = c0 / CPL;
-    y0 = __shfl_sync(kFull, y[0], base);
-    T inc = T(0);
+  } else if constexpr (MODE == MODE_PAR) {
+    const T m = __shfl_sync(kFull, y[0], base);
 #pragma unroll
-    for (int k = 0; k < CPL; ++k)
-      if (c0 + k >= 1) inc += y[k];
-#pragma unroll
-    for (int o = 1; o < NB; o <<= 1) {
-      const T t = __shfl_up_sync(kFull, inc, o);
-      if (blk >= o) inc += t;
+    for (int k = 0; k < CPL; ++k) {
+      const int c = c0 + k;
+      if (valid && c >= 1 && s_cand[c - 1] == r) y[k] = s_live[c - 1] ? m : T(0);
     }
-    const T t = __shfl_up_sync(kFull, inc, 1);
-    run = blk > 0 ? t : T(0);
-  }
-  bool special = false;  // r is one of the run's candidates (only units that hold one look)
-  if (maybe_cand) {
+  } else if constexpr (MODE == MODE_LOOK) {
+    constexpr int NB = C / CPL;  // column blocks of a group
+    T y0 = y[0];                 // column 0 sits in block 0, on the group's first lane
+    T run = T(0);                // sum of columns 1.. before this lane's
+    if constexpr (NB > 1) {
+      const int blk = c0 / CPL;
+      y0 = __shfl_sync(kFull, y[0], base);
+      T inc = T(0);
 #pragma unroll
-    for (int j = 0; j < C - 1; ++j) special |= valid && s_cand[j] == r;
-  }
-  const bool rare = maybe_cand && __any_sync(kFull, special);
-  T* M = static_cast<T*>(a.Mout);
+      for (int k = 0; k < CPL; ++k)
+        if (c0 + k >= 1) inc += y[k];
 #pragma unroll
-  for (int k = 0; k < CPL; ++k) {
-    const int d = c0 + k;
-    const T before = run;  // columns 1..d-1
-    if (d >= 1) run += y[k];
-    if (store && d <= C - 2) {  // table d = phi^miss(T_d): column 0 minus columns 1..d, 0 on c_1..c_d
-      T m = y0 - run;
-      m = m > T(0) ? m : T(0);
-      if (rare && special)
-        for (int j = 0; j < d; ++j)
-          if (s_cand[j] == r) m = T(0);
-      M[a.mout_stride * d + r] = m;
+      for (int o = 1; o < NB; o <<= 1) {
+        const T t = __shfl_up_sync(kFull, inc, o);
+        if (blk >= o) inc += t;
+      }
+      const T t = __shfl_up_sync(kFull, inc, 1);
+      run = blk > 0 ? t : T(0);
     }
-    // r = c_m: column m takes phi^miss(T_{m-1}) at r; columns beyond m run under sets that hold r
-    if (rare && special && d >= 1) {
-      if (s_cand[d - 1] == r) {
+#pragma unroll
+    for (int k = 0; k < CPL; ++k) {
+      const int c = c0 + k;
+      const T before = run;
+      if (c >= 1) run += y[k];
+      if (!valid || c < 1) continue;
+      if (s_cand[c - 1] == r) {
         const T e = y0 - before;
-        y[k] = e > T(0) ? e : T(0);
+        y[k] = s_live[c - 1] && e > T(0) ? e : T(0);
       } else {
-        for (int j = 0; j < d - 1; ++j)
+        for (int j = 0; j < c - 1; ++j)
           if (s_cand[j] == r) y[k] = T(0);
       }
     }
@@ -347,11 +302,11 @@ __device__ __forceinline__ void look_rows(const SweepArgs& a, const int* __restr
 // maybe_cand (warp-uniform): a candidate row may lie among the rows of this unit; otherwise the
 // per-row candidate test is skipped.
 template <typename T, int C, int MODE, int CPL>
-__device__ __forceinline__ void epilogue(const SweepArgs& a, const int* __restrict__ s_cand, int r, bool valid,
-                                         bool store, int c0, int base, T (&s)[CPL], ColAcc<T, CPL>& acc,
+__device__ __forceinline__ void epilogue(const SweepArgs& a, const int* __restrict__ s_cand,
+                                         const int* __restrict__ s_live, int r, bool valid, bool store, int c0, int base, T (&s)[CPL], ColAcc<T, CPL>& acc,
                                          bool maybe_cand) {
   T* Y = static_cast<T*>(a.Y);
-  constexpr bool kMasked = MODE == MODE_SCORE || MODE == MODE_FUSED || MODE == MODE_CAND || MODE == MODE_LOOK;
+  constexpr bool kMasked = MODE != MODE_TOTALS && MODE != MODE_PLAIN;
   const bool inS = kMasked && valid ? in_mask(a.mask, r) : false;
   // weighted graph: the row's scale s_r turns the gathered sum into the true value
   // alpha s_r (A x~)(r), which is summed, and the stored vector is x~ = s_r * value
@@ -382,13 +337,11 @@ __device__ __forceinline__ void epilogue(const SweepArgs& a, const int* __restri
     T y[CPL];
 #pragma unroll
     for (int k = 0; k < CPL; ++k) y[k] = inS ? T(0) : alpha * s[k];
-    if constexpr (MODE == MODE_LOOK) {
-      look_rows<T, C, CPL>(a, s_cand, r, valid, store, c0, base, y, maybe_cand);
-    } else if (Cands<MODE, C>::N > 0 && maybe_cand) {
+    if (Cands<MODE, C>::N > 0 && maybe_cand) {
       bool special = false;
 #pragma unroll
       for (int j = 0; j < Cands<MODE, C>::N; ++j) special |= s_cand[j] == r;
-      if (__any_sync(kFull, valid && special)) candidate_rows<T, C, MODE, CPL>(a, s_cand, r, valid, c0, base, y);
+      if (__any_sync(kFull, valid && special)) candidate_rows<T, C, MODE, CPL>(a, s_cand, s_live, r, valid, c0, base, y);
     }
     if constexpr (MODE == MODE_FUSED) {
       if (store && c0 == 0) static_cast<T*>(a.Mout)[r] = y[0];
@@ -432,7 +385,7 @@ __device__ __forceinline__ void write_slot(const SweepArgs& a, size_t slot, int 
 // Short rows (degree <= 2W): W lanes per row, at most two entries per lane, two rows per group.
 template <typename T, int C, int MODE, int LW, class Src>
 __device__ __forceinline__ void short_rows(const SweepArgs& a, const Src& src, const int4 u, int uidx, int lane,
-                                          int* s_rp, const int* s_cand) {
+                                          int* s_rp, const int* s_cand, const int* s_live) {
   constexpr int W = 1 << LW;
   constexpr int NG = 32 / W;
   using SC = Scatter<T, C, LW>;
@@ -486,8 +439,8 @@ __device__ __forceinline__ void short_rows(const SweepArgs& a, const Src& src, c
       sa[k] = acca[k];
       sb[k] = accb[k];
     }
-    epilogue<T, C, MODE, CPL>(a, s_cand, r0 + ra, va, va && owner, c0, base, sa, acc, maybe_cand);
-    epilogue<T, C, MODE, CPL>(a, s_cand, r0 + rb, vb, vb && owner, c0, base, sb, acc, maybe_cand);
+    epilogue<T, C, MODE, CPL>(a, s_cand, s_live, r0 + ra, va, va && owner, c0, base, sa, acc, maybe_cand);
+    epilogue<T, C, MODE, CPL>(a, s_cand, s_live, r0 + rb, vb, vb && owner, c0, base, sb, acc, maybe_cand);
   }
   // sum the groups' copies of each column (non-owners hold zeros), in FP64
   double cs[CPL];
@@ -503,7 +456,7 @@ __device__ __forceinline__ void short_rows(const SweepArgs& a, const Src& src, c
 // Long rows: one warp per row, entries strided over the lanes in groups of four loads.
 template <typename T, int C, int MODE, class Src>
 __device__ __forceinline__ void long_rows(const SweepArgs& a, const Src& src, const int4 u, int uidx, int lane,
-                                         int* s_rp, const int* s_cand) {
+                                         int* s_rp, const int* s_cand, const int* s_live) {
   using SC = Scatter<T, C, 5>;
   constexpr int CPL = SC::CPL;
   const int r0 = u.x, nrows = u.y - u.x;
@@ -536,7 +489,7 @@ __device__ __forceinline__ void long_rows(const SweepArgs& a, const Src& src, co
     T s[CPL];
 #pragma unroll
     for (int k = 0; k < CPL; ++k) s[k] = acc[k];
-    epilogue<T, C, MODE, CPL>(a, s_cand, r0 + rr, true, owner, c0, 0, s, cacc, maybe_cand);
+    epilogue<T, C, MODE, CPL>(a, s_cand, s_live, r0 + rr, true, owner, c0, 0, s, cacc, maybe_cand);
   }
   double cs[CPL];
 #pragma unroll
@@ -547,7 +500,7 @@ __device__ __forceinline__ void long_rows(const SweepArgs& a, const Src& src, co
 // Heavy slice: entries [u.y, u.z) of heavy row u.x, slice u.w.
 template <typename T, int C, int MODE, class Src>
 __device__ __forceinline__ void heavy_slice(const SweepArgs& a, const Src& src, const int4 u, int uidx, int lane,
-                                           const int* s_cand) {
+                                           const int* s_cand, const int* s_live) {
   using SC = Scatter<T, C, 5>;
   constexpr int CPL = SC::CPL;
   constexpr int NS = Sums<MODE, C>::N;
@@ -597,7 +550,7 @@ __device__ __forceinline__ void heavy_slice(const SweepArgs& a, const Src& src, 
     for (int k = 0; k < CPL; ++k) tot[k] += __ldcg(part + static_cast<size_t>(s) * C + c0 + k);
   ColAcc<T, CPL> cacc;
   cacc.zero();
-  epilogue<T, C, MODE, CPL>(a, s_cand, hr.x, true, owner, c0, 0, tot, cacc, true);
+  epilogue<T, C, MODE, CPL>(a, s_cand, s_live, hr.x, true, owner, c0, 0, tot, cacc, true);
   double cs[CPL];
 #pragma unroll
   for (int k = 0; k < CPL; ++k) cs[k] = cacc.get(k);
@@ -608,22 +561,22 @@ __device__ __forceinline__ void heavy_slice(const SweepArgs& a, const Src& src, 
 // Runs work unit uidx with the given gather source.
 template <typename T, int C, int MODE, class Src>
 __device__ __forceinline__ void run_unit(const SweepArgs& a, const Src& src, int uidx, int lane, int* rp,
-                                        const int* s_cand) {
+                                        const int* s_cand, const int* s_live) {
   const int4 u = a.units[uidx];
   if (u.w >= 0) {
-    heavy_slice<T, C, MODE>(a, src, u, uidx, lane, s_cand);
+    heavy_slice<T, C, MODE>(a, src, u, uidx, lane, s_cand, s_live);
     return;
   }
   switch (u.z) {
-    // the lookahead's 8-column rows of degree <= 2 take two lanes each: one lane holding all eight
+    // the runs' 8-column rows of degree <= 2 take two lanes each: one lane holding all eight
     // columns of two rows overflows the register budget of five CTAs per SM
-    case 0: short_rows<T, C, MODE, (MODE == MODE_LOOK && C == 8 && sizeof(T) == 4) ? 1 : 0>(a, src, u, uidx, lane, rp, s_cand); break;
-    case 1: short_rows<T, C, MODE, 1>(a, src, u, uidx, lane, rp, s_cand); break;
-    case 2: short_rows<T, C, MODE, 2>(a, src, u, uidx, lane, rp, s_cand); break;
-    case 3: short_rows<T, C, MODE, 3>(a, src, u, uidx, lane, rp, s_cand); break;
-    case 4: short_rows<T, C, MODE, 4>(a, src, u, uidx, lane, rp, s_cand); break;
-    case 5: short_rows<T, C, MODE, 5>(a, src, u, uidx, lane, rp, s_cand); break;
-    default: long_rows<T, C, MODE>(a, src, u, uidx, lane, rp, s_cand); break;
+    case 0: short_rows<T, C, MODE, ((MODE == MODE_LOOK || MODE == MODE_PAR) && C == 8 && sizeof(T) == 4) ? 1 : 0>(a, src, u, uidx, lane, rp, s_cand, s_live); break;
+    case 1: short_rows<T, C, MODE, 1>(a, src, u, uidx, lane, rp, s_cand, s_live); break;
+    case 2: short_rows<T, C, MODE, 2>(a, src, u, uidx, lane, rp, s_cand, s_live); break;
+    case 3: short_rows<T, C, MODE, 3>(a, src, u, uidx, lane, rp, s_cand, s_live); break;
+    case 4: short_rows<T, C, MODE, 4>(a, src, u, uidx, lane, rp, s_cand, s_live); break;
+    case 5: short_rows<T, C, MODE, 5>(a, src, u, uidx, lane, rp, s_cand, s_live); break;
+    default: long_rows<T, C, MODE>(a, src, u, uidx, lane, rp, s_cand, s_live); break;
   }
 }
 
@@ -638,7 +591,8 @@ constexpr int kCandSlots = 16;
 template <typename T, int C, int MODE>
 constexpr int min_ctas() {
   if (sizeof(T) == 8) return 1;
-  if (MODE == MODE_LOOK && C == 8) return 5;
+  if ((MODE == MODE_LOOK || MODE == MODE_PAR) && C == 8) return 5;
+  if ((MODE == MODE_LOOK || MODE == MODE_PAR) && C <= 4) return 6;
   if (MODE == MODE_CAND && C == 4) return 4;
   if ((MODE == MODE_FUSED || MODE == MODE_SCORE) && C <= 2) return 8;
   if (MODE == MODE_FUSED && C == 4) return 6;
@@ -649,16 +603,18 @@ constexpr int min_ctas() {
 // One warp per unit, one CTA per eight units.
 template <typename T, int C, int MODE>
 __global__ void __launch_bounds__(kThreads, (min_ctas<T, C, MODE>())) sweep_kernel(const SweepArgs a) {
-  __shared__ int s_cand[kCandSlots];
+  __shared__ int s_cand[kCandSlots], s_live[kCandSlots];
   __shared__ int s_rp[kWarps][kUnitRowsMax + 1];
-  if (threadIdx.x < kCandSlots)
-    s_cand[threadIdx.x] = (MODE == MODE_FUSED || MODE == MODE_CAND || MODE == MODE_LOOK) && a.cand ? a.cand[threadIdx.x] : -1;
+  if (Cands<MODE, C>::N > 0 && threadIdx.x < kCandSlots) {
+    s_cand[threadIdx.x] = a.cand[threadIdx.x];
+    if (MODE == MODE_LOOK || MODE == MODE_PAR) s_live[threadIdx.x] = a.live[threadIdx.x];
+  }
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int uidx = blockIdx.x * kWarps + warp;
   if (uidx >= a.num_units) return;
   const GlobalSrc<T, C> src{static_cast<const T*>(a.X), a.hub};
-  run_unit<T, C, MODE>(a, src, uidx, lane, s_rp[warp], s_cand);
+  run_unit<T, C, MODE>(a, src, uidx, lane, s_rp[warp], s_cand, s_live);
 }
 
 // [sweep-kernel-source-end]
@@ -744,29 +700,12 @@ int sweep_sums(int mode, int cols) {
     case MODE_SCORE:
       return 1;
     case MODE_FUSED:
-    case MODE_LOOK:
       return cols - 1;
     case MODE_CAND:
       return cols;
     default:
       return 0;
   }
-}
-
-gedwalk_status configure_sweep(int mode, bool fp64, int cols) {
-#define GW_CASE(M, T, C)                                     \
-  if (mode == M && fp64 == (sizeof(T) == 8) && cols == C) { \
-    configure<T, C, M>();                                    \
-    return GEDWALK_OK;                                       \
-  }
-  GW_CASE(MODE_LOOK, float, 4)
-  GW_CASE(MODE_LOOK, float, 8)
-  GW_CASE(MODE_LOOK, double, 4)
-  GW_CASE(MODE_CAND, float, 4)
-  GW_CASE(MODE_CAND, double, 4)
-#undef GW_CASE
-  return fail(GEDWALK_ERR_INVALID, "no sweep instantiation to configure for mode %d fp64 %d cols %d", mode,
-              int(fp64), cols);
 }
 
 gedwalk_status launch_sweep(int mode, bool fp64, int cols, const SweepArgs& a, cudaStream_t s, bool profile) {
@@ -783,13 +722,19 @@ gedwalk_status launch_sweep(int mode, bool fp64, int cols, const SweepArgs& a, c
   GW_CASE(MODE_FUSED, double, 2)
   GW_CASE(MODE_FUSED, double, 4)
   GW_CASE(MODE_CAND, float, 4)
-  GW_CASE(MODE_CAND, float, 8)
   GW_CASE(MODE_CAND, float, 16)
   GW_CASE(MODE_CAND, double, 4)
   GW_CASE(MODE_CAND, double, 8)
   GW_CASE(MODE_LOOK, float, 4)
   GW_CASE(MODE_LOOK, float, 8)
   GW_CASE(MODE_LOOK, double, 4)
+  GW_CASE(MODE_PAR, float, 2)
+  GW_CASE(MODE_PAR, float, 4)
+  GW_CASE(MODE_PAR, float, 8)
+  GW_CASE(MODE_PAR, float, 16)
+  GW_CASE(MODE_PAR, double, 2)
+  GW_CASE(MODE_PAR, double, 4)
+  GW_CASE(MODE_PAR, double, 8)
   GW_CASE(MODE_PLAIN, float, 4)
   GW_CASE(MODE_PLAIN, float, 8)
   GW_CASE(MODE_PLAIN, float, 16)
