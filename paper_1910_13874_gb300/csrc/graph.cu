@@ -723,8 +723,18 @@ static gedwalk_status finish_plan(Plan& plan, const std::vector<int4>& units, co
 // reverse CSR of a directed graph keeps the forward order, so its runs are shorter.
 // With `sorted` (the forward CSR) the runs are found by binary search over degrees and row
 // pointers; otherwise the rows are walked one by one.
+//
+// Size of a unit: its warp runs one iteration after the other (a chain of index load, gather,
+// reduction of 1.3 us or so), so few large units leave the chip waiting on latency, and many small
+// ones pay each unit's own start (unit, row pointers). A GB300 holds about 6,000 sweep warps; units
+// of nnz / 16384 entries, 128 to 1024, fill it a few times over. Measured, us per sweep with 1024 /
+// 512 / 256 / 128 entries: R-MAT scale 18 directed (4 M) 42 / 26 / 18 / 17; Erdos-Renyi 1.6 M 17 /
+// 15 / 14 / 14; R-MAT scale 20 (30 M) 127 / 122 / 129 / 141; Barabasi-Albert 16 M in FP64 352 / 357 /
+// 396 / 470; R-MAT scale 22 (128 M) 495 / 507 / 534 / 570.
 static gedwalk_status build_plan(Plan& plan, const std::vector<int32_t>& deg, const std::vector<int32_t>& rp,
                                  int32_t n_active, int32_t n, bool sorted) {
+  const int64_t unit_edges =
+      std::max<int64_t>(kUnitEdgesMin, std::min<int64_t>(kUnitEdges, static_cast<int64_t>(rp.back()) / kTargetUnits));
   if (!sorted) {
     std::vector<int4> units, heavy;
     int32_t slice = 0;
@@ -753,9 +763,9 @@ static gedwalk_status build_plan(Plan& plan, const std::vector<int32_t>& deg, co
       // a short-row unit takes up to kUnitRowsMax rows; on small graphs fewer, down to one
       // iteration of its warp (2 rows per lane group), so that every SM gets work
       const int32_t iter_rows = cls == 6 ? 1 : 2 * (32 >> cls);
-      const int32_t small_cap = std::max<int32_t>(iter_rows, n_active / kTargetUnits);
+      const int32_t small_cap = std::max<int32_t>(iter_rows, n_active / (kTargetUnits / 2));
       const int32_t max_rows = std::min<int32_t>(cls == 6 ? 32 : kUnitRowsMax, small_cap);
-      const int64_t max_edges = cls == 6 ? kLongUnitEdges : kUnitEdges;
+      const int64_t max_edges = cls == 6 ? 2 * unit_edges : unit_edges;
       int32_t r1 = r;
       int64_t edges = 0;
       while (r1 < n_active && deg[r1] <= kHeavyDeg && row_class(deg[r1]) == cls && r1 - r < max_rows &&
@@ -795,9 +805,9 @@ static gedwalk_status build_plan(Plan& plan, const std::vector<int32_t>& deg, co
     // a short-row unit takes up to kUnitRowsMax rows; on small graphs fewer, down to one
     // iteration of its warp (2 rows per lane group), so that every SM gets work
     const int32_t iter_rows = cls == 6 ? 1 : 2 * (32 >> cls);
-    const int32_t small_cap = std::max<int32_t>(iter_rows, n_active / kTargetUnits);
+    const int32_t small_cap = std::max<int32_t>(iter_rows, n_active / (kTargetUnits / 2));
     const int32_t max_rows = std::min<int32_t>(cls == 6 ? 32 : kUnitRowsMax, small_cap);
-    const int64_t max_edges = cls == 6 ? kLongUnitEdges : kUnitEdges;
+    const int64_t max_edges = cls == 6 ? 2 * unit_edges : unit_edges;
     while (r < cls_end) {
       // the most rows from r whose entries stay within max_edges (at least one row)
       const int64_t cap = static_cast<int64_t>(rp[r]) + max_edges;

@@ -92,10 +92,11 @@ struct DevBuf {
 constexpr int kThreads = 256;
 constexpr int kHeavyDeg = 1024;
 constexpr int kSliceEdges = 1024;
-constexpr int kUnitEdges = 1024;      // entries per short-row unit (at least one row)
-constexpr int kLongUnitEdges = 2048;  // entries per long-row unit (at least one row)
+constexpr int kUnitEdges = 1024;      // most entries of a short-row unit (at least one row); a
+                                      // long-row unit takes up to twice as many
+constexpr int kUnitEdgesMin = 128;    // fewest: a warp's iteration gathers up to 128 entries
 constexpr int kUnitRowsMax = 128;     // rows per unit (short classes); long units take <= 32
-constexpr int kTargetUnits = 4096;    // small graphs get units of fewer rows, aiming at this many
+constexpr int kTargetUnits = 16384;   // smaller graphs get smaller units, aiming at this many
 constexpr int kReduceParts = 64;      // first-stage parts of the deterministic slot reduction
 constexpr int64_t kL1HubBytes = 160 * 1024;  // x rows per SM kept in L1 with high priority
 
