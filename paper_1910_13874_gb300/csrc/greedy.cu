@@ -387,21 +387,6 @@ gedwalk_status run_sweeps(GreedyCtx& c, int mode, int cols, const std::vector<in
   });
 }
 
-// The stream a greedy run uses: the caller's, or (for the legacy default stream, which cannot
-// be captured) the workspace's own stream, ordered after the caller's.
-gedwalk_status greedy_stream(Workspace& ws, cudaStream_t caller, cudaStream_t* out) {
-  if (caller != nullptr) {
-    *out = caller;
-    return GEDWALK_OK;
-  }
-  if (!ws.own_stream) GW_CUDA(cudaStreamCreateWithFlags(&ws.own_stream, cudaStreamNonBlocking));
-  if (!ws.order_ev) GW_CUDA(cudaEventCreateWithFlags(&ws.order_ev, cudaEventDisableTiming));
-  GW_CUDA(cudaEventRecord(ws.order_ev, caller));
-  GW_CUDA(cudaStreamWaitEvent(ws.own_stream, ws.order_ev, 0));
-  *out = ws.own_stream;
-  return GEDWALK_OK;
-}
-
 }  // namespace
 
 gedwalk_status greedy_shape(const Graph& g, const Resolved& r, int32_t flags, GreedyShape* out) {
@@ -445,15 +430,12 @@ gedwalk_status greedy_shape(const Graph& g, const Resolved& r, int32_t flags, Gr
 }
 
 int64_t maximize_footprint(const Graph& g, const Resolved& r, int32_t flags, int32_t k) {
-  (void)k;
   GreedyShape sh{};
   if (greedy_shape(g, r, flags, &sh) != GEDWALK_OK) return 0;
   const int64_t n = g.n, es = r.fp64 ? 8 : 4;
   if (!g.directed) {
     int64_t b = run_bytes(g, sh.tab_L, sh.cols_max, r.fp64, (flags & GEDWALK_GAINS_ALL) == 0);
-    if (flags & GEDWALK_ADAPTIVE_L)  // the final group is scored at the full length
-      b += 2 * n * 2 * es + static_cast<int64_t>(std::max(g.plan.num_slots, 1)) * 2 * 8;
-    return b;
+    return b + 4 * static_cast<int64_t>(k);  // (the final group, where it has to be scored)
   }
   const int64_t slices = std::max(std::max(g.plan.num_slices, g.plan_r.num_slices), 1);
   const int64_t heavy = std::max(std::max(g.plan.num_heavy, g.plan_r.num_heavy), 1);
@@ -944,7 +926,7 @@ gedwalk_status maximize_impl(Graph& g, Workspace& ws, int32_t k, const Resolved&
   if (score) {
     // GED_{<=L} of the final group. From an empty start it is the sum of the picks' exact gains
     // g_L(S_j, c_j) = GED_{<=L}(S_j + c_j) - GED_{<=L}(S_j), telescoping from GED_{<=L}(empty) = 0;
-    // otherwise (an init group, or gains at shorter walk lengths) two-state sweeps over the group.
+    // otherwise (an init group, or gains at shorter walk lengths) the group is scored.
     if (init_int.empty() && !p.adaptive()) {
       double v = 0.0;
       for (int32_t j = 0; j < k; ++j) v += gains[j];

@@ -240,12 +240,13 @@ struct Graph {
 // ---------------------------------------------------------------- launchers
 enum SweepMode : int {
   MODE_TOTALS = 0,  // y = alpha A x, FP64, stores the column sum
-  MODE_SCORE = 1,   // two-state hit/miss step, sums h
+  MODE_SCORE = 1,   // directed scoring: two-state hit/miss step, sums h
   MODE_FUSED = 2,   // directed greedy: column 0 = phi^miss under S, columns 1.. candidate columns
   MODE_CAND = 3,    // directed greedy: candidate columns only; candidate rows read phi^miss from a table
   MODE_PLAIN = 4,   // batched scoring: y = alpha A x, no mask
   MODE_LOOK = 5,    // run, chain: phi^miss under S, then the walks through c_j avoiding S + {c_1..c_{j-1}}
-  MODE_PAR = 6      // run: phi^miss under S, then the walks through each c_j avoiding S
+  MODE_PAR = 6,     // run: phi^miss under S, then the walks through each c_j avoiding S
+  MODE_PAIR = 7     // scoring run: the two-state hit/miss step without its sum
 };
 
 struct SweepArgs {
@@ -355,6 +356,8 @@ gedwalk_status map_group(const Graph& g, const int32_t* S, int32_t s_len, std::v
 // Uploads the S bitmask (internal ids) into ws.mask.
 gedwalk_status upload_mask(Graph& g, Workspace& ws, const std::vector<int32_t>& S_int, cudaStream_t s);
 
+// GED_{<=L} of one group on an undirected graph, by a run of half the length (run.cu).
+gedwalk_status score_run(Graph& g, Workspace& ws, const std::vector<int32_t>& S_int, const Resolved& r, double* score);
 gedwalk_status score_one(Graph& g, Workspace& ws, const std::vector<int32_t>& S_int, const Resolved& r,
                          double* score);
 // Picks the batched-scoring column width for this graph (timed once, then cached).

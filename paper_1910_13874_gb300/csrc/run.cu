@@ -97,6 +97,21 @@ gedwalk_status run_sequence(Workspace& ws, cudaStream_t s, const Sequence& q,
   return GEDWALK_OK;
 }
 
+// The stream a run uses: the caller's, or (for the legacy default stream, which cannot
+// be captured) the workspace's own stream, ordered after the caller's.
+gedwalk_status greedy_stream(Workspace& ws, cudaStream_t caller, cudaStream_t* out) {
+  if (caller != nullptr) {
+    *out = caller;
+    return GEDWALK_OK;
+  }
+  if (!ws.own_stream) GW_CUDA(cudaStreamCreateWithFlags(&ws.own_stream, cudaStreamNonBlocking));
+  if (!ws.order_ev) GW_CUDA(cudaEventCreateWithFlags(&ws.order_ev, cudaEventDisableTiming));
+  GW_CUDA(cudaEventRecord(ws.order_ev, caller));
+  GW_CUDA(cudaStreamWaitEvent(ws.own_stream, ws.order_ev, 0));
+  *out = ws.own_stream;
+  return GEDWALK_OK;
+}
+
 void read_graph_timing(Workspace& ws) {
   for (SweepGraph& sg : ws.graphs) {
     if (!sg.timing_pending) continue;
@@ -132,9 +147,10 @@ __device__ __forceinline__ void join_set(const int32_t* __restrict__ list, int32
   }
 }
 
+// count: list[-1] when negative (a captured launch).
 __global__ void join_kernel(const int32_t* __restrict__ list, int32_t count, const int32_t* __restrict__ rp,
                             const int32_t* __restrict__ ci, uint32_t* __restrict__ mask, int32_t* __restrict__ cnt) {
-  join_set(list, count, rp, ci, mask, cnt);
+  join_set(list, count >= 0 ? count : list[-1], rp, ci, mask, cnt);
 }
 
 // Opens a run: the vertices that joined S, the exact gains known on the host, the pass's counters.
@@ -636,6 +652,100 @@ __global__ void __launch_bounds__(kThreads) guess_kernel(const float* __restrict
                 &d->out.lv[warp]);
 }
 
+// Scoring run, first stored vector, rows [0, n_active): (h, m) pairs. Unweighted: x_1 from the
+// counts: h_1 = alpha |N(v) cap S| (all of alpha deg on S), m_1 = alpha |N(v) \ S| (0 on S). Weighted
+// (rs): x_0 = the indicators of S and V \ S, scaled.
+template <typename T>
+__global__ void pair_init(T* __restrict__ X, const int32_t* __restrict__ rp, const int32_t* __restrict__ cnt,
+                          const uint32_t* __restrict__ mask, int32_t n_active, T alpha, const T* __restrict__ rs,
+                          int32_t* __restrict__ done) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *done = 0;
+  for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n_active; v += gridDim.x * blockDim.x) {
+    const bool inS = in_set(mask, v);
+    T h, m;
+    if (rs) {
+      h = inS ? rs[v] : T(0);
+      m = inS ? T(0) : rs[v];
+    } else {
+      const int32_t dg = rp[v + 1] - rp[v], c = cnt[v];
+      h = alpha * static_cast<T>(inS ? dg : c);
+      m = inS ? T(0) : alpha * static_cast<T>(dg - c);
+    }
+    if constexpr (sizeof(T) == 4) reinterpret_cast<float2*>(X)[v] = make_float2(h, m);
+    else reinterpret_cast<double2*>(X)[v] = make_double2(h, m);
+  }
+}
+
+// Walks of length a + b that hit S: the half of length a hits, or it misses and the half of length b
+// hits, so with b = H the lengths H + a, a = 1..L-H, number sum_v [h_a (h_H + m_H) + m_a h_H] and the
+// lengths up to H are plain sums of h_t. One thread per row; the last block adds the block sums.
+template <typename T>
+__global__ void __launch_bounds__(kThreads) pair_meet(const T* __restrict__ xs, int64_t stride, int32_t L, int32_t H,
+                                                      int32_t n_active, const T* __restrict__ rs,
+                                                      double* __restrict__ part, int32_t* __restrict__ done,
+                                                      double* __restrict__ out) {
+  constexpr int NW = kThreads / 32;
+  __shared__ double sg[NW];
+  __shared__ int is_last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool odd = (L & 1) != 0;
+  ColAcc<T, 1> acc;
+  acc.zero();
+  for (int32_t v = blockIdx.x * kThreads + threadIdx.x; v < n_active; v += gridDim.x * kThreads) {
+    T bh = T(0), bm = T(0), h = T(0), m = T(0);
+    const T* p = xs + 2 * static_cast<size_t>(v);
+#pragma unroll 4
+    for (int t = 1; t <= H; ++t, p += stride) {
+      T xh, xm;
+      if constexpr (sizeof(T) == 4) {
+        const float2 q = __ldcs(reinterpret_cast<const float2*>(p));
+        xh = q.x;
+        xm = q.y;
+      } else {
+        const double2 q = __ldcs(reinterpret_cast<const double2*>(p));
+        xh = q.x;
+        xm = q.y;
+      }
+      if (t < H) {
+        bh += xh;
+        bm += xm;
+      } else {
+        h = xh;
+        m = xm;
+      }
+    }
+    if (rs) {
+      const T inv = T(1) / rs[v];
+      bh *= inv;
+      bm *= inv;
+      h *= inv;
+      m *= inv;
+    }
+    const T vh = odd ? bh : bh + h, vm = odd ? bm : bm + m;
+    acc.add(0, (bh + h) + vh * (h + m) + vm * h);
+  }
+  double x = acc.get(0);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFullMask, x, o);
+  if (lane == 0) sg[warp] = x;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    x = 0.0;
+    for (int i = 0; i < NW; ++i) x += sg[i];
+    part[blockIdx.x] = x;
+    __threadfence();
+    is_last = atomicAdd(done, 1) == static_cast<int>(gridDim.x) - 1;
+  }
+  __syncthreads();
+  if (!is_last || warp != 0) return;
+  __threadfence();
+  x = 0.0;
+  for (int b = lane; b < static_cast<int>(gridDim.x); b += 32) x += __ldcg(part + b);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFullMask, x, o);
+  if (lane == 0) *out = x;
+}
+
 int grid_of(int64_t n) { return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 16))); }
 int meet_grid(int32_t n_scan) {
   return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(kMeetBlocks, (int64_t(n_scan) + kThreads - 1) / kThreads)));
@@ -683,6 +793,17 @@ int64_t run_bytes(const Graph& g, int32_t L_max, int cols, bool fp64, bool selec
   return b;
 }
 
+// The captured sequences copy from and to this block: it must outlive them at one address (a pinned
+// block freed and made again at the same address is another allocation to the driver).
+static gedwalk_status ensure_run_io(Workspace& ws) {
+  if (!ws.run_io && cudaMallocHost(&ws.run_io, sizeof(RunOut) + sizeof(RunIn)) != cudaSuccess) {
+    cudaGetLastError();
+    ws.run_io = nullptr;
+    return fail(GEDWALK_ERR_OOM, "pinned host allocation of %zu bytes failed", sizeof(RunOut) + sizeof(RunIn));
+  }
+  return GEDWALK_OK;
+}
+
 gedwalk_status RunEngine::setup(int32_t L_max, int cols, bool select, const std::vector<int32_t>& init) {
   const size_t n = static_cast<size_t>(g.n), H_max = static_cast<size_t>((L_max + 1) / 2), es = r.fp64 ? 8 : 4;
   const size_t row = static_cast<size_t>(g.n_active) * cols * es;
@@ -692,13 +813,7 @@ gedwalk_status RunEngine::setup(int32_t L_max, int cols, bool select, const std:
   GW_TRY(ws.mask.ensure(words * 4, s));
   GW_TRY(ws.parts.ensure(static_cast<size_t>(kMeetBlocks) * (cols - 1) * sizeof(double), s));
   GW_TRY(ws.small.ensure(sizeof(RunDev) + 256, s));
-  // the captured sequences copy from and to this block: it must outlive them at one address (a
-  // pinned block freed and made again at the same address is another allocation to the driver)
-  if (!ws.run_io && cudaMallocHost(&ws.run_io, sizeof(RunOut) + sizeof(RunIn)) != cudaSuccess) {
-    cudaGetLastError();
-    ws.run_io = nullptr;
-    return fail(GEDWALK_ERR_OOM, "pinned host allocation of %zu bytes failed", sizeof(RunOut) + sizeof(RunIn));
-  }
+  GW_TRY(ensure_run_io(ws));
   out = static_cast<RunOut*>(ws.run_io);
   in = reinterpret_cast<RunIn*>(out + 1);
   memset(in, 0, sizeof *in);
@@ -888,6 +1003,108 @@ gedwalk_status RunEngine::guess(int levels) {
   GW_CUDA(cudaStreamSynchronize(s));
   in->n_stale = 0;
   in->n_added = 0;
+  return GEDWALK_OK;
+}
+
+gedwalk_status score_run(Graph& g, Workspace& ws, const std::vector<int32_t>& S_int, const Resolved& r_in, double* score) {
+  Resolved r = r_in;
+  GW_TRY(greedy_stream(ws, r_in.stream, &r.stream));
+  struct Guard {  // nothing launched here still runs when a call leaves early
+    cudaStream_t s;
+    bool ok = false;
+    ~Guard() {
+      if (!ok) {
+        cudaStreamSynchronize(s);
+        cudaGetLastError();
+      }
+    }
+  } guard{r.stream};
+  cudaStream_t s = r.stream;
+  const bool fp64 = r.fp64;
+  const size_t n = static_cast<size_t>(g.n), es = fp64 ? 8 : 4;
+  const int32_t H = (r.L + 1) / 2;
+  const size_t row = static_cast<size_t>(g.n_active) * 2;
+  GW_TRY(ensure_run_io(ws));
+  GW_TRY(ws.xs.ensure(row * es * (H + (g.weighted ? 1 : 0)), s));
+  GW_TRY(ws.cnt.ensure(n * sizeof(int32_t), s));
+  const size_t words = (n + 31) / 32;
+  GW_TRY(ws.mask.ensure(words * 4, s));
+  GW_TRY(ws.parts.ensure(kMeetBlocks * sizeof(double), s));
+  GW_TRY(ws.small.ensure(64, s));
+  GW_TRY(ws.partial.ensure(static_cast<size_t>(std::max(g.plan.num_slices, 1)) * 2 * es, s));
+  const size_t cbytes = static_cast<size_t>(std::max(g.plan.num_heavy, 1)) * sizeof(unsigned);
+  if (ws.counters.bytes < cbytes || !ws.counters.p) GW_TRY(ws.counters.ensure(cbytes, s, /*zero=*/true));
+  // the group: its size, then its members
+  const int32_t count = static_cast<int32_t>(S_int.size());
+  GW_TRY(ws.members.ensure((S_int.size() + 1) * sizeof(int32_t), s));
+  GW_TRY(ws.ensure_pinned((S_int.size() + 1) * sizeof(int32_t)));
+  int32_t* st = static_cast<int32_t*>(ws.pinned);
+  st[0] = count;
+  std::copy(S_int.begin(), S_int.end(), st + 1);
+  GW_CUDA(cudaMemcpyAsync(ws.members.p, st, (S_int.size() + 1) * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+  int items = 1;  // blocks that walk the list, a power of two: few captured shapes
+  while (items < count && items < 256) items *= 2;
+  const int chunks = g.dmax > 4096 ? kChunks : 1;
+  double* d_sum = ws.small.as<double>();
+  int32_t* d_done = reinterpret_cast<int32_t*>(d_sum + 1);
+  double* h_sum = static_cast<double*>(ws.run_io);
+  auto issue = [&](bool profile, const std::vector<cudaEvent_t>* ev) -> gedwalk_status {
+    GW_CUDA(cudaMemsetAsync(ws.cnt.p, 0, n * sizeof(int32_t), s));
+    GW_CUDA(cudaMemsetAsync(ws.mask.p, 0, words * 4, s));
+    join_kernel<<<dim3(chunks, items), 256, 0, s>>>(ws.members.as<int32_t>() + 1, -1, g.rp.as<int32_t>(), g.ci.as<int32_t>(),
+                                                    ws.mask.as<uint32_t>(), ws.cnt.as<int32_t>());
+    GW_KCHECK();
+    char* xs = ws.xs.as<char>();
+    char* x0 = g.weighted ? xs + row * es * H : xs;
+    if (fp64)
+      pair_init<double><<<grid_of(g.n_active), 256, 0, s>>>(reinterpret_cast<double*>(x0), g.rp.as<int32_t>(),
+                                                            ws.cnt.as<int32_t>(), ws.mask.as<uint32_t>(), g.n_active, r.alpha,
+                                                            g.weighted ? g.rs_d.as<double>() : nullptr, d_done);
+    else
+      pair_init<float><<<grid_of(g.n_active), 256, 0, s>>>(reinterpret_cast<float*>(x0), g.rp.as<int32_t>(),
+                                                           ws.cnt.as<int32_t>(), ws.mask.as<uint32_t>(), g.n_active,
+                                                           static_cast<float>(r.alpha),
+                                                           g.weighted ? g.rs_f.as<float>() : nullptr, d_done);
+    GW_KCHECK();
+    SweepArgs a = base_args(g, ws);
+    a.alpha = r.alpha;
+    if (ev) GW_CUDA(cudaEventRecordWithFlags((*ev)[0], s, cudaEventRecordExternal));
+    for (int32_t t = g.weighted ? 1 : 2; t <= H; ++t) {
+      a.X = t == 1 ? x0 : xs + row * es * (t - 2);
+      a.Y = xs + row * es * (t - 1);
+      GW_TRY(launch_sweep(MODE_PAIR, fp64, 2, a, s, profile));
+    }
+    if (ev) GW_CUDA(cudaEventRecordWithFlags((*ev)[1], s, cudaEventRecordExternal));
+    if (fp64)
+      pair_meet<double><<<meet_grid(g.n_active), kThreads, 0, s>>>(reinterpret_cast<double*>(xs), static_cast<int64_t>(row), r.L,
+                                                                   H, g.n_active,
+                                                                   g.weighted ? g.rs_d.as<double>() : nullptr,
+                                                                   ws.parts.as<double>(), d_done, d_sum);
+    else
+      pair_meet<float><<<meet_grid(g.n_active), kThreads, 0, s>>>(reinterpret_cast<float*>(xs), static_cast<int64_t>(row), r.L, H,
+                                                                  g.n_active, g.weighted ? g.rs_f.as<float>() : nullptr,
+                                                                  ws.parts.as<double>(), d_done, d_sum);
+    GW_KCHECK();
+    GW_CUDA(cudaMemcpyAsync(h_sum, d_sum, sizeof(double), cudaMemcpyDeviceToHost, s));
+    return GEDWALK_OK;
+  };
+  const int swept = g.weighted ? H : H - 1;
+  uint64_t abits;
+  memcpy(&abits, &r.alpha, 8);
+  auto bits = [](const void* p) { return static_cast<uint64_t>(reinterpret_cast<uintptr_t>(p)); };
+  Sequence q;
+  q.key = mix_all({uint64_t(MODE_PAIR), uint64_t(fp64), uint64_t(r.L), uint64_t(items), abits, bits(&g), bits(s), bits(ws.xs.p),
+                   bits(ws.cnt.p), bits(ws.mask.p), bits(ws.parts.p), bits(ws.small.p), bits(ws.partial.p),
+                   bits(ws.counters.p), bits(ws.members.p), bits(ws.run_io), bits(g.rp.p), bits(g.ci.p), bits(g.plan.units.p)});
+  q.kernels = 3 + swept;
+  q.sweeps = swept;
+  q.bytes = sweep_bytes(MODE_PAIR, fp64, 2, g.n_active, g.nnz, g.weighted);
+  q.prof_key = (MODE_PAIR * 1000 + 2) * 2 + (fp64 ? 1 : 0);
+  GW_TRY(run_sequence(ws, s, q, issue));
+  GW_CUDA(cudaStreamSynchronize(s));
+  read_graph_timing(ws);
+  *score = *h_sum;
+  guard.ok = true;
   return GEDWALK_OK;
 }
 

@@ -63,6 +63,8 @@ struct Sequence {
 };
 gedwalk_status run_sequence(Workspace& ws, cudaStream_t s, const Sequence& q,
                             const std::function<gedwalk_status(bool profile, const std::vector<cudaEvent_t>* ev)>& issue);
+// The stream a run uses: the caller's, or the workspace's own for the legacy default stream.
+gedwalk_status greedy_stream(Workspace& ws, cudaStream_t caller, cudaStream_t* out);
 // After a synchronisation: hands the sweep timings of graph replays to the profiler.
 void read_graph_timing(Workspace& ws);
 uint64_t mix_all(std::initializer_list<uint64_t> vs);

@@ -12,13 +12,11 @@ namespace {
 
 // X0[v] = (h_0(v), m_0(v)) = (1_S(v), 1_{V\S}(v))
 template <typename T>
-__global__ void init_two_state(T* __restrict__ X, const uint32_t* __restrict__ mask, int32_t n,
-                               const T* __restrict__ rs) {
+__global__ void init_two_state(T* __restrict__ X, const uint32_t* __restrict__ mask, int32_t n) {
   for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
     const bool inS = (mask[v >> 5] >> (v & 31)) & 1u;
-    const T sv = rs ? rs[v] : T(1);  // weighted graph: the gathered vectors are scaled by s_v
-    X[2 * static_cast<size_t>(v)] = inS ? sv : T(0);
-    X[2 * static_cast<size_t>(v) + 1] = inS ? T(0) : sv;
+    X[2 * static_cast<size_t>(v)] = inS ? T(1) : T(0);
+    X[2 * static_cast<size_t>(v) + 1] = inS ? T(0) : T(1);
   }
 }
 
@@ -111,6 +109,7 @@ gedwalk_status score_one(Graph& g, Workspace& ws, const std::vector<int32_t>& S_
     *score = 0.0;
     return GEDWALK_OK;
   }
+  if (!g.directed) return score_run(g, ws, S_int, r, score);
   StreamGuard guard{s};
   const size_t es = r.fp64 ? 8 : 4;
   const size_t vbytes = static_cast<size_t>(g.n) * 2 * es;
@@ -120,11 +119,9 @@ gedwalk_status score_one(Graph& g, Workspace& ws, const std::vector<int32_t>& S_
   GW_TRY(ws.small.ensure(64, s));
   GW_TRY(upload_mask(g, ws, S_int, s));
   if (r.fp64)
-    init_two_state<double><<<blocks_for(g.n), 256, 0, s>>>(ws.x0.as<double>(), ws.mask.as<uint32_t>(), g.n,
-                                                            g.weighted ? g.rs_d.as<double>() : nullptr);
+    init_two_state<double><<<blocks_for(g.n), 256, 0, s>>>(ws.x0.as<double>(), ws.mask.as<uint32_t>(), g.n);
   else
-    init_two_state<float><<<blocks_for(g.n), 256, 0, s>>>(ws.x0.as<float>(), ws.mask.as<uint32_t>(), g.n,
-                                                           g.weighted ? g.rs_f.as<float>() : nullptr);
+    init_two_state<float><<<blocks_for(g.n), 256, 0, s>>>(ws.x0.as<float>(), ws.mask.as<uint32_t>(), g.n);
   GW_KCHECK();
   SweepArgs a = base_args(g, ws);
   a.alpha = r.alpha;

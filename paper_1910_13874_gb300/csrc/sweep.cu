@@ -313,7 +313,7 @@ __device__ __forceinline__ void epilogue(const SweepArgs& a, const int* __restri
   const T* rs = sizeof(T) == 8 ? reinterpret_cast<const T*>(a.rs_d) : reinterpret_cast<const T*>(a.rs_f);
   const T sv = rs && valid ? __ldg(rs + r) : T(1);
   const T alpha = static_cast<T>(a.alpha) * sv;
-  if constexpr (MODE == MODE_SCORE) {
+  if constexpr (MODE == MODE_SCORE || MODE == MODE_PAIR) {
     // Section 3.1.1: hit_i(v) = sum hit_{i-1}(u) + [v in S] sum miss_{i-1}(u);
     //                miss_i(v) = [v not in S] sum miss_{i-1}(u).  Columns: 0 = hit, 1 = miss.
     T sh, sm;
@@ -328,7 +328,7 @@ __device__ __forceinline__ void epilogue(const SweepArgs& a, const int* __restri
       T out[2];
       out[0] = alpha * (inS ? sh + sm : sh);
       out[1] = inS ? T(0) : alpha * sm;
-      acc.add(0, out[0]);
+      if (MODE == MODE_SCORE) acc.add(0, out[0]);
       out[0] *= sv;
       out[1] *= sv;
       store_vec<T, 2>(Y + static_cast<size_t>(r) * C, out);
@@ -391,8 +391,6 @@ __device__ __forceinline__ void short_rows(const SweepArgs& a, const Src& src, c
   using SC = Scatter<T, C, LW>;
   constexpr int CPL = SC::CPL;
   const int r0 = u.x, nrows = u.y - u.x;
-  for (int i = lane; i <= nrows; i += 32) s_rp[i] = __ldcs(a.rp + r0 + i);
-  __syncwarp();
   const bool maybe_cand = unit_has_cand<MODE, C>(s_cand, r0, r0 + nrows);
   const int g = lane >> LW, gl = lane & (W - 1);
   const int base = lane & ~(W - 1);
@@ -460,8 +458,6 @@ __device__ __forceinline__ void long_rows(const SweepArgs& a, const Src& src, co
   using SC = Scatter<T, C, 5>;
   constexpr int CPL = SC::CPL;
   const int r0 = u.x, nrows = u.y - u.x;
-  for (int i = lane; i <= nrows; i += 32) s_rp[i] = __ldcs(a.rp + r0 + i);
-  __syncwarp();
   const bool maybe_cand = unit_has_cand<MODE, C>(s_cand, r0, r0 + nrows);
   const int blk = lane & ((1 << SC::HS) - 1);
   const bool owner = (lane >> SC::HS) == 0;
@@ -560,9 +556,8 @@ __device__ __forceinline__ void heavy_slice(const SweepArgs& a, const Src& src, 
 
 // Runs work unit uidx with the given gather source.
 template <typename T, int C, int MODE, class Src>
-__device__ __forceinline__ void run_unit(const SweepArgs& a, const Src& src, int uidx, int lane, int* rp,
+__device__ __forceinline__ void run_unit(const SweepArgs& a, const Src& src, const int4 u, int uidx, int lane, int* rp,
                                         const int* s_cand, const int* s_live) {
-  const int4 u = a.units[uidx];
   if (u.w >= 0) {
     heavy_slice<T, C, MODE>(a, src, u, uidx, lane, s_cand, s_live);
     return;
@@ -594,27 +589,41 @@ constexpr int min_ctas() {
   if ((MODE == MODE_LOOK || MODE == MODE_PAR) && C == 8) return 5;
   if ((MODE == MODE_LOOK || MODE == MODE_PAR) && C <= 4) return 6;
   if (MODE == MODE_CAND && C == 4) return 4;
-  if ((MODE == MODE_FUSED || MODE == MODE_SCORE) && C <= 2) return 8;
+  if ((MODE == MODE_FUSED || MODE == MODE_SCORE || MODE == MODE_PAIR) && C <= 2) return 8;
   if (MODE == MODE_FUSED && C == 4) return 6;
   if (MODE == MODE_PLAIN) return C <= 8 ? 5 : C <= 16 ? 3 : C <= 32 ? 2 : 1;
   return 1;
 }
 
-// One warp per unit, one CTA per eight units.
+// One warp per unit, one CTA per eight units. The sweeps of a sequence are launched as programmatic
+// dependents: while the one before drains, a sweep's CTAs are scheduled and read what no kernel
+// writes (their unit and its row pointers), and wait for the earlier grid before anything else. On
+// small graphs, where a sweep is a chain of a few dependent loads, this hides the launch and two of
+// them.
 template <typename T, int C, int MODE>
 __global__ void __launch_bounds__(kThreads, (min_ctas<T, C, MODE>())) sweep_kernel(const SweepArgs a) {
   __shared__ int s_cand[kCandSlots], s_live[kCandSlots];
   __shared__ int s_rp[kWarps][kUnitRowsMax + 1];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int uidx = blockIdx.x * kWarps + warp;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  int4 u = make_int4(0, 0, 0, 0);
+  if (uidx < a.num_units) {
+    u = a.units[uidx];
+    if (u.w < 0) {  // light unit: its row pointers
+      const int nrows = u.y - u.x;
+      for (int i = lane; i <= nrows; i += 32) s_rp[warp][i] = __ldcs(a.rp + u.x + i);
+    }
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (Cands<MODE, C>::N > 0 && threadIdx.x < kCandSlots) {
     s_cand[threadIdx.x] = a.cand[threadIdx.x];
     if (MODE == MODE_LOOK || MODE == MODE_PAR) s_live[threadIdx.x] = a.live[threadIdx.x];
   }
   __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int uidx = blockIdx.x * kWarps + warp;
   if (uidx >= a.num_units) return;
   const GlobalSrc<T, C> src{static_cast<const T*>(a.X), a.hub};
-  run_unit<T, C, MODE>(a, src, uidx, lane, s_rp[warp], s_cand, s_live);
+  run_unit<T, C, MODE>(a, src, u, uidx, lane, s_rp[warp], s_cand, s_live);
 }
 
 // [sweep-kernel-source-end]
@@ -684,7 +693,16 @@ gedwalk_status run(const SweepArgs& a, cudaStream_t s, bool profile) {
   const int grid = (a.num_units + kWarps - 1) / kWarps;
   SweepArgs b = a;  // rows gathered with L1 priority: about kL1HubBytes of them
   b.hub = static_cast<int32_t>(std::min<int64_t>(a.n, kL1HubBytes / (sizeof(T) * C)));
-  sweep_kernel<T, C, MODE><<<grid, kThreads, 0, s>>>(b);
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kThreads);
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = prof ? 0 : 1;  // a timed launch runs alone between its events
+  GW_CUDA(cudaLaunchKernelEx(&cfg, sweep_kernel<T, C, MODE>, b));
   GW_KCHECK();
   if (prof)
     profile_end(s, ev, sweep_bytes(MODE, sizeof(T) == 8, C, a.n, a.nnz, a.rs_f != nullptr),
@@ -714,6 +732,8 @@ gedwalk_status launch_sweep(int mode, bool fp64, int cols, const SweepArgs& a, c
   GW_CASE(MODE_TOTALS, double, 1)
   GW_CASE(MODE_SCORE, double, 2)
   GW_CASE(MODE_SCORE, float, 2)
+  GW_CASE(MODE_PAIR, double, 2)
+  GW_CASE(MODE_PAIR, float, 2)
   GW_CASE(MODE_FUSED, float, 1)
   GW_CASE(MODE_FUSED, float, 2)
   GW_CASE(MODE_FUSED, float, 4)
