@@ -467,7 +467,7 @@ GEDWALK_API gedwalk_status gedwalk_serve_destroy(gedwalk_server_t srv);
  *    alpha^i-weighted count of the i-walks that hit S; the score is the sum over
  *    the L steps.
  *  stream: cudaStream_t (0 = default). The call is asynchronous.
- * Scratch: a fixed 512 KiB device array inside the library (per GPU, held until
+ * Scratch: a fixed 64 KiB device array inside the library (per GPU, held until
  * the process exits) limits n to 16,777,216; larger n returns
  * GEDWALK_ERR_INVALID. The first call on each device looks up that array's
  * address, so make the first call on a device before any stream capture. All
