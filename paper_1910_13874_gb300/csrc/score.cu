@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "device_util.cuh"
 #include "internal.h"
 
 namespace gw {
@@ -20,15 +21,14 @@ __global__ void init_two_state(T* __restrict__ X, const uint32_t* __restrict__ m
   }
 }
 
-// Batched scoring, first-visit form. Column j of a block is m_0 = 1_{V \ S_j}.
+// Batched scoring of a directed graph, first-visit form. Column j of a block is m_0 = 1_{V \ S_j}.
 // Isolated rows (r >= n_active) hold 0: the sweeps never write them and nothing gathers them,
-// so they read as the (zero) first-visit counts of such vertices.
-__global__ void init_batch(float* __restrict__ X, int32_t n, int32_t n_active, int32_t cols, int32_t active,
-                           const float* __restrict__ rs) {
+// so they read as the (zero) first-visit counts of such vertices. (The autotuner starts from it too.)
+__global__ void init_batch(float* __restrict__ X, int32_t n, int32_t n_active, int32_t cols, int32_t active) {
   const size_t total = static_cast<size_t>(n) * cols;
   const size_t live = static_cast<size_t>(n_active) * cols;
   for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < total; i += size_t(gridDim.x) * blockDim.x)
-    X[i] = (i < live && static_cast<int32_t>(i % cols) < active) ? (rs ? rs[i / cols] : 1.0f) : 0.0f;
+    X[i] = (i < live && static_cast<int32_t>(i % cols) < active) ? 1.0f : 0.0f;
 }
 
 __global__ void zero_members(float* __restrict__ X, int32_t cols, const int32_t* __restrict__ mrow,
@@ -40,11 +40,9 @@ __global__ void zero_members(float* __restrict__ X, int32_t cols, const int32_t*
 // After sweep p: Y_p(s, j) = alpha (A m_{p-1})(s) is alpha^p F_p(s), the weighted p-walks whose
 // first visit to S_j is their last vertex s. It meets every walk continuing from s:
 // acc += alpha^p F_p(s) * K_{L-p}(s), K_q(s) = sum_{r<=q} t_r(s). Then m_p(s) = 0.
-// On a weighted graph (rs = the vertex scales) Y and the table hold s times the true values.
 __global__ void batch_member_epilogue(float* __restrict__ Y, int32_t cols, const int32_t* __restrict__ mrow,
                                       const int32_t* __restrict__ mcol, double* __restrict__ acc, int32_t count,
-                                      const double* __restrict__ ttab, int32_t n, int32_t q,
-                                      const double* __restrict__ rs) {
+                                      const double* __restrict__ ttab, int32_t n, int32_t q) {
   const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const int32_t s = mrow[i];
@@ -52,24 +50,18 @@ __global__ void batch_member_epilogue(float* __restrict__ Y, int32_t cols, const
   const double f = static_cast<double>(*y);
   double K = 0.0;
   for (int32_t r = 0; r <= q; ++r) K += ttab[static_cast<size_t>(r) * n + s];
-  if (rs) {
-    const double sv = rs[s];
-    K = sv > 0.0 ? K / (sv * sv) : 0.0;  // a vertex without edges starts and ends no walk
-  }
   acc[i] += f * K;
   *y = 0.0f;
 }
 
 // acc starts with the p = 0 term: every walk that starts at s (length 1..L) hits S_j at s.
 __global__ void batch_member_init(const int32_t* __restrict__ mrow, double* __restrict__ acc, int32_t count,
-                                  const double* __restrict__ ttab, int32_t n, int32_t L,
-                                  const double* __restrict__ rs) {
+                                  const double* __restrict__ ttab, int32_t n, int32_t L) {
   const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const int32_t s = mrow[i];
   double K = 0.0;
   for (int32_t r = 1; r <= L; ++r) K += ttab[static_cast<size_t>(r) * n + s];
-  if (rs) K = rs[s] > 0.0 ? K / rs[s] : 0.0;
   acc[i] = K;
 }
 
@@ -82,6 +74,139 @@ __global__ void batch_group_sum(const double* __restrict__ acc, const int32_t* _
   for (int32_t i = goff[j]; i < goff[j + 1]; ++i) s += acc[i];
   out[j] = s;
 }
+
+// ---------------------------------------------------------------- half-length batches (undirected)
+// Column j of a block is the hit vector h_t(v) = the walks of length t that end at v and visit S_j:
+// h_t = alpha A h_{t-1}, and on S_j every walk that ends there, h_t(s) = t_t(s), a row of the
+// walk-total table. A walk of length H + a hits S_j in its half of length a or else in the other:
+//   sum_v [ h_a(v) t_H(v) + (t_a(v) - h_a(v)) h_H(v) ],
+// so ceil(L/2) vectors (the first from counts) and one pass over them replace L sweeps: 512 groups on
+// a Barabasi-Albert graph of n = 10^6 (L = 9, blocks of 16 columns) took 41.2 ms with the first-visit
+// sweeps of the full length.
+
+// t_H(v) and P(v) = sum_{a=1..L-H} t_a(v), true values in FP32.
+__global__ void batch_totals(const double* __restrict__ T, int64_t n, int32_t n_active, int32_t L, int32_t H,
+                             const double* __restrict__ rs, float* __restrict__ tH, float* __restrict__ P) {
+  for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n_active; v += gridDim.x * blockDim.x) {
+    const double inv = rs ? 1.0 / rs[v] : 1.0;
+    double p = 0.0;
+    for (int32_t a = 1; a <= L - H; ++a) p += T[static_cast<size_t>(a) * n + v];
+    tH[v] = static_cast<float>(T[static_cast<size_t>(H) * n + v] * inv);
+    P[v] = static_cast<float>(p * inv);
+  }
+}
+
+// h_1 outside the groups: alpha per neighbour in S_j (equal terms: their order does not matter). One
+// warp per member, gridDim.y warps on a hub's.
+__global__ void batch_scatter(float* __restrict__ X, int32_t cols, const int32_t* __restrict__ mrow,
+                              const int32_t* __restrict__ mcol, int32_t count, const int32_t* __restrict__ rp,
+                              const int32_t* __restrict__ ci, float alpha) {
+  const int lane = threadIdx.x & 31;
+  const int32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (i >= count) return;
+  const int32_t s = mrow[i], c = mcol[i];
+  const int64_t e1 = rp[s + 1];
+  for (int64_t e = rp[s] + static_cast<int64_t>(blockIdx.y) * 32 + lane; e < e1; e += 32 * static_cast<int64_t>(gridDim.y))
+    atomicAdd(X + static_cast<size_t>(ci[e]) * cols + c, alpha);
+}
+
+// h_t on the groups' own rows: a row of the table (as stored: times s on a weighted graph).
+__global__ void batch_own(float* __restrict__ X, int32_t cols, const int32_t* __restrict__ mrow,
+                          const int32_t* __restrict__ mcol, int32_t count, const double* __restrict__ row,
+                          int32_t n_active) {
+  const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= count || mrow[i] >= n_active) return;
+  X[static_cast<size_t>(mrow[i]) * cols + mcol[i]] = static_cast<float>(row[mrow[i]]);
+}
+
+// The stored vectors of a block: x_t sits at slot (t - 1) % kBatchRing; V holds the sum of those
+// already folded (walk lengths 1..folded).
+constexpr int kBatchRing = 5;
+struct BatchVecs {
+  const float* ring;
+  int64_t stride;
+  float* V;  // nullptr: nothing folded
+  int32_t folded, H;
+};
+
+// V (+)= x_{folded+1} .. x_{folded+4}.
+__global__ void batch_fold(const BatchVecs b, int64_t quads) {
+  for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < quads;
+       q += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+    float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (b.folded > 0) a = reinterpret_cast<const float4*>(b.V)[q];
+#pragma unroll
+    for (int t = 0; t < kBatchRing - 1; ++t) {
+      const float4 x = reinterpret_cast<const float4*>(b.ring + b.stride * ((b.folded + t) % kBatchRing))[q];
+      a.x += x.x;
+      a.y += x.y;
+      a.z += x.z;
+      a.w += x.w;
+    }
+    reinterpret_cast<float4*>(b.V)[q] = a;
+  }
+}
+
+// The halves meet: score_j = sum_v [K + V t_H + (P - V) h_H], K = h_1 + .. + h_H, V = h_1 + .. +
+// h_{L-H}. A thread takes four columns of a row (always the same four); FP32 terms are summed
+// compensated per thread, in FP64 over threads and blocks, in a fixed order.
+template <int C>
+__global__ void __launch_bounds__(kThreads) batch_meet(const BatchVecs b, int32_t odd, int32_t n_active,
+                                                       const float* __restrict__ tH, const float* __restrict__ P,
+                                                       const float* __restrict__ rs, double* __restrict__ part,
+                                                       unsigned* __restrict__ done, int32_t groups,
+                                                       double* __restrict__ out) {
+  constexpr int Q = C / 4;  // float4s of a row
+  __shared__ double sm[kThreads][4];
+  __shared__ int is_last;
+  ColAcc<float, 4> acc;
+  acc.zero();
+  const int64_t quads = static_cast<int64_t>(n_active) * Q;
+  for (int64_t q = blockIdx.x * static_cast<int64_t>(kThreads) + threadIdx.x; q < quads;
+       q += static_cast<int64_t>(gridDim.x) * kThreads) {
+    const int32_t v = static_cast<int32_t>(q / Q);
+    float k[4] = {0.0f, 0.0f, 0.0f, 0.0f}, h[4];
+    if (b.folded > 0) {
+      const float4 x = __ldcs(reinterpret_cast<const float4*>(b.V) + q);
+      k[0] = x.x, k[1] = x.y, k[2] = x.z, k[3] = x.w;
+    }
+    for (int t = b.folded + 1; t < b.H; ++t) {
+      const float4 x = __ldcs(reinterpret_cast<const float4*>(b.ring + b.stride * ((t - 1) % kBatchRing)) + q);
+      k[0] += x.x, k[1] += x.y, k[2] += x.z, k[3] += x.w;
+    }
+    {
+      const float4 x = __ldcs(reinterpret_cast<const float4*>(b.ring + b.stride * ((b.H - 1) % kBatchRing)) + q);
+      h[0] = x.x, h[1] = x.y, h[2] = x.z, h[3] = x.w;
+    }
+    const float inv = rs ? 1.0f / rs[v] : 1.0f, t = __ldg(tH + v), p = __ldg(P + v);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const float hh = h[c] * inv, below = k[c] * inv, kk = below + hh, vv = odd ? below : kk;
+      acc.add(c, kk + vv * t + fmaxf(p - vv, 0.0f) * hh);
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < 4; ++c) sm[threadIdx.x][c] = acc.get(c);
+  __syncthreads();
+  if (threadIdx.x < C) {  // column threadIdx.x: the threads that hold its four
+    double x = 0.0;
+    for (int i = threadIdx.x / 4; i < kThreads; i += Q) x += sm[i][threadIdx.x & 3];
+    part[static_cast<size_t>(blockIdx.x) * C + threadIdx.x] = x;
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) is_last = atomicInc(done, gridDim.x - 1) == gridDim.x - 1;  // back to 0 for the next
+  __syncthreads();
+  if (!is_last) return;
+  __threadfence();
+  if (static_cast<int>(threadIdx.x) < groups) {
+    double x = 0.0;
+#pragma unroll 8
+    for (int i = 0; i < static_cast<int>(gridDim.x); ++i) x += __ldcg(part + static_cast<size_t>(i) * C + threadIdx.x);
+    out[threadIdx.x] = x;
+  }
+}
+constexpr int kBatchMeetBlocks = 456;  // three per SM
 
 int blocks_for(int64_t n, int per = 256) { return static_cast<int>(std::min<int64_t>((n + per - 1) / per, 152 * 32)); }
 
@@ -158,16 +283,15 @@ gedwalk_status autotune_batch(Graph& g, Workspace& ws, const Resolved& r) {
   GW_CUDA(cudaEventCreate(&e1));
   g.tune_log.clear();
   for (int c : kCand) {
-    const size_t vbytes = static_cast<size_t>(g.n) * c * 4;
-    if (ws.x0.ensure(vbytes, s) != GEDWALK_OK || ws.x1.ensure(vbytes, s) != GEDWALK_OK) break;
+    const size_t vec = static_cast<size_t>(g.n) * c;
+    if (ws.xs.ensure(2 * vec * sizeof(float), s) != GEDWALK_OK) break;
     GW_TRY(ensure_sweep_scratch(g, ws, c, false, s));
-    init_batch<<<blocks_for(static_cast<int64_t>(g.n) * c), 256, 0, s>>>(ws.x0.as<float>(), g.n, g.n, c, c,
-                                                                          nullptr);
+    init_batch<<<blocks_for(static_cast<int64_t>(g.n) * c), 256, 0, s>>>(ws.xs.as<float>(), g.n, g.n, c, c);
     GW_KCHECK();
     SweepArgs a = base_args(g, ws);
     a.alpha = r.alpha;
-    a.X = ws.x0.p;
-    a.Y = ws.x1.p;
+    a.X = ws.xs.p;
+    a.Y = ws.xs.as<float>() + vec;
     for (int w = 0; w < 2; ++w) GW_TRY(launch_sweep(MODE_PLAIN, false, c, a, s));
     const int reps = 5;
     GW_CUDA(cudaEventRecord(e0, s));
@@ -192,12 +316,87 @@ gedwalk_status autotune_batch(Graph& g, Workspace& ws, const Resolved& r) {
 int64_t score_batch_footprint(const Graph& g, int64_t members, int32_t groups) {
   const int64_t C = g.batch_cols > 0 ? g.batch_cols : 32;  // before tuning: the widest width tried
   const int64_t n = g.n;
-  int64_t b = 2 * n * C * 4;                                      // walk vectors x0, x1
-  b += members * (4 + 4 + 8) + static_cast<int64_t>(groups + 1) * 4 + 256;  // members, columns, sums
+  int64_t b = members * (4 + 4 + 8) + static_cast<int64_t>(groups + 1) * 4 + 256;  // members, columns, sums
   b += static_cast<int64_t>(std::max(g.plan.num_slices, 1)) * C * 4 + std::max(g.plan.num_heavy, 1) * 4;
-  b += static_cast<int64_t>(std::max(g.plan.num_slots, 1)) * C * 8 + C * kReduceParts * 8;
   b += static_cast<int64_t>(groups) * 8 + 64;
+  if (!g.directed) {
+    b += static_cast<int64_t>(g.n_active) * C * 4 * (kBatchRing + 1);  // the stored vectors and their sum
+    b += 2 * n * 4 + kBatchMeetBlocks * C * 8;
+    return b;
+  }
+  b += 2 * n * C * 4;  // walk vectors x0, x1
+  b += static_cast<int64_t>(std::max(g.plan.num_slots, 1)) * C * 8 + C * kReduceParts * 8;
   return b;
+}
+
+// The blocks of an undirected graph's batch; the members (rows, columns) are on the device, the scores
+// go to ws.small. The table holds rows 0..L (the caller keeps its lock).
+static gedwalk_status batch_runs(Graph& g, Workspace& ws, int C, const int32_t* offsets, int32_t G, const int32_t* mrow,
+                                 const int32_t* mcol, const Resolved& r, cudaStream_t s) {
+  const int32_t L = r.L, H = (L + 1) / 2;
+  const int64_t vec = static_cast<int64_t>(g.n_active) * C;
+  // x_1 .. x_H in a ring of kBatchRing; beyond that the oldest are folded into one vector behind it
+  const int slots = H > kBatchRing ? kBatchRing + 1 : g.weighted ? kBatchRing : H;
+  GW_TRY(ws.xs.ensure(static_cast<size_t>(vec) * slots * sizeof(float), s));
+  GW_TRY(ws.tail.ensure(static_cast<size_t>(g.n) * sizeof(float), s));
+  GW_TRY(ws.bound.ensure(static_cast<size_t>(g.n) * sizeof(float), s));
+  GW_TRY(ws.partial.ensure(static_cast<size_t>(std::max(g.plan.num_slices, 1)) * C * sizeof(float), s));
+  const size_t cbytes = static_cast<size_t>(std::max(g.plan.num_heavy, 1)) * sizeof(unsigned);
+  if (ws.counters.bytes < cbytes || !ws.counters.p) GW_TRY(ws.counters.ensure(cbytes, s, /*zero=*/true));
+  GW_TRY(ws.parts.ensure((static_cast<size_t>(kBatchMeetBlocks) * C + 1) * sizeof(double), s));
+  double* part = ws.parts.as<double>() + 1;
+  unsigned* done = ws.parts.as<unsigned>();
+  GW_CUDA(cudaMemsetAsync(done, 0, sizeof(double), s));
+  const double* T = g.ttab.as<double>();
+  const float* rs = g.weighted ? g.rs_f.as<float>() : nullptr;
+  batch_totals<<<blocks_for(g.n_active), 256, 0, s>>>(T, g.n, g.n_active, L, H, g.weighted ? g.rs_d.as<double>() : nullptr,
+                                                      ws.tail.as<float>(), ws.bound.as<float>());
+  GW_KCHECK();
+  float* ring = ws.xs.as<float>();
+  auto slot = [&](int32_t t) { return ring + vec * ((t + kBatchRing - 1) % kBatchRing); };  // x_0: the last slot
+  float* V = ring + vec * kBatchRing;
+  SweepArgs a = base_args(g, ws);
+  a.alpha = r.alpha;
+  const int meet = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(kBatchMeetBlocks, (vec / 4 + kThreads - 1) / kThreads)));
+  for (int32_t g0 = 0; g0 < G; g0 += C) {
+    const int32_t g1 = std::min(G, g0 + C);
+    const int32_t m0 = offsets[g0], cnt = offsets[g1] - m0;
+    auto own = [&](int32_t t) -> gedwalk_status {
+      if (cnt == 0) return GEDWALK_OK;
+      batch_own<<<blocks_for(cnt), 256, 0, s>>>(slot(t), C, mrow + m0, mcol + m0, cnt, T + static_cast<size_t>(t) * g.n,
+                                                g.n_active);
+      GW_KCHECK();
+      return GEDWALK_OK;
+    };
+    int32_t t = g.weighted ? 0 : 1;  // the first vector: x_0 = the groups' indicators, or x_1 from counts
+    GW_CUDA(cudaMemsetAsync(slot(t), 0, static_cast<size_t>(vec) * sizeof(float), s));
+    if (!g.weighted && cnt > 0) {
+      batch_scatter<<<dim3((cnt + 7) / 8, g.dmax > 4096 ? 32 : 1), 256, 0, s>>>(slot(1), C, mrow + m0, mcol + m0, cnt, a.rp, a.ci,
+                                                                             static_cast<float>(r.alpha));
+      GW_KCHECK();
+    }
+    GW_TRY(own(t));
+    BatchVecs b{ring, vec, V, 0, H};
+    for (++t; t <= H; ++t) {
+      if (t - b.folded > kBatchRing) {  // x_t takes the slot of x_{t-5}: fold x_{t-5} .. x_{t-2}
+        batch_fold<<<blocks_for(vec / 4), 256, 0, s>>>(b, vec / 4);
+        GW_KCHECK();
+        b.folded += kBatchRing - 1;
+      }
+      a.X = slot(t - 1);
+      a.Y = slot(t);
+      GW_TRY(launch_sweep(MODE_PLAIN, false, C, a, s));
+      GW_TRY(own(t));
+    }
+    double* out = ws.small.as<double>() + g0;
+#define GW_MEET(CC) \
+  if (C == CC) \
+    batch_meet<CC><<<meet, kThreads, 0, s>>>(b, L & 1, g.n_active, ws.tail.as<float>(), ws.bound.as<float>(), rs, part, done, g1 - g0, out);
+    GW_MEET(8) GW_MEET(16) GW_MEET(32) GW_MEET(64)
+#undef GW_MEET
+    GW_KCHECK();
+  }
+  return GEDWALK_OK;
 }
 
 gedwalk_status score_batch_impl(Graph& g, Workspace& ws, const int32_t* offsets, const int32_t* members_int,
@@ -228,20 +427,27 @@ gedwalk_status score_batch_impl(Graph& g, Workspace& ws, const int32_t* offsets,
     for (int32_t i = offsets[j]; i < offsets[j + 1]; ++i) hst[total + i] = j % C;
   memcpy(hst + 2 * total, offsets, sizeof(int32_t) * (G + 1));
   GW_CUDA(cudaMemcpyAsync(mrow, hst, up, cudaMemcpyHostToDevice, s));
+  GW_TRY(ws.small.ensure(static_cast<size_t>(G) * sizeof(double) + 64, s));
+  const double* T = g.ttab.as<double>();
+  if (!g.directed) {
+    GW_TRY(batch_runs(g, ws, C, offsets, G, mrow, mcol, r, s));
+    GW_CUDA(cudaMemcpyAsync(ws.pinned, ws.small.p, sizeof(double) * G, cudaMemcpyDeviceToHost, s));
+    GW_CUDA(cudaStreamSynchronize(s));
+    memcpy(scores, ws.pinned, sizeof(double) * G);
+    guard.ok = true;
+    return GEDWALK_OK;
+  }
   const size_t vbytes = static_cast<size_t>(g.n) * C * 4;
   GW_TRY(ws.x0.ensure(vbytes, s));
   GW_TRY(ws.x1.ensure(vbytes, s));
   GW_TRY(ensure_sweep_scratch(g, ws, C, false, s));
-  GW_TRY(ws.small.ensure(static_cast<size_t>(G) * sizeof(double) + 64, s));
-  const double* T = g.ttab.as<double>();
-  const double* rsd = g.weighted ? g.rs_d.as<double>() : nullptr;
   SweepArgs a = base_args(g, ws);
   a.alpha = r.alpha;
   if (g.n_active < g.n)
     GW_CUDA(cudaMemsetAsync(ws.x1.as<float>() + static_cast<size_t>(g.n_active) * C, 0,
                             sizeof(float) * C * (static_cast<size_t>(g.n) - g.n_active), s));
   if (total > 0) {
-    batch_member_init<<<blocks_for(total), 256, 0, s>>>(mrow, acc, static_cast<int32_t>(total), T, g.n, r.L, rsd);
+    batch_member_init<<<blocks_for(total), 256, 0, s>>>(mrow, acc, static_cast<int32_t>(total), T, g.n, r.L);
     GW_KCHECK();
   }
   for (int32_t g0 = 0; g0 < G; g0 += C) {
@@ -249,8 +455,7 @@ gedwalk_status score_batch_impl(Graph& g, Workspace& ws, const int32_t* offsets,
     const int32_t m0 = offsets[g0], m1 = offsets[g1];
     const int32_t cnt = m1 - m0;
     init_batch<<<blocks_for(static_cast<int64_t>(g.n) * C), 256, 0, s>>>(ws.x0.as<float>(), g.n, g.n_active, C,
-                                                                          g1 - g0,
-                                                                          g.weighted ? g.rs_f.as<float>() : nullptr);
+                                                                          g1 - g0);
     GW_KCHECK();
     if (cnt > 0) {
       zero_members<<<blocks_for(cnt), 256, 0, s>>>(ws.x0.as<float>(), C, mrow + m0, mcol + m0, cnt);
@@ -264,7 +469,7 @@ gedwalk_status score_batch_impl(Graph& g, Workspace& ws, const int32_t* offsets,
       GW_TRY(launch_sweep(MODE_PLAIN, false, C, a, s));
       if (cnt > 0) {
         batch_member_epilogue<<<blocks_for(cnt), 256, 0, s>>>(static_cast<float*>(nxt), C, mrow + m0, mcol + m0,
-                                                               acc + m0, cnt, T, g.n, r.L - p, rsd);
+                                                               acc + m0, cnt, T, g.n, r.L - p);
         GW_KCHECK();
       }
       std::swap(cur, nxt);
