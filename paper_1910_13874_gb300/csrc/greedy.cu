@@ -435,6 +435,8 @@ int64_t maximize_footprint(const Graph& g, const Resolved& r, int32_t flags, int
   const int64_t n = g.n, es = r.fp64 ? 8 : 4;
   if (!g.directed) {
     int64_t b = run_bytes(g, sh.tab_L, sh.cols_max, r.fp64, (flags & GEDWALK_GAINS_ALL) == 0);
+    if ((flags & GEDWALK_GAINS_ALL) && small_gain_cols(g, r.fp64) > 0)  // one launch's table, vectors and gains
+      b += n * (es * ((sh.tab_L + 1) / 2 + 3) + 8) + static_cast<int64_t>(std::max(g.plan.num_slots, 1)) * 8;
     return b + 4 * static_cast<int64_t>(k);  // (the final group, where it has to be scored)
   }
   const int64_t slices = std::max(std::max(g.plan.num_slices, g.plan_r.num_slices), 1);
@@ -539,7 +541,19 @@ gedwalk_status maximize_runs(Graph& g, Workspace& ws, const Resolved& r, const G
       const unsigned long long z = iso.zero(g, inS, kNoZero);  // isolated vertices gain nothing
       if (z != kNoZero) best = Cand{0.0, zero_internal(z), zero_caller(z)};
       std::vector<int32_t> batch;
-      for (int32_t v = 0; v <= g.n_active; ++v) {
+      const bool small = small_gain_cols(g, r.fp64) > 0;
+      if (small) {
+        std::vector<double> got(g.n_active);
+        GW_TRY(small_gains(g, ws, r, *S_all, got.data()));
+        for (int32_t v = 0; v < g.n_active; ++v) {
+          if (inS[v]) continue;
+          const Cand e{got[v], v, g.perm[v]};
+          if (best.v < 0 || cand_before(e, best)) best = e;
+          ++ws.st_evals;
+        }
+        ++ws.st_batches;
+      }
+      for (int32_t v = 0; !small && v <= g.n_active; ++v) {
         if (v < g.n_active && !inS[v]) batch.push_back(v);
         if (static_cast<int>(batch.size()) < sh.cols_all - 1 && !(v == g.n_active && !batch.empty())) continue;
         GW_TRY(eng.run(false, sh.cols_all, false, batch));
@@ -952,6 +966,13 @@ gedwalk_status gains_impl(Graph& g, Workspace& ws, const std::vector<int32_t>& S
   for (int32_t v : S_int) inS[v] = 1;
   for (int32_t v = 0; v < g.n; ++v) gains_caller[v] = 0.0;
   std::vector<int32_t> batch;
+  if (small_gain_cols(g, r.fp64) > 0) {
+    std::vector<double> got(g.n_active);
+    GW_TRY(small_gains(g, ws, r, S_int, got.data()));
+    for (int32_t v = 0; v < g.n_active; ++v) gains_caller[g.perm[v]] = got[v];
+    guard.ok = true;
+    return GEDWALK_OK;
+  }
   if (!g.directed) {  // an isolated vertex gains nothing
     RunEngine eng(g, ws, r, s);
     GW_TRY(eng.setup(r.L, cols_all, false, S_int));

@@ -105,6 +105,7 @@ struct Plan {
   int32_t num_slices = 0;  // heavy slices (units [0, num_slices))
   int32_t num_heavy = 0;   // heavy rows (degree > kHeavyDeg)
   int32_t num_slots = 0;   // num_units + num_heavy column-sum slots
+  int32_t num_long = 0;    // sorted plans: rows above 64 entries, a prefix
   DevBuf units;            // int4[num_units]
   DevBuf heavy;            // int4[num_heavy]: {row, first slice, slice count, 0}
 };
@@ -366,6 +367,10 @@ gedwalk_status score_batch_impl(Graph& g, Workspace& ws, const int32_t* offsets,
                                 int32_t G, const Resolved& r, double* scores);
 gedwalk_status maximize_impl(Graph& g, Workspace& ws, int32_t k, const Resolved& r, int32_t flags,
                              const std::vector<int32_t>& init_int, int32_t* group, double* gains, double* score);
+// Every vertex's gain on a small undirected graph in one launch (gains.cu): columns per block (0: the
+// graph is too large), and the gains of the rows [0, n_active) by internal id.
+int small_gain_cols(const Graph& g, bool fp64);
+gedwalk_status small_gains(Graph& g, Workspace& ws, const Resolved& r, const std::vector<int32_t>& S, double* out);
 gedwalk_status gains_impl(Graph& g, Workspace& ws, const std::vector<int32_t>& S_int, const Resolved& r,
                           double* gains_caller);
 
