@@ -77,14 +77,52 @@ struct WarpList {
   int tag = 0;
 };
 
+// One compare-exchange step of a bitonic network: the lane keeps the better or the worse of its own
+// entry and that of lane ^ j.
+__device__ __forceinline__ void list_exchange(float& v, int& id, int& tag, int j, bool keep_better) {
+  const float ov = __shfl_xor_sync(kFullMask, v, j);
+  const int oi = __shfl_xor_sync(kFullMask, id, j);
+  const int ot = __shfl_xor_sync(kFullMask, tag, j);
+  if (better(ov, oi, v, id) == keep_better && oi != id) {
+    v = ov;
+    id = oi;
+    tag = ot;
+  }
+}
+
 // Offers every lane's (x, ix, tag) where `want` holds. Only the lanes that beat the list's last
-// entry are inserted, one at a time (lowest lane first); after each insertion the others are
-// checked again against the new last entry. Ids must be distinct. All 32 lanes take part.
+// entry go in: a few of them one at a time (lowest lane first; after each insertion the others are
+// checked again against the new last entry), many of them by sorting the 32 offers (15 steps) and
+// merging the best 16 with the list (5 steps). An insertion costs about as much as three of those
+// steps, and a warp's first offers would take some thirty. Ids must be distinct. All 32 lanes take
+// part.
 __device__ __forceinline__ void warp_list_offer(WarpList& w, bool want, float x, int ix, int tag) {
   const int lane = threadIdx.x & 31;
   float tv = __shfl_sync(kFullMask, w.v, kTopK - 1);
   int ti = __shfl_sync(kFullMask, w.id, kTopK - 1);
-  unsigned m = __ballot_sync(kFullMask, want && better(x, ix, tv, ti));
+  const bool enters = want && better(x, ix, tv, ti);
+  unsigned m = __ballot_sync(kFullMask, enters);
+  if (__popc(m) > 5) {
+    float v = enters ? x : -1.0f;
+    int id = enters ? ix : INT_MAX, tg = tag;
+#pragma unroll
+    for (int k = 2; k <= 32; k <<= 1)
+#pragma unroll
+      for (int j = k >> 1; j > 0; j >>= 1) list_exchange(v, id, tg, j, ((lane & j) == 0) == ((lane & k) == 0));
+    // the best of list[i] and offer[15 - i] are the best 16 of both, a bitonic sequence
+    const int src = (kTopK - 1 - lane) & 31;
+    const float rv = __shfl_sync(kFullMask, v, src);
+    const int ri = __shfl_sync(kFullMask, id, src);
+    const int rt = __shfl_sync(kFullMask, tg, src);
+    if (lane < kTopK && better(rv, ri, w.v, w.id)) {
+      w.v = rv;
+      w.id = ri;
+      w.tag = rt;
+    }
+#pragma unroll
+    for (int j = kTopK / 2; j > 0; j >>= 1) list_exchange(w.v, w.id, w.tag, j, (lane & j) == 0);
+    return;
+  }
   while (m) {
     const int src = __ffs(m) - 1;
     const float cv = __shfl_sync(kFullMask, x, src);

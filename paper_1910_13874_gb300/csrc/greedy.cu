@@ -503,6 +503,7 @@ gedwalk_status maximize_runs(Graph& g, Workspace& ws, const Resolved& r, const G
   const bool select = !p.gains_all();
   RunEngine eng(g, ws, r, r.stream);
   eng.n_scan = p.stochastic() ? g.n : g.n_active;
+  eng.draws = p.stochastic();
   GW_TRY(eng.setup(sh.tab_L, sh.cols_max, select, init));
   GW_TRY(eng.set_length(p.adaptive() ? 1 : r.L, select));
   std::vector<char> inS(g.n, 0);

@@ -298,7 +298,7 @@ struct MeetArgs {
   const uint32_t* mask;
   const int32_t* perm;
   const float* tail;
-  float* bound;        // the last level's bounds
+  float* bound;        // stochastic greedy: the last level's bounds (else nullptr)
   Stale* stale;
   const float* rs_f;
   const double* rs_d;
@@ -329,25 +329,35 @@ __device__ __forceinline__ T pos(T x) {
 __device__ __forceinline__ void merge_level(const float* __restrict__ sel_v, const int* __restrict__ sel_id, int blocks,
                                             LevelSel* __restrict__ out) {
   const int lane = threadIdx.x & 31;
-  WarpList h;
-  for (int b0 = 0; b0 < blocks; b0 += 32) {
-    const int blk = b0 + lane;
+  constexpr int NH = (kMeetBlocks + 31) / 32;
+  float hv[NH];  // all the loads first: one round trip
+  int hi[NH];
+#pragma unroll
+  for (int k = 0; k < NH; ++k) {
+    const int blk = k * 32 + lane;
     const bool ok = blk < blocks;
-    const float x = ok ? __ldcg(sel_v + static_cast<size_t>(blk) * kTopK) : -1.0f;
-    const int ix = ok ? __ldcg(sel_id + static_cast<size_t>(blk) * kTopK) : INT_MAX;
-    warp_list_offer(h, ix != INT_MAX, x, ix, blk);
+    hv[k] = ok ? __ldcg(sel_v + static_cast<size_t>(blk) * kTopK) : -1.0f;
+    hi[k] = ok ? __ldcg(sel_id + static_cast<size_t>(blk) * kTopK) : INT_MAX;
+  }
+  WarpList h;
+#pragma unroll
+  for (int k = 0; k < NH; ++k)
+    if (k * 32 < blocks) warp_list_offer(h, hi[k] != INT_MAX, hv[k], hi[k], k * 32 + lane);
+  constexpr int NE = kTopK / 2;
+  float ev[NE];
+  int ei[NE];
+#pragma unroll
+  for (int k = 0; k < NE; ++k) {
+    const int src = 2 * k + (lane >> 4);
+    const int tag = __shfl_sync(kFullMask, h.tag, src);
+    const bool ok = __shfl_sync(kFullMask, h.id, src) != INT_MAX;
+    const size_t e = static_cast<size_t>(ok ? tag : 0) * kTopK + (lane & 15);
+    ev[k] = ok ? __ldcg(sel_v + e) : -1.0f;
+    ei[k] = ok ? __ldcg(sel_id + e) : INT_MAX;
   }
   WarpList f;
 #pragma unroll
-  for (int j = 0; j < kTopK; j += 2) {
-    const int src = j + (lane >> 4);
-    const int tag = __shfl_sync(kFullMask, h.tag, src);
-    const int hid = __shfl_sync(kFullMask, h.id, src);
-    const size_t e = static_cast<size_t>(hid != INT_MAX ? tag : 0) * kTopK + (lane & 15);
-    const float x = hid != INT_MAX ? __ldcg(sel_v + e) : -1.0f;
-    const int ix = hid != INT_MAX ? __ldcg(sel_id + e) : INT_MAX;
-    warp_list_offer(f, ix != INT_MAX, x, ix, 0);
-  }
+  for (int k = 0; k < NE; ++k) warp_list_offer(f, ei[k] != INT_MAX, ev[k], ei[k], 0);
   if (lane < kTopK) {
     out->val[lane] = f.v;
     out->id[lane] = f.id;
@@ -389,9 +399,18 @@ __device__ __forceinline__ void block_levels(WarpList (&w)[NL], float* sv, int* 
 // T_d = S + {c_1..c_d}, phi(T_d) = column 0 - columns 1..d (a walk that avoids S avoids c_1..c_d or
 // has a first c_j among them, counted in column j); differences are clamped at 0, and a vertex
 // without a neighbour outside T_d (an exact count) has bound exactly 0. The last block to finish
-// merges the lists and adds the gain sums in block order. Bound by the H rows it streams.
+// merges the lists and adds the gain sums in block order.
+//
+// Meant to stream H rows of the vectors (R-MAT scale 22: 384 MB, 57 us at the copy rate). Bounds and
+// offers for seven levels cost five times that, so a warp skips them where none of its 32 rows can
+// enter any level's list: bounds fall with the level, so the first level's bound without its
+// correction, against the lowest last entry of the lists, decides. The rows come by decreasing
+// degree, so after a warp's first iteration few pass. A bound of exactly 0 matters only when every
+// bound is 0, so its vertex is recorded only while the warp's list is empty (an atomic per such row,
+// all to one address, would serialise). 279 -> 150 us; on
+// 10^5 rows, where a warp has one iteration, the lists cost most (device_util.cuh): 97 -> 63 us.
 template <typename T, int C, bool CHAIN, bool SEL>
-__global__ void __launch_bounds__(kThreads, 2) meet_kernel(const MeetArgs a) {
+__global__ void __launch_bounds__(kThreads, kMeetPerSM) meet_kernel(const MeetArgs a) {
   constexpr int D = C - 1;
   constexpr int NL = CHAIN ? D : 1;
   constexpr int NW = kThreads / 32;
@@ -426,122 +445,158 @@ __global__ void __launch_bounds__(kThreads, 2) meet_kernel(const MeetArgs a) {
   int nsampled[NL];
 #pragma unroll
   for (int l = 0; l < NL; ++l) nsampled[l] = 0;
+  float enter = -1.0f;     // lowest last entry of the warp's lists (-1: one is not full)
+  unsigned empty = ~0u;    // levels whose list is empty
   const int32_t stride = gridDim.x * kThreads;
   for (int32_t base = blockIdx.x * kThreads + warp * 32; base < a.n_scan; base += stride) {
     const int32_t v = base + lane;
     const bool ok = v < a.n_scan;
     const bool has = v < a.n_active;
-    // sums over t: B to H-1, A2 to H-2, A4 to H-4; x_1, x_2 and x_H
-    T B[C], A2[C], A4[C], f1[C], f2[C], xh[C];
+    const T* __restrict__ row = xs + static_cast<size_t>(has ? v : 0) * C;
+    // the row's sums over t = 1..H-1 and x_H
+    T B[C], xh[C];
 #pragma unroll
-    for (int c = 0; c < C; ++c) B[c] = A2[c] = A4[c] = f1[c] = f2[c] = xh[c] = T(0);
+    for (int c = 0; c < C; ++c) B[c] = xh[c] = T(0);
+    T inv = T(1);
     if (has) {
-      const T* p = xs + static_cast<size_t>(v) * C;
-#pragma unroll 2
-      for (int t = 1; t <= H; ++t, p += a.stride) {
-        T x[C];
+      const T* p = row;
+      auto load = [&](T (&x)[C]) {
         if constexpr (sizeof(T) * C >= 16) {
 #pragma unroll
           for (int k = 0; k < static_cast<int>(sizeof(T)) * C / 16; ++k) {
-            const float4 q = __ldcs(reinterpret_cast<const float4*>(p) + k);
+            const float4 q = __ldg(reinterpret_cast<const float4*>(p) + k);
             memcpy(&x[k * (16 / static_cast<int>(sizeof(T)))], &q, 16);
           }
         } else {
 #pragma unroll
-          for (int c = 0; c < C; ++c) x[c] = __ldcs(p + c);
+          for (int c = 0; c < C; ++c) x[c] = __ldg(p + c);
         }
+      };
+#pragma unroll 4
+      for (int t = 1; t < H; ++t, p += a.stride) {
+        T x[C];
+        load(x);
 #pragma unroll
-        for (int c = 0; c < C; ++c) {
-          if (SEL) {
-            if (t <= H - 4) A4[c] += x[c];
-            if (t <= H - 2) A2[c] += x[c];
-            if (t == 1) f1[c] = x[c];
-            if (t == 2) f2[c] = x[c];
-          }
-          if (t < H) B[c] += x[c];
-          else xh[c] = x[c];
-        }
+        for (int c = 0; c < C; ++c) B[c] += x[c];
       }
+      load(xh);
       if (rs) {
-        const T inv = T(1) / rs[v];
+        inv = T(1) / rs[v];
 #pragma unroll
         for (int c = 0; c < C; ++c) {
           B[c] *= inv;
           xh[c] *= inv;
-          if (SEL) {
-            A2[c] *= inv;
-            A4[c] *= inv;
-            f1[c] *= inv;
-            f2[c] *= inv;
-          }
         }
       }
     }
-    // running values of the level's phi: sums to H and to L - H, x_H, and what the bound needs
-    T rh = xh[0], rb = B[0];
-    T r2 = A2[0], r4 = A4[0], q1 = f1[0], q2 = f2[0];
-    bool out = false;
-    int dg = 0;
-    float tail = 0.0f;
-    Stale st{0.0f, -1};
-    uint32_t caller = 0;
-    if (SEL && ok) {
-      out = in_set(a.mask, v);
-      if (has) {
-        dg = a.rp[v + 1] - a.rp[v] - a.cnt[v];
-        tail = a.tail[v];
+    if (SEL) {
+      bool out = false;
+      int dg = 0;
+      float tail = 0.0f;
+      if (ok) {
+        out = in_set(a.mask, v);
+        if (has) {
+          dg = a.rp[v + 1] - a.rp[v] - a.cnt[v];
+          tail = a.tail[v];
+        }
       }
-      st = a.stale[v];
-      if (sampling) caller = static_cast<uint32_t>(__ldg(a.perm + v));
-    }
-    const float slack_u = __fmul_ru(e, f_up(B[0] + xh[0])), slack_2 = e * f_up(A2[0]), slack_4 = e * f_up(A4[0]);
-    const float slack_1 = e * f_up(f1[0]), slack_q = e * f_up(f2[0]), slack_h = e * f_up(xh[0]);
-    bool evaluated = false;
-    if (SEL && !CHAIN) {
+      const float K0 = f_up(B[0] + xh[0]);
+      const float most_u = __fmul_ru(K0, __fadd_ru(infl, e));
+      const float most = dg > 0 ? __fadd_ru(__fmaf_ru(most_u, most_u, __fadd_ru(most_u, most_u)), tail) : 0.0f;
+      // some row of the warp may enter a list
+      if (__any_sync(kFullMask, ok && !out && !(__fmul_ru(most, 1.00001f) < enter)) || a.bound) {
+        bool evaluated = false;
+        Stale st{0.0f, -1};
+        uint32_t caller = 0;
+        if (ok) {
+          st = a.stale[v];
+          if (sampling) caller = static_cast<uint32_t>(__ldg(a.perm + v));
+          if (!CHAIN) {
 #pragma unroll
-      for (int j = 0; j < D; ++j) evaluated |= s_cand[j] == v;
+            for (int j = 0; j < D; ++j) evaluated |= s_cand[j] == v;
+          }
+        }
+        // a column's sums over t to H-1, H-2 and H-4, x_1, x_2 and x_H (what is not at hand read again
+        // from the row: few warps come here on a large graph)
+        struct Col {
+          T b, b2, b4, f1, f2, h;
+        };
+        auto at = [&](int t, int c) {
+          return has && t >= 1 ? __ldg(row + static_cast<size_t>(t - 1) * a.stride + c) * inv : T(0);
+        };
+        auto column = [&](int c) {
+          Col k;
+          k.f1 = at(1, c);
+          k.f2 = H >= 2 ? at(2, c) : T(0);
+          const T x1 = at(H - 1, c), x2 = at(H - 2, c), x3 = at(H - 3, c);
+          k.b = B[c];
+          k.h = xh[c];
+          k.b2 = k.b - x1;
+          k.b4 = k.b2 - x2 - x3;
+          return k;
+        };
+        Col r = column(0);  // the level's phi
+        const Col r0 = r;
+#pragma unroll
+        for (int d = 0; d < NL; ++d) {
+          float ub = 0.0f;
+          if (dg > 0) {
+            const float U = __fmaf_ru(f_up(pos(r.b + r.h)), infl, __fmul_ru(e, K0));
+            const float p1lo = fmaxf(0.0f, __fsub_rd(f_down(pos(r.f1)), e * f_up(r0.f1)));
+            float s2, s4 = 0.0f;
+            if (rs) {  // Cauchy-Schwarz: sum of squared weights >= (their sum)^2 / their number
+              s2 = __fdiv_rd(__fmul_rd(p1lo, p1lo), static_cast<float>(dg));
+            } else {
+              s2 = __fmul_rd(al2, static_cast<float>(dg));
+              const float p2lo = fmaxf(0.0f, __fsub_rd(f_down(pos(r.f2)), e * f_up(r0.f2)));
+              const float p1up = __fadd_ru(f_up(pos(r.f1)), e * f_up(r0.f1));
+              s4 = fmaxf(0.0f, __fsub_rd(__fmul_rd(al2, p2lo), __fmul_ru(al3, p1up)));
+            }
+            float corr = 0.0f;
+            if (H >= 2) corr = __fmul_rd(s2, __fadd_rd(1.0f, fmaxf(0.0f, __fsub_rd(f_down(pos(r.b2)), e * f_up(r0.b2)))));
+            if (H >= 4)
+              corr = __fadd_rd(corr, __fmul_rd(s4, __fadd_rd(1.0f, fmaxf(0.0f, __fsub_rd(f_down(pos(r.b4)), e * f_up(r0.b4))))));
+            corr = __fmul_rd(corr, keep);
+            const float F = fmaxf(0.0f, __fsub_ru(U, corr));
+            ub = __fadd_ru(__fmaf_ru(F, U, __fadd_ru(F, U)), tail);
+            if (odd) {  // the pair (H, H) is longer than L
+              const float hlo = fmaxf(0.0f, __fsub_rd(f_down(pos(r.h)), e * f_up(r0.h)));
+              ub = __fsub_ru(ub, __fmul_rd(hlo, fmaxf(0.0f, __fsub_rd(hlo, corr))));
+            }
+            if (!(ub >= 0.0f)) ub = INFINITY;  // overflow: nothing is known
+            if (st.step >= 0 && st.ub < ub) ub = st.ub;
+          }
+          if (d == NL - 1 && ok && a.bound) a.bound[v] = ub;
+          bool want = ok && !out;
+          if (want && in.thr[d] != ~0ull) want = sample_hash(in.seed, static_cast<uint32_t>(step + d), caller) < in.thr[d];
+          nsampled[d] += want;
+          want = want && st.step != step + d && !(CHAIN ? s_cand[d] == v : evaluated);
+          if (want && ub == 0.0f && (empty >> d & 1u))
+            atomicMin(&a.d->out.lv[d].zero_min,
+                      (static_cast<unsigned long long>(__ldg(a.perm + v)) << 32) | static_cast<uint32_t>(v));
+          warp_list_offer(w[d], want && ub != 0.0f, ub, v, 0);
+          if ((empty >> d & 1u) && __shfl_sync(kFullMask, w[d].id, 0) != INT_MAX) empty &= ~(1u << d);
+          if (CHAIN && d + 1 < NL) {
+            const Col k = column(d + 1);
+            r.b -= k.b;
+            r.b2 -= k.b2;
+            r.b4 -= k.b4;
+            r.f1 -= k.f1;
+            r.f2 -= k.f2;
+            r.h -= k.h;
+            dg -= k.f1 > T(0);
+            out |= s_cand[d] == v;
+          }
+        }
+        enter = INFINITY;
+#pragma unroll
+        for (int l = 0; l < NL; ++l) enter = fminf(enter, __shfl_sync(kFullMask, w[l].v, kTopK - 1));
+      }
     }
+    // gain terms of candidate d + 1 under its base set
+    T rb = B[0], rh = xh[0];
 #pragma unroll
     for (int d = 0; d < D; ++d) {
-      if (SEL && d < NL) {
-        float ub = 0.0f;
-        if (dg > 0) {
-          const float U = __fmaf_ru(f_up(pos(rb + rh)), infl, slack_u);
-          const float p1lo = fmaxf(0.0f, __fsub_rd(f_down(pos(q1)), slack_1));
-          float s2, s4 = 0.0f;
-          if (rs) {  // Cauchy-Schwarz: sum of squared weights >= (their sum)^2 / their number
-            s2 = __fdiv_rd(__fmul_rd(p1lo, p1lo), static_cast<float>(dg));
-          } else {
-            s2 = __fmul_rd(al2, static_cast<float>(dg));
-            const float p2lo = fmaxf(0.0f, __fsub_rd(f_down(pos(q2)), slack_q));
-            const float p1up = __fadd_ru(f_up(pos(q1)), slack_1);
-            s4 = fmaxf(0.0f, __fsub_rd(__fmul_rd(al2, p2lo), __fmul_ru(al3, p1up)));
-          }
-          float corr = 0.0f;
-          if (H >= 2) corr = __fmul_rd(s2, __fadd_rd(1.0f, fmaxf(0.0f, __fsub_rd(f_down(pos(r2)), slack_2))));
-          if (H >= 4)
-            corr = __fadd_rd(corr, __fmul_rd(s4, __fadd_rd(1.0f, fmaxf(0.0f, __fsub_rd(f_down(pos(r4)), slack_4)))));
-          corr = __fmul_rd(corr, keep);
-          const float F = fmaxf(0.0f, __fsub_ru(U, corr));
-          ub = __fadd_ru(__fmaf_ru(F, U, __fadd_ru(F, U)), tail);
-          if (odd) {  // the pair (H, H) is longer than L
-            const float hlo = fmaxf(0.0f, __fsub_rd(f_down(pos(rh)), slack_h));
-            ub = __fsub_ru(ub, __fmul_rd(hlo, fmaxf(0.0f, __fsub_rd(hlo, corr))));
-          }
-          if (!(ub >= 0.0f)) ub = INFINITY;  // overflow: nothing is known
-          if (st.step >= 0 && st.ub < ub) ub = st.ub;
-        }
-        if (d == NL - 1 && ok && a.bound) a.bound[v] = ub;
-        bool want = ok && !out;
-        if (want && in.thr[d] != ~0ull) want = sample_hash(in.seed, static_cast<uint32_t>(step + d), caller) < in.thr[d];
-        nsampled[d] += want;
-        want = want && st.step != step + d && !(CHAIN ? s_cand[d] == v : evaluated);
-        if (want && ub == 0.0f)
-          atomicMin(&a.d->out.lv[d].zero_min,
-                    (static_cast<unsigned long long>(__ldg(a.perm + v)) << 32) | static_cast<uint32_t>(v));
-        warp_list_offer(w[d], want && ub != 0.0f, ub, v, 0);
-      }
-      // gain terms of candidate d + 1 under the level's set
       const T k = B[d + 1] + xh[d + 1];
       const T vv = odd ? B[d + 1] : k;
       const T pp = odd ? pos(rb) : pos(rb + rh);
@@ -549,14 +604,6 @@ __global__ void __launch_bounds__(kThreads, 2) meet_kernel(const MeetArgs a) {
       if (CHAIN) {
         rb -= B[d + 1];
         rh -= xh[d + 1];
-        if (SEL) {
-          r2 -= A2[d + 1];
-          r4 -= A4[d + 1];
-          q1 -= f1[d + 1];
-          q2 -= f2[d + 1];
-          dg -= f1[d + 1] > T(0);
-          out |= s_cand[d] == v;
-        }
       }
     }
   }
@@ -938,7 +985,7 @@ gedwalk_status RunEngine::issue(bool chain, int cols, bool select, bool profile,
   m.mask = ws.mask.as<uint32_t>();
   m.perm = g.perm_d.as<int32_t>();
   m.tail = ws.tail.as<float>();
-  m.bound = ws.bound.as<float>();
+  m.bound = draws ? ws.bound.as<float>() : nullptr;
   m.stale = ws.stale.as<Stale>();
   m.rs_f = g.weighted ? g.rs_f.as<float>() : nullptr;
   m.rs_d = g.weighted ? g.rs_d.as<double>() : nullptr;
@@ -969,7 +1016,7 @@ gedwalk_status RunEngine::run(bool chain, int cols, bool select, const std::vect
   memcpy(&abits, &r.alpha, 8);
   auto bits = [](const void* p) { return static_cast<uint64_t>(reinterpret_cast<uintptr_t>(p)); };
   Sequence q;
-  q.key = mix_all({uint64_t(mode), uint64_t(cols), uint64_t(r.fp64), uint64_t(L), uint64_t(select), uint64_t(n_scan), abits,
+  q.key = mix_all({uint64_t(mode), uint64_t(cols), uint64_t(r.fp64), uint64_t(L), uint64_t(select), uint64_t(n_scan), uint64_t(draws), abits,
                    bits(&g), bits(s), bits(ws.xs.p), bits(ws.cnt.p), bits(ws.mask.p), bits(ws.parts.p), bits(ws.small.p),
                    bits(ws.partial.p), bits(ws.counters.p), bits(ws.stale.p), bits(ws.sel.p), bits(ws.tail.p),
                    bits(ws.bound.p), bits(ws.run_io), bits(g.rp.p), bits(g.ci.p), bits(g.plan.units.p)});

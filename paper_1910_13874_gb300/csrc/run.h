@@ -13,7 +13,8 @@ namespace gw {
 constexpr int kRunCols = 16;            // widest run: column 0 and 15 candidates
 constexpr int kRunCands = kRunCols - 1;
 constexpr int kRunLevels = 7;           // lookahead levels with a selection of their own
-constexpr int kMeetBlocks = 304;        // two resident blocks of the meeting pass per SM
+constexpr int kMeetPerSM = 3;           // resident blocks of the meeting pass per SM
+constexpr int kMeetBlocks = 152 * kMeetPerSM;
 
 // What a run is told, copied to the device as its first operation.
 struct RunIn {
@@ -77,6 +78,7 @@ struct RunEngine {
   cudaStream_t s;
   int32_t L = 0, H = 0;
   int32_t n_scan = 0;  // rows of the selections (stochastic greedy scans isolated vertices too)
+  bool draws = false;  // stochastic greedy: the runs keep the last level's bounds for guess()
   int64_t sweeps = 0;
   RunIn* in = nullptr;   // pinned; step, seed, thr and the stale list are the caller's to fill
   RunOut* out = nullptr; // pinned; valid after run() or guess()
