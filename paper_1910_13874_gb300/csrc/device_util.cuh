@@ -149,30 +149,4 @@ __device__ __forceinline__ void warp_list_offer(WarpList& w, bool want, float x,
   }
 }
 
-// Merges the NW warp lists of a block into warp 0's list (staged through shared memory sv/si/st,
-// NW * kTopK entries each). Every thread of the block calls it.
-template <int NW>
-__device__ void block_list_merge(WarpList& w, float* sv, int* si, int* st) {
-  static_assert(kTopK == 16, "two warp lists per 32-lane offer");
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane < kTopK) {
-    sv[warp * kTopK + lane] = w.v;
-    si[warp * kTopK + lane] = w.id;
-    st[warp * kTopK + lane] = w.tag;
-  }
-  __syncthreads();
-  if (warp == 0) {
-    for (int j = 1; j < NW; j += 2) {  // lists j and j + 1 on lanes 0-15 and 16-31
-      const int src = j + (lane >> 4);
-      const bool ok = src < NW;
-      const int e = src * kTopK + (lane & 15);
-      const float x = ok ? sv[e] : -1.0f;
-      const int ix = ok ? si[e] : INT_MAX;
-      const int t = ok ? st[e] : 0;
-      warp_list_offer(w, ix != INT_MAX, x, ix, t);
-    }
-  }
-  __syncthreads();
-}
-
 }  // namespace gw

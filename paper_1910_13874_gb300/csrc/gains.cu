@@ -168,7 +168,7 @@ gedwalk_status small_gains(Graph& g, Workspace& ws, const Resolved& r, const std
     a.X = cur;
     a.Y = nxt;
     a.Mout = ws.mtab.as<char>() + static_cast<size_t>(t) * n * es;
-    GW_TRY(launch_sweep(MODE_FUSED, fp64, 1, a, s));
+    GW_TRY(launch_sweep(MODE_MISS, fp64, 1, a, s));
     std::swap(cur, nxt);
   }
   GainArgs q{};

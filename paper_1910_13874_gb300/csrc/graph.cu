@@ -112,7 +112,7 @@ double sweep_bytes(int mode, bool fp64, int cols, int32_t n, int64_t nnz, bool w
   const double es = mode == MODE_TOTALS ? 8.0 : (fp64 ? 8.0 : 4.0);
   double b = 4.0 * double(nnz) + 4.0 * (double(n) + 1.0) + 2.0 * cols * es * double(n);
   if (mode != MODE_TOTALS && mode != MODE_PLAIN) b += double(n) / 8.0;
-  if (mode == MODE_FUSED) b += es * double(n);
+  if (mode == MODE_MISS) b += es * double(n);
   if (weighted) b += es * double(n);  // the vertex scales
   return b;
 }
@@ -975,18 +975,21 @@ gedwalk_status ensure_totals(Graph& g, double alpha, int32_t rows, cudaStream_t 
   return GEDWALK_OK;
 }
 
-gedwalk_status totals_into(Graph& g, Workspace& ws, double* T, double alpha, int32_t rows, cudaStream_t s) {
+gedwalk_status totals_into(Graph& g, Workspace& ws, double* T, double alpha, int32_t from, int32_t rows, bool rev,
+                           cudaStream_t s) {
   const size_t n = static_cast<size_t>(g.n);
   GW_TRY(ensure_sweep_scratch(g, ws, 1, true, s));
-  if (g.weighted) {
-    GW_CUDA(cudaMemcpyAsync(T, g.rs_d.p, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
-  } else {
-    fill_f64_kernel<<<grid_for(g.n), 256, 0, s>>>(T, g.n, 1.0);
-    GW_KCHECK();
+  if (from == 0) {
+    if (g.weighted) {
+      GW_CUDA(cudaMemcpyAsync(T, g.rs_d.p, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    } else {
+      fill_f64_kernel<<<grid_for(g.n), 256, 0, s>>>(T, g.n, 1.0);
+      GW_KCHECK();
+    }
   }
-  SweepArgs a = base_args(g, ws);
+  SweepArgs a = rev ? base_args_rev(g, ws) : base_args(g, ws);
   a.alpha = alpha;
-  for (int32_t r = 1; r < rows; ++r) {
+  for (int32_t r = std::max(from, 1); r < rows; ++r) {
     a.X = T + static_cast<size_t>(r - 1) * n;
     a.Y = T + static_cast<size_t>(r) * n;
     if (g.n_active < g.n)
@@ -994,6 +997,29 @@ gedwalk_status totals_into(Graph& g, Workspace& ws, double* T, double alpha, int
                               sizeof(double) * (n - static_cast<size_t>(g.n_active)), s));
     GW_TRY(launch_sweep(MODE_TOTALS, true, 1, a, s));
   }
+  return GEDWALK_OK;
+}
+
+gedwalk_status ensure_totals_fwd(Graph& g, Workspace& ws, double alpha, int32_t rows, cudaStream_t s) {
+  {
+    std::shared_lock<std::shared_mutex> rl(g.tt_lock);
+    if (g.ttf_alpha == alpha && rows <= g.ttf_rows) return GEDWALK_OK;
+  }
+  std::unique_lock<std::shared_mutex> wl(g.tt_lock);
+  if (g.ttf_alpha != alpha) g.ttf_rows = 0;
+  if (g.ttf_alpha == alpha && rows <= g.ttf_rows) return GEDWALK_OK;
+  g.ttf_alpha = -1.0;  // not valid until its rows are done
+  const size_t need = static_cast<size_t>(rows) * g.n * sizeof(double);
+  int32_t from = g.ttf_rows;
+  g.ttf_rows = 0;
+  if (g.ttab_f.bytes < need) {
+    GW_TRY(g.ttab_f.ensure(need, s));
+    from = 0;
+  }
+  GW_TRY(totals_into(g, ws, g.ttab_f.as<double>(), alpha, from, rows, false, s));
+  GW_CUDA(cudaStreamSynchronize(s));
+  g.ttf_alpha = alpha;
+  g.ttf_rows = rows;
   return GEDWALK_OK;
 }
 

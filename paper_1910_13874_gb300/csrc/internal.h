@@ -137,8 +137,8 @@ struct SweepGraph {
 // creates one per concurrent request slot.
 struct Workspace {
   DevBuf x0, x1;     // walk vectors, [n][C]
-  DevBuf mtab;       // directed graphs: phi^miss table, [(L+1)][n]
-  DevBuf ztab;       // directed graphs: psi^miss table (walks in the other orientation), [(L+1)][n]
+  DevBuf mtab;       // gains of a small graph: phi^miss table, [(H+1)][n]
+  DevBuf ztab;       // runs without a shared walk-total table: the call's own, FP64
   DevBuf pvec;       // power iteration: three FP64 vectors and the statistics
   DevBuf partial;    // heavy-slice partial sums, [num_slices][C]
   DevBuf counters;   // heavy-row arrival counters, [num_heavy] (kept at 0 between launches)
@@ -213,6 +213,10 @@ struct Graph {
   int32_t tt_rows = 0;
   DevBuf ttab;
   std::vector<double> Wa;
+  // directed graphs: the table of the other orientation (walks that start at a vertex), made on demand
+  double ttf_alpha = -1.0;
+  int32_t ttf_rows = 0;
+  DevBuf ttab_f;
   DevBuf Wa_d;  // the same sums on the device, where the truncation test reads them
   // readers of ttab hold it shared; growing or replacing the table holds it exclusively
   std::shared_mutex tt_lock;
@@ -242,8 +246,7 @@ struct Graph {
 enum SweepMode : int {
   MODE_TOTALS = 0,  // y = alpha A x, FP64, stores the column sum
   MODE_SCORE = 1,   // directed scoring: two-state hit/miss step, sums h
-  MODE_FUSED = 2,   // directed greedy: column 0 = phi^miss under S, columns 1.. candidate columns
-  MODE_CAND = 3,    // directed greedy: candidate columns only; candidate rows read phi^miss from a table
+  MODE_MISS = 2,    // phi^miss under S, stored in a table too
   MODE_PLAIN = 4,   // batched scoring: y = alpha A x, no mask
   MODE_LOOK = 5,    // run, chain: phi^miss under S, then the walks through c_j avoiding S + {c_1..c_{j-1}}
   MODE_PAR = 6,     // run: phi^miss under S, then the walks through each c_j avoiding S
@@ -267,7 +270,6 @@ struct SweepArgs {
   double* slots;
   int32_t accumulate;
   void* Mout;
-  const void* Min;
   const int32_t* cand;
   const int32_t* live;  // runs: whether candidate j has a neighbour outside its base set
   int32_t hub;  // rows [0, hub) of x are gathered with L1 retention priority (set by the launcher)
@@ -329,7 +331,7 @@ struct Resolved {
 struct GreedyShape {
   int32_t levels;     // lookahead levels per run of sweeps (1 = no lookahead)
   int32_t cols_fused; // columns of the fused sweep (phi^miss + speculative candidates)
-  int32_t cols_cand;  // columns of a candidate batch (undirected: phi^miss and the candidates)
+  int32_t cols_cand;  // columns of a candidate batch (phi^miss and the candidates)
   int32_t cols_all;   // columns per batch of GEDWALK_GAINS_ALL
   int32_t tab_L;      // rows 0..tab_L of every phi^miss table
   int32_t ell_max;    // adaptive: the largest walk length it may reach (else L)
@@ -344,9 +346,12 @@ int64_t score_batch_footprint(const Graph& g, int64_t members, int32_t groups);
 gedwalk_status resolve(Graph& g, const gedwalk_params* p, double eps_override, Resolved* r);
 // Ensures the FP64 walk-total table holds rows 0..rows-1 for alpha.
 gedwalk_status ensure_totals(Graph& g, double alpha, int32_t rows, cudaStream_t s);
-// Walk totals t_0..t_{rows-1} (FP64, rows g.n apart) into a table of the caller's, with the caller's
-// workspace (undirected graphs).
-gedwalk_status totals_into(Graph& g, Workspace& ws, double* T, double alpha, int32_t rows, cudaStream_t s);
+// Walk totals t_from..t_{rows-1} (FP64, rows g.n apart) into a table of the caller's that holds the
+// rows before, with the caller's workspace: walks that start at a vertex, or (rev) that end there.
+gedwalk_status totals_into(Graph& g, Workspace& ws, double* T, double alpha, int32_t from, int32_t rows, bool rev,
+                           cudaStream_t s);
+// Directed graphs: the table of the walks that start at a vertex (ttab holds those that end there).
+gedwalk_status ensure_totals_fwd(Graph& g, Workspace& ws, double alpha, int32_t rows, cudaStream_t s);
 // Truncation length from the chosen tail bound (device-side test).
 gedwalk_status truncation_length(Graph& g, double alpha, double eps, int32_t* L, double* bound, cudaStream_t s,
                                  int32_t kind = 0);

@@ -1,5 +1,5 @@
-// Runs of the greedy maximisation on an undirected graph: sweeps of half the walk length and the
-// pass in which the halves meet.
+// Runs of the greedy maximisation: sweeps of half the walk length and the pass in which the halves
+// meet.
 //
 // With M = alpha 1_{V\S} A symmetric on V \ S, a walk of length a + b that avoids S is a walk of
 // length a and one of length b that end at the same vertex v (its vertex number a). So with
@@ -16,6 +16,12 @@
 // The first sweep is no sweep either: phi_1(v) = alpha |N(v) \ S| is a count kept per vertex, and
 // k_1 is alpha on the candidate's neighbours. (Weighted graphs sweep from the unit vectors.)
 //
+// Directed graphs keep two sets of vectors: walks that start at v (sweeps along the given rows) and
+// walks that end at v (sweeps along the reverse CSR). A walk of length H + a is a walk of length a
+// that ends at v and one of length H that starts there, so with the starting walks phi, k and the
+// ending walks psi, j:  gain(c) = sum_v [ K(v) + V(v) phi_H(v) + (P(v) - V(v)) k_H(v) ] with V and P
+// summed over j and psi. As many sweeps as the full length in one orientation, for up to seven steps.
+//
 // Bounds. The gain pairs first visits with continuations, sum_{1<=p+q<=L} f_p phi_q at c, where
 // f_p <= phi_p counts the walks whose only visit to c is their end: f_p = phi_p - sum_m s_m phi_{p-m}
 // with s_m the closed walks from c that return first at step m. Any lower bounds of s_m give an
@@ -23,7 +29,7 @@
 // v != c). With p, q <= H all pairs but (0,0) (and, for odd L, (H,H)) belong to the sum, so it is
 // F + U + F U with U = sum phi_t, F = sum f_t: no convolution. The pairs with p or q above H are
 // bounded once per maximisation by their value without S (walks avoiding S only get fewer as S
-// grows), from the walk-total table.
+// grows), from the walk-total tables. (Directed: F sums psi, U phi; the returns are not counted.)
 //
 // Measured on a GB300 (one maximisation, before: full-length sweeps that store every level's phi, a
 // bound pass per step and the visits-times-continuations bound): R-MAT scale 22, k = 100, FP32 143.2
@@ -133,32 +139,41 @@ __device__ __forceinline__ bool in_set(const uint32_t* __restrict__ mask, int32_
   return (__ldg(mask + (v >> 5)) >> (v & 31)) & 1u;
 }
 
-// S grows by list[0..count): the mask bits, and cnt[u] = |N(u) cap S| of every neighbour u.
-__device__ __forceinline__ void join_set(const int32_t* __restrict__ list, int32_t count,
-                                         const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                                         uint32_t* __restrict__ mask, int32_t* __restrict__ cnt) {
+// A graph's lists as the runs use them. o = 0: walks that start at a vertex, along its own row; o = 1
+// (directed): walks that end there, along its row of the reverse CSR. cnt[o][v] = |row o of v cap S|.
+struct Rows {
+  const int32_t* rp[2];
+  const int32_t* ci[2];
+  int32_t* cnt[2];
+  int directed;
+};
+
+// S grows by list[0..count): the mask bits, and the counts of every vertex whose row holds one of them.
+__device__ __forceinline__ void join_set(const int32_t* __restrict__ list, int32_t count, const Rows& g,
+                                         uint32_t* __restrict__ mask) {
   for (int32_t i = blockIdx.y; i < count; i += gridDim.y) {
     const int32_t v = list[i];
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(mask + (v >> 5), 1u << (v & 31));
-    const int64_t e1 = rp[v + 1];
-    for (int64_t j = rp[v] + static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; j < e1;
-         j += static_cast<int64_t>(gridDim.x) * blockDim.x)
-      atomicAdd(cnt + ci[j], 1);
+    for (int o = 0; o <= g.directed; ++o) {
+      const int r = g.directed ? 1 - o : 0;  // v is in row o of u where u is in v's other row
+      const int64_t e1 = g.rp[r][v + 1];
+      for (int64_t j = g.rp[r][v] + static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; j < e1;
+           j += static_cast<int64_t>(gridDim.x) * blockDim.x)
+        atomicAdd(g.cnt[o] + g.ci[r][j], 1);
+    }
   }
 }
 
 // count: list[-1] when negative (a captured launch).
-__global__ void join_kernel(const int32_t* __restrict__ list, int32_t count, const int32_t* __restrict__ rp,
-                            const int32_t* __restrict__ ci, uint32_t* __restrict__ mask, int32_t* __restrict__ cnt) {
-  join_set(list, count >= 0 ? count : list[-1], rp, ci, mask, cnt);
+__global__ void join_kernel(const int32_t* __restrict__ list, int32_t count, const Rows g, uint32_t* __restrict__ mask) {
+  join_set(list, count >= 0 ? count : list[-1], g, mask);
 }
 
 // Opens a run: the vertices that joined S, the exact gains known on the host, the pass's counters.
-__global__ void run_begin(RunDev* __restrict__ d, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                          uint32_t* __restrict__ mask, int32_t* __restrict__ cnt, Stale* __restrict__ stale) {
+__global__ void run_begin(RunDev* __restrict__ d, const Rows g, uint32_t* __restrict__ mask, Stale* __restrict__ stale) {
   if (blockIdx.x == 0 && blockIdx.y == 0) {
     const int t = threadIdx.x;
-    if (t < kRunCols) d->adj[t] = 0;
+    if (t < 2 * kRunCols) d->adj[t / kRunCols][t % kRunCols] = 0;
     if (t < kRunLevels) {
       d->out.lv[t].zero_min = kNoZero;
       d->out.lv[t].sampled = 0;
@@ -170,7 +185,7 @@ __global__ void run_begin(RunDev* __restrict__ d, const int32_t* __restrict__ rp
           stale[d->in.stale_id[j]] = Stale{__double2float_ru(d->in.stale_gain[j]), d->in.stale_step[j]};
     }
   }
-  join_set(d->in.added, d->in.n_added, rp, ci, mask, cnt);
+  join_set(d->in.added, d->in.n_added, g, mask);
 }
 
 template <typename T>
@@ -223,78 +238,88 @@ __global__ void run_init(T* __restrict__ X, const RunDev* __restrict__ d, const 
   }
 }
 
-// Unweighted x_1 of the candidate columns: alpha on the neighbours outside the column's base set
-// (S, with the earlier candidates in a chain), and, for a chain, the number of earlier candidates
-// next to each candidate. Weighted graphs take only the counts.
+// Unweighted x_1 of the candidate columns, one set of vectors per grid.z: alpha on the vertices whose
+// row holds the candidate and which lie outside the column's base set (S, with the earlier candidates
+// in a chain), and, for a chain, the number of earlier candidates in each candidate's row (found in
+// its other row's scan on a directed graph). Weighted graphs take only the counts.
 template <typename T, bool CHAIN>
-__global__ void run_scatter(T* __restrict__ X, int cols, RunDev* __restrict__ d, const int32_t* __restrict__ rp,
-                            const int32_t* __restrict__ ci, const uint32_t* __restrict__ mask, T alpha, int write) {
+__global__ void run_scatter(T* __restrict__ X, int64_t set, int cols, RunDev* __restrict__ d, const Rows g,
+                            const uint32_t* __restrict__ mask, T alpha, int write) {
   __shared__ int sc[kRunCols];
   if (threadIdx.x < kRunCols) sc[threadIdx.x] = d->in.cand[threadIdx.x];
   __syncthreads();
-  const int j = blockIdx.y;
+  const int j = blockIdx.y, o = blockIdx.z, r = g.directed ? 1 - o : 0;
   const int32_t c = sc[j];
   if (c < 0) return;
-  const int64_t e1 = rp[c + 1];
-  for (int64_t e = rp[c] + static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < e1;
+  X += set * o;
+  const int64_t e1 = g.rp[r][c + 1];
+  for (int64_t e = g.rp[r][c] + static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < e1;
        e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int32_t v = ci[e];
+    const int32_t v = g.ci[r][e];
     bool base = false;
     if (CHAIN)
       for (int i = 0; i < j; ++i) base |= sc[i] == v;
-    if (base) atomicAdd(&d->adj[j], 1);
+    if (base) atomicAdd(&d->adj[r][j], 1);
     else if (write && !in_set(mask, v)) X[static_cast<size_t>(v) * cols + j + 1] = alpha;
   }
 }
 
-// The candidates' own rows: live[j] says whether c_j has a neighbour outside its base set; x_1 there
-// is phi_1 under that set.
+// The candidates' own rows: live[o][j] says whether c_j's row o has an entry outside its base set; x_1
+// there is phi_1 under that set.
 template <typename T, bool CHAIN>
-__global__ void run_own(T* __restrict__ X, int cols, RunDev* __restrict__ d, const int32_t* __restrict__ rp,
-                        const int32_t* __restrict__ cnt, T alpha, int write) {
-  const int j = threadIdx.x;
+__global__ void run_own(T* __restrict__ X, int64_t set, int cols, RunDev* __restrict__ d, const Rows g, T alpha, int write) {
+  const int j = threadIdx.x, o = blockIdx.x;
   if (j >= kRunCols) return;
   const int32_t c = j < cols - 1 ? d->in.cand[j] : -1;
   int32_t dg = 0;
   if (c >= 0) {
-    dg = rp[c + 1] - rp[c] - cnt[c] - (CHAIN ? d->adj[j] : 0);
-    if (write) X[static_cast<size_t>(c) * cols + j + 1] = alpha * static_cast<T>(dg);
+    dg = g.rp[o][c + 1] - g.rp[o][c] - g.cnt[o][c] - (CHAIN ? d->adj[o][j] : 0);
+    if (write) X[set * o + static_cast<size_t>(c) * cols + j + 1] = alpha * static_cast<T>(dg);
   }
-  d->live[j] = dg > 0;
+  d->live[o][j] = dg > 0;
 }
 
-// Tail bounds from the walk-total table t_0..t_L (FP64, rows n apart; times s on a weighted graph):
-//   tail(v) = sum over pairs p + q <= L with p or q above H of t_p t_q = 2 sum_{a>H} t_a Q_{L-a},
-//   Q_q = t_0 + ... + t_q,
+// Tail bounds from the walk-total tables t_0..t_L of both orientations (FP64, rows n apart; times s on
+// a weighted graph; A = B unless directed):
+//   tail(v) = sum over pairs p + q <= L with p or q above H of b_p a_q
+//           = sum_{p>H} b_p Qa_{L-p} + sum_{q>H} a_q Qb_{L-q},  Q_q = t_0 + ... + t_q,
 // rounded up; and (about) the bound of the empty group, F + U + F U + tail, for the first guesses.
-__global__ void tail_kernel(const double* __restrict__ T, int64_t n, int32_t n_active, int32_t L, int32_t H,
-                            const double* __restrict__ rs, double alpha, float* __restrict__ tail,
+__global__ void tail_kernel(const double* __restrict__ A, const double* __restrict__ B, int64_t n, int32_t n_active,
+                            int32_t L, int32_t H, const double* __restrict__ rs, double alpha, float* __restrict__ tail,
                             float* __restrict__ bound) {
   for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n_active; v += gridDim.x * blockDim.x) {
     const double inv = rs ? 1.0 / rs[v] : 1.0;
-    double Q = 0.0, acc = 0.0;
+    double Qa = 0.0, Qb = 0.0, acc = 0.0, U = 0.0, F = 0.0;
     for (int32_t q = 0; q < L - H; ++q) {
-      Q += T[static_cast<size_t>(q) * n + v] * inv;
-      acc += T[static_cast<size_t>(L - q) * n + v] * inv * Q;
+      Qa += A[static_cast<size_t>(q) * n + v] * inv;
+      if (A == B) {
+        acc += 2.0 * A[static_cast<size_t>(L - q) * n + v] * inv * Qa;
+      } else {
+        Qb += B[static_cast<size_t>(q) * n + v];
+        acc += B[static_cast<size_t>(L - q) * n + v] * Qa + A[static_cast<size_t>(L - q) * n + v] * Qb;
+      }
     }
-    double U = 0.0;
-    for (int32_t t = 1; t <= H; ++t) U += T[static_cast<size_t>(t) * n + v] * inv;
-    acc *= 2.0 * (1.0 + 1e-12);
+    for (int32_t t = 1; t <= H; ++t) U += A[static_cast<size_t>(t) * n + v] * inv;
+    acc *= 1.0 + 1e-12;
     tail[v] = __double2float_ru(acc);
-    const double f1 = T[n + v] * inv, f2 = H >= 2 ? T[2 * n + v] * inv : 0.0;
-    const double s2 = rs ? 0.0 : alpha * f1, s4 = rs || H < 4 ? 0.0 : alpha * alpha * f2 - alpha * alpha * alpha * f1;
-    const double F = U - (H >= 2 ? (s2 + s4) * (1.0 + U) : 0.0);
+    if (A == B) {
+      const double f1 = A[n + v] * inv, f2 = H >= 2 ? A[2 * n + v] * inv : 0.0;
+      const double s2 = rs ? 0.0 : alpha * f1, s4 = rs || H < 4 ? 0.0 : alpha * alpha * f2 - alpha * alpha * alpha * f1;
+      F = U - (H >= 2 ? (s2 + s4) * (1.0 + U) : 0.0);
+    } else {
+      for (int32_t t = 1; t <= H; ++t) F += B[static_cast<size_t>(t) * n + v];
+    }
     bound[v] = static_cast<float>(F + U + F * U + acc);
   }
 }
 
 struct MeetArgs {
   const void* xs;      // x_1 .. x_H, each [n_active][C]
+  const void* xr;      // directed: the same of the walks that end at a vertex
   int64_t stride;      // elements from x_t to x_{t+1}
   int32_t L, H;
   int32_t n_scan, n_active;
-  const int32_t* rp;
-  const int32_t* cnt;
+  Rows g;
   const uint32_t* mask;
   const int32_t* perm;
   const float* tail;
@@ -409,8 +434,8 @@ __device__ __forceinline__ void block_levels(WarpList (&w)[NL], float* sv, int* 
 // bound is 0, so its vertex is recorded only while the warp's list is empty (an atomic per such row,
 // all to one address, would serialise). 279 -> 150 us; on
 // 10^5 rows, where a warp has one iteration, the lists cost most (device_util.cuh): 97 -> 63 us.
-template <typename T, int C, bool CHAIN, bool SEL>
-__global__ void __launch_bounds__(kThreads, kMeetPerSM) meet_kernel(const MeetArgs a) {
+template <typename T, int C, bool CHAIN, bool SEL, bool DIR>
+__global__ void __launch_bounds__(kThreads, DIR ? 2 : kMeetPerSM) meet_kernel(const MeetArgs a) {
   constexpr int D = C - 1;
   constexpr int NL = CHAIN ? D : 1;
   constexpr int NW = kThreads / 32;
@@ -453,14 +478,17 @@ __global__ void __launch_bounds__(kThreads, kMeetPerSM) meet_kernel(const MeetAr
     const bool ok = v < a.n_scan;
     const bool has = v < a.n_active;
     const T* __restrict__ row = xs + static_cast<size_t>(has ? v : 0) * C;
-    // the row's sums over t = 1..H-1 and x_H
-    T B[C], xh[C];
+    // the row's sums over t = 1..H-1 and x_H (directed: Br, xr of the walks that end here)
+    T B[C], xh[C], Br[DIR ? C : 1], xr[DIR ? C : 1];
 #pragma unroll
     for (int c = 0; c < C; ++c) B[c] = xh[c] = T(0);
+    if constexpr (DIR) {
+#pragma unroll
+      for (int c = 0; c < C; ++c) Br[c] = xr[c] = T(0);
+    }
     T inv = T(1);
     if (has) {
-      const T* p = row;
-      auto load = [&](T (&x)[C]) {
+      auto load = [&](const T* p, T (&x)[C]) {
         if constexpr (sizeof(T) * C >= 16) {
 #pragma unroll
           for (int k = 0; k < static_cast<int>(sizeof(T)) * C / 16; ++k) {
@@ -472,14 +500,26 @@ __global__ void __launch_bounds__(kThreads, kMeetPerSM) meet_kernel(const MeetAr
           for (int c = 0; c < C; ++c) x[c] = __ldg(p + c);
         }
       };
+      const T* p = row;
 #pragma unroll 4
       for (int t = 1; t < H; ++t, p += a.stride) {
         T x[C];
-        load(x);
+        load(p, x);
 #pragma unroll
         for (int c = 0; c < C; ++c) B[c] += x[c];
       }
-      load(xh);
+      load(p, xh);
+      if constexpr (DIR) {
+        p = static_cast<const T*>(a.xr) + static_cast<size_t>(v) * C;
+#pragma unroll 4
+        for (int t = 1; t < H; ++t, p += a.stride) {
+          T x[C];
+          load(p, x);
+#pragma unroll
+          for (int c = 0; c < C; ++c) Br[c] += x[c];
+        }
+        load(p, xr);
+      }
       if (rs) {
         inv = T(1) / rs[v];
 #pragma unroll
@@ -491,18 +531,24 @@ __global__ void __launch_bounds__(kThreads, kMeetPerSM) meet_kernel(const MeetAr
     }
     if (SEL) {
       bool out = false;
-      int dg = 0;
+      int dg = 0, dr = 0;  // entries of the vertex's rows outside the level's set
       float tail = 0.0f;
       if (ok) {
         out = in_set(a.mask, v);
         if (has) {
-          dg = a.rp[v + 1] - a.rp[v] - a.cnt[v];
+          dg = a.g.rp[0][v + 1] - a.g.rp[0][v] - a.g.cnt[0][v];
+          if (DIR) dr = a.g.rp[1][v + 1] - a.g.rp[1][v] - a.g.cnt[1][v];
           tail = a.tail[v];
         }
       }
       const float K0 = f_up(B[0] + xh[0]);
       const float most_u = __fmul_ru(K0, __fadd_ru(infl, e));
-      const float most = dg > 0 ? __fadd_ru(__fmaf_ru(most_u, most_u, __fadd_ru(most_u, most_u)), tail) : 0.0f;
+      float R0 = K0, most_f = most_u;
+      if constexpr (DIR) {
+        R0 = f_up(Br[0] + xr[0]);
+        most_f = __fmul_ru(R0, __fadd_ru(infl, e));
+      }
+      const float most = dg + dr > 0 ? __fadd_ru(__fmaf_ru(most_f, most_u, __fadd_ru(most_f, most_u)), tail) : 0.0f;
       // some row of the warp may enter a list
       if (__any_sync(kFullMask, ok && !out && !(__fmul_ru(most, 1.00001f) < enter)) || a.bound) {
         bool evaluated = false;
@@ -535,33 +581,44 @@ __global__ void __launch_bounds__(kThreads, kMeetPerSM) meet_kernel(const MeetAr
           k.b4 = k.b2 - x2 - x3;
           return k;
         };
+        T eb = T(0), eh = T(0);  // directed: the level's walks that end here, to H-1 and of length H
+        if constexpr (DIR) {
+          eb = Br[0];
+          eh = xr[0];
+        }
         Col r = column(0);  // the level's phi
         const Col r0 = r;
 #pragma unroll
         for (int d = 0; d < NL; ++d) {
           float ub = 0.0f;
-          if (dg > 0) {
+          if (dg + dr > 0) {
             const float U = __fmaf_ru(f_up(pos(r.b + r.h)), infl, __fmul_ru(e, K0));
-            const float p1lo = fmaxf(0.0f, __fsub_rd(f_down(pos(r.f1)), e * f_up(r0.f1)));
-            float s2, s4 = 0.0f;
-            if (rs) {  // Cauchy-Schwarz: sum of squared weights >= (their sum)^2 / their number
-              s2 = __fdiv_rd(__fmul_rd(p1lo, p1lo), static_cast<float>(dg));
+            float F, corr = 0.0f;
+            if constexpr (DIR) {
+              F = __fmaf_ru(f_up(pos(eb + eh)), infl, __fmul_ru(e, R0));
             } else {
-              s2 = __fmul_rd(al2, static_cast<float>(dg));
-              const float p2lo = fmaxf(0.0f, __fsub_rd(f_down(pos(r.f2)), e * f_up(r0.f2)));
-              const float p1up = __fadd_ru(f_up(pos(r.f1)), e * f_up(r0.f1));
-              s4 = fmaxf(0.0f, __fsub_rd(__fmul_rd(al2, p2lo), __fmul_ru(al3, p1up)));
+              const float p1lo = fmaxf(0.0f, __fsub_rd(f_down(pos(r.f1)), e * f_up(r0.f1)));
+              float s2, s4 = 0.0f;
+              if (rs) {  // Cauchy-Schwarz: sum of squared weights >= (their sum)^2 / their number
+                s2 = __fdiv_rd(__fmul_rd(p1lo, p1lo), static_cast<float>(dg));
+              } else {
+                s2 = __fmul_rd(al2, static_cast<float>(dg));
+                const float p2lo = fmaxf(0.0f, __fsub_rd(f_down(pos(r.f2)), e * f_up(r0.f2)));
+                const float p1up = __fadd_ru(f_up(pos(r.f1)), e * f_up(r0.f1));
+                s4 = fmaxf(0.0f, __fsub_rd(__fmul_rd(al2, p2lo), __fmul_ru(al3, p1up)));
+              }
+              if (H >= 2) corr = __fmul_rd(s2, __fadd_rd(1.0f, fmaxf(0.0f, __fsub_rd(f_down(pos(r.b2)), e * f_up(r0.b2)))));
+              if (H >= 4)
+                corr = __fadd_rd(corr, __fmul_rd(s4, __fadd_rd(1.0f, fmaxf(0.0f, __fsub_rd(f_down(pos(r.b4)), e * f_up(r0.b4))))));
+              corr = __fmul_rd(corr, keep);
+              F = fmaxf(0.0f, __fsub_ru(U, corr));
             }
-            float corr = 0.0f;
-            if (H >= 2) corr = __fmul_rd(s2, __fadd_rd(1.0f, fmaxf(0.0f, __fsub_rd(f_down(pos(r.b2)), e * f_up(r0.b2)))));
-            if (H >= 4)
-              corr = __fadd_rd(corr, __fmul_rd(s4, __fadd_rd(1.0f, fmaxf(0.0f, __fsub_rd(f_down(pos(r.b4)), e * f_up(r0.b4))))));
-            corr = __fmul_rd(corr, keep);
-            const float F = fmaxf(0.0f, __fsub_ru(U, corr));
             ub = __fadd_ru(__fmaf_ru(F, U, __fadd_ru(F, U)), tail);
             if (odd) {  // the pair (H, H) is longer than L
               const float hlo = fmaxf(0.0f, __fsub_rd(f_down(pos(r.h)), e * f_up(r0.h)));
-              ub = __fsub_ru(ub, __fmul_rd(hlo, fmaxf(0.0f, __fsub_rd(hlo, corr))));
+              float elo = hlo;
+              if constexpr (DIR) elo = fmaxf(0.0f, __fsub_rd(f_down(pos(eh)), e * f_up(xr[0])));
+              ub = __fsub_ru(ub, __fmul_rd(hlo, fmaxf(0.0f, __fsub_rd(elo, corr))));
             }
             if (!(ub >= 0.0f)) ub = INFINITY;  // overflow: nothing is known
             if (st.step >= 0 && st.ub < ub) ub = st.ub;
@@ -585,6 +642,11 @@ __global__ void __launch_bounds__(kThreads, kMeetPerSM) meet_kernel(const MeetAr
             r.f2 -= k.f2;
             r.h -= k.h;
             dg -= k.f1 > T(0);
+            if constexpr (DIR) {
+              eb -= Br[d + 1];
+              eh -= xr[d + 1];
+              dr -= has && __ldg(static_cast<const T*>(a.xr) + static_cast<size_t>(v) * C + d + 1) > T(0);
+            }
             out |= s_cand[d] == v;
           }
         }
@@ -594,16 +656,30 @@ __global__ void __launch_bounds__(kThreads, kMeetPerSM) meet_kernel(const MeetAr
       }
     }
     // gain terms of candidate d + 1 under its base set
-    T rb = B[0], rh = xh[0];
+    T rb = B[0], rh = xh[0], sb = T(0), sh = T(0);
+    if constexpr (DIR) {
+      sb = Br[0];
+      sh = xr[0];
+    }
 #pragma unroll
     for (int d = 0; d < D; ++d) {
       const T k = B[d + 1] + xh[d + 1];
-      const T vv = odd ? B[d + 1] : k;
-      const T pp = odd ? pos(rb) : pos(rb + rh);
+      T vv, pp;
+      if constexpr (DIR) {
+        vv = odd ? Br[d + 1] : Br[d + 1] + xr[d + 1];
+        pp = odd ? pos(sb) : pos(sb + sh);
+      } else {
+        vv = odd ? B[d + 1] : k;
+        pp = odd ? pos(rb) : pos(rb + rh);
+      }
       acc.add(d, k + vv * pos(rh) + pos(pp - vv) * xh[d + 1]);
       if (CHAIN) {
         rb -= B[d + 1];
         rh -= xh[d + 1];
+        if constexpr (DIR) {
+          sb -= Br[d + 1];
+          sh -= xr[d + 1];
+        }
       }
     }
   }
@@ -798,46 +874,62 @@ int meet_grid(int32_t n_scan) {
   return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(kMeetBlocks, (int64_t(n_scan) + kThreads - 1) / kThreads)));
 }
 
+Rows rows_of(const Graph& g, const Workspace& ws) {
+  Rows r{};
+  r.rp[0] = g.rp.as<int32_t>();
+  r.ci[0] = g.ci.as<int32_t>();
+  r.cnt[0] = ws.cnt.as<int32_t>();
+  r.directed = g.directed ? 1 : 0;
+  if (g.directed) {
+    r.rp[1] = g.rp_r.as<int32_t>();
+    r.ci[1] = g.ci_r.as<int32_t>();
+    r.cnt[1] = r.cnt[0] + g.n;
+  }
+  return r;
+}
+
+// X: the first stored vector; directed: that of the other set lies `set` elements behind it.
 template <typename T, int C>
-cudaError_t launch_init(cudaStream_t s, T* X, RunDev* d, const Graph& g, const Workspace& ws, bool chain, double alpha) {
+cudaError_t launch_init(cudaStream_t s, T* X, int64_t set, RunDev* d, const Graph& g, const Workspace& ws, bool chain,
+                        double alpha) {
   const T* rs = !g.weighted ? nullptr : sizeof(T) == 8 ? static_cast<const T*>(g.rs_d.p) : static_cast<const T*>(g.rs_f.p);
-  const int32_t* rp = g.rp.as<int32_t>();
-  const int32_t* ci = g.ci.as<int32_t>();
-  const int32_t* cnt = ws.cnt.as<int32_t>();
+  const Rows rows = rows_of(g, ws);
   const uint32_t* mask = ws.mask.as<uint32_t>();
   const T al = static_cast<T>(alpha);
-  const int write = g.weighted ? 0 : 1;
-  run_init<T, C><<<grid_of(static_cast<int64_t>(g.n_active) * C * sizeof(T) / 16), 256, 0, s>>>(X, d, rp, cnt, mask,
-                                                                                              g.n_active, al, rs);
+  const int write = g.weighted ? 0 : 1, sets = g.directed ? 2 : 1;
+  for (int o = 0; o < sets; ++o)
+    run_init<T, C><<<grid_of(static_cast<int64_t>(g.n_active) * C * sizeof(T) / 16), 256, 0, s>>>(
+        X + set * o, d, rows.rp[o], rows.cnt[o], mask, g.n_active, al, rs);
   if (chain) {
-    run_scatter<T, true><<<dim3(kChunks, C - 1), 256, 0, s>>>(X, C, d, rp, ci, mask, al, write);
-    run_own<T, true><<<1, 32, 0, s>>>(X, C, d, rp, cnt, al, write);
+    run_scatter<T, true><<<dim3(kChunks, C - 1, sets), 256, 0, s>>>(X, set, C, d, rows, mask, al, write);
+    run_own<T, true><<<sets, 32, 0, s>>>(X, set, C, d, rows, al, write);
   } else {
-    if (write) run_scatter<T, false><<<dim3(kChunks, C - 1), 256, 0, s>>>(X, C, d, rp, ci, mask, al, write);
-    run_own<T, false><<<1, 32, 0, s>>>(X, C, d, rp, cnt, al, write);
+    if (write) run_scatter<T, false><<<dim3(kChunks, C - 1, sets), 256, 0, s>>>(X, set, C, d, rows, mask, al, write);
+    run_own<T, false><<<sets, 32, 0, s>>>(X, set, C, d, rows, al, write);
   }
   return cudaGetLastError();
 }
 
 template <typename T, int C, bool CHAIN, bool SEL>
 cudaError_t launch_meet(cudaStream_t s, const MeetArgs& a) {
-  meet_kernel<T, C, CHAIN, SEL><<<meet_grid(a.n_scan), kThreads, 0, s>>>(a);
+  if (a.g.directed) meet_kernel<T, C, CHAIN, SEL, true><<<meet_grid(a.n_scan), kThreads, 0, s>>>(a);
+  else meet_kernel<T, C, CHAIN, SEL, false><<<meet_grid(a.n_scan), kThreads, 0, s>>>(a);
   return cudaGetLastError();
 }
 
 }  // namespace
 
 int64_t run_bytes(const Graph& g, int32_t L_max, int cols, bool fp64, bool select) {
-  const int64_t n = g.n, H = (L_max + 1) / 2, es = fp64 ? 8 : 4;
-  int64_t b = std::max<int64_t>(static_cast<int64_t>(g.n_active) * H * cols * es, 16);  // x_1 .. x_H (x_0: weighted)
-  if (g.weighted) b += static_cast<int64_t>(g.n_active) * cols * es;
-  b += n * 4 + (n + 31) / 32 * 4;                           // |N(v) cap S|, S bitmask
+  const int64_t n = g.n, H = (L_max + 1) / 2, es = fp64 ? 8 : 4, sets = g.directed ? 2 : 1;
+  const int64_t slices = std::max(std::max(g.plan.num_slices, g.directed ? g.plan_r.num_slices : 0), 1);
+  const int64_t heavy = std::max(std::max(g.plan.num_heavy, g.directed ? g.plan_r.num_heavy : 0), 1);
+  // x_1 .. x_H (x_0: weighted)
+  int64_t b = std::max<int64_t>(static_cast<int64_t>(g.n_active) * (sets * H + (g.weighted ? 1 : 0)) * cols * es, 16);
+  b += n * 4 * sets + (n + 31) / 32 * 4;                    // counts of S in the rows, S bitmask
   b += static_cast<int64_t>(kMeetBlocks) * (cols - 1) * 8;  // gain sums
   b += static_cast<int64_t>(sizeof(RunDev)) + 256;
   if (select) b += n * (4 + 4 + static_cast<int64_t>(sizeof(Stale))) + static_cast<int64_t>(kMeetBlocks) * kRunLevels * kTopK * 8;
-  const int64_t es_p = es;
-  b += static_cast<int64_t>(std::max(g.plan.num_slices, 1)) * cols * es_p + std::max(g.plan.num_heavy, 1) * 4;
-  return b;
+  return b + slices * cols * es + heavy * 4;
 }
 
 // The captured sequences copy from and to this block: it must outlive them at one address (a pinned
@@ -854,8 +946,9 @@ static gedwalk_status ensure_run_io(Workspace& ws) {
 gedwalk_status RunEngine::setup(int32_t L_max, int cols, bool select, const std::vector<int32_t>& init) {
   const size_t n = static_cast<size_t>(g.n), H_max = static_cast<size_t>((L_max + 1) / 2), es = r.fp64 ? 8 : 4;
   const size_t row = static_cast<size_t>(g.n_active) * cols * es;
-  GW_TRY(ws.xs.ensure(row * (H_max + (g.weighted ? 1 : 0)), s));
-  GW_TRY(ws.cnt.ensure(n * sizeof(int32_t), s));
+  const size_t sets = g.directed ? 2 : 1;
+  GW_TRY(ws.xs.ensure(row * (sets * H_max + (g.weighted ? 1 : 0)), s));
+  GW_TRY(ws.cnt.ensure(sets * n * sizeof(int32_t), s));
   const size_t words = (n + 31) / 32;
   GW_TRY(ws.mask.ensure(words * 4, s));
   GW_TRY(ws.parts.ensure(static_cast<size_t>(kMeetBlocks) * (cols - 1) * sizeof(double), s));
@@ -865,8 +958,10 @@ gedwalk_status RunEngine::setup(int32_t L_max, int cols, bool select, const std:
   in = reinterpret_cast<RunIn*>(out + 1);
   memset(in, 0, sizeof *in);
   for (uint64_t& t : in->thr) t = ~0ull;
-  GW_TRY(ws.partial.ensure(static_cast<size_t>(std::max(g.plan.num_slices, 1)) * cols * es, s));
-  const size_t cbytes = static_cast<size_t>(std::max(g.plan.num_heavy, 1)) * sizeof(unsigned);
+  const int32_t slices = std::max(g.plan.num_slices, g.directed ? g.plan_r.num_slices : 0);
+  const int32_t heavy = std::max(g.plan.num_heavy, g.directed ? g.plan_r.num_heavy : 0);
+  GW_TRY(ws.partial.ensure(static_cast<size_t>(std::max(slices, 1)) * cols * es, s));
+  const size_t cbytes = static_cast<size_t>(std::max(heavy, 1)) * sizeof(unsigned);
   if (ws.counters.bytes < cbytes || !ws.counters.p) GW_TRY(ws.counters.ensure(cbytes, s, /*zero=*/true));
   if (select) {
     GW_TRY(ws.stale.ensure(n * sizeof(Stale), s));
@@ -875,7 +970,7 @@ gedwalk_status RunEngine::setup(int32_t L_max, int cols, bool select, const std:
     GW_TRY(ws.bound.ensure(n * sizeof(float), s));
     GW_CUDA(cudaMemsetAsync(ws.stale.p, 0xff, n * sizeof(Stale), s));  // step -1
   }
-  GW_CUDA(cudaMemsetAsync(ws.cnt.p, 0, n * sizeof(int32_t), s));
+  GW_CUDA(cudaMemsetAsync(ws.cnt.p, 0, sets * n * sizeof(int32_t), s));
   GW_CUDA(cudaMemsetAsync(ws.mask.p, 0, words * 4, s));
   if (!init.empty()) {
     DevBuf& list = ws.members;
@@ -886,8 +981,7 @@ gedwalk_status RunEngine::setup(int32_t L_max, int cols, bool select, const std:
     GW_CUDA(cudaMemcpyAsync(list.p, st, init.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
     const int items = static_cast<int>(std::min<size_t>(init.size(), 4096));
     join_kernel<<<dim3(kChunks, items), 256, 0, s>>>(list.as<int32_t>(), static_cast<int32_t>(init.size()),
-                                                     g.rp.as<int32_t>(), g.ci.as<int32_t>(), ws.mask.as<uint32_t>(),
-                                                     ws.cnt.as<int32_t>());
+                                                     rows_of(g, ws), ws.mask.as<uint32_t>());
     GW_KCHECK();
   }
   return GEDWALK_OK;
@@ -897,23 +991,33 @@ gedwalk_status RunEngine::set_length(int32_t length, bool select) {
   L = length;
   H = (L + 1) / 2;
   if (!select || g.n_active == 0) return GEDWALK_OK;
-  // tail bounds from the walk totals; the table is read under its lock, to the end of the kernel
+  // tail bounds from the walk totals; the tables are read under their lock, to the end of the kernel
   const double* rs = g.weighted ? g.rs_d.as<double>() : nullptr;
+  bool table;
   {
     std::shared_lock<std::shared_mutex> rl(g.tt_lock);
-    if (g.tt_alpha == r.alpha && g.tt_rows >= L + 1) {
-      tail_kernel<<<grid_of(g.n_active), 256, 0, s>>>(g.ttab.as<double>(), g.n, g.n_active, L, H, rs, r.alpha, ws.tail.as<float>(),
-                                                      ws.bound.as<float>());
+    table = g.tt_alpha == r.alpha && g.tt_rows >= L + 1;
+  }
+  if (table && g.directed) GW_TRY(ensure_totals_fwd(g, ws, r.alpha, L + 1, s));
+  {
+    std::shared_lock<std::shared_mutex> rl(g.tt_lock);
+    if (g.tt_alpha == r.alpha && g.tt_rows >= L + 1 && (!g.directed || (g.ttf_alpha == r.alpha && g.ttf_rows >= L + 1))) {
+      const double* B = g.ttab.as<double>();
+      tail_kernel<<<grid_of(g.n_active), 256, 0, s>>>(g.directed ? g.ttab_f.as<double>() : B, B, g.n, g.n_active, L, H, rs,
+                                                      r.alpha, ws.tail.as<float>(), ws.bound.as<float>());
       GW_KCHECK();
       GW_CUDA(cudaStreamSynchronize(s));
       return GEDWALK_OK;
     }
   }
   // no table for this alpha (a forced L beyond the bound's reach): totals of this call's own
-  const size_t n = static_cast<size_t>(g.n);
-  GW_TRY(ws.ztab.ensure(static_cast<size_t>(L + 1) * n * sizeof(double), s));
-  GW_TRY(totals_into(g, ws, ws.ztab.as<double>(), r.alpha, L + 1, s));
-  tail_kernel<<<grid_of(g.n_active), 256, 0, s>>>(ws.ztab.as<double>(), g.n, g.n_active, L, H, rs, r.alpha, ws.tail.as<float>(),
+  const size_t n = static_cast<size_t>(g.n), rows = static_cast<size_t>(L + 1);
+  GW_TRY(ws.ztab.ensure((g.directed ? 2 : 1) * rows * n * sizeof(double), s));
+  double* A = ws.ztab.as<double>();
+  double* B = g.directed ? A + rows * n : A;
+  GW_TRY(totals_into(g, ws, A, r.alpha, 0, L + 1, false, s));
+  if (g.directed) GW_TRY(totals_into(g, ws, B, r.alpha, 0, L + 1, true, s));
+  tail_kernel<<<grid_of(g.n_active), 256, 0, s>>>(A, B, g.n, g.n_active, L, H, rs, r.alpha, ws.tail.as<float>(),
                                                   ws.bound.as<float>());
   GW_KCHECK();
   return GEDWALK_OK;
@@ -932,8 +1036,7 @@ gedwalk_status RunEngine::push_added() {
   while (added.size() > kRunCols) {
     std::copy(added.end() - kRunCols, added.end(), in->added);
     GW_CUDA(cudaMemcpyAsync(d->in.added, in->added, sizeof in->added, cudaMemcpyHostToDevice, s));
-    join_kernel<<<dim3(kChunks, kRunCols), 256, 0, s>>>(d->in.added, kRunCols, g.rp.as<int32_t>(), g.ci.as<int32_t>(),
-                                                        ws.mask.as<uint32_t>(), ws.cnt.as<int32_t>());
+    join_kernel<<<dim3(kChunks, kRunCols), 256, 0, s>>>(d->in.added, kRunCols, rows_of(g, ws), ws.mask.as<uint32_t>());
     GW_KCHECK();
     GW_CUDA(cudaStreamSynchronize(s));  // the pinned block is reused
     added.resize(added.size() - kRunCols);
@@ -950,38 +1053,43 @@ gedwalk_status RunEngine::issue(bool chain, int cols, bool select, bool profile,
   const size_t es = fp64 ? 8 : 4;
   const size_t row = static_cast<size_t>(g.n_active) * cols;
   GW_CUDA(cudaMemcpyAsync(&d->in, in, sizeof(RunIn), cudaMemcpyHostToDevice, s));
-  run_begin<<<dim3(kChunks, kRunCols), 256, 0, s>>>(d, g.rp.as<int32_t>(), g.ci.as<int32_t>(), ws.mask.as<uint32_t>(),
-                                                    ws.cnt.as<int32_t>(), select ? ws.stale.as<Stale>() : nullptr);
+  run_begin<<<dim3(kChunks, kRunCols), 256, 0, s>>>(d, rows_of(g, ws), ws.mask.as<uint32_t>(),
+                                                    select ? ws.stale.as<Stale>() : nullptr);
   GW_KCHECK();
-  // x_1 .. x_H; a weighted graph starts one sweep earlier, from x_0 behind them
+  // x_1 .. x_H; a weighted graph starts one sweep earlier, from x_0 behind them; a directed one has its
+  // second set behind the first
   char* xs = ws.xs.as<char>();
   char* x0 = g.weighted ? xs + row * es * H : xs;
+  const int64_t set = static_cast<int64_t>(row) * H;
 #define GW_RUN(T, C) \
-  if (fp64 == (sizeof(T) == 8) && cols == C) GW_CUDA((launch_init<T, C>(s, reinterpret_cast<T*>(x0), d, g, ws, chain, r.alpha)));
+  if (fp64 == (sizeof(T) == 8) && cols == C) GW_CUDA((launch_init<T, C>(s, reinterpret_cast<T*>(x0), set, d, g, ws, chain, r.alpha)));
   GW_RUN(float, 2) GW_RUN(float, 4) GW_RUN(float, 8) GW_RUN(float, 16) GW_RUN(double, 2) GW_RUN(double, 4) GW_RUN(double, 8)
 #undef GW_RUN
-  for (int i = 0; i < 3; ++i) count_launch();
-  SweepArgs a = base_args(g, ws);
-  a.alpha = r.alpha;
-  a.cand = d->in.cand;
-  a.live = d->live;
+  for (int i = 0; i < (g.directed ? 4 : 3); ++i) count_launch();
   const int mode = chain ? MODE_LOOK : MODE_PAR;
   if (ev) GW_CUDA(cudaEventRecordWithFlags((*ev)[0], s, cudaEventRecordExternal));
-  for (int32_t t = g.weighted ? 1 : 2; t <= H; ++t) {
-    a.X = t == 1 ? x0 : xs + row * es * (t - 2);
-    a.Y = xs + row * es * (t - 1);
-    GW_TRY(launch_sweep(mode, fp64, cols, a, s, profile));
+  for (int o = 0; o < (g.directed ? 2 : 1); ++o) {
+    SweepArgs a = o ? base_args_rev(g, ws) : base_args(g, ws);
+    a.alpha = r.alpha;
+    a.cand = d->in.cand;
+    a.live = d->live[o];
+    char* x = xs + static_cast<size_t>(set) * es * o;
+    for (int32_t t = g.weighted ? 1 : 2; t <= H; ++t) {
+      a.X = t == 1 ? x0 : x + row * es * (t - 2);
+      a.Y = x + row * es * (t - 1);
+      GW_TRY(launch_sweep(mode, fp64, cols, a, s, profile));
+    }
   }
   if (ev) GW_CUDA(cudaEventRecordWithFlags((*ev)[1], s, cudaEventRecordExternal));
   MeetArgs m{};
   m.xs = xs;
+  m.xr = xs + static_cast<size_t>(set) * es;
   m.stride = static_cast<int64_t>(row);
   m.L = L;
   m.H = H;
   m.n_scan = select ? n_scan : g.n_active;
   m.n_active = g.n_active;
-  m.rp = g.rp.as<int32_t>();
-  m.cnt = ws.cnt.as<int32_t>();
+  m.g = rows_of(g, ws);
   m.mask = ws.mask.as<uint32_t>();
   m.perm = g.perm_d.as<int32_t>();
   m.tail = ws.tail.as<float>();
@@ -1009,7 +1117,7 @@ gedwalk_status RunEngine::issue(bool chain, int cols, bool select, bool profile,
 gedwalk_status RunEngine::run(bool chain, int cols, bool select, const std::vector<int32_t>& cand) {
   for (int j = 0; j < kRunCols; ++j) in->cand[j] = j < static_cast<int>(cand.size()) && j < cols - 1 ? cand[j] : -1;
   GW_TRY(push_added());
-  const int swept = g.weighted ? H : H - 1;
+  const int swept = g.weighted ? H : (g.directed ? 2 : 1) * (H - 1);
   sweeps += swept;
   const int mode = chain ? MODE_LOOK : MODE_PAR;
   uint64_t abits;
@@ -1020,7 +1128,7 @@ gedwalk_status RunEngine::run(bool chain, int cols, bool select, const std::vect
                    bits(&g), bits(s), bits(ws.xs.p), bits(ws.cnt.p), bits(ws.mask.p), bits(ws.parts.p), bits(ws.small.p),
                    bits(ws.partial.p), bits(ws.counters.p), bits(ws.stale.p), bits(ws.sel.p), bits(ws.tail.p),
                    bits(ws.bound.p), bits(ws.run_io), bits(g.rp.p), bits(g.ci.p), bits(g.plan.units.p)});
-  q.kernels = 5 + swept;
+  q.kernels = (g.directed ? 6 : 5) + swept;
   q.sweeps = swept;
   q.bytes = sweep_bytes(mode, r.fp64, cols, g.n_active, g.nnz, g.weighted);
   q.prof_key = (mode * 1000 + cols) * 2 + (r.fp64 ? 1 : 0);
@@ -1038,8 +1146,7 @@ gedwalk_status RunEngine::guess(int levels) {
   RunDev* d = ws.small.as<RunDev>();
   GW_TRY(push_added());
   GW_CUDA(cudaMemcpyAsync(&d->in, in, sizeof(RunIn), cudaMemcpyHostToDevice, s));
-  run_begin<<<dim3(kChunks, kRunCols), 256, 0, s>>>(d, g.rp.as<int32_t>(), g.ci.as<int32_t>(), ws.mask.as<uint32_t>(),
-                                                    ws.cnt.as<int32_t>(), ws.stale.as<Stale>());
+  run_begin<<<dim3(kChunks, kRunCols), 256, 0, s>>>(d, rows_of(g, ws), ws.mask.as<uint32_t>(), ws.stale.as<Stale>());
   GW_KCHECK();
   float* sel_v = ws.sel.as<float>();
   guess_kernel<<<meet_grid(n_scan), kThreads, 0, s>>>(
@@ -1098,8 +1205,8 @@ gedwalk_status score_run(Graph& g, Workspace& ws, const std::vector<int32_t>& S_
   auto issue = [&](bool profile, const std::vector<cudaEvent_t>* ev) -> gedwalk_status {
     GW_CUDA(cudaMemsetAsync(ws.cnt.p, 0, n * sizeof(int32_t), s));
     GW_CUDA(cudaMemsetAsync(ws.mask.p, 0, words * 4, s));
-    join_kernel<<<dim3(chunks, items), 256, 0, s>>>(ws.members.as<int32_t>() + 1, -1, g.rp.as<int32_t>(), g.ci.as<int32_t>(),
-                                                    ws.mask.as<uint32_t>(), ws.cnt.as<int32_t>());
+    join_kernel<<<dim3(chunks, items), 256, 0, s>>>(ws.members.as<int32_t>() + 1, -1, rows_of(g, ws),
+                                                    ws.mask.as<uint32_t>());
     GW_KCHECK();
     char* xs = ws.xs.as<char>();
     char* x0 = g.weighted ? xs + row * es * H : xs;

@@ -48,8 +48,8 @@ struct RunOut {  // device -> host, one copy per run
 struct RunDev {  // device-side state of the runs of one workspace
   RunIn in;
   RunOut out;
-  int32_t live[kRunCols];  // whether candidate j has a neighbour outside its base set
-  int32_t adj[kRunCols];   // chain: earlier candidates that are neighbours of candidate j
+  int32_t live[2][kRunCols];  // per set of vectors: whether candidate j's row has an entry outside its base set
+  int32_t adj[2][kRunCols];   // chain: earlier candidates in candidate j's row
   int32_t done;            // blocks of the meeting (or guess) pass that have finished
 };
 
@@ -70,7 +70,7 @@ gedwalk_status greedy_stream(Workspace& ws, cudaStream_t caller, cudaStream_t* o
 void read_graph_timing(Workspace& ws);
 uint64_t mix_all(std::initializer_list<uint64_t> vs);
 
-// The runs of one maximisation (or one gains call) on an undirected graph.
+// The runs of one maximisation (or one gains call).
 struct RunEngine {
   Graph& g;
   Workspace& ws;

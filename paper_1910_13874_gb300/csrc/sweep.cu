@@ -210,19 +210,15 @@ struct Scatter {
 // Number of FP64 column sums a mode keeps.
 template <int MODE, int C>
 struct Sums {
-  static constexpr int N = MODE == MODE_TOTALS ? 1 : MODE == MODE_SCORE ? 1
-                           : MODE == MODE_FUSED ? C - 1 : MODE == MODE_CAND ? C : 0;
-  // the sum fed by column c, or -1 (MODE_FUSED: columns 1.., the candidates)
-  __device__ __forceinline__ static int slot(int c) {
-    constexpr int first = MODE == MODE_FUSED ? 1 : 0;
-    return c >= first && c - first < N ? c - first : -1;
-  }
+  static constexpr int N = MODE == MODE_TOTALS || MODE == MODE_SCORE ? 1 : 0;
+  // the sum fed by column c, or -1
+  __device__ __forceinline__ static int slot(int c) { return c < N ? c : -1; }
 };
 
 // Number of candidate ids a mode reads (the only rows whose epilogue differs from y = alpha s).
 template <int MODE, int C>
 struct Cands {
-  static constexpr int N = (MODE == MODE_FUSED || MODE == MODE_LOOK || MODE == MODE_PAR) ? C - 1 : MODE == MODE_CAND ? C : 0;
+  static constexpr int N = (MODE == MODE_LOOK || MODE == MODE_PAR) ? C - 1 : 0;
 };
 
 // The epilogue of the rows whose warp holds a candidate row (at most kCandSlots rows of the graph;
@@ -238,21 +234,7 @@ template <typename T, int C, int MODE, int CPL>
 __device__ __forceinline__ void candidate_rows(const SweepArgs& a, const int* __restrict__ s_cand,
                                                const int* __restrict__ s_live, int r, bool valid, int c0, int base,
                                                T (&y)[CPL]) {
-  if constexpr (MODE == MODE_FUSED) {
-    // column 0 is phi^miss under S; candidate column j >= 1 takes it at the candidate's row
-    // (every S-avoiding walk ending at c_j visits c_j)
-    const T m = __shfl_sync(kFull, y[0], base);
-#pragma unroll
-    for (int k = 0; k < CPL; ++k) {
-      const int c = c0 + k;
-      if (valid && c >= 1 && s_cand[c - 1] == r) y[k] = m;
-    }
-  } else if constexpr (MODE == MODE_CAND) {
-    const T* min = static_cast<const T*>(a.Min);
-#pragma unroll
-    for (int k = 0; k < CPL; ++k)
-      if (valid && s_cand[c0 + k] == r) y[k] = __ldg(min + r);
-  } else if constexpr (MODE == MODE_PAR) {
+  if constexpr (MODE == MODE_PAR) {
     const T m = __shfl_sync(kFull, y[0], base);
 #pragma unroll
     for (int k = 0; k < CPL; ++k) {
@@ -343,7 +325,7 @@ __device__ __forceinline__ void epilogue(const SweepArgs& a, const int* __restri
       for (int j = 0; j < Cands<MODE, C>::N; ++j) special |= s_cand[j] == r;
       if (__any_sync(kFull, valid && special)) candidate_rows<T, C, MODE, CPL>(a, s_cand, s_live, r, valid, c0, base, y);
     }
-    if constexpr (MODE == MODE_FUSED) {
+    if constexpr (MODE == MODE_MISS) {
       if (store && c0 == 0) static_cast<T*>(a.Mout)[r] = y[0];
     }
     if (store) {
@@ -588,9 +570,7 @@ constexpr int min_ctas() {
   if (sizeof(T) == 8) return 1;
   if ((MODE == MODE_LOOK || MODE == MODE_PAR) && C == 8) return 5;
   if ((MODE == MODE_LOOK || MODE == MODE_PAR) && C <= 4) return 6;
-  if (MODE == MODE_CAND && C == 4) return 4;
-  if ((MODE == MODE_FUSED || MODE == MODE_SCORE || MODE == MODE_PAIR) && C <= 2) return 8;
-  if (MODE == MODE_FUSED && C == 4) return 6;
+  if ((MODE == MODE_MISS || MODE == MODE_SCORE || MODE == MODE_PAIR) && C <= 2) return 8;
   if (MODE == MODE_PLAIN) return C <= 8 ? 5 : C <= 16 ? 3 : C <= 32 ? 2 : 1;
   return 1;
 }
@@ -618,7 +598,7 @@ __global__ void __launch_bounds__(kThreads, (min_ctas<T, C, MODE>())) sweep_kern
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (Cands<MODE, C>::N > 0 && threadIdx.x < kCandSlots) {
     s_cand[threadIdx.x] = a.cand[threadIdx.x];
-    if (MODE == MODE_LOOK || MODE == MODE_PAR) s_live[threadIdx.x] = a.live[threadIdx.x];
+    s_live[threadIdx.x] = a.live[threadIdx.x];
   }
   __syncthreads();
   if (uidx >= a.num_units) return;
@@ -717,10 +697,6 @@ int sweep_sums(int mode, int cols) {
     case MODE_TOTALS:
     case MODE_SCORE:
       return 1;
-    case MODE_FUSED:
-      return cols - 1;
-    case MODE_CAND:
-      return cols;
     default:
       return 0;
   }
@@ -734,17 +710,8 @@ gedwalk_status launch_sweep(int mode, bool fp64, int cols, const SweepArgs& a, c
   GW_CASE(MODE_SCORE, float, 2)
   GW_CASE(MODE_PAIR, double, 2)
   GW_CASE(MODE_PAIR, float, 2)
-  GW_CASE(MODE_FUSED, float, 1)
-  GW_CASE(MODE_FUSED, float, 2)
-  GW_CASE(MODE_FUSED, float, 4)
-  GW_CASE(MODE_FUSED, float, 8)
-  GW_CASE(MODE_FUSED, double, 1)
-  GW_CASE(MODE_FUSED, double, 2)
-  GW_CASE(MODE_FUSED, double, 4)
-  GW_CASE(MODE_CAND, float, 4)
-  GW_CASE(MODE_CAND, float, 16)
-  GW_CASE(MODE_CAND, double, 4)
-  GW_CASE(MODE_CAND, double, 8)
+  GW_CASE(MODE_MISS, float, 1)
+  GW_CASE(MODE_MISS, double, 1)
   GW_CASE(MODE_LOOK, float, 4)
   GW_CASE(MODE_LOOK, float, 8)
   GW_CASE(MODE_LOOK, double, 4)

@@ -112,3 +112,28 @@ def test_half_length_chain(name):
         base = base - k
         mask = mask.copy()
         mask[c] = 0.0
+
+
+@pytest.mark.parametrize("L", [1, 2, 5, 6, 9])
+def test_half_length_directed(L):
+    # walks that start at a vertex along the rows, walks that end there along the reverse lists
+    A = gg.random_digraph(40, 0.08, 7).to_dense().astype(float)
+    alpha = 1.0 / (1.0 + A.sum(1).max())
+    S, H = [1, 4], (L + 1) // 2
+    mask = np.ones(40)
+    mask[S] = 0.0
+    Ma, Mb = alpha * mask[:, None] * A, alpha * mask[:, None] * A.T
+    phi, psi = table(Ma, L, mask), table(Mb, L, mask)
+    fa, fb = table(alpha * A, L, np.ones(40)), table(alpha * A.T, L, np.ones(40))
+    Qa, Qb = fa.cumsum(0), fb.cumsum(0)
+    tail = sum((fb[p] * Qa[L - p] + fa[p] * Qb[L - p] for p in range(H + 1, L + 1)), np.zeros(40))
+    for c in range(40):
+        if c in S:
+            continue
+        k, j = column(Ma, phi, c, S), column(Mb, psi, c, S)
+        V, P = j[1:L - H + 1].sum(0), psi[1:L - H + 1].sum(0)
+        got = (k[1:H + 1].sum(0) + V * phi[H] + (P - V) * k[H]).sum()
+        assert got == pytest.approx(k[1:].sum(), rel=1e-12, abs=1e-15)
+        U, F = phi[1:H + 1, c].sum(), psi[1:H + 1, c].sum()
+        ub = F + U + F * U + tail[c] - (phi[H, c] * psi[H, c] if L % 2 else 0.0)
+        assert ub >= k[1:].sum() * (1 - 1e-12)
