@@ -148,6 +148,16 @@ __device__ __forceinline__ void add_row(T (&acc)[C], const T* __restrict__ X, in
   for (int c = 0; c < C; ++c) acc[c] += x[c];
 }
 
+// The first gather of a lane in FP64: a copy, where an addition to 0 would cost as much as any other
+// (64 times an FP32 one on a GB300). Barabasi-Albert, n = 10^6, 4 columns: 357 -> 283 us a sweep, and
+// with four CTAs per SM instead of two 270 us.
+template <typename T, int C>
+__device__ __forceinline__ void set_row(T (&acc)[C], const T* __restrict__ X, int v, int hub) {
+  const T* p = X + static_cast<size_t>(v) * C;
+  if (v < hub) gather_vec<T, C, true>(p, acc);
+  else gather_vec<T, C, false>(p, acc);
+}
+
 // Where gathered rows of x come from.
 // GlobalSrc: global memory, rows below `hub` with L1 retention priority.
 template <typename T, int C>
@@ -155,6 +165,7 @@ struct GlobalSrc {
   const T* __restrict__ X;
   int hub;
   __device__ __forceinline__ void add(T (&acc)[C], int v) const { add_row<T, C>(acc, X, v, hub); }
+  __device__ __forceinline__ void set(T (&acc)[C], int v) const { set_row<T, C>(acc, X, v, hub); }
 };
 
 // Column indices are streamed once per sweep: keep them out of L1 (which holds the gathered
@@ -407,9 +418,16 @@ __device__ __forceinline__ void short_rows(const SweepArgs& a, const Src& src, c
       acca[c] = T(0);
       accb[c] = T(0);
     }
-    if (va0 >= 0) src.add(acca, va0);
+    if constexpr (sizeof(T) == 8) {
+      if (va0 >= 0) src.set(acca, va0);
+      if (vb0 >= 0) src.set(accb, vb0);
+    } else {
+      if (va0 >= 0) src.add(acca, va0);
+    }
     if (va1 >= 0) src.add(acca, va1);
-    if (vb0 >= 0) src.add(accb, vb0);
+    if constexpr (sizeof(T) == 4) {
+      if (vb0 >= 0) src.add(accb, vb0);
+    }
     if (vb1 >= 0) src.add(accb, vb1);
     SC::run(acca, lane);
     SC::run(accb, lane);
@@ -561,13 +579,13 @@ constexpr int kCandSlots = 16;
 
 // Resident CTAs per SM each instantiation is compiled for (its register limit). The gathers wait
 // on memory, and more resident warps hide more of that latency than a few spilled registers cost:
-// the 8-column lookahead sweep is held to 48 registers (five CTAs per SM), the 4-column candidate
-// batch to 64 (four), the one-step fused and two-state sweeps of 1-2 columns to 32 (eight) and of 4
-// to 40 (six), and the batched-scoring widths to what their C-wide row sums need (measured on R-MAT
-// scale 22 and on the Barabasi-Albert graph with n = 10^6).
+// the 8-column sweeps of the runs are held to 48 registers (five CTAs per SM), the narrower ones to 40
+// (six), the two-state sweeps to 32 (eight), FP64 to 64 (four; five changed nothing), and the
+// batched-scoring widths to what their C-wide row sums need (measured on R-MAT scale 22 and on the
+// Barabasi-Albert graph with n = 10^6).
 template <typename T, int C, int MODE>
 constexpr int min_ctas() {
-  if (sizeof(T) == 8) return 1;
+  if (sizeof(T) == 8) return 4;
   if ((MODE == MODE_LOOK || MODE == MODE_PAR) && C == 8) return 5;
   if ((MODE == MODE_LOOK || MODE == MODE_PAR) && C <= 4) return 6;
   if ((MODE == MODE_MISS || MODE == MODE_SCORE || MODE == MODE_PAIR) && C <= 2) return 8;
