@@ -109,9 +109,9 @@ void profile_end(cudaStream_t s, cudaEvent_t a, double bytes, int key) {
 }
 
 double sweep_bytes(int mode, bool fp64, int cols, int32_t n, int64_t nnz, bool weighted) {
-  const double es = mode == MODE_TOTALS ? 8.0 : (fp64 ? 8.0 : 4.0);
+  const double es = fp64 ? 8.0 : 4.0;
   double b = 4.0 * double(nnz) + 4.0 * (double(n) + 1.0) + 2.0 * cols * es * double(n);
-  if (mode != MODE_TOTALS && mode != MODE_PLAIN) b += double(n) / 8.0;
+  if (mode != MODE_TOTALS && mode != MODE_WALKS && mode != MODE_PLAIN) b += double(n) / 8.0;
   if (mode == MODE_MISS) b += es * double(n);
   if (weighted) b += es * double(n);  // the vertex scales
   return b;
@@ -930,7 +930,8 @@ gedwalk_status reduce_slots(Graph& g, Workspace& ws, int nsum, double* out, cuda
 }
 
 // ---------------------------------------------------------------- walk totals
-gedwalk_status ensure_totals(Graph& g, double alpha, int32_t rows, cudaStream_t s) {
+gedwalk_status ensure_totals(Graph& g, double alpha, int32_t lengths, cudaStream_t s) {
+  const int32_t rows = walk_rows(g, lengths);
   {
     std::shared_lock<std::shared_mutex> rl(g.tt_lock);
     if (g.tt_alpha == alpha && rows <= g.tt_rows) return GEDWALK_OK;
@@ -955,18 +956,21 @@ gedwalk_status ensure_totals(Graph& g, double alpha, int32_t rows, cudaStream_t 
     g.ttab.swap(fresh);
     GW_CUDA(cudaStreamSynchronize(s));
   }
-  if (g.Wa_d.bytes < static_cast<size_t>(rows) * sizeof(double)) {
-    // grow the device sums, keeping the rows already computed
+  // W_0, then one sum per row, or (undirected) two: row r gives W_{2r-1} and W_{2r}
+  const int per = g.directed ? 1 : 2;
+  auto first = [&](int32_t r) { return r == 0 ? 0 : per * (r - 1) + 1; };
+  if (g.Wa_d.bytes < static_cast<size_t>(first(rows)) * sizeof(double)) {
+    // grow the device sums, keeping those already computed
     DevBuf fresh;
-    GW_TRY(fresh.ensure(static_cast<size_t>(std::max(rows, 64)) * sizeof(double), s));
+    GW_TRY(fresh.ensure(static_cast<size_t>(std::max(2 * first(rows), 64)) * sizeof(double), s));
     if (g.tt_rows > 0)
-      GW_CUDA(cudaMemcpyAsync(fresh.p, g.Wa_d.p, static_cast<size_t>(g.tt_rows) * sizeof(double),
+      GW_CUDA(cudaMemcpyAsync(fresh.p, g.Wa_d.p, static_cast<size_t>(first(g.tt_rows)) * sizeof(double),
                               cudaMemcpyDeviceToDevice, s));
     g.Wa_d.swap(fresh);
     GW_CUDA(cudaStreamSynchronize(s));
   }
   Workspace& ws = g.ws;
-  GW_TRY(ensure_sweep_scratch(g, ws, 1, true, s));
+  GW_TRY(ensure_sweep_scratch(g, ws, per, true, s));
   double* T = g.ttab.as<double>();
   double* dWa = g.Wa_d.as<double>();
   int32_t r0 = g.tt_rows;
@@ -995,14 +999,14 @@ gedwalk_status ensure_totals(Graph& g, double alpha, int32_t rows, cudaStream_t 
     if (g.n_active < g.n)  // isolated vertices start no walk of length >= 1
       GW_CUDA(cudaMemsetAsync(T + static_cast<size_t>(r) * n + g.n_active, 0,
                               sizeof(double) * (n - static_cast<size_t>(g.n_active)), s));
-    GW_TRY(launch_sweep(MODE_TOTALS, true, 1, a, s));
-    GW_TRY(reduce_slots(g, ws, 1, dWa + r, s, g.directed));
+    GW_TRY(launch_sweep(g.directed ? MODE_TOTALS : MODE_WALKS, true, 1, a, s));
+    if (g.plan.num_units > 0) GW_TRY(reduce_slots(g, ws, per, dWa + first(r), s, g.directed));
+    else GW_CUDA(cudaMemsetAsync(dWa + first(r), 0, sizeof(double) * per, s));  // no edges, no walks
   }
-  std::vector<double> tmp(rows);
-  GW_CUDA(cudaMemcpyAsync(tmp.data() + r0, dWa + r0, sizeof(double) * (rows - r0), cudaMemcpyDeviceToHost, s));
+  const int32_t w0 = first(r0), w1 = first(rows);
+  g.Wa.resize(w1);
+  if (w1 > w0) GW_CUDA(cudaMemcpyAsync(g.Wa.data() + w0, dWa + w0, sizeof(double) * (w1 - w0), cudaMemcpyDeviceToHost, s));
   GW_CUDA(cudaStreamSynchronize(s));
-  g.Wa.resize(rows);
-  for (int32_t r = r0; r < rows; ++r) g.Wa[r] = tmp[r];
   g.tt_rows = rows;
   return GEDWALK_OK;
 }
@@ -1217,10 +1221,11 @@ gedwalk_status truncation_length(Graph& g, double alpha, double eps, int32_t* L,
       return GEDWALK_OK;
     }
   const int32_t kCap = 4096;
-  int32_t rows = std::max(g.tt_alpha == alpha ? g.tt_rows : 0, 4);
+  int32_t rows = std::max(g.tt_alpha == alpha ? static_cast<int32_t>(g.Wa.size()) : 0, 4);
   Workspace& ws = g.ws;
   for (;;) {
-    GW_TRY(ensure_totals(g, alpha, rows, s));
+    GW_TRY(ensure_totals(g, alpha, std::min(rows, kCap), s));
+    rows = std::min(std::max(rows, static_cast<int32_t>(g.Wa.size())), kCap);  // as many as there are
     GW_TRY(ws.small.ensure(64, s));
     // the stop test reads the row sums where the sweeps' reductions left them
     double* db = ws.small.as<double>();

@@ -365,7 +365,7 @@ gedwalk_status maximize_impl(Graph& g, Workspace& ws, int32_t k, const Resolved&
     GW_TRY(bound_coef(g, r.alpha, r.bound_kind, r.stream, &p.coef));
     GW_TRY(ensure_totals(g, r.alpha, p.shape.ell_max + 1, r.stream));
     std::shared_lock<std::shared_mutex> rl(g.tt_lock);
-    if (g.tt_alpha != r.alpha || g.tt_rows < p.shape.ell_max + 1)
+    if (g.tt_alpha != r.alpha || static_cast<int32_t>(g.Wa.size()) < p.shape.ell_max + 1)
       return fail(GEDWALK_ERR_INVALID, "the walk-total table was replaced for another alpha during the call");
     p.Wa.assign(g.Wa.begin(), g.Wa.begin() + p.shape.ell_max + 1);
   }

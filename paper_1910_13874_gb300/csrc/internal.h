@@ -244,13 +244,14 @@ struct Graph {
 
 // ---------------------------------------------------------------- launchers
 enum SweepMode : int {
-  MODE_TOTALS = 0,  // y = alpha A x, FP64, stores the column sum
+  MODE_TOTALS = 0,  // directed walk totals, power iteration: y = alpha A x, FP64, stores the column sum
   MODE_SCORE = 1,   // directed scoring: two-state hit/miss step, sums h
   MODE_MISS = 2,    // phi^miss under S, stored in a table too
   MODE_PLAIN = 4,   // batched scoring: y = alpha A x, no mask
   MODE_LOOK = 5,    // run, chain: phi^miss under S, then the walks through c_j avoiding S + {c_1..c_{j-1}}
   MODE_PAR = 6,     // run: phi^miss under S, then the walks through each c_j avoiding S
-  MODE_PAIR = 7     // scoring run: the two-state hit/miss step without its sum
+  MODE_PAIR = 7,    // scoring run: the two-state hit/miss step without its sum
+  MODE_WALKS = 8    // walk totals of an undirected graph: y = alpha A x, sums <y, x> and <y, y>
 };
 
 struct SweepArgs {
@@ -344,7 +345,10 @@ int64_t maximize_footprint(const Graph& g, const Resolved& r, int32_t flags, int
 int64_t score_batch_footprint(const Graph& g, int64_t members, int32_t groups);
 // Resolves alpha (0 -> default), L (from epsilon unless forced) for a given epsilon.
 gedwalk_status resolve(Graph& g, const gedwalk_params* p, double eps_override, Resolved* r);
-// Ensures the FP64 walk-total table holds rows 0..rows-1 for alpha.
+// Rows of the walk-total table that give W_0..W_{lengths-1}: the walks of length a + b number
+// <t_a, t_b> on an undirected graph.
+inline int32_t walk_rows(const Graph& g, int32_t lengths) { return g.directed ? lengths : lengths / 2 + 1; }
+// Ensures the walk totals W_0..W_{rows-1} for alpha, and the walk_rows(g, rows) rows of the FP64 table.
 gedwalk_status ensure_totals(Graph& g, double alpha, int32_t rows, cudaStream_t s);
 // Walk totals t_from..t_{rows-1} (FP64, rows g.n apart) into a table of the caller's that holds the
 // rows before, with the caller's workspace: walks that start at a vertex, or (rev) that end there.

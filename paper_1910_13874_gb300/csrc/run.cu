@@ -279,36 +279,58 @@ __global__ void run_own(T* __restrict__ X, int64_t set, int cols, RunDev* __rest
   d->live[o][j] = dg > 0;
 }
 
-// Tail bounds from the walk-total tables t_0..t_L of both orientations (FP64, rows n apart; times s on
-// a weighted graph; A = B unless directed):
-//   tail(v) = sum over pairs p + q <= L with p or q above H of b_p a_q
-//           = sum_{p>H} b_p Qa_{L-p} + sum_{q>H} a_q Qb_{L-q},  Q_q = t_0 + ... + t_q,
-// rounded up; and (about) the bound of the empty group, F + U + F U + tail, for the first guesses.
-__global__ void tail_kernel(const double* __restrict__ A, const double* __restrict__ B, int64_t n, int32_t n_active,
-                            int32_t L, int32_t H, const double* __restrict__ rs, double alpha, float* __restrict__ tail,
-                            float* __restrict__ bound) {
+// Tail bounds from the walk-total tables (FP64, rows n apart; times s on a weighted graph): the pairs
+// p + q <= L with p or q above H.
+// Directed (A: walks that start at v, B: that end there, both to L):
+//   tail(v) = sum_{p>H} b_p Qa_{L-p} + sum_{q>H} a_q Qb_{L-q},  Q_q = t_0 + ... + t_q.
+// Undirected (A = B, rows 0..H): t_{H+b}(v) <= t_H(v) M_b, M_b the largest t_b (a walk of length H + b
+// from v is one of length H and one of length b from its end), so
+//   tail(v) = 2 t_H(v) sum_{b=1..L-H} M_b Q_{L-H-b}.
+// Rounded up; and (about) the bound of the empty group, F + U + F U + tail, for the first guesses.
+__global__ void row_max_kernel(const double* __restrict__ A, int64_t n, int32_t n_active, const double* __restrict__ rs,
+                               unsigned long long* __restrict__ M) {
+  const double* row = A + static_cast<size_t>(blockIdx.y + 1) * n;
+  double m = 0.0;
+  for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n_active; v += gridDim.x * blockDim.x)
+    m = fmax(m, rs ? row[v] / rs[v] : row[v]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(kFullMask, m, o));
+  if ((threadIdx.x & 31) == 0) atomicMax(M + blockIdx.y + 1, static_cast<unsigned long long>(__double_as_longlong(m)));
+}
+
+__global__ void tail_kernel(const double* __restrict__ A, const double* __restrict__ B, const double* __restrict__ M,
+                            int64_t n, int32_t n_active, int32_t L, int32_t H, const double* __restrict__ rs, double alpha,
+                            float* __restrict__ tail, float* __restrict__ bound) {
   for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n_active; v += gridDim.x * blockDim.x) {
     const double inv = rs ? 1.0 / rs[v] : 1.0;
     double Qa = 0.0, Qb = 0.0, acc = 0.0, U = 0.0, F = 0.0;
-    for (int32_t q = 0; q < L - H; ++q) {
-      Qa += A[static_cast<size_t>(q) * n + v] * inv;
-      if (A == B) {
-        acc += 2.0 * A[static_cast<size_t>(L - q) * n + v] * inv * Qa;
-      } else {
-        Qb += B[static_cast<size_t>(q) * n + v];
-        acc += B[static_cast<size_t>(L - q) * n + v] * Qa + A[static_cast<size_t>(L - q) * n + v] * Qb;
-      }
-    }
-    for (int32_t t = 1; t <= H; ++t) U += A[static_cast<size_t>(t) * n + v] * inv;
-    acc *= 1.0 + 1e-12;
-    tail[v] = __double2float_ru(acc);
     if (A == B) {
+      for (int32_t q = 0; q < L - H; ++q) {
+        const double t = A[static_cast<size_t>(q) * n + v] * inv;
+        Qa += t;
+        if (q > 0) U += t;
+        acc += __ldg(M + (L - H - q)) * Qa;
+      }
+      for (int32_t t = std::max(L - H, 1); t < H; ++t) U += A[static_cast<size_t>(t) * n + v] * inv;
+      const double tH = A[static_cast<size_t>(H) * n + v] * inv;
+      U += tH;
+      acc *= 2.0 * tH;
       const double f1 = A[n + v] * inv, f2 = H >= 2 ? A[2 * n + v] * inv : 0.0;
       const double s2 = rs ? 0.0 : alpha * f1, s4 = rs || H < 4 ? 0.0 : alpha * alpha * f2 - alpha * alpha * alpha * f1;
       F = U - (H >= 2 ? (s2 + s4) * (1.0 + U) : 0.0);
     } else {
-      for (int32_t t = 1; t <= H; ++t) F += B[static_cast<size_t>(t) * n + v];
+      for (int32_t q = 0; q < L - H; ++q) {
+        Qa += A[static_cast<size_t>(q) * n + v];
+        Qb += B[static_cast<size_t>(q) * n + v];
+        acc += B[static_cast<size_t>(L - q) * n + v] * Qa + A[static_cast<size_t>(L - q) * n + v] * Qb;
+      }
+      for (int32_t t = 1; t <= H; ++t) {
+        U += A[static_cast<size_t>(t) * n + v];
+        F += B[static_cast<size_t>(t) * n + v];
+      }
     }
+    acc *= 1.0 + 1e-12;
+    tail[v] = __double2float_ru(acc);
     bound[v] = static_cast<float>(F + U + F * U + acc);
   }
 }
@@ -993,34 +1015,42 @@ gedwalk_status RunEngine::set_length(int32_t length, bool select) {
   if (!select || g.n_active == 0) return GEDWALK_OK;
   // tail bounds from the walk totals; the tables are read under their lock, to the end of the kernel
   const double* rs = g.weighted ? g.rs_d.as<double>() : nullptr;
+  const int32_t rows = walk_rows(g, L + 1);
+  // the largest entries of rows 1..L-H (the selections' lists are free here)
+  unsigned long long* M = ws.sel.as<unsigned long long>();
+  auto tails = [&](const double* A, const double* B) -> gedwalk_status {
+    if (!g.directed && L > H) {
+      GW_CUDA(cudaMemsetAsync(M, 0, sizeof(*M) * (L - H + 1), s));
+      row_max_kernel<<<dim3(std::min(grid_of(g.n_active), 304), L - H), 256, 0, s>>>(A, g.n, g.n_active, rs, M);
+      GW_KCHECK();
+    }
+    tail_kernel<<<grid_of(g.n_active), 256, 0, s>>>(A, B, reinterpret_cast<const double*>(M), g.n, g.n_active, L, H, rs, r.alpha,
+                                                    ws.tail.as<float>(), ws.bound.as<float>());
+    GW_KCHECK();
+    return GEDWALK_OK;
+  };
   bool table;
   {
     std::shared_lock<std::shared_mutex> rl(g.tt_lock);
-    table = g.tt_alpha == r.alpha && g.tt_rows >= L + 1;
+    table = g.tt_alpha == r.alpha && g.tt_rows >= rows;
   }
-  if (table && g.directed) GW_TRY(ensure_totals_fwd(g, ws, r.alpha, L + 1, s));
+  if (table && g.directed) GW_TRY(ensure_totals_fwd(g, ws, r.alpha, rows, s));
   {
     std::shared_lock<std::shared_mutex> rl(g.tt_lock);
-    if (g.tt_alpha == r.alpha && g.tt_rows >= L + 1 && (!g.directed || (g.ttf_alpha == r.alpha && g.ttf_rows >= L + 1))) {
-      const double* B = g.ttab.as<double>();
-      tail_kernel<<<grid_of(g.n_active), 256, 0, s>>>(g.directed ? g.ttab_f.as<double>() : B, B, g.n, g.n_active, L, H, rs,
-                                                      r.alpha, ws.tail.as<float>(), ws.bound.as<float>());
-      GW_KCHECK();
+    if (g.tt_alpha == r.alpha && g.tt_rows >= rows && (!g.directed || (g.ttf_alpha == r.alpha && g.ttf_rows >= rows))) {
+      GW_TRY(tails(g.directed ? g.ttab_f.as<double>() : g.ttab.as<double>(), g.ttab.as<double>()));
       GW_CUDA(cudaStreamSynchronize(s));
       return GEDWALK_OK;
     }
   }
   // no table for this alpha (a forced L beyond the bound's reach): totals of this call's own
-  const size_t n = static_cast<size_t>(g.n), rows = static_cast<size_t>(L + 1);
-  GW_TRY(ws.ztab.ensure((g.directed ? 2 : 1) * rows * n * sizeof(double), s));
+  const size_t cells = static_cast<size_t>(rows) * g.n;
+  GW_TRY(ws.ztab.ensure((g.directed ? 2 : 1) * cells * sizeof(double), s));
   double* A = ws.ztab.as<double>();
-  double* B = g.directed ? A + rows * n : A;
-  GW_TRY(totals_into(g, ws, A, r.alpha, 0, L + 1, false, s));
-  if (g.directed) GW_TRY(totals_into(g, ws, B, r.alpha, 0, L + 1, true, s));
-  tail_kernel<<<grid_of(g.n_active), 256, 0, s>>>(A, B, g.n, g.n_active, L, H, rs, r.alpha, ws.tail.as<float>(),
-                                                  ws.bound.as<float>());
-  GW_KCHECK();
-  return GEDWALK_OK;
+  double* B = g.directed ? A + cells : A;
+  GW_TRY(totals_into(g, ws, A, r.alpha, 0, rows, false, s));
+  if (g.directed) GW_TRY(totals_into(g, ws, B, r.alpha, 0, rows, true, s));
+  return tails(A, B);
 }
 
 void RunEngine::stale(int32_t v, double gain, int32_t step) {

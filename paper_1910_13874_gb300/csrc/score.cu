@@ -330,7 +330,7 @@ int64_t score_batch_footprint(const Graph& g, int64_t members, int32_t groups) {
 }
 
 // The blocks of an undirected graph's batch; the members (rows, columns) are on the device, the scores
-// go to ws.small. The table holds rows 0..L (the caller keeps its lock).
+// go to ws.small. The table holds rows 0..H (the caller keeps its lock).
 static gedwalk_status batch_runs(Graph& g, Workspace& ws, int C, const int32_t* offsets, int32_t G, const int32_t* mrow,
                                  const int32_t* mcol, const Resolved& r, cudaStream_t s) {
   const int32_t L = r.L, H = (L + 1) / 2;
@@ -404,9 +404,9 @@ gedwalk_status score_batch_impl(Graph& g, Workspace& ws, const int32_t* offsets,
   cudaStream_t s = r.stream;
   if (G == 0) return GEDWALK_OK;
   StreamGuard guard{s};
-  // the caller has made the walk-total table hold rows 0..L for alpha and tuned the width
+  // the caller has made the walk-total table for alpha and L, and tuned the width
   std::shared_lock<std::shared_mutex> rl(g.tt_lock);
-  if (g.tt_alpha != r.alpha || g.tt_rows < r.L + 1 || g.batch_cols <= 0)
+  if (g.tt_alpha != r.alpha || g.tt_rows < walk_rows(g, r.L + 1) || g.batch_cols <= 0)
     return fail(GEDWALK_ERR_INVALID, "walk-total table or column width not prepared for this batch");
   const int C = g.batch_cols;
   const int64_t total = offsets[G];

@@ -221,9 +221,15 @@ struct Scatter {
 // Number of FP64 column sums a mode keeps.
 template <int MODE, int C>
 struct Sums {
-  static constexpr int N = MODE == MODE_TOTALS || MODE == MODE_SCORE ? 1 : 0;
+  static constexpr int N = MODE == MODE_WALKS ? 2 : MODE == MODE_TOTALS || MODE == MODE_SCORE ? 1 : 0;
   // the sum fed by column c, or -1
   __device__ __forceinline__ static int slot(int c) { return c < N ? c : -1; }
+};
+
+// Sums a lane keeps: one per column it holds, or MODE_WALKS' two.
+template <int MODE, int CPL>
+struct LaneSums {
+  static constexpr int N = MODE == MODE_WALKS ? 2 : CPL;
 };
 
 // Number of candidate ids a mode reads (the only rows whose epilogue differs from y = alpha s).
@@ -296,10 +302,10 @@ __device__ __forceinline__ void candidate_rows(const SweepArgs& a, const int* __
 // per-row candidate test is skipped.
 template <typename T, int C, int MODE, int CPL>
 __device__ __forceinline__ void epilogue(const SweepArgs& a, const int* __restrict__ s_cand,
-                                         const int* __restrict__ s_live, int r, bool valid, bool store, int c0, int base, T (&s)[CPL], ColAcc<T, CPL>& acc,
+                                         const int* __restrict__ s_live, int r, bool valid, bool store, int c0, int base, T (&s)[CPL], ColAcc<T, LaneSums<MODE, CPL>::N>& acc,
                                          bool maybe_cand) {
   T* Y = static_cast<T*>(a.Y);
-  constexpr bool kMasked = MODE != MODE_TOTALS && MODE != MODE_PLAIN;
+  constexpr bool kMasked = MODE != MODE_TOTALS && MODE != MODE_WALKS && MODE != MODE_PLAIN;
   const bool inS = kMasked && valid ? in_mask(a.mask, r) : false;
   // weighted graph: the row's scale s_r turns the gathered sum into the true value
   // alpha s_r (A x~)(r), which is summed, and the stored vector is x~ = s_r * value
@@ -340,7 +346,12 @@ __device__ __forceinline__ void epilogue(const SweepArgs& a, const int* __restri
       if (store && c0 == 0) static_cast<T*>(a.Mout)[r] = y[0];
     }
     if (store) {
-      if constexpr (Sums<MODE, C>::N > 0) {
+      if constexpr (MODE == MODE_WALKS) {
+        // W_{2r-1} = <t_r, t_{r-1}> and W_{2r} = <t_r, t_r>: the two halves of a walk meet
+        const T x = __ldg(static_cast<const T*>(a.X) + r);
+        acc.add(0, y[0] * (rs ? x / sv : x));
+        acc.add(1, y[0] * y[0]);
+      } else if constexpr (Sums<MODE, C>::N > 0) {
 #pragma unroll
         for (int k = 0; k < CPL; ++k)
           if (Sums<MODE, C>::slot(c0 + k) >= 0) acc.add(k, y[k]);
@@ -363,12 +374,13 @@ __device__ __forceinline__ bool unit_has_cand(const int* __restrict__ s_cand, in
 
 // Writes this lane's column sums (already reduced over the warp) to slot `slot`.
 template <int MODE, int C, int CPL>
-__device__ __forceinline__ void write_slot(const SweepArgs& a, size_t slot, int c0, const double (&cs)[CPL]) {
+__device__ __forceinline__ void write_slot(const SweepArgs& a, size_t slot, int c0,
+                                           const double (&cs)[LaneSums<MODE, CPL>::N]) {
   constexpr int NS = Sums<MODE, C>::N;
   if constexpr (NS > 0) {
     double* dst = a.slots + slot * NS;
 #pragma unroll
-    for (int k = 0; k < CPL; ++k) {
+    for (int k = 0; k < LaneSums<MODE, CPL>::N; ++k) {
       const int j = Sums<MODE, C>::slot(c0 + k);
       if (j >= 0) dst[j] = a.accumulate ? dst[j] + cs[k] : cs[k];
     }
@@ -392,7 +404,8 @@ __device__ __forceinline__ void short_rows(const SweepArgs& a, const Src& src, c
   const int c0 = blk * CPL;
   const int32_t* __restrict__ ci = a.ci;
   const uint64_t pol = stream_policy();
-  ColAcc<T, CPL> acc;
+  constexpr int NL = LaneSums<MODE, CPL>::N;
+  ColAcc<T, NL> acc;
   acc.zero();
   for (int it = 0; it < nrows; it += 2 * NG) {
     const int ra = it + g, rb = it + NG + g;
@@ -441,13 +454,13 @@ __device__ __forceinline__ void short_rows(const SweepArgs& a, const Src& src, c
     epilogue<T, C, MODE, CPL>(a, s_cand, s_live, r0 + rb, vb, vb && owner, c0, base, sb, acc, maybe_cand);
   }
   // sum the groups' copies of each column (non-owners hold zeros), in FP64
-  double cs[CPL];
+  double cs[NL];
 #pragma unroll
-  for (int k = 0; k < CPL; ++k) cs[k] = acc.get(k);
+  for (int k = 0; k < NL; ++k) cs[k] = acc.get(k);
 #pragma unroll
   for (int o = W; o < 32; o <<= 1)
 #pragma unroll
-    for (int k = 0; k < CPL; ++k) cs[k] += __shfl_xor_sync(kFull, cs[k], o);
+    for (int k = 0; k < NL; ++k) cs[k] += __shfl_xor_sync(kFull, cs[k], o);
   if (lane < W && owner) write_slot<MODE, C, CPL>(a, static_cast<size_t>(uidx), c0, cs);
 }
 
@@ -464,7 +477,8 @@ __device__ __forceinline__ void long_rows(const SweepArgs& a, const Src& src, co
   const int c0 = blk * CPL;
   const int32_t* __restrict__ ci = a.ci;
   const uint64_t pol = stream_policy();
-  ColAcc<T, CPL> cacc;
+  constexpr int NL = LaneSums<MODE, CPL>::N;
+  ColAcc<T, NL> cacc;
   cacc.zero();
   for (int rr = 0; rr < nrows; ++rr) {
     const int e0 = s_rp[rr], e1 = s_rp[rr + 1];
@@ -487,9 +501,9 @@ __device__ __forceinline__ void long_rows(const SweepArgs& a, const Src& src, co
     for (int k = 0; k < CPL; ++k) s[k] = acc[k];
     epilogue<T, C, MODE, CPL>(a, s_cand, s_live, r0 + rr, true, owner, c0, 0, s, cacc, maybe_cand);
   }
-  double cs[CPL];
+  double cs[NL];
 #pragma unroll
-  for (int k = 0; k < CPL; ++k) cs[k] = cacc.get(k);
+  for (int k = 0; k < NL; ++k) cs[k] = cacc.get(k);
   if (owner) write_slot<MODE, C, CPL>(a, static_cast<size_t>(uidx), c0, cs);
 }
 
@@ -544,12 +558,13 @@ __device__ __forceinline__ void heavy_slice(const SweepArgs& a, const Src& src, 
   for (int s = hr.y; s < hr.y + hr.z; ++s)
 #pragma unroll
     for (int k = 0; k < CPL; ++k) tot[k] += __ldcg(part + static_cast<size_t>(s) * C + c0 + k);
-  ColAcc<T, CPL> cacc;
+  constexpr int NL = LaneSums<MODE, CPL>::N;
+  ColAcc<T, NL> cacc;
   cacc.zero();
   epilogue<T, C, MODE, CPL>(a, s_cand, s_live, hr.x, true, owner, c0, 0, tot, cacc, true);
-  double cs[CPL];
+  double cs[NL];
 #pragma unroll
-  for (int k = 0; k < CPL; ++k) cs[k] = cacc.get(k);
+  for (int k = 0; k < NL; ++k) cs[k] = cacc.get(k);
   if (owner) write_slot<MODE, C, CPL>(a, static_cast<size_t>(a.num_units + u.x), c0, cs);
   if (lane == 0) a.counters[u.x] = 0u;  // ready for the next launch
 }
@@ -656,12 +671,13 @@ __global__ void __launch_bounds__(kThreads) reduce_slots_part(const double* __re
   if (threadIdx.x == 0) parts[c * kReduceParts + part] = v;
 }
 
-__global__ void reduce_slots_final(const double* __restrict__ parts, int32_t nsum, double* __restrict__ out) {
-  const int c = threadIdx.x;
-  if (c >= nsum) return;
+// One warp per column.
+__global__ void reduce_slots_final(const double* __restrict__ parts, double* __restrict__ out) {
   double s = 0.0;
-  for (int p = 0; p < kReduceParts; ++p) s += parts[c * kReduceParts + p];
-  out[c] = s;
+  for (int p = threadIdx.x; p < kReduceParts; p += 32) s += parts[blockIdx.x * kReduceParts + p];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+  if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
 
 // Sets the instantiation's shared-memory carveout on the current device, once per device: a small
@@ -712,6 +728,8 @@ gedwalk_status run(const SweepArgs& a, cudaStream_t s, bool profile) {
 
 int sweep_sums(int mode, int cols) {
   switch (mode) {
+    case MODE_WALKS:
+      return 2;
     case MODE_TOTALS:
     case MODE_SCORE:
       return 1;
@@ -724,6 +742,7 @@ gedwalk_status launch_sweep(int mode, bool fp64, int cols, const SweepArgs& a, c
 #define GW_CASE(M, T, C) \
   if (mode == M && fp64 == (sizeof(T) == 8) && cols == C) return run<T, C, M>(a, s, profile);
   GW_CASE(MODE_TOTALS, double, 1)
+  GW_CASE(MODE_WALKS, double, 1)
   GW_CASE(MODE_SCORE, double, 2)
   GW_CASE(MODE_SCORE, float, 2)
   GW_CASE(MODE_PAIR, double, 2)
@@ -754,7 +773,7 @@ gedwalk_status launch_reduce_slots(const double* slots, int32_t num_slots, int32
   if (nsum <= 0) return GEDWALK_OK;
   reduce_slots_part<<<dim3(kReduceParts, nsum), kThreads, 0, s>>>(slots, num_slots, nsum, parts);
   GW_KCHECK();
-  reduce_slots_final<<<1, 32, 0, s>>>(parts, nsum, out);
+  reduce_slots_final<<<nsum, 32, 0, s>>>(parts, out);
   GW_KCHECK();
   return GEDWALK_OK;
 }
