@@ -47,7 +47,7 @@ def parse():
     ap.add_argument("--k", type=int, default=100)
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--device-loop", action="store_true",
-                    help="greedy: run the k steps as one device-resident CUDA graph (its kernels are hidden from ncu)")
+                    help="greedy: pass GEDWALK_DEVICE_LOOP (accepted; the same loop runs)")
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--batch-cols", type=int, default=0,
                     help="batch workload: pin the column-block width (0 = the autotuner picks it)")
@@ -149,8 +149,8 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
-MODE_NAMES = {0: "totals", 1: "two-state score", 2: "fused greedy", 3: "candidate batch", 4: "batched scoring",
-              5: "lookahead greedy"}
+MODE_NAMES = {0: "totals", 1: "two-state score", 2: "phi^miss", 4: "batched scoring", 5: "greedy chain run",
+              6: "greedy candidate run", 7: "two-state score", 8: "totals"}
 
 
 def recorded_traffic(top, workload_key):
@@ -161,7 +161,7 @@ def recorded_traffic(top, workload_key):
     """
     from paper_1910_13874_gb300.kernel_hash import sweep_kernel_hash
 
-    files = {("rmat22", 2, 2, 0): "sweep_fused_f2_rmat22.md", ("rmat22", 5, 8, 0): "sweep_look_f8_rmat22.md"}
+    files = {("rmat22", 5, 8, 0): "sweep_look_f8_rmat22.md"}
     name = files.get((workload_key, top["top_mode"], top["top_cols"], top["top_fp64"]))
     if not name:
         return None

@@ -96,10 +96,11 @@ typedef struct {
   uint64_t seed;           /* stochastic greedy: seed of the counter-based sample draws */
   int32_t bound;           /* GEDWALK_BOUND_COMBINATORIAL (default) or GEDWALK_BOUND_SPECTRAL */
   int32_t lookahead;       /* maximize: greedy steps carried by one run of sweeps (see gedwalk_maximize):
-                              0 = default (7 in FP32, 3 in FP64), 1 = off, 3 or (FP32) 7 */
-  int32_t spec_cols;       /* maximize without lookahead: columns of the fused sweep (phi^miss plus
-                              speculative candidates): 0 = default (2; 4 with GEDWALK_ADAPTIVE_L), 2, 4
-                              or (FP32) 8 */
+                              0 = default (7; 3 in FP64 on very large graphs), 1 = off, 3 or
+                              (FP32) 7 */
+  int32_t spec_cols;       /* maximize without lookahead: columns of the one-step run (phi^miss plus
+                              speculative candidates): 0 = default (2), 2, 4 or (FP32) 8; on a directed
+                              graph or with a flag a value other than 0 turns the lookahead off */
   int32_t reserved;        /* 0 */
 } gedwalk_params;
 
@@ -241,9 +242,12 @@ GEDWALK_API gedwalk_status gedwalk_score(gedwalk_graph_t g, const int32_t* S, in
 
 /*
  * Scores G groups at once (problem (i) for many groups). Group j is
- * members[offsets[j] .. offsets[j+1]). Groups become the columns of one masked
+ * members[offsets[j] .. offsets[j+1]). Groups become the columns of one
  * FP32 SpMM over column blocks whose width an on-device autotuner picks; the
- * per-group hit sums are FP64. The hits are counted by first visits:
+ * per-group hit sums are FP64. On an undirected graph a column holds the walks
+ * that end at a vertex and hit the group, to half the length; a walk of length
+ * a + b hits it in its first half or else in its second. On a directed graph the
+ * hits are counted by first visits over the full length:
  *   GED_{<=L}(S) = sum_{s in S} sum_{p=0..L} alpha^p F_p(s) * K_{L-p}(s),
  * F_p(s) the p-walks ending at s whose earlier vertices avoid S, and K_q(s) the
  * alpha-weighted walks of length <= q starting at s (the p = 0 term excludes
@@ -315,7 +319,7 @@ GEDWALK_API gedwalk_status gedwalk_gains(gedwalk_graph_t g, const int32_t* S, in
  * guessed needs no sweep. Every pick is still certified against the bounds of
  * the actual group, so the results do not depend on it. params->lookahead
  * (1 = off, 3; 7 in FP32; read without a flag) sets the number of steps per run
- * (0: 7 in FP32, 3 in FP64); params->spec_cols the width of the one-step run
+ * (0: 7, or 3 in FP64 on very large graphs); params->spec_cols the width of the one-step run
  * when the lookahead is off. Other values return INVALID. The host drives the
  * steps with one synchronisation per run.
  * GEDWALK_ADAPTIVE_L runs the lazy greedy of Algorithm 2 (Section 3.2.3): the
@@ -490,11 +494,11 @@ typedef struct {
   double sweep_ms;         /* summed device time of those launches (CUDA events on their stream) */
   double sweep_bytes;      /* summed algorithmic bytes of those launches: per launch the CSR (4 nnz
                               + 4 (n+1)), x read and y written once (2 C s n for C columns of s
-                              bytes), the S mask (n/8) where masked, the phi^miss rows written
-                              (s n fused, (C-1) s n lookahead) and the vertex scales (s n, weighted) */
+                              bytes), the S mask (n/8) where masked, a phi^miss row written
+                              (mode 2) and the vertex scales (s n, weighted) */
   /* the sweep instantiation with the largest summed time: */
-  int32_t top_mode;        /* 0 totals, 1 two-state score, 2 fused greedy, 3 candidates, 4 batched,
-                              5 greedy lookahead */
+  int32_t top_mode;        /* 0 and 8 totals, 1 and 7 two-state score, 2 phi^miss, 4 batched, 5 greedy
+                              chain run, 6 greedy candidate run */
   int32_t top_cols;        /* columns per row */
   int32_t top_fp64;        /* 1 for FP64 rows */
   int32_t top_pad;

@@ -46,11 +46,16 @@ gedwalk_status greedy_shape(const Graph& g, const Resolved& r, int32_t flags, Gr
   // Lookahead: one run carries `levels` steps, level d under S + {c_1..c_d} with
   // the guessed winners c_d; a step whose winner was guessed needs no run of its own. The run's rows
   // hold levels + 1 columns. A gather costs one L2 sector request whatever the row width up to 32
-  // bytes, so 7 FP32 levels (3 FP64) cost little more per sweep than one.
+  // bytes, so 7 FP32 levels cost little more per sweep than one.
   const bool plain = (flags & (GEDWALK_ADAPTIVE_L | GEDWALK_STOCHASTIC | GEDWALK_GAINS_ALL)) == 0;
   sh.levels = 1;
   if (!(flags & GEDWALK_GAINS_ALL)) {
-    sh.levels = r.fp64 ? 3 : 7;
+    // FP64: 64-byte rows, two sectors a gather, but seven steps for them: a sweep of 8 columns takes
+    // 456 us instead of 270 on Barabasi-Albert n = 10^6 (k = 25: 9.2 -> 7.4 ms). Three levels where the
+    // stored vectors would outgrow kWideBytes.
+    constexpr int64_t kWideBytes = int64_t(32) << 30;
+    const int64_t wide = static_cast<int64_t>(g.n_active) * ((r.L + 1) / 2) * 64;
+    sh.levels = r.fp64 && wide > kWideBytes ? 3 : 7;
     if (plain && !g.directed && r.lookahead != 0) {
       if (!(r.lookahead == 1 || r.lookahead == 3 || (!r.fp64 && r.lookahead == 7)))
         return fail(GEDWALK_ERR_INVALID, "lookahead must be 0, 1, 3 or (FP32) 7");
@@ -58,8 +63,8 @@ gedwalk_status greedy_shape(const Graph& g, const Resolved& r, int32_t flags, Gr
     }
     if ((!plain || g.directed) && r.spec_cols != 0) sh.levels = 1;  // the caller fixed the one-step width
   }
-  // Candidate batches run when the evaluated guess is not certified: as wide as one sector carries.
-  sh.cols_cand = r.fp64 ? 4 : 8;
+  // Candidate batches run when the evaluated guess is not certified: as wide as the chains.
+  sh.cols_cand = sh.levels == 3 && r.fp64 ? 4 : 8;
   sh.cols_all = r.fp64 ? 8 : 16;
   sh.ell_max = 1;
   while (adaptive && sh.ell_max < r.L) sh.ell_max *= 2;
@@ -165,6 +170,11 @@ gedwalk_status maximize_runs(Graph& g, Workspace& ws, const Resolved& r, const G
   if (select && p.k > 0) GW_TRY(guess(0, &spec));
   RunOut look{};                // the last run's answers, and
   std::vector<int32_t> look_c;  // its guesses
+  // FP64 rows of 8 columns cost more than rows of 4 in every sweep, so they wait for a chain that held
+  // for three steps (on a small graph one winner changes the order of the next ones).
+  const bool two_widths = r.fp64 && sh.levels == 7;
+  int width = two_widths && g.n_active < 20000 ? 3 : n_spec;
+  int held = -1;                // steps the last chain has carried (-1: none yet)
   int lvl = -1;                 // its level that stands under the current S (-1: none)
 
   for (int32_t step = 0; step < p.k; ++step) {
@@ -201,10 +211,12 @@ gedwalk_status maximize_runs(Graph& g, Workspace& ws, const Resolved& r, const G
       for (;;) {  // one attempt per walk length (a single attempt unless adaptive)
         std::vector<Cand> E;  // evaluated with the current S
         if (lvl < 0) {
+          if (two_widths && held >= 0) width = held >= 3 ? 7 : 3;
+          held = 0;
           look_c = spec;
-          look_c.resize(n_spec, -1);
+          look_c.resize(width, -1);
           draws(step);
-          GW_TRY(eng.run(chain, n_spec + 1, true, look_c));
+          GW_TRY(eng.run(chain, width + 1, true, look_c));
           look = *eng.out;
           lvl = 0;
           for (int32_t v : look_c) ws.st_evals += v >= 0;
@@ -224,6 +236,7 @@ gedwalk_status maximize_runs(Graph& g, Workspace& ws, const Resolved& r, const G
           sel = eng.out->lv[0];
         }
         bool first_batch = true, separated = true;
+        const int cols_cand = two_widths && width == 3 ? 4 : sh.cols_cand;
         std::vector<Cand> X;  // exact values for the current S, best first
         std::vector<int32_t> top;
         const int32_t left = g.n - static_cast<int32_t>(S_all->size());
@@ -265,10 +278,10 @@ gedwalk_status maximize_runs(Graph& g, Workspace& ws, const Resolved& r, const G
             for (const Cand& e : E) eng.stale(e.v, e.g, step);
           }
           first_batch = false;
-          std::vector<int32_t> last(top.begin(), top.begin() + std::min<size_t>(top.size(), sh.cols_cand - 1));
+          std::vector<int32_t> last(top.begin(), top.begin() + std::min<size_t>(top.size(), cols_cand - 1));
           draws(step);
           if (everyone) eng.in->thr[0] = ~0ull;
-          GW_TRY(eng.run(false, sh.cols_cand, true, last));
+          GW_TRY(eng.run(false, cols_cand, true, last));
           for (size_t j = 0; j < last.size(); ++j) E.push_back(Cand{eng.out->gains[j], last[j], g.perm[last[j]]});
           ws.st_evals += static_cast<int64_t>(last.size());
           ++ws.st_batches;
@@ -293,7 +306,9 @@ gedwalk_status maximize_runs(Graph& g, Workspace& ws, const Resolved& r, const G
         lvl = -1;
       }
       // the next level is valid only when this step took the vertex it assumed
-      if (chain && best.v == look_c[lvl] && lvl + 1 < sh.levels && look_c[lvl + 1] >= 0) ++lvl;
+      const bool taken = chain && best.v == look_c[lvl];
+      held += taken;
+      if (taken && lvl + 1 < width && look_c[lvl + 1] >= 0) ++lvl;
       else lvl = -1;
     }
     if (best.v < 0) return fail(GEDWALK_ERR_INVALID, "no vertex left to add");

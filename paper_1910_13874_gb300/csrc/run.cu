@@ -457,7 +457,7 @@ __device__ __forceinline__ void block_levels(WarpList (&w)[NL], float* sv, int* 
 // all to one address, would serialise). 279 -> 150 us; on
 // 10^5 rows, where a warp has one iteration, the lists cost most (device_util.cuh): 97 -> 63 us.
 template <typename T, int C, bool CHAIN, bool SEL, bool DIR>
-__global__ void __launch_bounds__(kThreads, DIR ? 2 : kMeetPerSM) meet_kernel(const MeetArgs a) {
+__global__ void __launch_bounds__(kThreads, DIR || sizeof(T) * C > 32 ? 2 : kMeetPerSM) meet_kernel(const MeetArgs a) {
   constexpr int D = C - 1;
   constexpr int NL = CHAIN ? D : 1;
   constexpr int NW = kThreads / 32;
@@ -1134,9 +1134,9 @@ gedwalk_status RunEngine::issue(bool chain, int cols, bool select, bool profile,
   m.d = d;
 #define GW_MEET(T, C, CH, SE) \
   if (fp64 == (sizeof(T) == 8) && cols == C && chain == CH && select == SE) GW_CUDA((launch_meet<T, C, CH, SE>(s, m)));
-  GW_MEET(float, 4, true, true) GW_MEET(float, 8, true, true) GW_MEET(double, 4, true, true)
+  GW_MEET(float, 4, true, true) GW_MEET(float, 8, true, true) GW_MEET(double, 4, true, true) GW_MEET(double, 8, true, true)
   GW_MEET(float, 2, false, true) GW_MEET(float, 4, false, true) GW_MEET(float, 8, false, true)
-  GW_MEET(double, 2, false, true) GW_MEET(double, 4, false, true)
+  GW_MEET(double, 2, false, true) GW_MEET(double, 4, false, true) GW_MEET(double, 8, false, true)
   GW_MEET(float, 16, false, false) GW_MEET(double, 8, false, false)
 #undef GW_MEET
   count_launch();

@@ -600,7 +600,7 @@ constexpr int kCandSlots = 16;
 // Barabasi-Albert graph with n = 10^6).
 template <typename T, int C, int MODE>
 constexpr int min_ctas() {
-  if (sizeof(T) == 8) return 4;
+  if (sizeof(T) == 8) return C <= 4 ? 4 : 2;
   if ((MODE == MODE_LOOK || MODE == MODE_PAR) && C == 8) return 5;
   if ((MODE == MODE_LOOK || MODE == MODE_PAR) && C <= 4) return 6;
   if ((MODE == MODE_MISS || MODE == MODE_SCORE || MODE == MODE_PAIR) && C <= 2) return 8;
@@ -752,6 +752,7 @@ gedwalk_status launch_sweep(int mode, bool fp64, int cols, const SweepArgs& a, c
   GW_CASE(MODE_LOOK, float, 4)
   GW_CASE(MODE_LOOK, float, 8)
   GW_CASE(MODE_LOOK, double, 4)
+  GW_CASE(MODE_LOOK, double, 8)
   GW_CASE(MODE_PAR, float, 2)
   GW_CASE(MODE_PAR, float, 4)
   GW_CASE(MODE_PAR, float, 8)

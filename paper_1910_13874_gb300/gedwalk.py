@@ -197,7 +197,7 @@ def make_params(alpha: float = 0.0, epsilon: float = 1e-4, L: int = 0, precision
                 lookahead: int = 0, spec_cols: int = 0, device_loop: bool = False) -> Params:
     """gedwalk_params from keywords: precision "fp32"/"fp64", eps_rule "over_k"/"plain", bound
     "combinatorial"/"spectral", the flags as booleans; 0 keeps the library's default (alpha
-    1/(1+d_max), L from the bound, lookahead 7 in FP32 and 3 in FP64)."""
+    1/(1+d_max), L from the bound, lookahead 7)."""
     p = Params()
     load().gedwalk_params_default(ctypes.byref(p))
     p.alpha = alpha
