@@ -195,7 +195,7 @@ Workspace::~Workspace() {
   if (order_ev) cudaEventDestroy(order_ev);
   if (own_stream) cudaStreamDestroy(own_stream);
   if (pinned) cudaFreeHost(pinned);
-  if (run_io) cudaFreeHost(run_io);
+  release_run_io(run_io);
 }
 
 gedwalk_status Workspace::ensure_pinned(size_t need) {

@@ -133,6 +133,8 @@ struct SweepGraph {
 };
 
 // ---------------------------------------------------------------- workspaces
+void release_run_io(void* p);  // a workspace's run_io block, no longer referred to
+
 // Per-request scratch. The graph owns one for the synchronous API; the server
 // creates one per concurrent request slot.
 struct Workspace {
@@ -272,6 +274,7 @@ struct SweepArgs {
   int32_t accumulate;
   void* Mout;
   const int32_t* cand;
+  const uint32_t* nz;   // MODE_PLAIN: bit per row of X that may hold a nonzero (nullptr: all may)
   const int32_t* live;  // runs: whether candidate j has a neighbour outside its base set
   int32_t hub;  // rows [0, hub) of x are gathered with L1 retention priority (set by the launcher)
   // Vertex scales s of a weighted graph (nullptr: unweighted). Vectors are then gathered in the

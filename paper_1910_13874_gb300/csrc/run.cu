@@ -67,7 +67,7 @@ gedwalk_status run_sequence(Workspace& ws, cudaStream_t s, const Sequence& q,
   SweepGraph& sg = *hit;
   sg.last_use = ++ws.graph_clock;
   if (!sg.exec) {
-    if (sg.uses++ < 1) return issue(true, nullptr);  // set-up happens outside capture
+    if (sg.uses++ < (q.nnz > kLateEntries ? 3 : 1)) return issue(true, nullptr);  // set-up happens outside capture
     sg.ev.assign(2, nullptr);
     for (cudaEvent_t& e : sg.ev) GW_CUDA(cudaEventCreate(&e));
     GW_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
@@ -955,14 +955,45 @@ int64_t run_bytes(const Graph& g, int32_t L_max, int cols, bool fp64, bool selec
 }
 
 // The captured sequences copy from and to this block: it must outlive them at one address (a pinned
-// block freed and made again at the same address is another allocation to the driver).
+// block freed and made again at the same address is another allocation to the driver). Blocks go back to
+// a pool (at most kIoPool, the rest are freed): pinning one takes longer than a run on a small graph.
+namespace {
+constexpr size_t kIoPool = 64;
+std::mutex g_io_mu;
+std::vector<void*>& io_pool() {
+  static std::vector<void*>* p = new std::vector<void*>();  // lives until exit
+  return *p;
+}
+}  // namespace
+
 static gedwalk_status ensure_run_io(Workspace& ws) {
-  if (!ws.run_io && cudaMallocHost(&ws.run_io, sizeof(RunOut) + sizeof(RunIn)) != cudaSuccess) {
+  if (ws.run_io) return GEDWALK_OK;
+  {
+    std::lock_guard<std::mutex> lk(g_io_mu);
+    if (!io_pool().empty()) {
+      ws.run_io = io_pool().back();
+      io_pool().pop_back();
+      return GEDWALK_OK;
+    }
+  }
+  if (cudaMallocHost(&ws.run_io, sizeof(RunOut) + sizeof(RunIn)) != cudaSuccess) {
     cudaGetLastError();
     ws.run_io = nullptr;
     return fail(GEDWALK_ERR_OOM, "pinned host allocation of %zu bytes failed", sizeof(RunOut) + sizeof(RunIn));
   }
   return GEDWALK_OK;
+}
+
+void release_run_io(void* p) {
+  if (!p) return;
+  {
+    std::lock_guard<std::mutex> lk(g_io_mu);
+    if (io_pool().size() < kIoPool) {
+      io_pool().push_back(p);
+      return;
+    }
+  }
+  cudaFreeHost(p);
 }
 
 gedwalk_status RunEngine::setup(int32_t L_max, int cols, bool select, const std::vector<int32_t>& init) {
@@ -1162,6 +1193,7 @@ gedwalk_status RunEngine::run(bool chain, int cols, bool select, const std::vect
   q.sweeps = swept;
   q.bytes = sweep_bytes(mode, r.fp64, cols, g.n_active, g.nnz, g.weighted);
   q.prof_key = (mode * 1000 + cols) * 2 + (r.fp64 ? 1 : 0);
+  q.nnz = g.nnz;
   GW_TRY(run_sequence(ws, s, q, [&](bool profile, const std::vector<cudaEvent_t>* ev) {
     return issue(chain, cols, select, profile, ev);
   }));
@@ -1284,6 +1316,7 @@ gedwalk_status score_run(Graph& g, Workspace& ws, const std::vector<int32_t>& S_
   q.sweeps = swept;
   q.bytes = sweep_bytes(MODE_PAIR, fp64, 2, g.n_active, g.nnz, g.weighted);
   q.prof_key = (MODE_PAIR * 1000 + 2) * 2 + (fp64 ? 1 : 0);
+  q.nnz = g.nnz;
   GW_TRY(run_sequence(ws, s, q, issue));
   GW_CUDA(cudaStreamSynchronize(s));
   read_graph_timing(ws);

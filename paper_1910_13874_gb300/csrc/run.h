@@ -53,14 +53,18 @@ struct RunDev {  // device-side state of the runs of one workspace
   int32_t done;            // blocks of the meeting (or guess) pass that have finished
 };
 
-// Runs a launch sequence, captured once per configuration (on its second use) and replayed as a
-// CUDA graph; directly on the legacy default stream. `issue` gets the two timing events of a
+// Runs a launch sequence, captured once per configuration and replayed as a CUDA graph; directly on the
+// legacy default stream. The capture comes with the second use, above kLateEntries entries with the
+// fourth: sweeps outlast their launches there, and a new graph's short maximisation (two runs on R-MAT
+// scale 20) spent 0.3 of its 1.9 ms on capturing and instantiating. `issue` gets the two timing events of a
 // capture (or null).
+constexpr int64_t kLateEntries = int64_t(4) << 20;
 struct Sequence {
   uint64_t key;
   int kernels, sweeps;
   double bytes;
   int prof_key;
+  int64_t nnz;
 };
 gedwalk_status run_sequence(Workspace& ws, cudaStream_t s, const Sequence& q,
                             const std::function<gedwalk_status(bool profile, const std::vector<cudaEvent_t>* ev)>& issue);

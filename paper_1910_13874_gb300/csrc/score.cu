@@ -96,26 +96,31 @@ __global__ void batch_totals(const double* __restrict__ T, int64_t n, int32_t n_
   }
 }
 
-// h_1 outside the groups: alpha per neighbour in S_j (equal terms: their order does not matter). One
-// warp per member, gridDim.y warps on a hub's.
+// h_1 outside the groups: alpha per neighbour in S_j (equal terms: their order does not matter), and its
+// rows' bits in nz. One warp per member, gridDim.y warps on a hub's.
 __global__ void batch_scatter(float* __restrict__ X, int32_t cols, const int32_t* __restrict__ mrow,
                               const int32_t* __restrict__ mcol, int32_t count, const int32_t* __restrict__ rp,
-                              const int32_t* __restrict__ ci, float alpha) {
+                              const int32_t* __restrict__ ci, float alpha, uint32_t* __restrict__ nz) {
   const int lane = threadIdx.x & 31;
   const int32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (i >= count) return;
   const int32_t s = mrow[i], c = mcol[i];
   const int64_t e1 = rp[s + 1];
   for (int64_t e = rp[s] + static_cast<int64_t>(blockIdx.y) * 32 + lane; e < e1; e += 32 * static_cast<int64_t>(gridDim.y))
-    atomicAdd(X + static_cast<size_t>(ci[e]) * cols + c, alpha);
+  {
+    const int32_t u = ci[e];
+    atomicAdd(X + static_cast<size_t>(u) * cols + c, alpha);
+    if (!((nz[u >> 5] >> (u & 31)) & 1u)) atomicOr(nz + (u >> 5), 1u << (u & 31));
+  }
 }
 
 // h_t on the groups' own rows: a row of the table (as stored: times s on a weighted graph).
 __global__ void batch_own(float* __restrict__ X, int32_t cols, const int32_t* __restrict__ mrow,
                           const int32_t* __restrict__ mcol, int32_t count, const double* __restrict__ row,
-                          int32_t n_active) {
+                          int32_t n_active, uint32_t* __restrict__ nz) {
   const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count || mrow[i] >= n_active) return;
+  if (nz) atomicOr(nz + (mrow[i] >> 5), 1u << (mrow[i] & 31));
   X[static_cast<size_t>(mrow[i]) * cols + mcol[i]] = static_cast<float>(row[mrow[i]]);
 }
 
@@ -318,7 +323,7 @@ int64_t score_batch_footprint(const Graph& g, int64_t members, int32_t groups) {
   const int64_t n = g.n;
   int64_t b = members * (4 + 4 + 8) + static_cast<int64_t>(groups + 1) * 4 + 256;  // members, columns, sums
   b += static_cast<int64_t>(std::max(g.plan.num_slices, 1)) * C * 4 + std::max(g.plan.num_heavy, 1) * 4;
-  b += static_cast<int64_t>(groups) * 8 + 64;
+  b += static_cast<int64_t>(groups) * 8 + 64 + (n + 31) / 32 * 4;
   if (!g.directed) {
     b += static_cast<int64_t>(g.n_active) * C * 4 * (kBatchRing + 1);  // the stored vectors and their sum
     b += 2 * n * 4 + kBatchMeetBlocks * C * 8;
@@ -340,6 +345,9 @@ static gedwalk_status batch_runs(Graph& g, Workspace& ws, int C, const int32_t* 
   GW_TRY(ws.xs.ensure(static_cast<size_t>(vec) * slots * sizeof(float), s));
   GW_TRY(ws.tail.ensure(static_cast<size_t>(g.n) * sizeof(float), s));
   GW_TRY(ws.bound.ensure(static_cast<size_t>(g.n) * sizeof(float), s));
+  const size_t nz_bytes = (static_cast<size_t>(g.n) + 31) / 32 * sizeof(uint32_t);
+  GW_TRY(ws.mask.ensure(nz_bytes, s));
+  uint32_t* nz = ws.mask.as<uint32_t>();
   GW_TRY(ws.partial.ensure(static_cast<size_t>(std::max(g.plan.num_slices, 1)) * C * sizeof(float), s));
   const size_t cbytes = static_cast<size_t>(std::max(g.plan.num_heavy, 1)) * sizeof(unsigned);
   if (ws.counters.bytes < cbytes || !ws.counters.p) GW_TRY(ws.counters.ensure(cbytes, s, /*zero=*/true));
@@ -361,21 +369,23 @@ static gedwalk_status batch_runs(Graph& g, Workspace& ws, int C, const int32_t* 
   for (int32_t g0 = 0; g0 < G; g0 += C) {
     const int32_t g1 = std::min(G, g0 + C);
     const int32_t m0 = offsets[g0], cnt = offsets[g1] - m0;
-    auto own = [&](int32_t t) -> gedwalk_status {
+    auto own = [&](int32_t t, uint32_t* bits) -> gedwalk_status {
       if (cnt == 0) return GEDWALK_OK;
       batch_own<<<blocks_for(cnt), 256, 0, s>>>(slot(t), C, mrow + m0, mcol + m0, cnt, T + static_cast<size_t>(t) * g.n,
-                                                g.n_active);
+                                                g.n_active, bits);
       GW_KCHECK();
       return GEDWALK_OK;
     };
     int32_t t = g.weighted ? 0 : 1;  // the first vector: x_0 = the groups' indicators, or x_1 from counts
     GW_CUDA(cudaMemsetAsync(slot(t), 0, static_cast<size_t>(vec) * sizeof(float), s));
+    GW_CUDA(cudaMemsetAsync(nz, 0, nz_bytes, s));
     if (!g.weighted && cnt > 0) {
       batch_scatter<<<dim3((cnt + 7) / 8, g.dmax > 4096 ? 32 : 1), 256, 0, s>>>(slot(1), C, mrow + m0, mcol + m0, cnt, a.rp, a.ci,
-                                                                             static_cast<float>(r.alpha));
+                                                                             static_cast<float>(r.alpha), nz);
       GW_KCHECK();
     }
-    GW_TRY(own(t));
+    GW_TRY(own(t, nz));
+    a.nz = nz;  // the first vector is zero but next to the groups: its sweep gathers those rows alone
     BatchVecs b{ring, vec, V, 0, H};
     for (++t; t <= H; ++t) {
       if (t - b.folded > kBatchRing) {  // x_t takes the slot of x_{t-5}: fold x_{t-5} .. x_{t-2}
@@ -386,7 +396,8 @@ static gedwalk_status batch_runs(Graph& g, Workspace& ws, int C, const int32_t* 
       a.X = slot(t - 1);
       a.Y = slot(t);
       GW_TRY(launch_sweep(MODE_PLAIN, false, C, a, s));
-      GW_TRY(own(t));
+      a.nz = nullptr;
+      GW_TRY(own(t, nullptr));
     }
     double* out = ws.small.as<double>() + g0;
 #define GW_MEET(CC) \

@@ -159,12 +159,17 @@ __device__ __forceinline__ void set_row(T (&acc)[C], const T* __restrict__ X, in
 }
 
 // Where gathered rows of x come from.
-// GlobalSrc: global memory, rows below `hub` with L1 retention priority.
-template <typename T, int C>
+// GlobalSrc: global memory, rows below `hub` with L1 retention priority. SPARSE: rows without their bit in
+// nz (if given) are zero and not gathered.
+template <typename T, int C, bool SPARSE>
 struct GlobalSrc {
   const T* __restrict__ X;
   int hub;
-  __device__ __forceinline__ void add(T (&acc)[C], int v) const { add_row<T, C>(acc, X, v, hub); }
+  const uint32_t* __restrict__ nz;
+  __device__ __forceinline__ void add(T (&acc)[C], int v) const {
+    if (SPARSE && nz && !((__ldg(nz + (v >> 5)) >> (v & 31)) & 1u)) return;
+    add_row<T, C>(acc, X, v, hub);
+  }
   __device__ __forceinline__ void set(T (&acc)[C], int v) const { set_row<T, C>(acc, X, v, hub); }
 };
 
@@ -635,7 +640,7 @@ __global__ void __launch_bounds__(kThreads, (min_ctas<T, C, MODE>())) sweep_kern
   }
   __syncthreads();
   if (uidx >= a.num_units) return;
-  const GlobalSrc<T, C> src{static_cast<const T*>(a.X), a.hub};
+  const GlobalSrc<T, C, MODE == MODE_PLAIN> src{static_cast<const T*>(a.X), a.hub, a.nz};
   run_unit<T, C, MODE>(a, src, u, uidx, lane, s_rp[warp], s_cand, s_live);
 }
 
