@@ -35,6 +35,9 @@ bool cand_before(const Cand& a, const Cand& b) { return a.g > b.g || (a.g == b.g
 gedwalk_status greedy_shape(const Graph& g, const Resolved& r, int32_t flags, GreedyShape* out) {
   GreedyShape sh{};
   const bool adaptive = (flags & GEDWALK_ADAPTIVE_L) != 0;
+  sh.ell_max = 1;
+  while (adaptive && sh.ell_max < r.L) sh.ell_max *= 2;
+  const int32_t tab_L = adaptive ? sh.ell_max : r.L;
   // One-step runs (lookahead off, spec_cols): phi^miss and the candidates likely to win. One certifies
   // most steps (a miss costs one candidate batch).
   sh.cols_fused = 2;
@@ -51,11 +54,8 @@ gedwalk_status greedy_shape(const Graph& g, const Resolved& r, int32_t flags, Gr
   sh.levels = 1;
   if (!(flags & GEDWALK_GAINS_ALL)) {
     // FP64: 64-byte rows, two sectors a gather, but seven steps for them: a sweep of 8 columns takes
-    // 456 us instead of 270 on Barabasi-Albert n = 10^6 (k = 25: 9.2 -> 7.4 ms). Three levels where the
-    // stored vectors would outgrow kWideBytes.
-    constexpr int64_t kWideBytes = int64_t(32) << 30;
-    const int64_t wide = static_cast<int64_t>(g.n_active) * ((r.L + 1) / 2) * 64;
-    sh.levels = r.fp64 && wide > kWideBytes ? 3 : 7;
+    // 456 us instead of 270 on Barabasi-Albert n = 10^6 (k = 25: 9.2 -> 7.4 ms).
+    sh.levels = run_width(g, tab_L, 8, r.fp64) - 1;
     if (plain && !g.directed && r.lookahead != 0) {
       if (!(r.lookahead == 1 || r.lookahead == 3 || (!r.fp64 && r.lookahead == 7)))
         return fail(GEDWALK_ERR_INVALID, "lookahead must be 0, 1, 3 or (FP32) 7");
@@ -64,11 +64,9 @@ gedwalk_status greedy_shape(const Graph& g, const Resolved& r, int32_t flags, Gr
     if ((!plain || g.directed) && r.spec_cols != 0) sh.levels = 1;  // the caller fixed the one-step width
   }
   // Candidate batches run when the evaluated guess is not certified: as wide as the chains.
-  sh.cols_cand = sh.levels == 3 && r.fp64 ? 4 : 8;
-  sh.cols_all = r.fp64 ? 8 : 16;
-  sh.ell_max = 1;
-  while (adaptive && sh.ell_max < r.L) sh.ell_max *= 2;
-  sh.tab_L = adaptive ? sh.ell_max : r.L;
+  sh.cols_cand = run_width(g, tab_L, 8, r.fp64);
+  sh.cols_all = run_width(g, tab_L, r.fp64 ? 8 : 16, r.fp64);
+  sh.tab_L = tab_L;
   sh.cols_max = std::max({sh.levels > 1 ? sh.levels + 1 : sh.cols_fused, sh.cols_cand,
                           (flags & GEDWALK_GAINS_ALL) ? sh.cols_all : 0, 2});
   *out = sh;
@@ -411,7 +409,7 @@ gedwalk_status gains_impl(Graph& g, Workspace& ws, const std::vector<int32_t>& S
   GW_TRY(greedy_stream(ws, r_in.stream, &r.stream));
   SyncOnError guard{r.stream};
   cudaStream_t s = r.stream;
-  const int cols_all = r.fp64 ? 8 : 16;
+  const int cols_all = run_width(g, r.L, r.fp64 ? 8 : 16, r.fp64);
   std::vector<char> inS(g.n, 0);
   for (int32_t v : S_int) inS[v] = 1;
   for (int32_t v = 0; v < g.n; ++v) gains_caller[v] = 0.0;  // an isolated vertex gains nothing

@@ -824,9 +824,10 @@ __global__ void pair_init(T* __restrict__ X, const int32_t* __restrict__ rp, con
 // Walks of length a + b that hit S: the half of length a hits, or it misses and the half of length b
 // hits, so with b = H the lengths H + a, a = 1..L-H, number sum_v [h_a (h_H + m_H) + m_a h_H] and the
 // lengths up to H are plain sums of h_t. One thread per row; the last block adds the block sums.
+// x_t sits at slot (t - 1) % ring; with folded > 0 the slot behind the ring holds x_1 + .. + x_folded.
 template <typename T>
-__global__ void __launch_bounds__(kThreads) pair_meet(const T* __restrict__ xs, int64_t stride, int32_t L, int32_t H,
-                                                      int32_t n_active, const T* __restrict__ rs,
+__global__ void __launch_bounds__(kThreads) pair_meet(const T* __restrict__ xs, int64_t stride, int32_t ring, int32_t folded,
+                                                      int32_t L, int32_t H, int32_t n_active, const T* __restrict__ rs,
                                                       double* __restrict__ part, int32_t* __restrict__ done,
                                                       double* __restrict__ out) {
   constexpr int NW = kThreads / 32;
@@ -838,9 +839,14 @@ __global__ void __launch_bounds__(kThreads) pair_meet(const T* __restrict__ xs, 
   acc.zero();
   for (int32_t v = blockIdx.x * kThreads + threadIdx.x; v < n_active; v += gridDim.x * kThreads) {
     T bh = T(0), bm = T(0), h = T(0), m = T(0);
-    const T* p = xs + 2 * static_cast<size_t>(v);
+    const T* row = xs + 2 * static_cast<size_t>(v);
+    if (folded > 0) {
+      bh = row[stride * ring];
+      bm = row[stride * ring + 1];
+    }
 #pragma unroll 4
-    for (int t = 1; t <= H; ++t, p += stride) {
+    for (int t = folded + 1; t <= H; ++t) {
+      const T* p = row + stride * ((t - 1) % ring);
       T xh, xm;
       if constexpr (sizeof(T) == 4) {
         const float2 q = __ldcs(reinterpret_cast<const float2*>(p));
@@ -889,6 +895,18 @@ __global__ void __launch_bounds__(kThreads) pair_meet(const T* __restrict__ xs, 
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFullMask, x, o);
   if (lane == 0) *out = x;
+}
+
+// acc (+)= x_{from+1} .. x_{from+count}, elementwise.
+template <typename T>
+__global__ void pair_fold(T* __restrict__ xs, int64_t stride, int32_t ring, int32_t from, int32_t count) {
+  T* acc = xs + stride * ring;
+  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < stride;
+       i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+    T a = from > 0 ? acc[i] : T(0);
+    for (int32_t t = 0; t < count; ++t) a += xs[stride * ((from + t) % ring) + i];
+    acc[i] = a;
+  }
 }
 
 int grid_of(int64_t n) { return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 16))); }
@@ -1168,7 +1186,9 @@ gedwalk_status RunEngine::issue(bool chain, int cols, bool select, bool profile,
   GW_MEET(float, 4, true, true) GW_MEET(float, 8, true, true) GW_MEET(double, 4, true, true) GW_MEET(double, 8, true, true)
   GW_MEET(float, 2, false, true) GW_MEET(float, 4, false, true) GW_MEET(float, 8, false, true)
   GW_MEET(double, 2, false, true) GW_MEET(double, 4, false, true) GW_MEET(double, 8, false, true)
-  GW_MEET(float, 16, false, false) GW_MEET(double, 8, false, false)
+  GW_MEET(float, 2, false, false) GW_MEET(float, 4, false, false) GW_MEET(float, 8, false, false)
+  GW_MEET(float, 16, false, false)
+  GW_MEET(double, 2, false, false) GW_MEET(double, 4, false, false) GW_MEET(double, 8, false, false)
 #undef GW_MEET
   count_launch();
   GW_CUDA(cudaMemcpyAsync(out, &d->out, sizeof(RunOut), cudaMemcpyDeviceToHost, s));
@@ -1241,7 +1261,11 @@ gedwalk_status score_run(Graph& g, Workspace& ws, const std::vector<int32_t>& S_
   const int32_t H = (r.L + 1) / 2;
   const size_t row = static_cast<size_t>(g.n_active) * 2;
   GW_TRY(ensure_run_io(ws));
-  GW_TRY(ws.xs.ensure(row * es * (H + (g.weighted ? 1 : 0)), s));
+  // x_1 .. x_H, or, where they would outgrow kWideBytes, a ring of the last ones and the sum of the
+  // older; x_0 (weighted) sits where x_ring goes later
+  const int32_t ring = static_cast<int32_t>(std::max<int64_t>(
+      3, std::min<int64_t>(H + (g.weighted ? 1 : 0), kWideBytes / std::max<int64_t>(static_cast<int64_t>(row * es), 1))));
+  GW_TRY(ws.xs.ensure(row * es * (ring + (H > ring ? 1 : 0)), s));
   GW_TRY(ws.cnt.ensure(n * sizeof(int32_t), s));
   const size_t words = (n + 31) / 32;
   GW_TRY(ws.mask.ensure(words * 4, s));
@@ -1271,7 +1295,7 @@ gedwalk_status score_run(Graph& g, Workspace& ws, const std::vector<int32_t>& S_
                                                     ws.mask.as<uint32_t>());
     GW_KCHECK();
     char* xs = ws.xs.as<char>();
-    char* x0 = g.weighted ? xs + row * es * H : xs;
+    char* x0 = g.weighted ? xs + row * es * (ring - 1) : xs;
     if (fp64)
       pair_init<double><<<grid_of(g.n_active), 256, 0, s>>>(reinterpret_cast<double*>(x0), g.rp.as<int32_t>(),
                                                             ws.cnt.as<int32_t>(), ws.mask.as<uint32_t>(), g.n_active, r.alpha,
@@ -1285,19 +1309,31 @@ gedwalk_status score_run(Graph& g, Workspace& ws, const std::vector<int32_t>& S_
     SweepArgs a = base_args(g, ws);
     a.alpha = r.alpha;
     if (ev) GW_CUDA(cudaEventRecordWithFlags((*ev)[0], s, cudaEventRecordExternal));
+    int32_t folded = 0;
     for (int32_t t = g.weighted ? 1 : 2; t <= H; ++t) {
-      a.X = t == 1 ? x0 : xs + row * es * (t - 2);
-      a.Y = xs + row * es * (t - 1);
+      if (t - folded > ring) {  // x_t takes the slot of x_{t-ring}: fold all before x_{t-1}
+        const int32_t count = ring - 1;
+        if (fp64)
+          pair_fold<double><<<grid_of(static_cast<int64_t>(row)), 256, 0, s>>>(reinterpret_cast<double*>(xs),
+                                                                              static_cast<int64_t>(row), ring, folded, count);
+        else
+          pair_fold<float><<<grid_of(static_cast<int64_t>(row)), 256, 0, s>>>(reinterpret_cast<float*>(xs),
+                                                                             static_cast<int64_t>(row), ring, folded, count);
+        GW_KCHECK();
+        folded += count;
+      }
+      a.X = t == 1 ? x0 : xs + row * es * ((t - 2) % ring);
+      a.Y = xs + row * es * ((t - 1) % ring);
       GW_TRY(launch_sweep(MODE_PAIR, fp64, 2, a, s, profile));
     }
     if (ev) GW_CUDA(cudaEventRecordWithFlags((*ev)[1], s, cudaEventRecordExternal));
     if (fp64)
-      pair_meet<double><<<meet_grid(g.n_active), kThreads, 0, s>>>(reinterpret_cast<double*>(xs), static_cast<int64_t>(row), r.L,
+      pair_meet<double><<<meet_grid(g.n_active), kThreads, 0, s>>>(reinterpret_cast<double*>(xs), static_cast<int64_t>(row), ring, folded, r.L,
                                                                    H, g.n_active,
                                                                    g.weighted ? g.rs_d.as<double>() : nullptr,
                                                                    ws.parts.as<double>(), d_done, d_sum);
     else
-      pair_meet<float><<<meet_grid(g.n_active), kThreads, 0, s>>>(reinterpret_cast<float*>(xs), static_cast<int64_t>(row), r.L, H,
+      pair_meet<float><<<meet_grid(g.n_active), kThreads, 0, s>>>(reinterpret_cast<float*>(xs), static_cast<int64_t>(row), ring, folded, r.L, H,
                                                                   g.n_active, g.weighted ? g.rs_f.as<float>() : nullptr,
                                                                   ws.parts.as<double>(), d_done, d_sum);
     GW_KCHECK();
@@ -1312,7 +1348,7 @@ gedwalk_status score_run(Graph& g, Workspace& ws, const std::vector<int32_t>& S_
   q.key = mix_all({uint64_t(MODE_PAIR), uint64_t(fp64), uint64_t(r.L), uint64_t(items), abits, bits(&g), bits(s), bits(ws.xs.p),
                    bits(ws.cnt.p), bits(ws.mask.p), bits(ws.parts.p), bits(ws.small.p), bits(ws.partial.p),
                    bits(ws.counters.p), bits(ws.members.p), bits(ws.run_io), bits(g.rp.p), bits(g.ci.p), bits(g.plan.units.p)});
-  q.kernels = 3 + swept;
+  q.kernels = 3 + swept + (H > ring ? (H - ring - 1) / (ring - 1) + 1 : 0);
   q.sweeps = swept;
   q.bytes = sweep_bytes(MODE_PAIR, fp64, 2, g.n_active, g.nnz, g.weighted);
   q.prof_key = (MODE_PAIR * 1000 + 2) * 2 + (fp64 ? 1 : 0);

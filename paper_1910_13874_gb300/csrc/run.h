@@ -74,6 +74,16 @@ gedwalk_status greedy_stream(Workspace& ws, cudaStream_t caller, cudaStream_t* o
 void read_graph_timing(Workspace& ws);
 uint64_t mix_all(std::initializer_list<uint64_t> vs);
 
+// Stored vectors are kept to about this size: beyond it rows get narrower (fewer steps or candidates a
+// run) and scoring keeps a ring of vectors.
+constexpr int64_t kWideBytes = int64_t(32) << 30;
+// The widest rows of at most `cols` columns, at least 2, whose ceil(L/2) stored vectors stay below it.
+inline int run_width(const Graph& g, int32_t L, int cols, bool fp64) {
+  const int64_t cell = static_cast<int64_t>(g.n_active) * ((L + 1) / 2) * (g.directed ? 2 : 1) * (fp64 ? 8 : 4);
+  while (cols > 2 && cell * cols > kWideBytes) cols /= 2;
+  return cols;
+}
+
 // The runs of one maximisation (or one gains call).
 struct RunEngine {
   Graph& g;

@@ -7,6 +7,7 @@
 
 #include "device_util.cuh"
 #include "internal.h"
+#include "run.h"
 
 namespace gw {
 namespace {
@@ -124,25 +125,26 @@ __global__ void batch_own(float* __restrict__ X, int32_t cols, const int32_t* __
   X[static_cast<size_t>(mrow[i]) * cols + mcol[i]] = static_cast<float>(row[mrow[i]]);
 }
 
-// The stored vectors of a block: x_t sits at slot (t - 1) % kBatchRing; V holds the sum of those
-// already folded (walk lengths 1..folded).
+// The stored vectors of a block: x_t sits at slot (t - 1) % slots; V holds the sum of those already
+// folded (walk lengths 1..folded). Five slots hold the walks of L <= 10; two where five would outgrow
+// kWideBytes.
 constexpr int kBatchRing = 5;
 struct BatchVecs {
   const float* ring;
   int64_t stride;
+  int slots;
   float* V;  // nullptr: nothing folded
   int32_t folded, H;
 };
 
-// V (+)= x_{folded+1} .. x_{folded+4}.
+// V (+)= x_{folded+1} .. x_{folded+slots-1}.
 __global__ void batch_fold(const BatchVecs b, int64_t quads) {
   for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < quads;
        q += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (b.folded > 0) a = reinterpret_cast<const float4*>(b.V)[q];
-#pragma unroll
-    for (int t = 0; t < kBatchRing - 1; ++t) {
-      const float4 x = reinterpret_cast<const float4*>(b.ring + b.stride * ((b.folded + t) % kBatchRing))[q];
+    for (int t = 0; t < b.slots - 1; ++t) {
+      const float4 x = reinterpret_cast<const float4*>(b.ring + b.stride * ((b.folded + t) % b.slots))[q];
       a.x += x.x;
       a.y += x.y;
       a.z += x.z;
@@ -176,11 +178,11 @@ __global__ void __launch_bounds__(kThreads) batch_meet(const BatchVecs b, int32_
       k[0] = x.x, k[1] = x.y, k[2] = x.z, k[3] = x.w;
     }
     for (int t = b.folded + 1; t < b.H; ++t) {
-      const float4 x = __ldcs(reinterpret_cast<const float4*>(b.ring + b.stride * ((t - 1) % kBatchRing)) + q);
+      const float4 x = __ldcs(reinterpret_cast<const float4*>(b.ring + b.stride * ((t - 1) % b.slots)) + q);
       k[0] += x.x, k[1] += x.y, k[2] += x.z, k[3] += x.w;
     }
     {
-      const float4 x = __ldcs(reinterpret_cast<const float4*>(b.ring + b.stride * ((b.H - 1) % kBatchRing)) + q);
+      const float4 x = __ldcs(reinterpret_cast<const float4*>(b.ring + b.stride * ((b.H - 1) % b.slots)) + q);
       h[0] = x.x, h[1] = x.y, h[2] = x.z, h[3] = x.w;
     }
     const float inv = rs ? 1.0f / rs[v] : 1.0f, t = __ldg(tH + v), p = __ldg(P + v);
@@ -318,6 +320,10 @@ gedwalk_status autotune_batch(Graph& g, Workspace& ws, const Resolved& r) {
   return GEDWALK_OK;
 }
 
+static int batch_ring(const Graph& g, int64_t C) {
+  return static_cast<int64_t>(g.n_active) * C * 4 * kBatchRing > kWideBytes ? 2 : kBatchRing;
+}
+
 int64_t score_batch_footprint(const Graph& g, int64_t members, int32_t groups) {
   const int64_t C = g.batch_cols > 0 ? g.batch_cols : 32;  // before tuning: the widest width tried
   const int64_t n = g.n;
@@ -325,7 +331,7 @@ int64_t score_batch_footprint(const Graph& g, int64_t members, int32_t groups) {
   b += static_cast<int64_t>(std::max(g.plan.num_slices, 1)) * C * 4 + std::max(g.plan.num_heavy, 1) * 4;
   b += static_cast<int64_t>(groups) * 8 + 64 + (n + 31) / 32 * 4;
   if (!g.directed) {
-    b += static_cast<int64_t>(g.n_active) * C * 4 * (kBatchRing + 1);  // the stored vectors and their sum
+    b += static_cast<int64_t>(g.n_active) * C * 4 * (batch_ring(g, C) + 1);  // the stored vectors and their sum
     b += 2 * n * 4 + kBatchMeetBlocks * C * 8;
     return b;
   }
@@ -340,9 +346,10 @@ static gedwalk_status batch_runs(Graph& g, Workspace& ws, int C, const int32_t* 
                                  const int32_t* mcol, const Resolved& r, cudaStream_t s) {
   const int32_t L = r.L, H = (L + 1) / 2;
   const int64_t vec = static_cast<int64_t>(g.n_active) * C;
-  // x_1 .. x_H in a ring of kBatchRing; beyond that the oldest are folded into one vector behind it
-  const int slots = H > kBatchRing ? kBatchRing + 1 : g.weighted ? kBatchRing : H;
-  GW_TRY(ws.xs.ensure(static_cast<size_t>(vec) * slots * sizeof(float), s));
+  // x_1 .. x_H in a ring; beyond that the oldest are folded into one vector behind it
+  const int ring_slots = batch_ring(g, C);
+  const int stored = H > ring_slots ? ring_slots + 1 : g.weighted ? ring_slots : H;
+  GW_TRY(ws.xs.ensure(static_cast<size_t>(vec) * stored * sizeof(float), s));
   GW_TRY(ws.tail.ensure(static_cast<size_t>(g.n) * sizeof(float), s));
   GW_TRY(ws.bound.ensure(static_cast<size_t>(g.n) * sizeof(float), s));
   const size_t nz_bytes = (static_cast<size_t>(g.n) + 31) / 32 * sizeof(uint32_t);
@@ -361,8 +368,8 @@ static gedwalk_status batch_runs(Graph& g, Workspace& ws, int C, const int32_t* 
                                                       ws.tail.as<float>(), ws.bound.as<float>());
   GW_KCHECK();
   float* ring = ws.xs.as<float>();
-  auto slot = [&](int32_t t) { return ring + vec * ((t + kBatchRing - 1) % kBatchRing); };  // x_0: the last slot
-  float* V = ring + vec * kBatchRing;
+  auto slot = [&](int32_t t) { return ring + vec * ((t + ring_slots - 1) % ring_slots); };  // x_0: the last slot
+  float* V = ring + vec * ring_slots;
   SweepArgs a = base_args(g, ws);
   a.alpha = r.alpha;
   const int meet = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(kBatchMeetBlocks, (vec / 4 + kThreads - 1) / kThreads)));
@@ -386,12 +393,12 @@ static gedwalk_status batch_runs(Graph& g, Workspace& ws, int C, const int32_t* 
     }
     GW_TRY(own(t, nz));
     a.nz = nz;  // the first vector is zero but next to the groups: its sweep gathers those rows alone
-    BatchVecs b{ring, vec, V, 0, H};
+    BatchVecs b{ring, vec, ring_slots, V, 0, H};
     for (++t; t <= H; ++t) {
-      if (t - b.folded > kBatchRing) {  // x_t takes the slot of x_{t-5}: fold x_{t-5} .. x_{t-2}
+      if (t - b.folded > ring_slots) {  // x_t takes the slot of x_{t-slots}: fold all before x_{t-1}
         batch_fold<<<blocks_for(vec / 4), 256, 0, s>>>(b, vec / 4);
         GW_KCHECK();
-        b.folded += kBatchRing - 1;
+        b.folded += ring_slots - 1;
       }
       a.X = slot(t - 1);
       a.Y = slot(t);
