@@ -488,10 +488,48 @@ __global__ void __launch_bounds__(kRadixThreads) radix_scatter_kernel(const uint
   }
 }
 
-// key[v] = dmax - degree(v): ascending keys order the rows by decreasing degree
-__global__ void degree_key_kernel(const int32_t* __restrict__ rp, int32_t n, int32_t dmax, uint32_t* __restrict__ key) {
-  for (int64_t v = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; v < n; v += int64_t(gridDim.x) * blockDim.x)
-    key[v] = static_cast<uint32_t>(dmax - (rp[v + 1] - rp[v]));
+// key[i] = dmax - degree(v), v = order[i] (null: i): ascending keys order the rows by decreasing degree
+__global__ void degree_key_kernel(const int32_t* __restrict__ rp, const int32_t* __restrict__ order, int32_t n, int32_t dmax,
+                                  uint32_t* __restrict__ key) {
+  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
+    const int32_t v = order ? order[i] : static_cast<int32_t>(i);
+    key[i] = static_cast<uint32_t>(dmax - (rp[v + 1] - rp[v]));
+  }
+}
+
+// Directed graphs: deg[u] = entries that name u.
+__global__ void reverse_degree_kernel(const int32_t* __restrict__ ci, int64_t nnz, int32_t* __restrict__ deg) {
+  for (int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; j < nnz; j += int64_t(gridDim.x) * blockDim.x)
+    atomicAdd(deg + ci[j], 1);
+}
+
+__global__ void max_kernel(const int32_t* __restrict__ x, int32_t n, int32_t* __restrict__ out) {
+  int32_t m = 0;
+  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
+    m = max(m, x[i]);
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(out, m);
+}
+
+// key[v] = top - x[v]
+__global__ void key_kernel(const int32_t* __restrict__ x, int32_t n, int32_t top, uint32_t* __restrict__ key) {
+  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
+    key[i] = static_cast<uint32_t>(top - x[i]);
+}
+
+// out[i] = x[perm[i]]
+__global__ void permute_kernel(const int32_t* __restrict__ x, const int32_t* __restrict__ perm, int32_t n,
+                               uint32_t* __restrict__ out) {
+  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
+    out[i] = static_cast<uint32_t>(x[perm[i]]);
+}
+
+// row[j] = the row of entry j; one warp per row
+__global__ void row_of_kernel(const int32_t* __restrict__ rp, int32_t n, int32_t* __restrict__ row) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t(gridDim.x) * blockDim.x) >> 5;
+  for (int64_t i = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; i < n; i += warps)
+    for (int64_t j = rp[i] + lane; j < rp[i + 1]; j += 32) row[j] = static_cast<int32_t>(i);
 }
 
 // inv[perm[i]] = i and deg[i] = dmax - key[i] (the sorted keys)
@@ -503,29 +541,26 @@ __global__ void perm_finish_kernel(const int32_t* __restrict__ perm, const uint3
   }
 }
 
-// perm: new -> caller id (decreasing degree, equal degrees by caller id), inv its inverse, deg
-// and rp the relabelled degrees and row pointers (rp[n] = nnz), all on the device.
-static gedwalk_status degree_order(const int32_t* raw_rp, int32_t n, int32_t dmax, int32_t* perm, int32_t* inv,
-                                   int32_t* deg, int32_t* rp) {
-  const int64_t blocks = (int64_t(n) + kRadixTile - 1) / kRadixTile;
-  DevBuf k0, k1, v1, counts, offs;
-  GW_TRY(k0.ensure(static_cast<size_t>(n) * sizeof(uint32_t), 0));
-  GW_TRY(k1.ensure(static_cast<size_t>(n) * sizeof(uint32_t), 0));
-  GW_TRY(v1.ensure(static_cast<size_t>(n) * sizeof(int32_t), 0));
+static int radix_passes(uint32_t top) {
+  int bits = 0;
+  while (bits < 32 && (top >> bits) != 0) ++bits;
+  return std::max(1, (bits + 7) / 8);
+}
+
+// Stable sort of n pairs by key in `passes` digits: the values (null: the indices) end in `vals`, with
+// `vals_tmp` between the passes (neither may be vals_in); *keys_out: where the sorted keys are, k0 or k1
+// (keys_in is read once and may be k0).
+static gedwalk_status radix_sort(const uint32_t* keys_in, const int32_t* vals_in, int64_t n, int passes, uint32_t* k0,
+                                 uint32_t* k1, int32_t* vals, int32_t* vals_tmp, const uint32_t** keys_out) {
+  const int64_t blocks = (n + kRadixTile - 1) / kRadixTile;
+  DevBuf counts, offs;
   GW_TRY(counts.ensure(static_cast<size_t>(blocks) * 256 * sizeof(uint32_t), 0));
   GW_TRY(offs.ensure(static_cast<size_t>(blocks) * 256 * sizeof(uint32_t), 0));
-  degree_key_kernel<<<grid_for(n), 256>>>(raw_rp, n, dmax, k0.as<uint32_t>());
-  GW_KCHECK();
-  int bits = 0;
-  while (bits < 32 && (static_cast<uint32_t>(dmax) >> bits) != 0) ++bits;
-  const int passes = std::max(1, (bits + 7) / 8);
-  // ping-pong so that the last pass writes perm: passes odd -> k0/perm first
-  uint32_t* kin = k0.as<uint32_t>();
-  const int32_t* vin = nullptr;
+  const uint32_t* kin = keys_in;
+  const int32_t* vin = vals_in;
   for (int ps = 0; ps < passes; ++ps) {
-    const bool last_to_perm = ((passes - 1 - ps) % 2) == 0;
-    uint32_t* kout = (kin == k0.as<uint32_t>()) ? k1.as<uint32_t>() : k0.as<uint32_t>();
-    int32_t* vout = last_to_perm ? perm : v1.as<int32_t>();
+    uint32_t* kout = (kin == k0) ? k1 : k0;
+    int32_t* vout = ((passes - 1 - ps) % 2) == 0 ? vals : vals_tmp;
     radix_count_kernel<<<static_cast<int>(blocks), kRadixThreads>>>(kin, n, 8 * ps, counts.as<uint32_t>());
     GW_KCHECK();
     GW_TRY(exclusive_scan(counts.as<uint32_t>(), blocks * 256, offs.as<uint32_t>(), nullptr));
@@ -535,11 +570,56 @@ static gedwalk_status degree_order(const int32_t* raw_rp, int32_t n, int32_t dma
     kin = kout;
     vin = vout;
   }
-  perm_finish_kernel<<<grid_for(n), 256>>>(perm, kin, n, dmax, inv, reinterpret_cast<uint32_t*>(deg));
+  if (keys_out) *keys_out = kin;
+  return GEDWALK_OK;
+}
+
+// perm: new -> caller id (decreasing degree, equal degrees by decreasing rdeg if given, then by caller
+// id), inv its inverse, deg and rp the relabelled degrees and row pointers (rp[n] = nnz), all on the
+// device.
+static gedwalk_status degree_order(const int32_t* raw_rp, int32_t n, int32_t dmax, const int32_t* rdeg, int32_t rdmax,
+                                   int32_t* perm, int32_t* inv, int32_t* deg, int32_t* rp) {
+  DevBuf k0, k1, v1;
+  GW_TRY(k0.ensure(static_cast<size_t>(n) * sizeof(uint32_t), 0));
+  GW_TRY(k1.ensure(static_cast<size_t>(n) * sizeof(uint32_t), 0));
+  GW_TRY(v1.ensure(static_cast<size_t>(n) * sizeof(int32_t), 0));
+  const int passes = radix_passes(static_cast<uint32_t>(dmax));
+  const int32_t* order = nullptr;
+  if (rdeg) {  // the less significant key first, into the buffer the second sort does not write first
+    int32_t* to = passes % 2 ? v1.as<int32_t>() : perm;
+    key_kernel<<<grid_for(n), 256>>>(rdeg, n, rdmax, k0.as<uint32_t>());
+    GW_KCHECK();
+    GW_TRY(radix_sort(k0.as<uint32_t>(), nullptr, n, radix_passes(static_cast<uint32_t>(rdmax)), k0.as<uint32_t>(),
+                      k1.as<uint32_t>(), to, to == perm ? v1.as<int32_t>() : perm, nullptr));
+    order = to;
+  }
+  degree_key_kernel<<<grid_for(n), 256>>>(raw_rp, order, n, dmax, k0.as<uint32_t>());
+  GW_KCHECK();
+  const uint32_t* keys = nullptr;
+  GW_TRY(radix_sort(k0.as<uint32_t>(), order, n, passes, k0.as<uint32_t>(), k1.as<uint32_t>(), perm, v1.as<int32_t>(), &keys));
+  perm_finish_kernel<<<grid_for(n), 256>>>(perm, keys, n, dmax, inv, reinterpret_cast<uint32_t*>(deg));
   GW_KCHECK();
   GW_TRY(exclusive_scan(reinterpret_cast<const uint32_t*>(deg), n, reinterpret_cast<uint32_t*>(rp),
                         reinterpret_cast<uint32_t*>(rp + n)));
   return GEDWALK_OK;
+}
+
+// The reverse lists of a relabelled CSR: its entries sorted by column, stably, so that every reverse row
+// holds its rows in increasing order. (On the host this walk over the entries, with the two-key order,
+// took 50 of the 51 ms of a directed R-MAT scale 18 upload, 4 M entries; now 1.6 ms in all.)
+static gedwalk_status transpose_rows(const int32_t* rp, const int32_t* ci, int32_t n, int64_t nnz, int32_t* ci_r) {
+  if (nnz == 0) return GEDWALK_OK;
+  DevBuf k0, k1, rows, tmp;
+  const size_t bytes = static_cast<size_t>(nnz) * sizeof(int32_t);
+  GW_TRY(k0.ensure(bytes, 0));
+  GW_TRY(k1.ensure(bytes, 0));
+  GW_TRY(rows.ensure(bytes, 0));
+  GW_TRY(tmp.ensure(bytes, 0));
+  row_of_kernel<<<static_cast<int>(std::min<int64_t>((static_cast<int64_t>(n) * 32 + 255) / 256, 152 * 32)), 256>>>(
+      rp, n, rows.as<int32_t>());
+  GW_KCHECK();
+  return radix_sort(reinterpret_cast<const uint32_t*>(ci), rows.as<int32_t>(), nnz, radix_passes(static_cast<uint32_t>(n - 1)),
+                    k0.as<uint32_t>(), k1.as<uint32_t>(), ci_r, tmp.as<int32_t>(), nullptr);
 }
 
 // Relabelled CSR with sorted rows: each row's entries are read from the caller's CSR, mapped to new ids,
@@ -761,15 +841,16 @@ static gedwalk_status finish_plan(Plan& plan, const std::vector<int4>& units, co
 // 512 / 256 / 128 entries: R-MAT scale 18 directed (4 M) 42 / 26 / 18 / 17; Erdos-Renyi 1.6 M 17 /
 // 15 / 14 / 14; R-MAT scale 20 (30 M) 127 / 122 / 129 / 141; Barabasi-Albert 16 M in FP64 352 / 357 /
 // 396 / 470; R-MAT scale 22 (128 M) 495 / 507 / 534 / 570.
-static gedwalk_status build_plan(Plan& plan, const std::vector<int32_t>& deg, const std::vector<int32_t>& rp,
+static gedwalk_status build_plan(Plan& plan, const std::vector<int32_t>& rp,
                                  int32_t n_active, int32_t n, bool sorted) {
   const int64_t unit_edges =
       std::max<int64_t>(kUnitEdgesMin, std::min<int64_t>(kUnitEdges, static_cast<int64_t>(rp.back()) / kTargetUnits));
+  auto deg_at = [&](int32_t i) { return rp[i + 1] - rp[i]; };
   if (!sorted) {
     std::vector<int4> units, heavy;
     int32_t slice = 0;
     for (int32_t r = 0; r < n_active; ++r) {
-      const int32_t d = deg[r];
+      const int32_t d = deg_at(r);
       if (d <= kHeavyDeg) continue;
       const int32_t ns = (d + kSliceEdges - 1) / kSliceEdges;
       const int32_t hi = static_cast<int32_t>(heavy.size());
@@ -785,11 +866,11 @@ static gedwalk_status build_plan(Plan& plan, const std::vector<int32_t>& deg, co
     plan.num_heavy = static_cast<int32_t>(heavy.size());
     int32_t r = 0;
     while (r < n_active) {
-      if (deg[r] > kHeavyDeg) {
+      if (deg_at(r) > kHeavyDeg) {
         ++r;
         continue;
       }
-      const int cls = row_class(deg[r]);
+      const int cls = row_class(deg_at(r));
       // a short-row unit takes up to kUnitRowsMax rows; on small graphs fewer, down to one
       // iteration of its warp (2 rows per lane group), so that every SM gets work
       const int32_t iter_rows = cls == 6 ? 1 : 2 * (32 >> cls);
@@ -798,9 +879,9 @@ static gedwalk_status build_plan(Plan& plan, const std::vector<int32_t>& deg, co
       const int64_t max_edges = cls == 6 ? 2 * unit_edges : unit_edges;
       int32_t r1 = r;
       int64_t edges = 0;
-      while (r1 < n_active && deg[r1] <= kHeavyDeg && row_class(deg[r1]) == cls && r1 - r < max_rows &&
-             (r1 == r || edges + deg[r1] <= max_edges)) {
-        edges += deg[r1];
+      while (r1 < n_active && deg_at(r1) <= kHeavyDeg && row_class(deg_at(r1)) == cls && r1 - r < max_rows &&
+             (r1 == r || edges + deg_at(r1) <= max_edges)) {
+        edges += deg_at(r1);
         ++r1;
       }
       units.push_back(make_int4(r, r1, cls, -1));
@@ -810,7 +891,6 @@ static gedwalk_status build_plan(Plan& plan, const std::vector<int32_t>& deg, co
   }
   // rows are ordered by decreasing degree: the heavy rows form a prefix, then runs of one class
   // (row lengths from the row pointers)
-  auto deg_at = [&](int32_t i) { return rp[i + 1] - rp[i]; };
   std::vector<int4> units, heavy;
   int32_t slice = 0;
   int32_t r = 0;
@@ -1448,18 +1528,22 @@ static gedwalk_status upload_impl(const int32_t* row_ptr, const int32_t* col_idx
   g->n = n;
   g->nnz = nnz;
   g->directed = directed;
-  // degrees by caller id (weighted and directed graphs): the rows' own lengths; for a directed
-  // graph also the reverse (in) degree
-  std::vector<int32_t> deg_old, rdeg_old;
-  if (weighted || directed) {
+  // degrees by caller id: the rows' own lengths; for a directed graph also the reverse (in) degrees
+  std::vector<int32_t> deg_old;
+  if (weighted) {
     deg_old.resize(n);
     for (int32_t v = 0; v < n; ++v) deg_old[v] = row_ptr[v + 1] - row_ptr[v];
   }
   int32_t rdmax = 0;
+  DevBuf rdeg;  // by caller id, then the largest
   if (directed) {
-    rdeg_old.assign(n, 0);
-    for (int64_t j = 0; j < nnz; ++j) rdeg_old[col_idx[j]]++;
-    for (int32_t v = 0; v < n; ++v) rdmax = std::max(rdmax, rdeg_old[v]);
+    GW_TRY(rdeg.ensure((static_cast<size_t>(n) + 1) * sizeof(int32_t), 0));
+    GW_CUDA(cudaMemset(rdeg.p, 0, (static_cast<size_t>(n) + 1) * sizeof(int32_t)));
+    reverse_degree_kernel<<<grid_for(std::max<int64_t>(nnz, 1)), 256>>>(raw_ci.as<int32_t>(), nnz, rdeg.as<int32_t>());
+    GW_KCHECK();
+    max_kernel<<<grid_for(n), 256>>>(rdeg.as<int32_t>(), n, rdeg.as<int32_t>() + n);
+    GW_KCHECK();
+    GW_CUDA(cudaMemcpy(&rdmax, rdeg.as<int32_t>() + n, sizeof rdmax, cudaMemcpyDeviceToHost));
   }
   g->dmax = dmax;
   // W_{l+1} <= d W_l with d = d_max; on a digraph an l-walk extends at its end along at most
@@ -1501,39 +1585,30 @@ static gedwalk_status upload_impl(const int32_t* row_ptr, const int32_t* col_idx
   GW_TRY(g->perm_d.ensure(static_cast<size_t>(n) * sizeof(int32_t), 0));
   DevBuf inv_d;
   GW_TRY(inv_d.ensure(static_cast<size_t>(n) * sizeof(int32_t), 0));
-  if (!directed) {
+  {
     // on the device: a stable radix sort by degree, the inverse, the new degrees and row pointers
     DevBuf deg_d;
     GW_TRY(deg_d.ensure(static_cast<size_t>(n) * sizeof(int32_t), 0));
-    GW_TRY(degree_order(raw_rp.as<int32_t>(), n, dmax, g->perm_d.as<int32_t>(), inv_d.as<int32_t>(),
-                        deg_d.as<int32_t>(), g->rp.as<int32_t>()));
+    GW_TRY(degree_order(raw_rp.as<int32_t>(), n, dmax, directed ? rdeg.as<int32_t>() : nullptr, rdmax,
+                        g->perm_d.as<int32_t>(), inv_d.as<int32_t>(), deg_d.as<int32_t>(), g->rp.as<int32_t>()));
     GW_CUDA(cudaMemcpy(g->perm.data(), g->perm_d.p, static_cast<size_t>(n) * sizeof(int32_t), cudaMemcpyDeviceToHost));
     GW_CUDA(cudaMemcpy(g->inv.data(), inv_d.p, static_cast<size_t>(n) * sizeof(int32_t), cudaMemcpyDeviceToHost));
     GW_CUDA(cudaMemcpy(rp.data(), g->rp.p, rp.size() * sizeof(int32_t), cudaMemcpyDeviceToHost));
-  } else {
-    g->deg.resize(n);
-    for (int32_t v = 0; v < n; ++v) g->perm[v] = v;
-    std::stable_sort(g->perm.begin(), g->perm.end(), [&](int32_t a, int32_t b) {
-      if (deg_old[a] != deg_old[b]) return deg_old[a] > deg_old[b];
-      return rdeg_old[a] > rdeg_old[b];
-    });
-    for (int32_t i = 0; i < n; ++i) g->inv[g->perm[i]] = i;
-    rp[0] = 0;
-    for (int32_t i = 0; i < n; ++i) {
-      g->deg[i] = deg_old[g->perm[i]];
-      rp[i + 1] = rp[i] + g->deg[i];
-    }
-    GW_CUDA(cudaMemcpy(g->rp.p, rp.data(), rp.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-    GW_CUDA(cudaMemcpy(g->perm_d.p, g->perm.data(), static_cast<size_t>(n) * sizeof(int32_t), cudaMemcpyHostToDevice));
-    GW_CUDA(cudaMemcpy(inv_d.p, g->inv.data(), static_cast<size_t>(n) * sizeof(int32_t), cudaMemcpyHostToDevice));
   }
-  // rows from n_active on are isolated: no entry in either direction
-  g->n_active = n;
-  if (!directed) {
-    g->n_active = first_row(0, n, [&](int32_t i) { return rp[i + 1] == rp[i]; });
-  } else {
-    while (g->n_active > 0 && g->deg[g->n_active - 1] == 0 && rdeg_old[g->perm[g->n_active - 1]] == 0) --g->n_active;
+  std::vector<int32_t> rpr;  // directed: the reverse lists' row pointers by new id
+  if (directed) {
+    DevBuf deg_d;
+    rpr.resize(static_cast<size_t>(n) + 1);
+    GW_TRY(deg_d.ensure(static_cast<size_t>(n) * sizeof(uint32_t), 0));
+    GW_TRY(g->rp_r.ensure(rpr.size() * sizeof(int32_t), 0));
+    permute_kernel<<<grid_for(n), 256>>>(rdeg.as<int32_t>(), g->perm_d.as<int32_t>(), n, deg_d.as<uint32_t>());
+    GW_KCHECK();
+    GW_TRY(exclusive_scan(deg_d.as<uint32_t>(), n, g->rp_r.as<uint32_t>(), g->rp_r.as<uint32_t>() + n));
+    GW_CUDA(cudaMemcpy(rpr.data(), g->rp_r.p, rpr.size() * sizeof(int32_t), cudaMemcpyDeviceToHost));
   }
+  // rows from n_active on are isolated: no entry in either direction (directed: among the rows without
+  // entries of their own the order is by falling reverse degree)
+  g->n_active = first_row(0, n, [&](int32_t i) { return rp[i + 1] == rp[i] && (!directed || rpr[i + 1] == rpr[i]); });
   {
     GW_CUDA(cudaMemset(g->ci.as<int32_t>() + nnz, 0, 4 * sizeof(int32_t)));
     // rows by falling length (a prefix above each length): one launch per network size
@@ -1591,24 +1666,13 @@ static gedwalk_status upload_impl(const int32_t* row_ptr, const int32_t* col_idx
     GW_CUDA(cudaMemcpy(g->rs_d.p, sd.data(), sd.size() * sizeof(double), cudaMemcpyHostToDevice));
     GW_CUDA(cudaMemcpy(g->rs_f.p, sf.data(), sf.size() * sizeof(float), cudaMemcpyHostToDevice));
   }
-  GW_TRY(build_plan(g->plan, g->deg, rp, g->n_active, n, true));
+  GW_TRY(build_plan(g->plan, rp, g->n_active, n, true));
   if (directed) {
     // the reverse CSR (row v: the u with an arc u -> v), same ids, rows sorted
-    g->deg_r.assign(n, 0);
-    for (int32_t i = 0; i < n; ++i) g->deg_r[i] = rdeg_old[g->perm[i]];
-    std::vector<int32_t> rpr(static_cast<size_t>(n) + 1, 0);
-    for (int32_t i = 0; i < n; ++i) rpr[i + 1] = rpr[i] + g->deg_r[i];
-    std::vector<int32_t> cir(static_cast<size_t>(nnz) + 4, 0);
-    std::vector<int32_t> fill(rpr.begin(), rpr.end() - 1);
-    for (int32_t i = 0; i < n; ++i) {  // rows i in increasing order: every reverse row comes out sorted
-      const int32_t v = g->perm[i];
-      for (int32_t j = row_ptr[v]; j < row_ptr[v + 1]; ++j) cir[fill[g->inv[col_idx[j]]]++] = i;
-    }
-    GW_TRY(g->rp_r.ensure(rpr.size() * sizeof(int32_t), 0));
-    GW_TRY(g->ci_r.ensure(cir.size() * sizeof(int32_t), 0));
-    GW_CUDA(cudaMemcpy(g->rp_r.p, rpr.data(), rpr.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-    GW_CUDA(cudaMemcpy(g->ci_r.p, cir.data(), cir.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-    GW_TRY(build_plan(g->plan_r, g->deg_r, rpr, g->n_active, n, false));
+    GW_TRY(g->ci_r.ensure((static_cast<size_t>(nnz) + 4) * sizeof(int32_t), 0));
+    GW_CUDA(cudaMemset(g->ci_r.as<int32_t>() + nnz, 0, 4 * sizeof(int32_t)));
+    GW_TRY(transpose_rows(g->rp.as<int32_t>(), g->ci.as<int32_t>(), n, nnz, g->ci_r.as<int32_t>()));
+    GW_TRY(build_plan(g->plan_r, rpr, g->n_active, n, false));
   }
   *out = reinterpret_cast<gedwalk_graph_t>(g.release());
   return GEDWALK_OK;

@@ -199,14 +199,12 @@ struct Graph {
   bool directed = false;
   DevBuf rp_r, ci_r;
   Plan plan_r;
-  std::vector<int32_t> deg_r;
   // certified upper bound of sigma_max (0: not computed) and the last Rayleigh estimate
   double sigma_up = 0.0, sigma_lo = 0.0;
   DevBuf rp, ci;            // relabelled CSR (new ids), ci padded by 4 entries
   DevBuf perm_d;            // int32[n]: new -> caller id
   std::vector<int32_t> perm;  // new -> caller id
   std::vector<int32_t> inv;   // caller id -> new
-  std::vector<int32_t> deg;   // degree by new id (directed graphs only; else the row pointers give it)
   Plan plan;
 
   // alpha-scaled walk totals t_r = alpha A t_{r-1}, t_0 = 1 (FP64, [rows][n]; on a weighted graph
