@@ -32,10 +32,11 @@
 // grows), from the walk-total tables. (Directed: F sums psi, U phi; the returns are not counted.)
 //
 // Measured on a GB300 (one maximisation, before: full-length sweeps that store every level's phi, a
-// bound pass per step and the visits-times-continuations bound): R-MAT scale 22, k = 100, FP32 143.2
-// -> 40.9 ms (60 + 8 sweeps of 495 us instead of 135 of 587 and 54 of 498); Erdos-Renyi n = 100,003,
-// degree 16, k = 27 19.4 -> 2.3 ms (the sharper bound leaves one candidate batch); Barabasi-Albert
-// n = 10^6, k = 25, FP64 38.1 -> 12.4 ms; Algorithm 2 on R-MAT scale 20, k = 50 94.1 -> 11.1 ms.
+// bound pass per step and the visits-times-continuations bound): R-MAT scale 22, k = 100, FP32 144.3
+// -> 34.5 ms (60 to 64 sweeps of 493 us instead of 135 of 587 and 54 of 498); Erdos-Renyi n = 100,003,
+// degree 16, k = 27 18.1 -> 2.0 ms (the sharper bound leaves one or two candidate batches);
+// Barabasi-Albert n = 10^6, k = 25, FP64 38.2 -> 7.4 ms; Algorithm 2 on R-MAT scale 20, k = 50 93.6 ->
+// 9.9 ms.
 #include <algorithm>
 #include <cmath>
 
@@ -454,8 +455,9 @@ __device__ __forceinline__ void block_levels(WarpList (&w)[NL], float* sv, int* 
 // correction, against the lowest last entry of the lists, decides. The rows come by decreasing
 // degree, so after a warp's first iteration few pass. A bound of exactly 0 matters only when every
 // bound is 0, so its vertex is recorded only while the warp's list is empty (an atomic per such row,
-// all to one address, would serialise). 279 -> 150 us; on
-// 10^5 rows, where a warp has one iteration, the lists cost most (device_util.cuh): 97 -> 63 us.
+// all to one address, would serialise). 279 -> 123 us (418 MB
+// of traffic at 3.4 TB/s, 37% of the warps resident: a row's vectors and sums take the registers); on 10^5
+// rows, where a warp has one iteration, the lists cost most (device_util.cuh): 97 -> 63 us.
 template <typename T, int C, bool CHAIN, bool SEL, bool DIR>
 __global__ void __launch_bounds__(kThreads, DIR || sizeof(T) * C > 32 ? 2 : kMeetPerSM) meet_kernel(const MeetArgs a) {
   constexpr int D = C - 1;
