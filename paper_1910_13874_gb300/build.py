@@ -36,8 +36,12 @@ def _sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cpp")))
 
 
+def _headers():
+    return [p for d, ext in ((CSRC, "*.h"), (CSRC, "*.cuh"), (INCLUDE, "*.h")) for p in glob.glob(os.path.join(d, ext))]
+
+
 def _deps():
-    return _sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(INCLUDE, "*.h"))
+    return _sources() + _headers()
 
 
 def up_to_date() -> bool:
@@ -52,7 +56,7 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
         return LIB
     nvcc = _nvcc()
     os.makedirs(OUT, exist_ok=True)
-    hdr_time = max(os.path.getmtime(d) for d in _deps() if d.endswith(".h"))
+    hdr_time = max(os.path.getmtime(d) for d in _headers())
 
     def compile_one(src):
         obj = os.path.join(OUT, os.path.basename(src) + ".o")
