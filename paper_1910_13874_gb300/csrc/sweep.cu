@@ -50,26 +50,7 @@ struct Log2<1> {
   static constexpr int v = 0;
 };
 
-// p[0..N) -> out with the widest aligned vector loads (through the read-only path).
-template <typename T, int N>
-__device__ __forceinline__ void load_vec(const T* __restrict__ p, T (&out)[N]) {
-  constexpr int kBytes = int(sizeof(T)) * N;
-  if constexpr (kBytes % 16 == 0) {
-    constexpr int kPer = 16 / int(sizeof(T));
-#pragma unroll
-    for (int k = 0; k < kBytes / 16; ++k) {
-      const float4 t = __ldg(reinterpret_cast<const float4*>(p) + k);
-      memcpy(&out[k * kPer], &t, 16);
-    }
-  } else if constexpr (kBytes == 8) {
-    const float2 t = __ldg(reinterpret_cast<const float2*>(p));
-    memcpy(out, &t, 8);
-  } else {
-#pragma unroll
-    for (int e = 0; e < N; ++e) out[e] = __ldg(p + e);
-  }
-}
-
+// v -> p[0..N) with the widest aligned vector stores.
 template <typename T, int N>
 __device__ __forceinline__ void store_vec(T* __restrict__ p, const T (&v)[N]) {
   constexpr int kBytes = int(sizeof(T)) * N;
@@ -94,15 +75,18 @@ __device__ __forceinline__ void store_vec(T* __restrict__ p, const T (&v)[N]) {
 // Gathers of x rows. Vertices are numbered by decreasing degree, so the rows with the
 // lowest ids are gathered most often: rows below the hub limit are loaded with high L1
 // retention priority, all others without allocating in L1, so the stream of cold rows
-// cannot flush the hot ones. 32-byte rows take a single 256-bit load.
-#define GW_LD1(Q, TY, R, x, p) asm volatile("ld.global.nc." Q "." TY " %0, [%1];" : "=" R(x[0]) : "l"(p))
+// cannot flush the hot ones. 32-byte rows take a single 256-bit load. These are coherent loads, not
+// ld.global.nc: the sweep before writes x while this one is already resident (programmatic dependents),
+// and the non-coherent path is only defined for data that no one writes while the kernel runs. Row
+// pointers, indices, units, scales and masks are such data.
+#define GW_LD1(Q, TY, R, x, p) asm volatile("ld.global." Q "." TY " %0, [%1];" : "=" R(x[0]) : "l"(p))
 #define GW_LD2(Q, TY, R, x, p) \
-  asm volatile("ld.global.nc." Q ".v2." TY " {%0,%1}, [%2];" : "=" R(x[0]), "=" R(x[1]) : "l"(p))
+  asm volatile("ld.global." Q ".v2." TY " {%0,%1}, [%2];" : "=" R(x[0]), "=" R(x[1]) : "l"(p))
 #define GW_LD4(Q, TY, R, x, p)                                                                        \
-  asm volatile("ld.global.nc." Q ".v4." TY " {%0,%1,%2,%3}, [%4];" : "=" R(x[0]), "=" R(x[1]), "=" R(x[2]), \
+  asm volatile("ld.global." Q ".v4." TY " {%0,%1,%2,%3}, [%4];" : "=" R(x[0]), "=" R(x[1]), "=" R(x[2]), \
                "=" R(x[3]) : "l"(p))
 #define GW_LD8(Q, x, p)                                                                                 \
-  asm volatile("ld.global.nc." Q ".v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"                              \
+  asm volatile("ld.global." Q ".v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"                              \
                : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(x[4]), "=f"(x[5]), "=f"(x[6]), \
                  "=f"(x[7])                                                                             \
                : "l"(p))
@@ -353,7 +337,7 @@ __device__ __forceinline__ void epilogue(const SweepArgs& a, const int* __restri
     if (store) {
       if constexpr (MODE == MODE_WALKS) {
         // W_{2r-1} = <t_r, t_{r-1}> and W_{2r} = <t_r, t_r>: the two halves of a walk meet
-        const T x = __ldg(static_cast<const T*>(a.X) + r);
+        const T x = __ldcg(static_cast<const T*>(a.X) + r);  // coherent, as the gathers
         acc.add(0, y[0] * (rs ? x / sv : x));
         acc.add(1, y[0] * y[0]);
       } else if constexpr (Sums<MODE, C>::N > 0) {
