@@ -236,7 +236,9 @@ __global__ void __launch_bounds__(kThreads) batch_meet(const BatchVecs b, int32_
 }
 constexpr int kBatchMeetBlocks = 456;  // three per SM
 
-int blocks_for(int64_t n, int per = 256) { return static_cast<int>(std::min<int64_t>((n + per - 1) / per, 152 * 32)); }
+int blocks_for(int64_t n, int per = 256) {
+  return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((n + per - 1) / per, 152 * 32)));
+}
 
 }  // namespace
 
@@ -365,6 +367,10 @@ int64_t score_batch_footprint(const Graph& g, int64_t members, int32_t groups) {
 // go to ws.small. The table holds rows 0..H (the caller keeps its lock).
 static gedwalk_status batch_runs(Graph& g, Workspace& ws, int C, const int32_t* offsets, int32_t G, const int32_t* mrow,
                                  const int32_t* mcol, const Resolved& r, cudaStream_t s) {
+  if (g.n_active == 0) {  // no edges, no walks
+    GW_CUDA(cudaMemsetAsync(ws.small.p, 0, sizeof(double) * G, s));
+    return GEDWALK_OK;
+  }
   const int32_t L = r.L, H = (L + 1) / 2;
   const int64_t vec = static_cast<int64_t>(g.n_active) * C;
   // x_1 .. x_H in a ring; beyond that the oldest are folded into one vector behind it
