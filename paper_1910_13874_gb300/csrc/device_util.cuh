@@ -9,6 +9,50 @@
 
 namespace gw {
 
+// Pairs of FP32 values hi + lo, |lo| about 2^-24 |hi|: values and sums to about 2^-46 where a GB300's FP64
+// units would take 64 times as long. Exact sum and product of two floats (Knuth; Dekker, with fma):
+__device__ __forceinline__ float two_sum(float a, float b, float* err) {
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  *err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+  return s;
+}
+__device__ __forceinline__ float two_prod(float a, float b, float* err) {
+  const float p = __fmul_rn(a, b);
+  *err = __fmaf_rn(a, b, -p);
+  return p;
+}
+struct Pair {
+  float hi, lo;
+  __device__ __forceinline__ void add(float x) {
+    float e;
+    hi = two_sum(hi, x, &e);
+    lo = __fadd_rn(lo, e);
+  }
+  __device__ __forceinline__ void add(const Pair& x) {
+    float e;
+    hi = two_sum(hi, x.hi, &e);
+    lo = __fadd_rn(lo, __fadd_rn(e, x.lo));
+  }
+  __device__ __forceinline__ void sub(const Pair& x) { add(Pair{-x.hi, -x.lo}); }
+  __device__ __forceinline__ Pair times(const Pair& x) const {
+    float e;
+    const float p = two_prod(hi, x.hi, &e);
+    return Pair{p, __fmaf_rn(hi, x.lo, __fmaf_rn(lo, x.hi, e))};
+  }
+  __device__ __forceinline__ Pair times(float x) const {
+    float e;
+    const float p = two_prod(hi, x, &e);
+    return Pair{p, __fmaf_rn(lo, x, e)};
+  }
+  // at least 0: differences of rounded values that would be >= 0 exactly
+  __device__ __forceinline__ Pair pos() const { return __fadd_rn(hi, lo) > 0.0f ? *this : Pair{0.0f, 0.0f}; }
+  __device__ __forceinline__ double get() const { return static_cast<double>(hi) + static_cast<double>(lo); }
+};
+__device__ __forceinline__ Pair to_pair(double x) {
+  const float hi = static_cast<float>(x);
+  return Pair{hi, static_cast<float>(x - static_cast<double>(hi))};
+}
+
 // Per-lane column sums over the rows of one unit. FP64 vectors sum in FP64. FP32 vectors sum with
 // compensated FP32 additions (Kahan: the error is at most 2u * sum |y| + O(m u^2), u = 2^-24, over
 // m <= 128 rows) and convert once per unit to FP64, in which every later sum (over lanes, units and

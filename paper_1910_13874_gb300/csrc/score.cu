@@ -85,15 +85,23 @@ __global__ void batch_group_sum(const double* __restrict__ acc, const int32_t* _
 // a Barabasi-Albert graph of n = 10^6 (L = 9, blocks of 16 columns) took 41.2 ms with the first-visit
 // sweeps of the full length.
 
-// t_H(v) and P(v) = sum_{a=1..L-H} t_a(v), true values in FP32.
+// What a vertex contributes beside the hit vectors, as pairs (hi, lo) from the FP64 table: with x the
+// stored vectors (s h on a weighted graph, i = 1 / s; s = 1 else) its term of the score is
+//   i K(x) + i t_H V(x) + (s P - V(x)) i^2 x_H,   P = t_1 + .. + t_{L-H}.
+struct BatchRow {
+  Pair t, p;  // i t_H and s P
+};
+struct BatchScale {
+  Pair i, i2;
+};
 __global__ void batch_totals(const double* __restrict__ T, int64_t n, int32_t n_active, int32_t L, int32_t H,
-                             const double* __restrict__ rs, float* __restrict__ tH, float* __restrict__ P) {
+                             const double* __restrict__ rs, BatchRow* __restrict__ row, BatchScale* __restrict__ scale) {
   for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n_active; v += gridDim.x * blockDim.x) {
     const double inv = rs ? 1.0 / rs[v] : 1.0;
     double p = 0.0;
     for (int32_t a = 1; a <= L - H; ++a) p += T[static_cast<size_t>(a) * n + v];
-    tH[v] = static_cast<float>(T[static_cast<size_t>(H) * n + v] * inv);
-    P[v] = static_cast<float>(p * inv);
+    row[v] = BatchRow{to_pair(T[static_cast<size_t>(H) * n + v] * inv * inv), to_pair(p)};
+    if (rs) scale[v] = BatchScale{to_pair(inv), to_pair(inv * inv)};
   }
 }
 
@@ -154,67 +162,89 @@ struct BatchVecs {
   const float* ring;
   int64_t stride;
   int slots;
-  float* V;  // nullptr: nothing folded
+  float* V;  // hi and lo parts, `stride` elements each
   int32_t folded, H;
 };
 
 // V (+)= x_{folded+1} .. x_{folded+slots-1}.
 __global__ void batch_fold(const BatchVecs b, int64_t quads) {
+  float4* hi = reinterpret_cast<float4*>(b.V);
+  float4* lo = reinterpret_cast<float4*>(b.V + b.stride);
   for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < quads;
        q += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    if (b.folded > 0) a = reinterpret_cast<const float4*>(b.V)[q];
+    Pair a[4] = {};
+    if (b.folded > 0) {
+      const float4 h = hi[q], l = lo[q];
+      a[0] = Pair{h.x, l.x}, a[1] = Pair{h.y, l.y}, a[2] = Pair{h.z, l.z}, a[3] = Pair{h.w, l.w};
+    }
     for (int t = 0; t < b.slots - 1; ++t) {
       const float4 x = reinterpret_cast<const float4*>(b.ring + b.stride * ((b.folded + t) % b.slots))[q];
-      a.x += x.x;
-      a.y += x.y;
-      a.z += x.z;
-      a.w += x.w;
+      a[0].add(x.x), a[1].add(x.y), a[2].add(x.z), a[3].add(x.w);
     }
-    reinterpret_cast<float4*>(b.V)[q] = a;
+    hi[q] = make_float4(a[0].hi, a[1].hi, a[2].hi, a[3].hi);
+    lo[q] = make_float4(a[0].lo, a[1].lo, a[2].lo, a[3].lo);
   }
 }
 
 // The halves meet: score_j = sum_v [K + V t_H + (P - V) h_H], K = h_1 + .. + h_H, V = h_1 + .. +
-// h_{L-H}. A thread takes four columns of a row (always the same four); FP32 terms are summed
-// compensated per thread, in FP64 over threads and blocks, in a fixed order.
-template <int C>
+// h_{L-H}. A thread takes four columns of a row (always the same four). Nothing beyond the stored vectors
+// is rounded to FP32: sums over t, products and the thread's sum are kept as pairs, and summed in FP64
+// over threads and blocks in a fixed order.
+template <int C, bool WEIGHTED>
 __global__ void __launch_bounds__(kThreads) batch_meet(const BatchVecs b, int32_t odd, int32_t n_active,
-                                                       const float* __restrict__ tH, const float* __restrict__ P,
-                                                       const float* __restrict__ rs, double* __restrict__ part,
+                                                       const BatchRow* __restrict__ row,
+                                                       const BatchScale* __restrict__ scale, double* __restrict__ part,
                                                        unsigned* __restrict__ done, int32_t groups,
                                                        double* __restrict__ out) {
   constexpr int Q = C / 4;  // float4s of a row
   __shared__ double sm[kThreads][4];
   __shared__ int is_last;
-  ColAcc<float, 4> acc;
-  acc.zero();
+  Pair acc[4] = {};
   const int64_t quads = static_cast<int64_t>(n_active) * Q;
   for (int64_t q = blockIdx.x * static_cast<int64_t>(kThreads) + threadIdx.x; q < quads;
        q += static_cast<int64_t>(gridDim.x) * kThreads) {
     const int32_t v = static_cast<int32_t>(q / Q);
-    float k[4] = {0.0f, 0.0f, 0.0f, 0.0f}, h[4];
+    Pair k[4] = {};
+    float h[4];
     if (b.folded > 0) {
       const float4 x = __ldcs(reinterpret_cast<const float4*>(b.V) + q);
-      k[0] = x.x, k[1] = x.y, k[2] = x.z, k[3] = x.w;
+      const float4 y = __ldcs(reinterpret_cast<const float4*>(b.V + b.stride) + q);
+      k[0] = Pair{x.x, y.x}, k[1] = Pair{x.y, y.y}, k[2] = Pair{x.z, y.z}, k[3] = Pair{x.w, y.w};
     }
     for (int t = b.folded + 1; t < b.H; ++t) {
       const float4 x = __ldcs(reinterpret_cast<const float4*>(b.ring + b.stride * ((t - 1) % b.slots)) + q);
-      k[0] += x.x, k[1] += x.y, k[2] += x.z, k[3] += x.w;
+      k[0].add(x.x), k[1].add(x.y), k[2].add(x.z), k[3].add(x.w);
     }
     {
       const float4 x = __ldcs(reinterpret_cast<const float4*>(b.ring + b.stride * ((b.H - 1) % b.slots)) + q);
       h[0] = x.x, h[1] = x.y, h[2] = x.z, h[3] = x.w;
     }
-    const float inv = rs ? 1.0f / rs[v] : 1.0f, t = __ldg(tH + v), p = __ldg(P + v);
+    const float4 rw = __ldg(reinterpret_cast<const float4*>(row) + v);
+    const Pair t{rw.x, rw.y}, p{rw.z, rw.w};
+    Pair i{1.0f, 0.0f}, i2{1.0f, 0.0f};
+    if constexpr (WEIGHTED) {
+      const float4 sc = __ldg(reinterpret_cast<const float4*>(scale) + v);
+      i = Pair{sc.x, sc.y}, i2 = Pair{sc.z, sc.w};
+    }
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      const float hh = h[c] * inv, below = k[c] * inv, kk = below + hh, vv = odd ? below : kk;
-      acc.add(c, kk + vv * t + fmaxf(p - vv, 0.0f) * hh);
+      Pair kk = k[c];
+      kk.add(h[c]);
+      const Pair vv = odd ? k[c] : kk;
+      Pair rest = p;
+      rest.sub(vv);
+      if constexpr (WEIGHTED) {
+        acc[c].add(kk.times(i));
+        acc[c].add(rest.pos().times(i2.times(h[c])));
+      } else {
+        acc[c].add(kk);
+        acc[c].add(rest.pos().times(h[c]));
+      }
+      acc[c].add(vv.times(t));
     }
   }
 #pragma unroll
-  for (int c = 0; c < 4; ++c) sm[threadIdx.x][c] = acc.get(c);
+  for (int c = 0; c < 4; ++c) sm[threadIdx.x][c] = acc[c].get();
   __syncthreads();
   if (threadIdx.x < C) {  // column threadIdx.x: the threads that hold its four
     double x = 0.0;
@@ -354,8 +384,8 @@ int64_t score_batch_footprint(const Graph& g, int64_t members, int32_t groups) {
   b += static_cast<int64_t>(std::max(g.plan.num_slices, 1)) * C * 4 + std::max(g.plan.num_heavy, 1) * 4;
   b += static_cast<int64_t>(groups) * 8 + 64 + (n + 31) / 32 * 4;
   if (!g.directed) {
-    b += static_cast<int64_t>(g.n_active) * C * 4 * (batch_ring(g, C) + 1);  // the stored vectors and their sum
-    b += 2 * n * 4 + kBatchMeetBlocks * C * 8;
+    b += static_cast<int64_t>(g.n_active) * C * 4 * (batch_ring(g, C) + 2);  // the stored vectors, their sum's parts
+    b += n * (g.weighted ? 32 : 16) + kBatchMeetBlocks * C * 8;
     return b;
   }
   b += 2 * n * C * 4;  // walk vectors x0, x1
@@ -373,12 +403,12 @@ static gedwalk_status batch_runs(Graph& g, Workspace& ws, int C, const int32_t* 
   }
   const int32_t L = r.L, H = (L + 1) / 2;
   const int64_t vec = static_cast<int64_t>(g.n_active) * C;
-  // x_1 .. x_H in a ring; beyond that the oldest are folded into one vector behind it
+  // x_1 .. x_H in a ring; beyond that the oldest are folded into two vectors (hi, lo) behind it
   const int ring_slots = batch_ring(g, C);
-  const int stored = H > ring_slots ? ring_slots + 1 : g.weighted ? ring_slots : H;
+  const int stored = H > ring_slots ? ring_slots + 2 : g.weighted ? ring_slots : H;
   GW_TRY(ws.xs.ensure(static_cast<size_t>(vec) * stored * sizeof(float), s));
-  GW_TRY(ws.tail.ensure(static_cast<size_t>(g.n) * sizeof(float), s));
-  GW_TRY(ws.bound.ensure(static_cast<size_t>(g.n) * sizeof(float), s));
+  GW_TRY(ws.tail.ensure(static_cast<size_t>(g.n) * sizeof(BatchRow), s));
+  if (g.weighted) GW_TRY(ws.bound.ensure(static_cast<size_t>(g.n) * sizeof(BatchScale), s));
   const size_t nz_bytes = (static_cast<size_t>(g.n) + 31) / 32 * sizeof(uint32_t);
   GW_TRY(ws.mask.ensure(nz_bytes, s));
   uint32_t* nz = ws.mask.as<uint32_t>();
@@ -390,9 +420,10 @@ static gedwalk_status batch_runs(Graph& g, Workspace& ws, int C, const int32_t* 
   unsigned* done = ws.parts.as<unsigned>();
   GW_CUDA(cudaMemsetAsync(done, 0, sizeof(double), s));
   const double* T = g.ttab.as<double>();
-  const float* rs = g.weighted ? g.rs_f.as<float>() : nullptr;
+  BatchRow* row = ws.tail.as<BatchRow>();
+  BatchScale* scale = ws.bound.as<BatchScale>();
   batch_totals<<<blocks_for(g.n_active), 256, 0, s>>>(T, g.n, g.n_active, L, H, g.weighted ? g.rs_d.as<double>() : nullptr,
-                                                      ws.tail.as<float>(), ws.bound.as<float>());
+                                                      row, scale);
   GW_KCHECK();
   float* ring = ws.xs.as<float>();
   auto slot = [&](int32_t t) { return ring + vec * ((t + ring_slots - 1) % ring_slots); };  // x_0: the last slot
@@ -436,9 +467,13 @@ static gedwalk_status batch_runs(Graph& g, Workspace& ws, int C, const int32_t* 
       GW_TRY(own(t, nullptr));
     }
     double* out = ws.small.as<double>() + g0;
-#define GW_MEET(CC) \
-  if (C == CC) \
-    batch_meet<CC><<<meet, kThreads, 0, s>>>(b, L & 1, g.n_active, ws.tail.as<float>(), ws.bound.as<float>(), rs, part, done, g1 - g0, out);
+#define GW_MEET(CC)                                                                                                     \
+  if (C == CC) {                                                                                                        \
+    if (g.weighted)                                                                                                     \
+      batch_meet<CC, true><<<meet, kThreads, 0, s>>>(b, L & 1, g.n_active, row, scale, part, done, g1 - g0, out);       \
+    else                                                                                                                \
+      batch_meet<CC, false><<<meet, kThreads, 0, s>>>(b, L & 1, g.n_active, row, nullptr, part, done, g1 - g0, out);    \
+  }
     GW_MEET(8) GW_MEET(16) GW_MEET(32) GW_MEET(64)
 #undef GW_MEET
     GW_KCHECK();
