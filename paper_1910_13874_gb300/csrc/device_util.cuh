@@ -48,6 +48,43 @@ struct Pair {
   __device__ __forceinline__ Pair pos() const { return __fadd_rn(hi, lo) > 0.0f ? *this : Pair{0.0f, 0.0f}; }
   __device__ __forceinline__ double get() const { return static_cast<double>(hi) + static_cast<double>(lo); }
 };
+// The same interface in FP64, for kernels of either precision: Wide<T> holds what must not be rounded to T
+// when T is FP32.
+struct Double {
+  double v;
+  __device__ __forceinline__ void add(double x) { v += x; }
+  __device__ __forceinline__ void add(const Double& x) { v += x.v; }
+  __device__ __forceinline__ void sub(const Double& x) { v -= x.v; }
+  __device__ __forceinline__ Double times(const Double& x) const { return Double{v * x.v}; }
+  __device__ __forceinline__ Double times(double x) const { return Double{v * x}; }
+  __device__ __forceinline__ Double pos() const { return Double{v > 0.0 ? v : 0.0}; }
+  __device__ __forceinline__ double get() const { return v; }
+};
+template <typename T>
+struct WideOf {
+  using type = Double;
+  __device__ __forceinline__ static Double make(double hi, double) { return Double{hi}; }
+  __device__ __forceinline__ static Double inverse(double x) { return Double{1.0 / x}; }
+  // a + x, the rounding error added to lo
+  __device__ __forceinline__ static void accumulate(double& a, double&, double x) { a += x; }
+};
+template <>
+struct WideOf<float> {
+  using type = Pair;
+  __device__ __forceinline__ static Pair make(float hi, float lo) { return Pair{hi, lo}; }
+  __device__ __forceinline__ static Pair inverse(float x) {
+    const float r = 1.0f / x;
+    return Pair{r, __fmul_rn(r, __fmaf_rn(-x, r, 1.0f))};
+  }
+  __device__ __forceinline__ static void accumulate(float& a, float& lo, float x) {
+    float e;
+    a = two_sum(a, x, &e);
+    lo = __fadd_rn(lo, e);
+  }
+};
+template <typename T>
+using Wide = typename WideOf<T>::type;
+
 __device__ __forceinline__ Pair to_pair(double x) {
   const float hi = static_cast<float>(x);
   return Pair{hi, static_cast<float>(x - static_cast<double>(hi))};

@@ -488,8 +488,8 @@ __global__ void __launch_bounds__(kThreads, DIR || sizeof(T) * C > 32 ? 2 : kMee
 #pragma unroll
     for (int l = 0; l < NL; ++l) sampling |= in.thr[l] != ~0ull;
   }
-  ColAcc<T, D> acc;
-  acc.zero();
+  using W = WideOf<T>;
+  Wide<T> acc[D] = {};
   WarpList w[NL];
   int nsampled[NL];
 #pragma unroll
@@ -502,15 +502,16 @@ __global__ void __launch_bounds__(kThreads, DIR || sizeof(T) * C > 32 ? 2 : kMee
     const bool ok = v < a.n_scan;
     const bool has = v < a.n_active;
     const T* __restrict__ row = xs + static_cast<size_t>(has ? v : 0) * C;
-    // the row's sums over t = 1..H-1 and x_H (directed: Br, xr of the walks that end here)
-    T B[C], xh[C], Br[DIR ? C : 1], xr[DIR ? C : 1];
+    // the row's sums over t = 1..H-1 with their low parts, and x_H (directed: Br, xr of the walks that end here)
+    T B[C], Bl[C], xh[C], Br[DIR ? C : 1], Brl[DIR ? C : 1], xr[DIR ? C : 1];
 #pragma unroll
-    for (int c = 0; c < C; ++c) B[c] = xh[c] = T(0);
+    for (int c = 0; c < C; ++c) B[c] = Bl[c] = xh[c] = T(0);
     if constexpr (DIR) {
 #pragma unroll
-      for (int c = 0; c < C; ++c) Br[c] = xr[c] = T(0);
+      for (int c = 0; c < C; ++c) Br[c] = Brl[c] = xr[c] = T(0);
     }
     T inv = T(1);
+    Wide<T> winv = W::make(T(1), T(0));
     if (has) {
       auto load = [&](const T* p, T (&x)[C]) {
         if constexpr (sizeof(T) * C >= 16) {
@@ -530,7 +531,7 @@ __global__ void __launch_bounds__(kThreads, DIR || sizeof(T) * C > 32 ? 2 : kMee
         T x[C];
         load(p, x);
 #pragma unroll
-        for (int c = 0; c < C; ++c) B[c] += x[c];
+        for (int c = 0; c < C; ++c) W::accumulate(B[c], Bl[c], x[c]);
       }
       load(p, xh);
       if constexpr (DIR) {
@@ -540,17 +541,61 @@ __global__ void __launch_bounds__(kThreads, DIR || sizeof(T) * C > 32 ? 2 : kMee
           T x[C];
           load(p, x);
 #pragma unroll
-          for (int c = 0; c < C; ++c) Br[c] += x[c];
+          for (int c = 0; c < C; ++c) W::accumulate(Br[c], Brl[c], x[c]);
         }
         load(p, xr);
       }
       if (rs) {
+        winv = W::inverse(rs[v]);
         inv = T(1) / rs[v];
+      }
+    }
+    // gain terms of candidate d + 1 under its base set; nothing beyond the stored vectors is rounded to T
+    {
+      auto value = [&](T hi, T lo) { return rs ? W::make(hi, lo).times(winv) : W::make(hi, lo); };
+      Wide<T> rb = value(B[0], Bl[0]), rh = value(xh[0], T(0)), sb = W::make(T(0), T(0)), sh = sb;
+      if constexpr (DIR) {
+        sb = W::make(Br[0], Brl[0]);
+        sh = W::make(xr[0], T(0));
+      }
 #pragma unroll
-        for (int c = 0; c < C; ++c) {
-          B[c] *= inv;
-          xh[c] *= inv;
+      for (int d = 0; d < D; ++d) {
+        const Wide<T> kb = value(B[d + 1], Bl[d + 1]), kh = value(xh[d + 1], T(0));
+        Wide<T> k = kb, vv, pp;
+        k.add(kh);
+        if constexpr (DIR) {
+          const Wide<T> jh = W::make(xr[d + 1], T(0));
+          vv = W::make(Br[d + 1], Brl[d + 1]);
+          pp = sb;
+          if (!odd) {
+            vv.add(jh);
+            pp.add(sh);
+          }
+          if (CHAIN) {
+            sb.sub(W::make(Br[d + 1], Brl[d + 1]));
+            sh.sub(jh);
+          }
+        } else {
+          vv = odd ? kb : k;
+          pp = rb;
+          if (!odd) pp.add(rh);
         }
+        pp = pp.pos();
+        pp.sub(vv);
+        acc[d].add(k);
+        acc[d].add(vv.times(rh.pos()));
+        acc[d].add(pp.pos().times(kh));
+        if (CHAIN) {
+          rb.sub(kb);
+          rh.sub(kh);
+        }
+      }
+    }
+    if (rs) {
+#pragma unroll
+      for (int c = 0; c < C; ++c) {
+        B[c] *= inv;
+        xh[c] *= inv;
       }
     }
     if (SEL) {
@@ -679,38 +724,11 @@ __global__ void __launch_bounds__(kThreads, DIR || sizeof(T) * C > 32 ? 2 : kMee
         for (int l = 0; l < NL; ++l) enter = fminf(enter, __shfl_sync(kFullMask, w[l].v, kTopK - 1));
       }
     }
-    // gain terms of candidate d + 1 under its base set
-    T rb = B[0], rh = xh[0], sb = T(0), sh = T(0);
-    if constexpr (DIR) {
-      sb = Br[0];
-      sh = xr[0];
-    }
-#pragma unroll
-    for (int d = 0; d < D; ++d) {
-      const T k = B[d + 1] + xh[d + 1];
-      T vv, pp;
-      if constexpr (DIR) {
-        vv = odd ? Br[d + 1] : Br[d + 1] + xr[d + 1];
-        pp = odd ? pos(sb) : pos(sb + sh);
-      } else {
-        vv = odd ? B[d + 1] : k;
-        pp = odd ? pos(rb) : pos(rb + rh);
-      }
-      acc.add(d, k + vv * pos(rh) + pos(pp - vv) * xh[d + 1]);
-      if (CHAIN) {
-        rb -= B[d + 1];
-        rh -= xh[d + 1];
-        if constexpr (DIR) {
-          sb -= Br[d + 1];
-          sh -= xr[d + 1];
-        }
-      }
-    }
   }
   // gain sums of the block
 #pragma unroll
   for (int d = 0; d < D; ++d) {
-    double x = acc.get(d);
+    double x = acc[d].get();
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFullMask, x, o);
     if (lane == 0) sg[warp][d] = x;
