@@ -844,7 +844,8 @@ __global__ void pair_init(T* __restrict__ X, const int32_t* __restrict__ rp, con
 // Walks of length a + b that hit S: the half of length a hits, or it misses and the half of length b
 // hits, so with b = H the lengths H + a, a = 1..L-H, number sum_v [h_a (h_H + m_H) + m_a h_H] and the
 // lengths up to H are plain sums of h_t. One thread per row; the last block adds the block sums.
-// x_t sits at slot (t - 1) % ring; with folded > 0 the slot behind the ring holds x_1 + .. + x_folded.
+// x_t sits at slot (t - 1) % ring; with folded > 0 the two slots behind the ring hold x_1 + .. + x_folded (hi
+// and lo parts). Nothing beyond the stored vectors is rounded to FP32.
 template <typename T>
 __global__ void __launch_bounds__(kThreads) pair_meet(const T* __restrict__ xs, int64_t stride, int32_t ring, int32_t folded,
                                                       int32_t L, int32_t H, int32_t n_active, const T* __restrict__ rs,
@@ -855,14 +856,17 @@ __global__ void __launch_bounds__(kThreads) pair_meet(const T* __restrict__ xs, 
   __shared__ int is_last;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool odd = (L & 1) != 0;
-  ColAcc<T, 1> acc;
-  acc.zero();
+  using W = WideOf<T>;
+  Wide<T> acc = W::make(T(0), T(0));
   for (int32_t v = blockIdx.x * kThreads + threadIdx.x; v < n_active; v += gridDim.x * kThreads) {
-    T bh = T(0), bm = T(0), h = T(0), m = T(0);
+    T bh = T(0), bm = T(0), lh = T(0), lm = T(0), h = T(0), m = T(0);  // sums over t < H and their low parts
     const T* row = xs + 2 * static_cast<size_t>(v);
     if (folded > 0) {
-      bh = row[stride * ring];
-      bm = row[stride * ring + 1];
+      const T* f = row + stride * ring;
+      bh = f[0];
+      bm = f[1];
+      lh = f[stride];
+      lm = f[stride + 1];
     }
 #pragma unroll 4
     for (int t = folded + 1; t <= H; ++t) {
@@ -878,24 +882,33 @@ __global__ void __launch_bounds__(kThreads) pair_meet(const T* __restrict__ xs, 
         xm = q.y;
       }
       if (t < H) {
-        bh += xh;
-        bm += xm;
+        W::accumulate(bh, lh, xh);
+        W::accumulate(bm, lm, xm);
       } else {
         h = xh;
         m = xm;
       }
     }
+    Wide<T> vh = W::make(bh, lh), vm = W::make(bm, lm), wh = W::make(h, T(0)), wm = W::make(m, T(0));
     if (rs) {
-      const T inv = T(1) / rs[v];
-      bh *= inv;
-      bm *= inv;
-      h *= inv;
-      m *= inv;
+      const Wide<T> inv = W::inverse(rs[v]);
+      vh = vh.times(inv);
+      vm = vm.times(inv);
+      wh = wh.times(inv);
+      wm = wm.times(inv);
     }
-    const T vh = odd ? bh : bh + h, vm = odd ? bm : bm + m;
-    acc.add(0, (bh + h) + vh * (h + m) + vm * h);
+    Wide<T> k = vh, both = wh;
+    k.add(wh);
+    both.add(wm);
+    if (!odd) {
+      vh = k;
+      vm.add(wm);
+    }
+    acc.add(k);
+    acc.add(vh.times(both));
+    acc.add(vm.times(wh));
   }
-  double x = acc.get(0);
+  double x = acc.get();
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFullMask, x, o);
   if (lane == 0) sg[warp] = x;
@@ -917,15 +930,16 @@ __global__ void __launch_bounds__(kThreads) pair_meet(const T* __restrict__ xs, 
   if (lane == 0) *out = x;
 }
 
-// acc (+)= x_{from+1} .. x_{from+count}, elementwise.
+// The sum behind the ring, hi and lo parts `stride` apart, (+)= x_{from+1} .. x_{from+count}, elementwise.
 template <typename T>
 __global__ void pair_fold(T* __restrict__ xs, int64_t stride, int32_t ring, int32_t from, int32_t count) {
-  T* acc = xs + stride * ring;
+  T* sum = xs + stride * ring;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < stride;
        i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    T a = from > 0 ? acc[i] : T(0);
-    for (int32_t t = 0; t < count; ++t) a += xs[stride * ((from + t) % ring) + i];
-    acc[i] = a;
+    T a = from > 0 ? sum[i] : T(0), lo = from > 0 ? sum[stride + i] : T(0);
+    for (int32_t t = 0; t < count; ++t) WideOf<T>::accumulate(a, lo, xs[stride * ((from + t) % ring) + i]);
+    sum[i] = a;
+    sum[stride + i] = lo;
   }
 }
 
@@ -1285,7 +1299,7 @@ gedwalk_status score_run(Graph& g, Workspace& ws, const std::vector<int32_t>& S_
   // older; x_0 (weighted) sits where x_ring goes later
   const int32_t ring = static_cast<int32_t>(std::max<int64_t>(
       3, std::min<int64_t>(H + (g.weighted ? 1 : 0), kWideBytes / std::max<int64_t>(static_cast<int64_t>(row * es), 1))));
-  GW_TRY(ws.xs.ensure(row * es * (ring + (H > ring ? 1 : 0)), s));
+  GW_TRY(ws.xs.ensure(row * es * (ring + (H > ring ? 2 : 0)), s));
   GW_TRY(ws.cnt.ensure(n * sizeof(int32_t), s));
   const size_t words = (n + 31) / 32;
   GW_TRY(ws.mask.ensure(words * 4, s));

@@ -85,3 +85,16 @@ def test_gains_by_candidate_runs(cuda_device, weighted):
         for x in (0, 1, 17, 600, 6000, 12_999):
             assert rel(gains[x], oracle.gain(g, S, x, ALPHA, L, w=w)) < TOL, (L, x)
     G.free()
+
+
+@pytest.mark.parametrize("weighted", [False, True])
+def test_score(cuda_device, weighted):
+    g = ba(700)
+    G, w = upload(g, weighted)
+    for L in (1, 2, 3, 4, 5, 6, 7, 8):
+        if weighted and L > 6:
+            continue
+        for S in ([0], [5, 699, 41], list(range(0, 700, 3))):
+            got, _, _ = G.score(S, precision="fp32", alpha=ALPHA, L=L)
+            assert rel(got, oracle.score(g, S, ALPHA, L, w=w)) < TOL, (L, len(S))
+    G.free()
