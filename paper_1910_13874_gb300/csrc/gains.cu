@@ -14,12 +14,13 @@ namespace {
 
 constexpr int kGainThreads = 1024;
 constexpr int kGroup = 8;  // lanes of a short row (K columns, kGroup / K entries at a time)
+constexpr int kParts = 8;  // partial sums a lane keeps of its entries of a row
 constexpr size_t kGainSmem = 200 * 1024;
 
 struct GainArgs {
   const int32_t* rp;
   const int32_t* ci;
-  int32_t n_active, n_long;  // rows [0, n_long) take a warp each
+  int32_t n_active, n_long;  // rows [0, n_long) take a warp each: above 64 entries, 32 with 8 columns
   int64_t phi_stride;
   const uint32_t* mask;
   const void* phi;  // phi_0 .. phi_H under S, true values
@@ -30,19 +31,32 @@ struct GainArgs {
   double* out;  // by internal id
 };
 
-// One step for one row on W lanes: lane l holds column l % K and the entries l / K, + W / K, ..
+// One step for one row on W lanes: lane l holds column l % K and the entries l / K, + W / K, .. in kParts
+// partial sums taken in turn, so a row has kParts W / K of them, added up as a tree: as few additions in
+// a row as the sweeps' (one running sum over 64 equal entries can drift by 16 units in the last place).
+// Nothing else is rounded to FP32: the gain terms are pairs.
 template <typename T, int K, int W>
 __device__ __forceinline__ void gain_row(const GainArgs& a, const T* __restrict__ x, T* __restrict__ y,
                                          const T* __restrict__ phi1, const T* __restrict__ phi0,
                                          const T* __restrict__ rs, int32_t v, bool ok, int32_t c, int l, bool both,
-                                         ColAcc<T, 1>& acc) {
+                                         Wide<T>& acc) {
   const int col = l % K;
-  T s = T(0);
+  T part[kParts];
+#pragma unroll
+  for (int p = 0; p < kParts; ++p) part[p] = T(0);
   if (ok) {
     const int64_t e1 = a.rp[v + 1];
-#pragma unroll 4
-    for (int64_t e = a.rp[v] + l / K; e < e1; e += W / K) s += x[static_cast<size_t>(__ldg(a.ci + e)) * K + col];
+    for (int64_t e = a.rp[v] + l / K; e < e1; e += kParts * (W / K)) {
+#pragma unroll
+      for (int p = 0; p < kParts; ++p)
+        if (e + p * (W / K) < e1) part[p] += x[static_cast<size_t>(__ldg(a.ci + e + p * (W / K))) * K + col];
+    }
   }
+#pragma unroll
+  for (int p = kParts / 2; p > 0; p /= 2)
+#pragma unroll
+    for (int q = 0; q < p; ++q) part[q] += part[q + p];
+  T s = part[0];
 #pragma unroll
   for (int o = K; o < W; o <<= 1) s += __shfl_xor_sync(kFullMask, s, o);
   if (!ok || l >= K) return;
@@ -52,12 +66,21 @@ __device__ __forceinline__ void gain_row(const GainArgs& a, const T* __restrict_
   T k1 = inS ? T(0) : static_cast<T>(a.alpha) * sv * s;
   if (v == c) k1 = f1;
   const size_t i = static_cast<size_t>(v) * K + col;
-  const T k0 = rs ? x[i] / sv : x[i];
+  using WT = WideOf<T>;
+  Wide<T> k0 = WT::make(x[i], T(0));
+  if (rs) k0 = k0.times(WT::inverse(sv));
   // walks of length 2t - 1 (halves t and t - 1) and 2t (halves t and t)
-  const T m0 = f0 - k0, m1 = f1 - k1;
-  T w = m0 > T(0) ? m0 : T(0);
-  if (both) w += f1 + (m1 > T(0) ? m1 : T(0));
-  acc.add(0, k1 * w + f1 * k0);
+  Wide<T> w = WT::make(f0, T(0));
+  w.sub(k0);
+  w = w.pos();
+  if (both) {
+    Wide<T> m1 = WT::make(f1, T(0));
+    m1.sub(WT::make(k1, T(0)));
+    w.add(f1);
+    w.add(m1.pos());
+  }
+  acc.add(w.times(k1));
+  acc.add(k0.times(f1));
   y[i] = k1 * sv;
 }
 
@@ -80,8 +103,7 @@ __global__ void __launch_bounds__(kGainThreads) gains_kernel(const GainArgs a) {
   __syncthreads();
   int32_t c = first + lane % K;  // this lane's candidate
   if (!live(c)) c = -1;
-  ColAcc<T, 1> acc;
-  acc.zero();
+  Wide<T> acc = WideOf<T>::make(T(0), T(0));
   constexpr int NW = kGainThreads / 32, GW = 32 / kGroup;
   for (int32_t t = 1; t <= a.H; ++t) {
     const T* phi1 = static_cast<const T*>(a.phi) + a.phi_stride * t;
@@ -97,7 +119,7 @@ __global__ void __launch_bounds__(kGainThreads) gains_kernel(const GainArgs a) {
     x = y;
     y = z;
   }
-  double g = acc.get(0);
+  double g = acc.get();
 #pragma unroll
   for (int o = K; o < 32; o <<= 1) g += __shfl_xor_sync(kFullMask, g, o);
   if (lane < K) sums[warp][lane] = g;
@@ -175,7 +197,7 @@ gedwalk_status small_gains(Graph& g, Workspace& ws, const Resolved& r, const std
   q.rp = g.rp.as<int32_t>();
   q.ci = g.ci.as<int32_t>();
   q.n_active = g.n_active;
-  q.n_long = g.plan.num_long;
+  q.n_long = small_gain_cols(g, fp64) == 8 ? g.plan.num_mid : g.plan.num_long;
   q.phi_stride = static_cast<int64_t>(n);
   q.mask = ws.mask.as<uint32_t>();
   q.phi = ws.mtab.p;

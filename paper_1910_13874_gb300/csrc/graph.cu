@@ -909,6 +909,7 @@ static gedwalk_status build_plan(Plan& plan, const std::vector<int32_t>& rp,
   plan.num_slices = slice;
   plan.num_heavy = static_cast<int32_t>(heavy.size());
   plan.num_long = first_row(0, n_active, [&](int32_t i) { return deg_at(i) <= 64; });
+  plan.num_mid = first_row(0, n_active, [&](int32_t i) { return deg_at(i) <= 32; });
   while (r < n_active) {
     const int cls = row_class(deg_at(r));
     // the run of this class: classes do not increase along the rows

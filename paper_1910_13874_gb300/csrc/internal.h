@@ -106,6 +106,7 @@ struct Plan {
   int32_t num_heavy = 0;   // heavy rows (degree > kHeavyDeg)
   int32_t num_slots = 0;   // num_units + num_heavy column-sum slots
   int32_t num_long = 0;    // sorted plans: rows above 64 entries, a prefix
+  int32_t num_mid = 0;     // the same above 32
   DevBuf units;            // int4[num_units]
   DevBuf heavy;            // int4[num_heavy]: {row, first slice, slice count, 0}
 };

@@ -98,3 +98,33 @@ def test_score(cuda_device, weighted):
             got, _, _ = G.score(S, precision="fp32", alpha=ALPHA, L=L)
             assert rel(got, oracle.score(g, S, ALPHA, L, w=w)) < TOL, (L, len(S))
     G.free()
+
+
+@pytest.mark.parametrize("n", [700, 5000, 9000])  # 8, 4 and 2 columns a block
+@pytest.mark.parametrize("weighted", [False, True])
+def test_gains_from_shared_memory(cuda_device, n, weighted):
+    g = ba(n)
+    G, w = upload(g, weighted)
+    S = [3, 44, 611]
+    for L in (1, 2, 3, 4, 5, 6):
+        gains, _ = G.gains(S, precision="fp32", alpha=ALPHA, L=L)
+        for x in (0, 1, 17, 600, n - 1):
+            assert rel(gains[x], oracle.gain(g, S, x, ALPHA, L, w=w)) < TOL, (L, x)
+    G.free()
+
+
+def test_row_sums_of_the_small_gains(cuda_device):
+    # 500 vertices joined to the same 63: most of a gain is sums of 63 equal terms, of a value whose running
+    # FP32 sum drifts by 16 units in the last place (6e-7 of the gain). As a tree a sum takes six additions
+    # of half a unit each, on both factors at most: 7 units, 4.2e-7.
+    from paper_1910_13874_gb300 import gedwalk
+
+    m, mids = 500, 63
+    a, b = np.meshgrid(np.arange(m), m + np.arange(mids), indexing="ij")
+    g = gg.from_edges(m + mids, np.stack([a.ravel(), b.ravel()], 1))
+    alpha = float.fromhex("0x1.f08ccp+0")
+    G = gedwalk.Graph.from_host(g)
+    gains, _ = G.gains([], precision="fp32", alpha=alpha, L=4)
+    for x in (0, 250, 499, m, m + 62):
+        assert rel(gains[x], oracle.gain(g, [], x, alpha, 4)) < 4.2e-7, x
+    G.free()
