@@ -47,6 +47,10 @@ struct Pair {
   // at least 0: differences of rounded values that would be >= 0 exactly
   __device__ __forceinline__ Pair pos() const { return __fadd_rn(hi, lo) > 0.0f ? *this : Pair{0.0f, 0.0f}; }
   __device__ __forceinline__ double get() const { return static_cast<double>(hi) + static_cast<double>(lo); }
+  __device__ __forceinline__ float rounded() const { return __fadd_rn(hi, lo); }
+  __device__ __forceinline__ Pair from_lane_xor(int o) const {
+    return Pair{__shfl_xor_sync(0xffffffffu, hi, o), __shfl_xor_sync(0xffffffffu, lo, o)};
+  }
 };
 // The same interface in FP64, for kernels of either precision: Wide<T> holds what must not be rounded to T
 // when T is FP32.
@@ -59,6 +63,8 @@ struct Double {
   __device__ __forceinline__ Double times(double x) const { return Double{v * x}; }
   __device__ __forceinline__ Double pos() const { return Double{v > 0.0 ? v : 0.0}; }
   __device__ __forceinline__ double get() const { return v; }
+  __device__ __forceinline__ double rounded() const { return v; }
+  __device__ __forceinline__ Double from_lane_xor(int o) const { return Double{__shfl_xor_sync(0xffffffffu, v, o)}; }
 };
 template <typename T>
 struct WideOf {

@@ -18,7 +18,7 @@
 //    over the lanes in groups of four loads;
 //  - heavy rows (degree > kHeavyDeg): cut into slices of about kSliceEdges
 //    entries, one warp per slice; each writes its partial sum and the last warp
-//    to arrive (atomic counter) adds the partials in slice order and finishes
+//    to arrive (atomic counter) adds the partials in a fixed order and finishes
 //    the row. No warp ever waits for another.
 // A row's C-wide sum is reduce-scattered across its lanes (halving the columns
 // at every shuffle step), so each lane ends with its own columns and the
@@ -541,12 +541,21 @@ __device__ __forceinline__ void heavy_slice(const SweepArgs& a, const Src& src, 
   prev = __shfl_sync(kFull, prev, 0);
   if (prev != static_cast<unsigned>(hr.z - 1)) return;  // warp-uniform
   __threadfence();
+  // the slices' sums, compensated in FP32: the lanes that hold a column block take slices in turn and add
+  // their sums up, so a row's error does not grow with its slices (160 in a row on R-MAT scale 22)
+  Wide<T> sum[CPL];
+#pragma unroll
+  for (int k = 0; k < CPL; ++k) sum[k] = WideOf<T>::make(T(0), T(0));
+  for (int s = hr.y + (lane >> SC::HS); s < hr.y + hr.z; s += 32 >> SC::HS)
+#pragma unroll
+    for (int k = 0; k < CPL; ++k) sum[k].add(__ldcg(part + static_cast<size_t>(s) * C + c0 + k));
+#pragma unroll
+  for (int o = 1 << SC::HS; o < 32; o <<= 1)
+#pragma unroll
+    for (int k = 0; k < CPL; ++k) sum[k].add(sum[k].from_lane_xor(o));
   T tot[CPL];
 #pragma unroll
-  for (int k = 0; k < CPL; ++k) tot[k] = T(0);
-  for (int s = hr.y; s < hr.y + hr.z; ++s)
-#pragma unroll
-    for (int k = 0; k < CPL; ++k) tot[k] += __ldcg(part + static_cast<size_t>(s) * C + c0 + k);
+  for (int k = 0; k < CPL; ++k) tot[k] = sum[k].rounded();
   constexpr int NL = LaneSums<MODE, CPL>::N;
   ColAcc<T, NL> cacc;
   cacc.zero();

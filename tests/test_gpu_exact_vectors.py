@@ -128,3 +128,21 @@ def test_row_sums_of_the_small_gains(cuda_device):
     for x in (0, 250, 499, m, m + 62):
         assert rel(gains[x], oracle.gain(g, [], x, alpha, 4)) < 4.2e-7, x
     G.free()
+
+
+def test_hub_row_of_many_slices(cuda_device):
+    # a hub's row is summed in slices of 1024 entries, here 488 equal ones. alpha has 19 bits, so a slice is
+    # exact, and its multiples round the same way in a running sum: 7e-6 of the score. Compensated, a
+    # handful of roundings of 6e-8 are left: 1e-6.
+    from paper_1910_13874_gb300 import gedwalk
+
+    g = gg.star(488 * 1024)
+    alpha = 0x40007 * 2.0 ** -22
+    want = oracle.score(g, [1], alpha, 6)
+    G = gedwalk.Graph.from_host(g)
+    assert rel(G.score([1], precision="fp32", alpha=alpha, L=6)[0], want) < 1e-6
+    for width in (8, 64):
+        G.batch_set_width(width)
+        scores, _ = G.score_batch([0, 1, 2], [1, 7], alpha=alpha, L=6)
+        assert rel(scores[0], want) < 1e-6 and rel(scores[1], want) < 1e-6
+    G.free()
