@@ -171,3 +171,17 @@ def test_fp64_chain_widths(cuda_device):
         ref, ref_gains, _ = oracle.greedy(g, 16, alpha, L, "lazy")
         check_sequence(grp, gains, 1e-12, ref, ref_gains, *oracle_greedy_checker(oracle, g, alpha, L))
         G.free()
+
+
+@pytest.mark.parametrize("kw", [{}, dict(lookahead=1)])
+def test_long_walks_are_certified(cuda_device, kw):
+    # 30 sweeps a run: the rounding a certification allows for grows with them (2.5e-7 each, so 1e-5)
+    from paper_1910_13874_gb300 import gedwalk
+
+    g = gg.erdos_renyi(2000, 8, 5)
+    alpha = oracle.default_alpha(g)
+    G = gedwalk.Graph.from_host(g)
+    grp, gains, _, _ = G.maximize(12, precision="fp32", L=61, **kw)
+    ref, ref_gains, _ = oracle.greedy(g, 12, alpha, 61, "lazy")
+    check_sequence(grp, gains, 1e-5, ref, ref_gains, *oracle_greedy_checker(oracle, g, alpha, 61))
+    G.free()
