@@ -71,7 +71,11 @@ gedwalk_status run_sequence(Workspace& ws, cudaStream_t s, const Sequence& q,
     if (sg.uses++ < (q.nnz > kLateEntries ? 3 : 1)) return issue(true, nullptr);  // set-up happens outside capture
     sg.ev.assign(2, nullptr);
     for (cudaEvent_t& e : sg.ev) GW_CUDA(cudaEventCreate(&e));
-    GW_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+    if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+      cudaGetLastError();  // a stream that cannot be captured: directly, as ever
+      sg.reset();
+      return issue(true, nullptr);
+    }
     set_capturing(true);
     const gedwalk_status st = issue(false, &sg.ev);
     set_capturing(false);
@@ -104,10 +108,10 @@ gedwalk_status run_sequence(Workspace& ws, cudaStream_t s, const Sequence& q,
   return GEDWALK_OK;
 }
 
-// The stream a run uses: the caller's, or (for the legacy default stream, which cannot
-// be captured) the workspace's own stream, ordered after the caller's.
+// The stream a run uses: the caller's, or (for the legacy default stream, handle 0 or cudaStreamLegacy,
+// which cannot be captured) the workspace's own stream, ordered after the caller's.
 gedwalk_status greedy_stream(Workspace& ws, cudaStream_t caller, cudaStream_t* out) {
-  if (caller != nullptr) {
+  if (caller != nullptr && caller != cudaStreamLegacy) {
     *out = caller;
     return GEDWALK_OK;
   }
