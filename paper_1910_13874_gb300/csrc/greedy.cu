@@ -73,6 +73,18 @@ gedwalk_status greedy_shape(const Graph& g, const Resolved& r, int32_t flags, Gr
   return GEDWALK_OK;
 }
 
+gedwalk_status ensure_run_tables(Graph& g, Workspace& ws, const Resolved& r, const GreedyShape& sh, int32_t flags) {
+  const bool adaptive = (flags & GEDWALK_ADAPTIVE_L) != 0;
+  if (adaptive) GW_TRY(ensure_totals(g, r.alpha, sh.ell_max + 1, r.stream));
+  if (!g.directed || g.n_active == 0 || (flags & GEDWALK_GAINS_ALL)) return GEDWALK_OK;
+  const int32_t rows = walk_rows(g, (adaptive ? sh.ell_max : r.L) + 1);
+  {
+    std::shared_lock<std::shared_mutex> rl(g.tt_lock);
+    if (g.tt_alpha != r.alpha || g.tt_rows < rows) return GEDWALK_OK;
+  }
+  return ensure_totals_fwd(g, ws, r.alpha, rows, r.stream);
+}
+
 int64_t maximize_footprint(const Graph& g, const Resolved& r, int32_t flags, int32_t k) {
   GreedyShape sh{};
   if (greedy_shape(g, r, flags, &sh) != GEDWALK_OK) return 0;
@@ -83,7 +95,7 @@ int64_t maximize_footprint(const Graph& g, const Resolved& r, int32_t flags, int
   // (directed: the sums of the walk totals; adaptive: the final group is scored)
   if (g.directed) b += static_cast<int64_t>(std::max(std::max(g.plan.num_slots, g.plan_r.num_slots), 1)) * 2 * 8;
   if (g.directed && (flags & GEDWALK_ADAPTIVE_L)) b += 2 * n * 2 * es;
-  return b + 4 * static_cast<int64_t>(k);
+  return b + 4 * (static_cast<int64_t>(k) + 1);
 }
 
 namespace {
@@ -376,7 +388,7 @@ gedwalk_status maximize_impl(Graph& g, Workspace& ws, int32_t k, const Resolved&
   p.eps_sep = r.eps;
   if (p.adaptive()) {
     GW_TRY(bound_coef(g, r.alpha, r.bound_kind, r.stream, &p.coef));
-    GW_TRY(ensure_totals(g, r.alpha, p.shape.ell_max + 1, r.stream));
+    GW_TRY(ensure_run_tables(g, ws, r, p.shape, flags));
     std::shared_lock<std::shared_mutex> rl(g.tt_lock);
     if (g.tt_alpha != r.alpha || static_cast<int32_t>(g.Wa.size()) < p.shape.ell_max + 1)
       return fail(GEDWALK_ERR_INVALID, "the walk-total table was replaced for another alpha during the call");

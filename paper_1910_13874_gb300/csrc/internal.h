@@ -341,6 +341,9 @@ struct GreedyShape {
   int32_t cols_max;   // widest sweep of the run (walk vectors are sized for it)
 };
 gedwalk_status greedy_shape(const Graph& g, const Resolved& r, int32_t flags, GreedyShape* out);
+// The walk-total tables of the graph that a maximisation reads at any of its walk lengths, where the bound
+// applies to its alpha (its own totals serve otherwise): made once, before it starts.
+gedwalk_status ensure_run_tables(Graph& g, Workspace& ws, const Resolved& r, const GreedyShape& sh, int32_t flags);
 // Device bytes a maximisation of k vertices with this configuration needs in its workspace.
 int64_t maximize_footprint(const Graph& g, const Resolved& r, int32_t flags, int32_t k);
 // Device bytes a batched scoring of `groups` groups with `members` members needs in its workspace.

@@ -391,6 +391,7 @@ gedwalk_status gedwalk_serve_submit(gedwalk_server_t h, int32_t graph, int32_t k
       GW_TRY(resolve(g, &p, eps, &q->r));
       GreedyShape sh{};
       GW_TRY(greedy_shape(g, q->r, q->flags, &sh));  // rejects bad lookahead / spec_cols now
+      GW_TRY(ensure_run_tables(g, g.ws, q->r, sh, q->flags));  // the graph's, not the request's
       q->need = maximize_footprint(g, q->r, q->flags, q->k);
     }
   }
