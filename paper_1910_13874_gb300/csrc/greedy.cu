@@ -66,6 +66,10 @@ gedwalk_status greedy_shape(const Graph& g, const Resolved& r, int32_t flags, Gr
   // Candidate batches run when the evaluated guess is not certified: as wide as the chains.
   sh.cols_cand = run_width(g, tab_L, 8, r.fp64);
   sh.cols_all = run_width(g, tab_L, r.fp64 ? 8 : 16, r.fp64);
+  if (r.max_cols > 0) {
+    sh.levels = std::min(sh.levels, r.max_cols - 1);
+    for (int32_t* c : {&sh.cols_fused, &sh.cols_cand, &sh.cols_all}) *c = std::min(*c, r.max_cols);
+  }
   sh.tab_L = tab_L;
   sh.cols_max = std::max({sh.levels > 1 ? sh.levels + 1 : sh.cols_fused, sh.cols_cand,
                           (flags & GEDWALK_GAINS_ALL) ? sh.cols_all : 0, 2});
@@ -394,10 +398,18 @@ gedwalk_status maximize_impl(Graph& g, Workspace& ws, int32_t k, const Resolved&
       return fail(GEDWALK_ERR_INVALID, "the walk-total table was replaced for another alpha during the call");
     p.Wa.assign(g.Wa.begin(), g.Wa.begin() + p.shape.ell_max + 1);
   }
-  ws.st_evals = ws.st_batches = ws.st_sweeps = ws.st_spec_miss = ws.st_sep_fail = 0;
-  ws.st_ell.clear();
   std::vector<int32_t> S_all;
-  GW_TRY(maximize_runs(g, ws, r, p, init_int, group, gains, &S_all));
+  for (;;) {
+    ws.st_evals = ws.st_batches = ws.st_sweeps = ws.st_spec_miss = ws.st_sep_fail = 0;
+    ws.st_ell.clear();
+    const gedwalk_status st = maximize_runs(g, ws, r, p, init_int, group, gains, &S_all);
+    if (st == GEDWALK_OK) break;
+    if (st != GEDWALK_ERR_OOM || p.shape.cols_max <= 2) return st;
+    // the device cannot hold rows this wide: again with half the columns (the results do not depend on them)
+    GW_CUDA(cudaStreamSynchronize(r.stream));
+    r.max_cols = p.shape.cols_max / 2;
+    GW_TRY(greedy_shape(g, r, flags, &p.shape));
+  }
   if (score) {
     // GED_{<=L} of the final group. From an empty start it is the sum of the picks' exact gains
     // g_L(S_j, c_j) = GED_{<=L}(S_j + c_j) - GED_{<=L}(S_j), telescoping from GED_{<=L}(empty) = 0;
@@ -421,7 +433,7 @@ gedwalk_status gains_impl(Graph& g, Workspace& ws, const std::vector<int32_t>& S
   GW_TRY(greedy_stream(ws, r_in.stream, &r.stream));
   SyncOnError guard{r.stream};
   cudaStream_t s = r.stream;
-  const int cols_all = run_width(g, r.L, r.fp64 ? 8 : 16, r.fp64);
+  int cols_all = run_width(g, r.L, r.fp64 ? 8 : 16, r.fp64);
   std::vector<char> inS(g.n, 0);
   for (int32_t v : S_int) inS[v] = 1;
   for (int32_t v = 0; v < g.n; ++v) gains_caller[v] = 0.0;  // an isolated vertex gains nothing
@@ -433,7 +445,12 @@ gedwalk_status gains_impl(Graph& g, Workspace& ws, const std::vector<int32_t>& S
     return GEDWALK_OK;
   }
   RunEngine eng(g, ws, r, s);
-  GW_TRY(eng.setup(r.L, cols_all, false, S_int));
+  for (;; cols_all /= 2) {  // narrower where the device cannot hold the vectors
+    const gedwalk_status st = eng.setup(r.L, cols_all, false, S_int);
+    if (st == GEDWALK_OK) break;
+    if (st != GEDWALK_ERR_OOM || cols_all <= 2) return st;
+    GW_CUDA(cudaStreamSynchronize(s));
+  }
   GW_TRY(eng.set_length(r.L, false));
   std::vector<int32_t> batch;
   for (int32_t v = 0; v <= g.n_active; ++v) {

@@ -327,6 +327,7 @@ struct Resolved {
   int32_t bound_kind = 0;  // GEDWALK_BOUND_COMBINATORIAL or GEDWALK_BOUND_SPECTRAL
   int32_t lookahead = 0;   // gedwalk_params.lookahead (0 = default)
   int32_t spec_cols = 0;   // gedwalk_params.spec_cols (0 = default)
+  int32_t max_cols = 0;    // maximize: columns a run may have at most (0: as many as it likes); little memory
 };
 
 // The configuration of one greedy maximisation (sweep widths, lookahead levels, table rows),
@@ -346,8 +347,9 @@ gedwalk_status greedy_shape(const Graph& g, const Resolved& r, int32_t flags, Gr
 gedwalk_status ensure_run_tables(Graph& g, Workspace& ws, const Resolved& r, const GreedyShape& sh, int32_t flags);
 // Device bytes a maximisation of k vertices with this configuration needs in its workspace.
 int64_t maximize_footprint(const Graph& g, const Resolved& r, int32_t flags, int32_t k);
-// Device bytes a batched scoring of `groups` groups with `members` members needs in its workspace.
-int64_t score_batch_footprint(const Graph& g, int64_t members, int32_t groups);
+// Device bytes a batched scoring of `groups` groups with `members` members by walks up to L needs in its
+// workspace.
+int64_t score_batch_footprint(const Graph& g, int64_t members, int32_t groups, int32_t L);
 // Resolves alpha (0 -> default), L (from epsilon unless forced) for a given epsilon.
 gedwalk_status resolve(Graph& g, const gedwalk_params* p, double eps_override, Resolved* r);
 // Rows of the walk-total table that give W_0..W_{lengths-1}: the walks of length a + b number

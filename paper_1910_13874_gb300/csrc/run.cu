@@ -1299,11 +1299,15 @@ gedwalk_status score_run(Graph& g, Workspace& ws, const std::vector<int32_t>& S_
   const int32_t H = (r.L + 1) / 2;
   const size_t row = static_cast<size_t>(g.n_active) * 2;
   GW_TRY(ensure_run_io(ws));
-  // x_1 .. x_H, or, where they would outgrow kWideBytes, a ring of the last ones and the sum of the
-  // older; x_0 (weighted) sits where x_ring goes later
-  const int32_t ring = static_cast<int32_t>(std::max<int64_t>(
+  // x_1 .. x_H, or, where they would outgrow kWideBytes or the device, a ring of the last ones (three at
+  // least) and the sum of the older; x_0 (weighted) sits where x_ring goes later
+  int32_t ring = static_cast<int32_t>(std::max<int64_t>(
       3, std::min<int64_t>(H + (g.weighted ? 1 : 0), kWideBytes / std::max<int64_t>(static_cast<int64_t>(row * es), 1))));
-  GW_TRY(ws.xs.ensure(row * es * (ring + (H > ring ? 2 : 0)), s));
+  for (;; ring = std::max(3, ring / 2)) {
+    const gedwalk_status st = ws.xs.ensure(row * es * (ring + (H > ring ? 2 : 0)), s);
+    if (st == GEDWALK_OK) break;
+    if (st != GEDWALK_ERR_OOM || ring <= 3) return st;
+  }
   GW_TRY(ws.cnt.ensure(n * sizeof(int32_t), s));
   const size_t words = (n + 31) / 32;
   GW_TRY(ws.mask.ensure(words * 4, s));
@@ -1383,7 +1387,7 @@ gedwalk_status score_run(Graph& g, Workspace& ws, const std::vector<int32_t>& S_
   memcpy(&abits, &r.alpha, 8);
   auto bits = [](const void* p) { return static_cast<uint64_t>(reinterpret_cast<uintptr_t>(p)); };
   Sequence q;
-  q.key = mix_all({uint64_t(MODE_PAIR), uint64_t(fp64), uint64_t(r.L), uint64_t(items), abits, bits(&g), bits(s), bits(ws.xs.p),
+  q.key = mix_all({uint64_t(MODE_PAIR), uint64_t(fp64), uint64_t(r.L), uint64_t(items), uint64_t(ring), abits, bits(&g), bits(s), bits(ws.xs.p),
                    bits(ws.cnt.p), bits(ws.mask.p), bits(ws.parts.p), bits(ws.small.p), bits(ws.partial.p),
                    bits(ws.counters.p), bits(ws.members.p), bits(ws.run_io), bits(g.rp.p), bits(g.ci.p), bits(g.plan.units.p)});
   q.kernels = 3 + swept + (H > ring ? (H - ring - 1) / (ring - 1) + 1 : 0);

@@ -84,8 +84,8 @@ gedwalk_status greedy_stream(Workspace& ws, cudaStream_t caller, cudaStream_t* o
 void read_graph_timing(Workspace& ws);
 uint64_t mix_all(std::initializer_list<uint64_t> vs);
 
-// Stored vectors are kept to about this size: beyond it rows get narrower (fewer steps or candidates a
-// run) and scoring keeps a ring of vectors.
+// Stored vectors are kept to about this size: beyond it, and where the device cannot hold them, rows get
+// narrower (fewer steps or candidates a run) and scoring keeps a ring of vectors.
 constexpr int64_t kWideBytes = int64_t(32) << 30;
 // The widest rows of at most `cols` columns, at least 2, whose ceil(L/2) stored vectors stay below it.
 inline int run_width(const Graph& g, int32_t L, int cols, bool fp64) {

@@ -12,13 +12,14 @@
 namespace gw {
 namespace {
 
-// X0[v] = (h_0(v), m_0(v)) = (1_S(v), 1_{V\S}(v))
+// X0[v] = (h_0(v), m_0(v)) = (1_S(v), 1_{V\S}(v)), times s on a weighted graph
 template <typename T>
-__global__ void init_two_state(T* __restrict__ X, const uint32_t* __restrict__ mask, int32_t n) {
+__global__ void init_two_state(T* __restrict__ X, const uint32_t* __restrict__ mask, int32_t n, const T* __restrict__ rs) {
   for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
     const bool inS = (mask[v >> 5] >> (v & 31)) & 1u;
-    X[2 * static_cast<size_t>(v)] = inS ? T(1) : T(0);
-    X[2 * static_cast<size_t>(v) + 1] = inS ? T(0) : T(1);
+    const T x = rs ? rs[v] : T(1);
+    X[2 * static_cast<size_t>(v)] = inS ? x : T(0);
+    X[2 * static_cast<size_t>(v) + 1] = inS ? T(0) : x;
   }
 }
 
@@ -156,7 +157,7 @@ __global__ void batch_own(float* __restrict__ X, int32_t cols, const int32_t* __
 
 // The stored vectors of a block: x_t sits at slot (t - 1) % slots; V holds the sum of those already
 // folded (walk lengths 1..folded). Five slots hold the walks of L <= 10; two where five would outgrow
-// kWideBytes.
+// kWideBytes or the device.
 constexpr int kBatchRing = 5;
 struct BatchVecs {
   const float* ring;
@@ -294,7 +295,11 @@ gedwalk_status score_one(Graph& g, Workspace& ws, const std::vector<int32_t>& S_
     *score = 0.0;
     return GEDWALK_OK;
   }
-  if (!g.directed) return score_run(g, ws, S_int, r, score);
+  if (!g.directed) {
+    const gedwalk_status st = score_run(g, ws, S_int, r, score);
+    if (st != GEDWALK_ERR_OOM) return st;
+    // no memory for the half-length run's five vectors: sweeps of the full length keep two
+  }
   StreamGuard guard{s};
   const size_t es = r.fp64 ? 8 : 4;
   const size_t vbytes = static_cast<size_t>(g.n) * 2 * es;
@@ -304,9 +309,11 @@ gedwalk_status score_one(Graph& g, Workspace& ws, const std::vector<int32_t>& S_
   GW_TRY(ws.small.ensure(64, s));
   GW_TRY(upload_mask(g, ws, S_int, s));
   if (r.fp64)
-    init_two_state<double><<<blocks_for(g.n), 256, 0, s>>>(ws.x0.as<double>(), ws.mask.as<uint32_t>(), g.n);
+    init_two_state<double><<<blocks_for(g.n), 256, 0, s>>>(ws.x0.as<double>(), ws.mask.as<uint32_t>(), g.n,
+                                                           g.weighted ? g.rs_d.as<double>() : nullptr);
   else
-    init_two_state<float><<<blocks_for(g.n), 256, 0, s>>>(ws.x0.as<float>(), ws.mask.as<uint32_t>(), g.n);
+    init_two_state<float><<<blocks_for(g.n), 256, 0, s>>>(ws.x0.as<float>(), ws.mask.as<uint32_t>(), g.n,
+                                                          g.weighted ? g.rs_f.as<float>() : nullptr);
   GW_KCHECK();
   SweepArgs a = base_args(g, ws);
   a.alpha = r.alpha;
@@ -373,18 +380,24 @@ gedwalk_status autotune_batch(Graph& g, Workspace& ws, const Resolved& r) {
   return GEDWALK_OK;
 }
 
+// Vectors of a batch's ring, and those it stores in all: x_1 .. x_H in the ring (x_0 of a weighted graph in
+// its last slot); beyond the ring the oldest are folded into two vectors (hi, lo) behind it.
 static int batch_ring(const Graph& g, int64_t C) {
   return static_cast<int64_t>(g.n_active) * C * 4 * kBatchRing > kWideBytes ? 2 : kBatchRing;
 }
+static int batch_stored(const Graph& g, int32_t L, int ring) {
+  const int H = (L + 1) / 2;
+  return H > ring ? ring + 2 : g.weighted ? ring : H;
+}
 
-int64_t score_batch_footprint(const Graph& g, int64_t members, int32_t groups) {
+int64_t score_batch_footprint(const Graph& g, int64_t members, int32_t groups, int32_t L) {
   const int64_t C = g.batch_cols > 0 ? g.batch_cols : 32;  // before tuning: the widest width tried
   const int64_t n = g.n;
   int64_t b = members * (4 + 4 + 8) + static_cast<int64_t>(groups + 1) * 4 + 256;  // members, columns, sums
   b += static_cast<int64_t>(std::max(g.plan.num_slices, 1)) * C * 4 + std::max(g.plan.num_heavy, 1) * 4;
   b += static_cast<int64_t>(groups) * 8 + 64 + (n + 31) / 32 * 4;
   if (!g.directed) {
-    b += static_cast<int64_t>(g.n_active) * C * 4 * (batch_ring(g, C) + 2);  // the stored vectors, their sum's parts
+    b += static_cast<int64_t>(g.n_active) * C * 4 * batch_stored(g, L, batch_ring(g, C));
     b += n * (g.weighted ? 32 : 16) + kBatchMeetBlocks * C * 8;
     return b;
   }
@@ -395,7 +408,7 @@ int64_t score_batch_footprint(const Graph& g, int64_t members, int32_t groups) {
 
 // The blocks of an undirected graph's batch; the members (rows, columns) are on the device, the scores
 // go to ws.small. The table holds rows 0..H (the caller keeps its lock).
-static gedwalk_status batch_runs(Graph& g, Workspace& ws, int C, const int32_t* offsets, int32_t G, const int32_t* mrow,
+static gedwalk_status batch_runs(Graph& g, Workspace& ws, int C, int ring_slots, const int32_t* offsets, int32_t G, const int32_t* mrow,
                                  const int32_t* mcol, const Resolved& r, cudaStream_t s) {
   if (g.n_active == 0) {  // no edges, no walks
     GW_CUDA(cudaMemsetAsync(ws.small.p, 0, sizeof(double) * G, s));
@@ -403,10 +416,6 @@ static gedwalk_status batch_runs(Graph& g, Workspace& ws, int C, const int32_t* 
   }
   const int32_t L = r.L, H = (L + 1) / 2;
   const int64_t vec = static_cast<int64_t>(g.n_active) * C;
-  // x_1 .. x_H in a ring; beyond that the oldest are folded into two vectors (hi, lo) behind it
-  const int ring_slots = batch_ring(g, C);
-  const int stored = H > ring_slots ? ring_slots + 2 : g.weighted ? ring_slots : H;
-  GW_TRY(ws.xs.ensure(static_cast<size_t>(vec) * stored * sizeof(float), s));
   GW_TRY(ws.tail.ensure(static_cast<size_t>(g.n) * sizeof(BatchRow), s));
   if (g.weighted) GW_TRY(ws.bound.ensure(static_cast<size_t>(g.n) * sizeof(BatchScale), s));
   const size_t nz_bytes = (static_cast<size_t>(g.n) + 31) / 32 * sizeof(uint32_t);
@@ -474,7 +483,7 @@ static gedwalk_status batch_runs(Graph& g, Workspace& ws, int C, const int32_t* 
     else                                                                                                                \
       batch_meet<CC, false><<<meet, kThreads, 0, s>>>(b, L & 1, g.n_active, row, nullptr, part, done, g1 - g0, out);    \
   }
-    GW_MEET(8) GW_MEET(16) GW_MEET(32) GW_MEET(64)
+    GW_MEET(4) GW_MEET(8) GW_MEET(16) GW_MEET(32) GW_MEET(64)
 #undef GW_MEET
     GW_KCHECK();
   }
@@ -490,7 +499,20 @@ gedwalk_status score_batch_impl(Graph& g, Workspace& ws, const int32_t* offsets,
   std::shared_lock<std::shared_mutex> rl(g.tt_lock);
   if (g.tt_alpha != r.alpha || g.tt_rows < walk_rows(g, r.L + 1) || g.batch_cols <= 0)
     return fail(GEDWALK_ERR_INVALID, "walk-total table or column width not prepared for this batch");
-  const int C = g.batch_cols;
+  int C = g.batch_cols;
+  int ring = 0;
+  if (!g.directed) {
+    // the stored vectors, with a shorter ring and then narrower blocks where the device cannot hold them
+    // (at four columns as much as two vectors of eight, the least that full-length sweeps would take)
+    for (ring = batch_ring(g, C);;) {
+      const size_t vec = static_cast<size_t>(g.n_active) * C * sizeof(float);
+      const gedwalk_status st = ws.xs.ensure(vec * batch_stored(g, r.L, ring), s);
+      if (st == GEDWALK_OK) break;
+      if (st != GEDWALK_ERR_OOM || (ring == 2 && C == 4)) return st;
+      if (ring > 2) ring = 2;
+      else C /= 2;
+    }
+  }
   const int64_t total = offsets[G];
   // members: row (internal id), column within its block, accumulator; group offsets
   const size_t mbytes = static_cast<size_t>(total) * (4 + 4 + 8) + static_cast<size_t>(G + 1) * 4 + 256;
@@ -512,7 +534,7 @@ gedwalk_status score_batch_impl(Graph& g, Workspace& ws, const int32_t* offsets,
   GW_TRY(ws.small.ensure(static_cast<size_t>(G) * sizeof(double) + 64, s));
   const double* T = g.ttab.as<double>();
   if (!g.directed) {
-    GW_TRY(batch_runs(g, ws, C, offsets, G, mrow, mcol, r, s));
+    GW_TRY(batch_runs(g, ws, C, ring, offsets, G, mrow, mcol, r, s));
     GW_CUDA(cudaMemcpyAsync(ws.pinned, ws.small.p, sizeof(double) * G, cudaMemcpyDeviceToHost, s));
     GW_CUDA(cudaStreamSynchronize(s));
     memcpy(scores, ws.pinned, sizeof(double) * G);

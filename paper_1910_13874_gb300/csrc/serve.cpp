@@ -45,6 +45,9 @@ struct Request {
   int32_t flags = 0;
   Resolved r{};
   int64_t need = 0;  // maximise: the footprint of its run
+  // maximise: {widest rows, footprint}, the default first and then narrower ones, which take less memory and
+  // more runs (the results are the same)
+  std::vector<std::pair<int32_t, int64_t>> widths;
   bool admitted = false;
   bool waited = false;  // not admitted by the call that submitted it
   Clock::time_point t_submit, t_done;
@@ -62,6 +65,7 @@ struct Lane {  // one per graph: batched scoring
   std::deque<ReqPtr> queue;
   int64_t q_members = 0;     // members of the queued requests
   int32_t q_groups = 0;      // queued requests
+  int32_t q_L = 0;           // their longest walk length
   bool busy = false;
   int64_t need_running = 0;  // footprint of the batch being scored
   int64_t held = 0;          // device bytes of the workspace when it was last idle
@@ -104,7 +108,7 @@ struct Server {
     int64_t c = l.held;
     if (l.busy) c = std::max(c, l.need_running);
     if (l.q_groups > 0)
-      c = std::max(c, score_batch_footprint(*graphs[l.graph], l.q_members, std::min(l.q_groups, max_batch)));
+      c = std::max(c, score_batch_footprint(*graphs[l.graph], l.q_members, std::min(l.q_groups, max_batch), l.q_L));
     return c;
   }
   static int64_t worker_charge(const Worker& w) { return w.job ? std::max(w.held, w.job->need) : w.held; }
@@ -161,14 +165,18 @@ struct Server {
       Lane& l = *lanes[q->graph];
       const int64_t members = static_cast<int64_t>(q->S.size());
       const int64_t before = lane_charge(l);
+      const int32_t L_before = l.q_L;
       l.q_members += members;  // the lane's charge with q queued
       ++l.q_groups;
+      l.q_L = std::max(l.q_L, q->r.L);
       const int64_t delta = lane_charge(l) - before;
       l.q_members -= members;
       --l.q_groups;
+      l.q_L = L_before;
       if (!make_room(delta, &l, nullptr) && total() - lane_charge(l) > 0) break;  // wait
       l.q_members += members;
       ++l.q_groups;
+      l.q_L = std::max(l.q_L, q->r.L);
       pending.pop_front();
       mark_admitted(q, q.get() == submitting);
       l.queue.push_back(q);
@@ -176,19 +184,26 @@ struct Server {
     }
     while (!pending_max.empty()) {  // then maximise requests, one per free worker
       ReqPtr q = pending_max.front();
-      Worker* pick = nullptr;  // a free worker: the smallest held bytes that fit q, else the largest
-      for (auto& w : workers) {
-        if (w->job) continue;
-        if (!pick) {
-          pick = w.get();
-          continue;
+      Worker* pick = nullptr;
+      bool admit = false;
+      for (const auto& width : q->widths) {
+        q->r.max_cols = width.first;
+        q->need = width.second;
+        pick = nullptr;  // a free worker: the smallest held bytes that fit q, else the largest
+        for (auto& w : workers) {
+          if (w->job) continue;
+          if (!pick) {
+            pick = w.get();
+            continue;
+          }
+          const bool fits = w->held >= q->need, pfits = pick->held >= q->need;
+          if ((fits && (!pfits || w->held < pick->held)) || (!fits && !pfits && w->held > pick->held)) pick = w.get();
         }
-        const bool fits = w->held >= q->need, pfits = pick->held >= q->need;
-        if ((fits && (!pfits || w->held < pick->held)) || (!fits && !pfits && w->held > pick->held)) pick = w.get();
+        if (!pick) break;
+        admit = make_room(std::max(pick->held, q->need) - pick->held, nullptr, pick);
+        if (admit) break;
       }
-      if (!pick) break;
-      const int64_t delta = std::max(pick->held, q->need) - pick->held;
-      if (!make_room(delta, nullptr, pick) && total() - pick->held > 0) break;
+      if (!pick || (!admit && total() - pick->held > 0)) break;
       pending_max.pop_front();
       mark_admitted(q, q.get() == submitting);
       pick->job = q;
@@ -227,7 +242,9 @@ struct Server {
         }
         lane.q_members -= members;
         lane.q_groups -= static_cast<int32_t>(batch.size());
-        lane.need_running = score_batch_footprint(g, members, static_cast<int32_t>(batch.size()));
+        lane.q_L = 0;
+        for (const ReqPtr& q : lane.queue) lane.q_L = std::max(lane.q_L, q->r.L);
+        lane.need_running = score_batch_footprint(g, members, static_cast<int32_t>(batch.size()), first->r.L);
         lane.busy = true;
       }
       std::vector<int32_t> off(1, 0), mem;
@@ -392,7 +409,15 @@ gedwalk_status gedwalk_serve_submit(gedwalk_server_t h, int32_t graph, int32_t k
       GreedyShape sh{};
       GW_TRY(greedy_shape(g, q->r, q->flags, &sh));  // rejects bad lookahead / spec_cols now
       GW_TRY(ensure_run_tables(g, g.ws, q->r, sh, q->flags));  // the graph's, not the request's
-      q->need = maximize_footprint(g, q->r, q->flags, q->k);
+      q->widths.emplace_back(0, maximize_footprint(g, q->r, q->flags, q->k));
+      // Rows of eight columns took the place of a table and narrow sweeps in directed, stochastic and
+      // l-doubling runs, four times the memory: they may run narrower rather than wait for it.
+      if (g.directed || (q->flags & (GEDWALK_STOCHASTIC | GEDWALK_ADAPTIVE_L | GEDWALK_GAINS_ALL)))
+        for (int32_t cols = sh.cols_max / 2; cols >= 2; cols /= 2) {
+          Resolved narrow = q->r;
+          narrow.max_cols = cols;
+          q->widths.emplace_back(cols, maximize_footprint(g, narrow, q->flags, q->k));
+        }
     }
   }
   std::lock_guard<std::mutex> lk(srv->mu);
