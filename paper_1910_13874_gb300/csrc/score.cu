@@ -394,15 +394,17 @@ int64_t score_batch_footprint(const Graph& g, int64_t members, int32_t groups, i
   const int64_t C = g.batch_cols > 0 ? g.batch_cols : 32;  // before tuning: the widest width tried
   const int64_t n = g.n;
   int64_t b = members * (4 + 4 + 8) + static_cast<int64_t>(groups + 1) * 4 + 256;  // members, columns, sums
-  b += static_cast<int64_t>(std::max(g.plan.num_slices, 1)) * C * 4 + std::max(g.plan.num_heavy, 1) * 4;
+  // the scratch fits the larger of a directed graph's two plans
+  auto larger = [&](int32_t a, int32_t rev) { return static_cast<int64_t>(std::max({a, g.directed ? rev : 0, 1})); };
+  b += larger(g.plan.num_slices, g.plan_r.num_slices) * C * 4 + larger(g.plan.num_heavy, g.plan_r.num_heavy) * 4;
   b += static_cast<int64_t>(groups) * 8 + 64 + (n + 31) / 32 * 4;
   if (!g.directed) {
     b += static_cast<int64_t>(g.n_active) * C * 4 * batch_stored(g, L, batch_ring(g, C));
-    b += n * (g.weighted ? 32 : 16) + kBatchMeetBlocks * C * 8;
+    b += n * (g.weighted ? 32 : 16) + (kBatchMeetBlocks * C + 1) * 8;
     return b;
   }
   b += 2 * n * C * 4;  // walk vectors x0, x1
-  b += static_cast<int64_t>(std::max(g.plan.num_slots, 1)) * C * 8 + C * kReduceParts * 8;
+  b += larger(g.plan.num_slots, g.plan_r.num_slots) * C * 8 + C * kReduceParts * 8;
   return b;
 }
 

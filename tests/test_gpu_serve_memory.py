@@ -54,3 +54,26 @@ def test_charge_covers_what_a_maximisation_allocates(cuda_device, directed, kw):
         gedwalk._torch_hooks = None
         gedwalk.use_torch_allocator()
     assert 0 < state["peak"] <= charged
+
+
+@pytest.mark.parametrize("kind", ["plain", "weighted", "directed"])
+@pytest.mark.parametrize("L", [4, 9, 15])
+def test_charge_covers_what_a_scoring_allocates(cuda_device, kind, L):
+    from paper_1910_13874_gb300 import gedwalk
+
+    state = {"blocks": {}, "now": 0, "peak": 0}
+    counting_allocator(state)
+    try:
+        G = gedwalk.Graph.from_host(gg.rmat(13, 8, seed=3, directed=kind == "directed"), directed=kind == "directed",
+                                    weighted=kind == "weighted")
+        srv = gedwalk.Server([G], mem_budget=1 << 34)
+        state.update(now=0, peak=0)
+        srv.poll(srv.submit_score(0, [1, 2, 3, 100], L=L))
+        charged = srv.stats()["peak_bytes"]
+        srv.close()
+        G.free()
+    finally:
+        gedwalk.load().gedwalk_set_allocator(gedwalk._ALLOC_FN(), gedwalk._FREE_FN(), None)
+        gedwalk._torch_hooks = None
+        gedwalk.use_torch_allocator()
+    assert 0 < state["peak"] <= charged
