@@ -1547,6 +1547,7 @@ static gedwalk_status upload_impl(const int32_t* row_ptr, const int32_t* col_idx
     GW_CUDA(cudaMemcpy(&rdmax, rdeg.as<int32_t>() + n, sizeof rdmax, cudaMemcpyDeviceToHost));
   }
   g->dmax = dmax;
+  g->rdmax = rdmax;
   // W_{l+1} <= d W_l with d = d_max; on a digraph an l-walk extends at its end along at most
   // max out-degree arcs and at its start along at most max in-degree arcs, so the smaller counts
   g->delta = directed ? std::min(dmax, rdmax) : dmax;

@@ -186,6 +186,7 @@ struct Graph {
   int32_t n = 0;
   int64_t nnz = 0;
   int32_t dmax = 0;
+  int32_t rdmax = 0;        // directed: the largest reverse degree
   int32_t n_active = 0;     // rows with at least one entry; isolated rows are [n_active, n)
   double alpha_default = 0;
   // Weighted walks (Section 5.4) with vertex-separable weights w(v,u) = s_v s_u: rs_* hold s by

@@ -169,9 +169,42 @@ __device__ __forceinline__ void join_set(const int32_t* __restrict__ list, int32
   }
 }
 
-// count: list[-1] when negative (a captured launch).
+// The same for a whole group, which may be half of the graph. With blockIdx.y = 0 a warp takes a member at a
+// time and up to kJoinRow entries of its row; the other slices of the grid (where rows are longer than that)
+// look through 32 members at a time for the rest of hubs' rows, which they share. A block per member took
+// 30 ms for half of R-MAT scale 20, the sweeps 0.35. count: list[-1] when negative (a captured launch).
+constexpr int kJoinRow = 256;
 __global__ void join_kernel(const int32_t* __restrict__ list, int32_t count, const Rows g, uint32_t* __restrict__ mask) {
-  join_set(list, count >= 0 ? count : list[-1], g, mask);
+  if (count < 0) count = list[-1];
+  const int lane = threadIdx.x & 31;
+  const int32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, warps = (gridDim.x * blockDim.x) >> 5;
+  if (blockIdx.y == 0) {
+    for (int32_t i = warp; i < count; i += warps) {
+      const int32_t v = list[i];
+      if (lane == 0) atomicOr(mask + (v >> 5), 1u << (v & 31));
+      for (int o = 0; o <= g.directed; ++o) {
+        const int r = g.directed ? 1 - o : 0;  // v is in row o of u where u is in v's other row
+        const int64_t e0 = g.rp[r][v], e1 = min(static_cast<int64_t>(g.rp[r][v + 1]), e0 + kJoinRow);
+        for (int64_t e = e0 + lane; e < e1; e += 32) atomicAdd(g.cnt[o] + g.ci[r][e], 1);
+      }
+    }
+    return;
+  }
+  const int slice = static_cast<int>(blockIdx.y) - 1, slices = static_cast<int>(gridDim.y) - 1;
+  for (int64_t i0 = 32 * static_cast<int64_t>(warp); i0 < count; i0 += 32 * static_cast<int64_t>(warps)) {
+    const int32_t mine = i0 + lane < count ? list[i0 + lane] : -1;
+    for (int o = 0; o <= g.directed; ++o) {
+      const int r = g.directed ? 1 - o : 0;
+      const bool hub = mine >= 0 && g.rp[r][mine + 1] - g.rp[r][mine] > kJoinRow;
+      for (unsigned m = __ballot_sync(kFullMask, hub); m; m &= m - 1) {
+        const int32_t v = __shfl_sync(kFullMask, mine, __ffs(m) - 1);
+        const int64_t e1 = g.rp[r][v + 1];
+#pragma unroll 4
+        for (int64_t e = static_cast<int64_t>(g.rp[r][v]) + kJoinRow + slice * 32 + lane; e < e1; e += 32 * slices)
+          atomicAdd(g.cnt[o] + g.ci[r][e], 1);
+      }
+    }
+  }
 }
 
 // Opens a run: the vertices that joined S, the exact gains known on the host, the pass's counters.
@@ -948,9 +981,18 @@ __global__ void pair_fold(T* __restrict__ xs, int64_t stride, int32_t ring, int3
 }
 
 int grid_of(int64_t n) { return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 16))); }
+// Blocks of join_kernel for a group of `count`, a power of two: few captured shapes.
+dim3 join_grid(int64_t count, int32_t longest) {
+  int x = 1;
+  while (x * 8 < count && x < 2048) x *= 2;
+  return dim3(x, longest > kJoinRow ? kChunks : 1);
+}
 int meet_grid(int32_t n_scan) {
   return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(kMeetBlocks, (int64_t(n_scan) + kThreads - 1) / kThreads)));
 }
+
+// The longest row of a graph, in either orientation.
+int32_t longest_row(const Graph& g) { return std::max(g.dmax, g.rdmax); }
 
 Rows rows_of(const Graph& g, const Workspace& ws) {
   Rows r{};
@@ -1088,9 +1130,8 @@ gedwalk_status RunEngine::setup(int32_t L_max, int cols, bool select, const std:
     int32_t* st = static_cast<int32_t*>(ws.pinned);
     std::copy(init.begin(), init.end(), st);
     GW_CUDA(cudaMemcpyAsync(list.p, st, init.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    const int items = static_cast<int>(std::min<size_t>(init.size(), 4096));
-    join_kernel<<<dim3(kChunks, items), 256, 0, s>>>(list.as<int32_t>(), static_cast<int32_t>(init.size()),
-                                                     rows_of(g, ws), ws.mask.as<uint32_t>());
+    join_kernel<<<join_grid(init.size(), longest_row(g)), 256, 0, s>>>(list.as<int32_t>(), static_cast<int32_t>(init.size()),
+                                                                      rows_of(g, ws), ws.mask.as<uint32_t>());
     GW_KCHECK();
   }
   return GEDWALK_OK;
@@ -1153,7 +1194,8 @@ gedwalk_status RunEngine::push_added() {
   while (added.size() > kRunCols) {
     std::copy(added.end() - kRunCols, added.end(), in->added);
     GW_CUDA(cudaMemcpyAsync(d->in.added, in->added, sizeof in->added, cudaMemcpyHostToDevice, s));
-    join_kernel<<<dim3(kChunks, kRunCols), 256, 0, s>>>(d->in.added, kRunCols, rows_of(g, ws), ws.mask.as<uint32_t>());
+    join_kernel<<<join_grid(kRunCols, longest_row(g)), 256, 0, s>>>(d->in.added, kRunCols, rows_of(g, ws),
+                                                                   ws.mask.as<uint32_t>());
     GW_KCHECK();
     GW_CUDA(cudaStreamSynchronize(s));  // the pinned block is reused
     added.resize(added.size() - kRunCols);
@@ -1324,17 +1366,14 @@ gedwalk_status score_run(Graph& g, Workspace& ws, const std::vector<int32_t>& S_
   st[0] = count;
   std::copy(S_int.begin(), S_int.end(), st + 1);
   GW_CUDA(cudaMemcpyAsync(ws.members.p, st, (S_int.size() + 1) * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-  int items = 1;  // blocks that walk the list, a power of two: few captured shapes
-  while (items < count && items < 256) items *= 2;
-  const int chunks = g.dmax > 4096 ? kChunks : 1;
+  const dim3 join = join_grid(count, longest_row(g));
   double* d_sum = ws.small.as<double>();
   int32_t* d_done = reinterpret_cast<int32_t*>(d_sum + 1);
   double* h_sum = static_cast<double*>(ws.run_io);
   auto issue = [&](bool profile, const std::vector<cudaEvent_t>* ev) -> gedwalk_status {
     GW_CUDA(cudaMemsetAsync(ws.cnt.p, 0, n * sizeof(int32_t), s));
     GW_CUDA(cudaMemsetAsync(ws.mask.p, 0, words * 4, s));
-    join_kernel<<<dim3(chunks, items), 256, 0, s>>>(ws.members.as<int32_t>() + 1, -1, rows_of(g, ws),
-                                                    ws.mask.as<uint32_t>());
+    join_kernel<<<join, 256, 0, s>>>(ws.members.as<int32_t>() + 1, -1, rows_of(g, ws), ws.mask.as<uint32_t>());
     GW_KCHECK();
     char* xs = ws.xs.as<char>();
     char* x0 = g.weighted ? xs + row * es * (ring - 1) : xs;
@@ -1387,7 +1426,7 @@ gedwalk_status score_run(Graph& g, Workspace& ws, const std::vector<int32_t>& S_
   memcpy(&abits, &r.alpha, 8);
   auto bits = [](const void* p) { return static_cast<uint64_t>(reinterpret_cast<uintptr_t>(p)); };
   Sequence q;
-  q.key = mix_all({uint64_t(MODE_PAIR), uint64_t(fp64), uint64_t(r.L), uint64_t(items), uint64_t(ring), abits, bits(&g), bits(s), bits(ws.xs.p),
+  q.key = mix_all({uint64_t(MODE_PAIR), uint64_t(fp64), uint64_t(r.L), uint64_t(join.x), uint64_t(ring), abits, bits(&g), bits(s), bits(ws.xs.p),
                    bits(ws.cnt.p), bits(ws.mask.p), bits(ws.parts.p), bits(ws.small.p), bits(ws.partial.p),
                    bits(ws.counters.p), bits(ws.members.p), bits(ws.run_io), bits(g.rp.p), bits(g.ci.p), bits(g.plan.units.p)});
   q.kernels = 3 + swept + (H > ring ? (H - ring - 1) / (ring - 1) + 1 : 0);

@@ -185,3 +185,28 @@ def test_long_walks_are_certified(cuda_device, kw):
     ref, ref_gains, _ = oracle.greedy(g, 12, alpha, 61, "lazy")
     check_sequence(grp, gains, 1e-5, ref, ref_gains, *oracle_greedy_checker(oracle, g, alpha, 61))
     G.free()
+
+
+@pytest.mark.parametrize("directed", [False, True])
+@pytest.mark.parametrize("size", [1, 7, 9, 2000])
+def test_groups_of_every_size(cuda_device, directed, size):
+    # one warp per member and more slices for the rows above 256 entries: a hub of 2500, groups with and
+    # without it, up to half of the graph, scored and as an init group
+    from paper_1910_13874_gb300 import gedwalk
+
+    n = 4000
+    rng = np.random.default_rng(size)
+    arcs = np.concatenate([rng.integers(0, n, size=(8 * n, 2)), [(0, v) for v in range(1, 2501)], [(v, 1) for v in range(2, 1500)]])
+    g = gg.from_arcs(n, arcs) if directed else gg.from_edges(n, arcs)
+    alpha = oracle.default_alpha(g, directed=directed)
+    G = gedwalk.Graph.from_host(g, directed=directed)
+    rest = rng.permutation(np.arange(2, n))
+    for S in (rest[:size], np.concatenate([[0, 1], rest[:size]])):
+        for _ in range(3):  # direct and captured
+            got, _, _ = G.score(S, precision="fp64", L=5)
+        assert rel(got, oracle.score(g, S, alpha, 5)) < 1e-12
+        _, gains, score, _ = G.maximize(1, precision="fp64", L=5, init=S)
+        _, ref_gains, _ = oracle.greedy(g, 1, alpha, 5, "lazy", init=list(S), directed=directed)
+        assert rel(gains[0], ref_gains[0]) < 1e-12
+        assert rel(score, oracle.score(g, S, alpha, 5) + ref_gains[0]) < 1e-12
+    G.free()
