@@ -491,8 +491,8 @@ __device__ __forceinline__ void block_levels(WarpList (&w)[NL], float* sv, int* 
 // enter any level's list: bounds fall with the level, so the first level's bound without its
 // correction, against the lowest last entry of the lists, decides. The rows come by decreasing
 // degree, so after a warp's first iteration few pass. A bound of exactly 0 matters only when every
-// bound is 0, so its vertex is recorded only while the warp's list is empty (an atomic per such row,
-// all to one address, would serialise). 279 -> 123 us (418 MB
+// bound is 0, so its vertex is recorded only while the warp's list is empty, and by one atomic per block
+// (one per row, all to one address, serialise: k = 1 on a star of 100,000 leaves, 0.44 ms). 279 -> 123 us (418 MB
 // of traffic at 3.4 TB/s, 37% of the warps resident: a row's vectors and sums take the registers); on 10^5
 // rows, where a warp has one iteration, the lists cost most (device_util.cuh): 97 -> 63 us.
 template <typename T, int C, bool CHAIN, bool SEL, bool DIR>
@@ -504,8 +504,10 @@ __global__ void __launch_bounds__(kThreads, DIR || sizeof(T) * C > 32 ? 2 : kMee
   __shared__ float sv[SEL ? NL * NW * kTopK : 1];
   __shared__ int si[SEL ? NL * NW * kTopK : 1];
   __shared__ double sg[NW][D];
+  __shared__ unsigned long long s_zero[SEL ? NL : 1];  // the block's smallest vertex with bound 0, per level
   __shared__ int is_last;
   const RunIn& in = a.d->in;
+  if (SEL && threadIdx.x < NL) s_zero[threadIdx.x] = kNoZero;
   if (threadIdx.x < D) s_cand[threadIdx.x] = in.cand[threadIdx.x];
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -734,9 +736,11 @@ __global__ void __launch_bounds__(kThreads, DIR || sizeof(T) * C > 32 ? 2 : kMee
           if (want && in.thr[d] != ~0ull) want = sample_hash(in.seed, static_cast<uint32_t>(step + d), caller) < in.thr[d];
           nsampled[d] += want;
           want = want && st.step != step + d && !(CHAIN ? s_cand[d] == v : evaluated);
-          if (want && ub == 0.0f && (empty >> d & 1u))
-            atomicMin(&a.d->out.lv[d].zero_min,
-                      (static_cast<unsigned long long>(__ldg(a.perm + v)) << 32) | static_cast<uint32_t>(v));
+          if (want && ub == 0.0f && (empty >> d & 1u)) {
+            const unsigned long long z =
+                (static_cast<unsigned long long>(__ldg(a.perm + v)) << 32) | static_cast<uint32_t>(v);
+            if (z < s_zero[d]) atomicMin(&s_zero[d], z);
+          }
           warp_list_offer(w[d], want && ub != 0.0f, ub, v, 0);
           if ((empty >> d & 1u) && __shfl_sync(kFullMask, w[d].id, 0) != INT_MAX) empty &= ~(1u << d);
           if (CHAIN && d + 1 < NL) {
@@ -783,6 +787,8 @@ __global__ void __launch_bounds__(kThreads, DIR || sizeof(T) * C > 32 ? 2 : kMee
     block_levels<NL>(w, sv, si, a.sel_v, a.sel_id);
   }
   __syncthreads();
+  if (SEL && threadIdx.x < NL && s_zero[threadIdx.x] != kNoZero)
+    atomicMin(&a.d->out.lv[threadIdx.x].zero_min, s_zero[threadIdx.x]);
   if (threadIdx.x < D) {
     double x = 0.0;
     for (int i = 0; i < NW; ++i) x += sg[i][threadIdx.x];

@@ -38,3 +38,27 @@ def test_serving_an_edgeless_graph(cuda_device):
     assert srv.poll(t, wait_us=30_000_000)["score"] == 0.0
     srv.close()
     G.free()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_zero_gains_in_the_sample_go_to_the_lowest_id(cuda_device, prec):
+    # ten stars: once the centres are taken, bounds of 0 decide, in every block of the pass, and the lowest id
+    # wins; in a sample, the leaves of an open star have equal gains (to rounding: the checker allows any of
+    # them) and those of a taken one 0
+    import oracle
+    from seqcheck import check_sequence, oracle_stochastic_checker
+    from paper_1910_13874_gb300 import gedwalk
+
+    leaves, stars = 400, 10
+    c = np.arange(stars) * (leaves + 1)
+    e = np.concatenate([np.stack([np.full(leaves, x), x + 1 + np.arange(leaves)], 1) for x in c])
+    g = gg.from_edges(stars * (leaves + 1), e)
+    alpha = oracle.default_alpha(g)
+    G = gedwalk.Graph.from_host(g)
+    grp, gains, _, _ = G.maximize(16, precision=prec, L=6)
+    assert sorted(grp[:10]) == list(c) and list(grp[10:]) == [1, 2, 3, 4, 5, 6] and not np.any(gains[10:])
+    k, eta, tol = 60, 0.2, {"fp64": 1e-12, "fp32": 1e-5}[prec]
+    grp, gains, _, _ = G.maximize(k, precision=prec, L=4, stochastic=True, eta=eta, seed=3)
+    ref, ref_gains, _ = oracle.greedy_stochastic(g, k, alpha, 4, eta, 3)
+    check_sequence(grp, gains, tol, ref, ref_gains, *oracle_stochastic_checker(oracle, g, alpha, 4, k, eta, 3))
+    G.free()
