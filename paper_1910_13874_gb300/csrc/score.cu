@@ -106,22 +106,41 @@ __global__ void batch_totals(const double* __restrict__ T, int64_t n, int32_t n_
   }
 }
 
-// |N(v) cap S_j| outside the groups, as whole numbers in X's cells, and its rows' bits in nz: one warp per
-// member, gridDim.y warps on a hub's. batch_count_scale makes them h_1 = alpha |N(v) cap S_j|, rounded once
-// (adding alpha up in FP32 drifts with the count: 2.7e-4 of the score on a star of 100,000 leaves).
+// |N(v) cap S_j| outside the groups, as whole numbers in X's cells, and its rows' bits in nz.
+// batch_count_scale makes them h_1 = alpha |N(v) cap S_j|, rounded once (adding alpha up in FP32 drifts with
+// the count: 2.7e-4 of the score on a star of 100,000 leaves). With blockIdx.y = 0 a warp takes a member and
+// up to kScatterRow entries of its row; the other slices of the grid (where rows are longer) look through
+// 32 members at a time for the rest of hubs' rows, which they share.
+constexpr int kScatterRow = 256;
 __global__ void batch_scatter(int32_t* __restrict__ X, int32_t cols, const int32_t* __restrict__ mrow,
                               const int32_t* __restrict__ mcol, int32_t count, const int32_t* __restrict__ rp,
                               const int32_t* __restrict__ ci, uint32_t* __restrict__ nz) {
   const int lane = threadIdx.x & 31;
-  const int32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (i >= count) return;
-  const int32_t s = mrow[i], c = mcol[i];
-  const int64_t e1 = rp[s + 1];
-  for (int64_t e = rp[s] + static_cast<int64_t>(blockIdx.y) * 32 + lane; e < e1; e += 32 * static_cast<int64_t>(gridDim.y))
-  {
+  const int32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, warps = (gridDim.x * blockDim.x) >> 5;
+  auto add = [&](int64_t e, int32_t c) {
     const int32_t u = ci[e];
     atomicAdd(X + static_cast<size_t>(u) * cols + c, 1);
     if (!((nz[u >> 5] >> (u & 31)) & 1u)) atomicOr(nz + (u >> 5), 1u << (u & 31));
+  };
+  if (blockIdx.y == 0) {
+    for (int32_t i = warp; i < count; i += warps) {
+      const int32_t s = mrow[i], c = mcol[i];
+      const int64_t e0 = rp[s], e1 = min(static_cast<int64_t>(rp[s + 1]), e0 + kScatterRow);
+#pragma unroll 4
+      for (int64_t e = e0 + lane; e < e1; e += 32) add(e, c);
+    }
+    return;
+  }
+  const int slice = static_cast<int>(blockIdx.y) - 1, slices = static_cast<int>(gridDim.y) - 1;
+  for (int64_t i0 = 32 * static_cast<int64_t>(warp); i0 < count; i0 += 32 * static_cast<int64_t>(warps)) {
+    const int32_t mine = i0 + lane < count ? mrow[i0 + lane] : -1, col = i0 + lane < count ? mcol[i0 + lane] : 0;
+    const bool hub = mine >= 0 && rp[mine + 1] - rp[mine] > kScatterRow;
+    for (unsigned m = __ballot_sync(kFullMask, hub); m; m &= m - 1) {
+      const int32_t s = __shfl_sync(kFullMask, mine, __ffs(m) - 1), c = __shfl_sync(kFullMask, col, __ffs(m) - 1);
+      const int64_t e1 = rp[s + 1];
+#pragma unroll 4
+      for (int64_t e = static_cast<int64_t>(rp[s]) + kScatterRow + slice * 32 + lane; e < e1; e += 32 * slices) add(e, c);
+    }
   }
 }
 
@@ -456,7 +475,7 @@ static gedwalk_status batch_runs(Graph& g, Workspace& ws, int C, int ring_slots,
     GW_CUDA(cudaMemsetAsync(slot(t), 0, static_cast<size_t>(vec) * sizeof(float), s));
     GW_CUDA(cudaMemsetAsync(nz, 0, nz_bytes, s));
     if (!g.weighted && cnt > 0) {
-      batch_scatter<<<dim3((cnt + 7) / 8, g.dmax > 4096 ? 32 : 1), 256, 0, s>>>(
+      batch_scatter<<<dim3(static_cast<unsigned>(std::min((cnt + 7) / 8, 2048)), g.dmax > kScatterRow ? 32 : 1), 256, 0, s>>>(
           reinterpret_cast<int32_t*>(slot(1)), C, mrow + m0, mcol + m0, cnt, a.rp, a.ci, nz);
       GW_KCHECK();
       batch_count_scale<<<blocks_for(g.n_active), 256, 0, s>>>(slot(1), C, g.n_active, static_cast<float>(r.alpha), nz);
