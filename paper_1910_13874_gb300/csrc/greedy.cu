@@ -162,7 +162,8 @@ gedwalk_status maximize_runs(Graph& g, Workspace& ws, const Resolved& r, const G
   // Relative inflation of bounds against the rounding of the values a certification compares, beyond what
   // the bounds themselves allow for: each of the H - 1 sweeps' (run.h), 1e-6 at least. More costs runs where
   // gains lie close: R-MAT scale 22, k = 100 takes 35.5 ms with 1e-6, 39.8 with 3e-6 and 55 to 66 with 1e-5
-  // (1, 3 and 10 of 100 steps not certified by their guess); the other graphs measured do not care.
+  // (1, 3 and 10 of 100 steps not certified by their guess), and 37.8 with four times the bounds' own slack
+  // (run.cu); the other graphs measured do not care.
   auto tol = [&]() { return r.fp64 ? 1e-11 : std::max(1e-6, static_cast<double>(sweep_rounding<float>()) * (eng.H - 1)); };
   auto draws = [&](int32_t step) {
     eng.in->step = step;
@@ -254,7 +255,6 @@ gedwalk_status maximize_runs(Graph& g, Workspace& ws, const Resolved& r, const G
           sel = eng.out->lv[0];
         }
         bool first_batch = true, separated = true;
-        const int cols_cand = two_widths && width == 3 ? 4 : sh.cols_cand;
         std::vector<Cand> X;  // exact values for the current S, best first
         std::vector<int32_t> top;
         const int32_t left = g.n - static_cast<int32_t>(S_all->size());
@@ -295,6 +295,8 @@ gedwalk_status maximize_runs(Graph& g, Workspace& ws, const Resolved& r, const G
             ws.st_spec_miss += guessed;
             for (const Cand& e : E) eng.stale(e.v, e.g, step);
           }
+          // rows of four columns for the first batch where the chain's are; more candidates at a time after it
+          const int cols_cand = two_widths && width == 3 && first_batch ? 4 : sh.cols_cand;
           first_batch = false;
           std::vector<int32_t> last(top.begin(), top.begin() + std::min<size_t>(top.size(), cols_cand - 1));
           draws(step);

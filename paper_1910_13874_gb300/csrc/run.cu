@@ -516,8 +516,9 @@ __global__ void __launch_bounds__(kThreads, DIR || sizeof(T) * C > 32 ? 2 : kMee
   const T* __restrict__ xs = static_cast<const T*>(a.xs);
   const T* __restrict__ rs = sizeof(T) == 8 ? reinterpret_cast<const T*>(a.rs_d) : reinterpret_cast<const T*>(a.rs_f);
   // directed rounding keeps a bound above that of the stored vectors; e covers the vectors' own
-  // rounding where differences of columns cancel, keep the returns' where they reduce f
-  const float e = sweep_rounding<T>() * static_cast<float>(H > 2 ? H - 1 : 1);
+  // rounding where differences of columns cancel (sweeps' errors are independent and average over a row's
+  // neighbours, so like the root of their number), keep the returns' where they reduce f
+  const float e = sweep_rounding<T>() * sqrtf(fmaxf(1.0f, 0.25f * static_cast<float>(H - 1)));
   constexpr float keep = 1.0f - 2e-6f;
   const float infl = __fadd_ru(1.0f, __fmul_ru(static_cast<float>(H), 1.2e-7f));
   const float al2 = __double2float_rd(a.alpha * a.alpha), al3 = __double2float_ru(a.alpha * a.alpha * a.alpha);
