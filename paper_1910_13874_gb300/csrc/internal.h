@@ -141,7 +141,7 @@ void release_run_io(void* p);  // a workspace's run_io block, no longer referred
 struct Workspace {
   DevBuf x0, x1;     // walk vectors, [n][C]
   DevBuf mtab;       // gains of a small graph: phi^miss table, [(H+1)][n]
-  DevBuf ztab;       // runs without a shared walk-total table: the call's own, FP64
+  DevBuf ztab;       // runs without a shared walk-total table: the call's own, in the runs' precision
   DevBuf pvec;       // power iteration: three FP64 vectors and the statistics
   DevBuf partial;    // heavy-slice partial sums, [num_slices][C]
   DevBuf counters;   // heavy-row arrival counters, [num_heavy] (kept at 0 between launches)

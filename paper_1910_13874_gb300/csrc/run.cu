@@ -317,14 +317,15 @@ __global__ void run_own(T* __restrict__ X, int64_t set, int cols, RunDev* __rest
   d->live[o][j] = dg > 0;
 }
 
-// Tail bounds from the walk-total tables (FP64, rows n apart; times s on a weighted graph): the pairs
-// p + q <= L with p or q above H.
-// Directed (A: walks that start at v, B: that end there, both to L):
+// Tail bounds from tables of walk totals (rows n apart; times s on a weighted graph): the pairs p + q <= L
+// with p or q above H.
+// A: walks that start at v, B: that end there, both to L (the same on an undirected graph):
 //   tail(v) = sum_{p>H} b_p Qa_{L-p} + sum_{q>H} a_q Qb_{L-q},  Q_q = t_0 + ... + t_q.
-// Undirected (A = B, rows 0..H): t_{H+b}(v) <= t_H(v) M_b, M_b the largest t_b (a walk of length H + b
-// from v is one of length H and one of length b from its end), so
+// With M, an undirected graph's table of rows 0..H: t_{H+b}(v) <= t_H(v) M_b, M_b the largest t_b (a walk of
+// length H + b from v is one of length H and one of length b from its end), so
 //   tail(v) = 2 t_H(v) sum_{b=1..L-H} M_b Q_{L-H-b}.
-// Rounded up; and (about) the bound of the empty group, F + U + F U + tail, for the first guesses.
+// Rounded up, times `grow` for the table's own rounding; and (about) the bound of the empty group,
+// F + U + F U + tail, for the first guesses.
 __global__ void row_max_kernel(const double* __restrict__ A, int64_t n, int32_t n_active, const double* __restrict__ rs,
                                unsigned long long* __restrict__ M) {
   const double* row = A + static_cast<size_t>(blockIdx.y + 1) * n;
@@ -336,41 +337,51 @@ __global__ void row_max_kernel(const double* __restrict__ A, int64_t n, int32_t 
   if ((threadIdx.x & 31) == 0) atomicMax(M + blockIdx.y + 1, static_cast<unsigned long long>(__double_as_longlong(m)));
 }
 
-__global__ void tail_kernel(const double* __restrict__ A, const double* __restrict__ B, const double* __restrict__ M,
-                            int64_t n, int32_t n_active, int32_t L, int32_t H, const double* __restrict__ rs, double alpha,
-                            float* __restrict__ tail, float* __restrict__ bound) {
+template <typename T>
+__global__ void tail_kernel(const T* __restrict__ A, const T* __restrict__ B, const double* __restrict__ M,
+                            int64_t n, int32_t n_active, int32_t L, int32_t H, const T* __restrict__ rs, double alpha,
+                            double grow, float* __restrict__ tail, float* __restrict__ bound) {
   for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n_active; v += gridDim.x * blockDim.x) {
     const double inv = rs ? 1.0 / rs[v] : 1.0;
+    auto a = [&](int32_t t) { return A[static_cast<size_t>(t) * n + v] * inv; };
+    auto b = [&](int32_t t) { return B[static_cast<size_t>(t) * n + v] * inv; };
     double Qa = 0.0, Qb = 0.0, acc = 0.0, U = 0.0, F = 0.0;
-    if (A == B) {
+    if (M) {
       for (int32_t q = 0; q < L - H; ++q) {
-        const double t = A[static_cast<size_t>(q) * n + v] * inv;
+        const double t = a(q);
         Qa += t;
         if (q > 0) U += t;
         acc += __ldg(M + (L - H - q)) * Qa;
       }
-      for (int32_t t = std::max(L - H, 1); t < H; ++t) U += A[static_cast<size_t>(t) * n + v] * inv;
-      const double tH = A[static_cast<size_t>(H) * n + v] * inv;
+      for (int32_t t = std::max(L - H, 1); t < H; ++t) U += a(t);
+      const double tH = a(H);
       U += tH;
       acc *= 2.0 * tH;
-      const double f1 = A[n + v] * inv, f2 = H >= 2 ? A[2 * n + v] * inv : 0.0;
+      const double f1 = a(1), f2 = H >= 2 ? a(2) : 0.0;
       const double s2 = rs ? 0.0 : alpha * f1, s4 = rs || H < 4 ? 0.0 : alpha * alpha * f2 - alpha * alpha * alpha * f1;
       F = U - (H >= 2 ? (s2 + s4) * (1.0 + U) : 0.0);
     } else {
       for (int32_t q = 0; q < L - H; ++q) {
-        Qa += A[static_cast<size_t>(q) * n + v];
-        Qb += B[static_cast<size_t>(q) * n + v];
-        acc += B[static_cast<size_t>(L - q) * n + v] * Qa + A[static_cast<size_t>(L - q) * n + v] * Qb;
+        Qa += a(q);
+        Qb += b(q);
+        acc += b(L - q) * Qa + a(L - q) * Qb;
       }
       for (int32_t t = 1; t <= H; ++t) {
-        U += A[static_cast<size_t>(t) * n + v];
-        F += B[static_cast<size_t>(t) * n + v];
+        U += a(t);
+        F += b(t);
       }
     }
-    acc *= 1.0 + 1e-12;
+    acc *= grow;
     tail[v] = __double2float_ru(acc);
     bound[v] = static_cast<float>(F + U + F * U + acc);
   }
+}
+
+// Row 0 of a call's own table: 1 outside S (times s).
+template <typename T>
+__global__ void own_row0(T* __restrict__ row, const uint32_t* __restrict__ mask, int32_t n_active, const T* __restrict__ rs) {
+  for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n_active; v += gridDim.x * blockDim.x)
+    row[v] = in_set(mask, v) ? T(0) : rs ? rs[v] : T(1);
 }
 
 struct MeetArgs {
@@ -1149,18 +1160,21 @@ gedwalk_status RunEngine::set_length(int32_t length, bool select) {
   H = (L + 1) / 2;
   if (!select || g.n_active == 0) return GEDWALK_OK;
   // tail bounds from the walk totals; the tables are read under their lock, to the end of the kernel
-  const double* rs = g.weighted ? g.rs_d.as<double>() : nullptr;
   const int32_t rows = walk_rows(g, L + 1);
   // the largest entries of rows 1..L-H (the selections' lists are free here)
   unsigned long long* M = ws.sel.as<unsigned long long>();
   auto tails = [&](const double* A, const double* B) -> gedwalk_status {
-    if (!g.directed && L > H) {
+    const double* rs = g.weighted ? g.rs_d.as<double>() : nullptr;
+    if (!g.directed) {
       GW_CUDA(cudaMemsetAsync(M, 0, sizeof(*M) * (L - H + 1), s));
-      row_max_kernel<<<dim3(std::min(grid_of(g.n_active), 304), L - H), 256, 0, s>>>(A, g.n, g.n_active, rs, M);
-      GW_KCHECK();
+      if (L > H) {
+        row_max_kernel<<<dim3(std::min(grid_of(g.n_active), 304), L - H), 256, 0, s>>>(A, g.n, g.n_active, rs, M);
+        GW_KCHECK();
+      }
     }
-    tail_kernel<<<grid_of(g.n_active), 256, 0, s>>>(A, B, reinterpret_cast<const double*>(M), g.n, g.n_active, L, H, rs, r.alpha,
-                                                    ws.tail.as<float>(), ws.bound.as<float>());
+    tail_kernel<double><<<grid_of(g.n_active), 256, 0, s>>>(A, B, g.directed ? nullptr : reinterpret_cast<const double*>(M),
+                                                            g.n, g.n_active, L, H, rs, r.alpha, 1.0 + 1e-12,
+                                                            ws.tail.as<float>(), ws.bound.as<float>());
     GW_KCHECK();
     return GEDWALK_OK;
   };
@@ -1178,14 +1192,40 @@ gedwalk_status RunEngine::set_length(int32_t length, bool select) {
       return GEDWALK_OK;
     }
   }
-  // no table for this alpha (a forced L beyond the bound's reach): totals of this call's own
-  const size_t cells = static_cast<size_t>(rows) * g.n;
-  GW_TRY(ws.ztab.ensure((g.directed ? 2 : 1) * cells * sizeof(double), s));
-  double* A = ws.ztab.as<double>();
-  double* B = g.directed ? A + cells : A;
-  GW_TRY(totals_into(g, ws, A, r.alpha, 0, rows, false, s));
-  if (g.directed) GW_TRY(totals_into(g, ws, B, r.alpha, 0, rows, true, s));
-  return tails(A, B);
+  return r.fp64 ? own_tails<double>() : own_tails<float>();
+}
+
+// No table for this alpha (a forced L beyond the bound's reach): totals of this call's own, of the walks that
+// avoid the S it starts from, to the full length (where walks multiply with their length the largest
+// entries of the other form are far off) and in the runs' precision: in FP64 R-MAT scale 20, L = 9, spent
+// 1.2 ms on them, more than on the run.
+template <typename T>
+gedwalk_status RunEngine::own_tails() {
+  const size_t cells = static_cast<size_t>(L + 1) * g.n;
+  const int sets = g.directed ? 2 : 1;
+  GW_TRY(ws.ztab.ensure(sets * cells * sizeof(T), s));
+  GW_TRY(ws.x0.ensure(static_cast<size_t>(g.n) * sizeof(T), s));  // the sweeps' unscaled values, unused
+  T* tab = ws.ztab.as<T>();
+  const T* rs = !g.weighted ? nullptr : sizeof(T) == 8 ? static_cast<const T*>(g.rs_d.p) : static_cast<const T*>(g.rs_f.p);
+  for (int o = 0; o < sets; ++o) {
+    T* row = tab + o * cells;
+    own_row0<T><<<grid_of(g.n_active), 256, 0, s>>>(row, ws.mask.as<uint32_t>(), g.n_active, rs);
+    GW_KCHECK();
+    SweepArgs a = o ? base_args_rev(g, ws) : base_args(g, ws);
+    a.alpha = r.alpha;
+    a.Mout = ws.x0.p;
+    for (int32_t t = 1; t <= L; ++t, row += g.n) {
+      a.X = row;
+      a.Y = row + g.n;
+      GW_TRY(launch_sweep(MODE_MISS, sizeof(T) == 8, 1, a, s));
+    }
+  }
+  // a sweep rounds a value by at most 41 units (run.h), and two values meet
+  const double grow = 1.0 + 2.0 * (L + 1) * (sizeof(T) == 8 ? 5e-15 : 2.5e-6);
+  tail_kernel<T><<<grid_of(g.n_active), 256, 0, s>>>(tab, tab + (sets - 1) * cells, nullptr, g.n, g.n_active, L, H, rs, r.alpha,
+                                                     grow, ws.tail.as<float>(), ws.bound.as<float>());
+  GW_KCHECK();
+  return GEDWALK_OK;
 }
 
 void RunEngine::stale(int32_t v, double gain, int32_t step) {

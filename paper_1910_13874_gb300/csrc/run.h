@@ -120,6 +120,8 @@ struct RunEngine {
   void stale(int32_t v, double gain, int32_t step);
 
  private:
+  template <typename T>
+  gedwalk_status own_tails();
   gedwalk_status push_added();
   gedwalk_status issue(bool chain, int cols, bool select, bool profile, const std::vector<cudaEvent_t>* ev);
 };

@@ -210,3 +210,26 @@ def test_groups_of_every_size(cuda_device, directed, size):
         assert rel(gains[0], ref_gains[0]) < 1e-12
         assert rel(score, oracle.score(g, S, alpha, 5) + ref_gains[0]) < 1e-12
     G.free()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("kind", ["plain", "weighted", "directed"])
+def test_alpha_beyond_the_bound(cuda_device, prec, kind):
+    # a forced length with alpha * d_max > 1: no table of walk totals applies, the call makes its own
+    from paper_1910_13874_gb300 import gedwalk
+
+    directed = kind == "directed"
+    g = gg.rmat(9, 8, seed=6, directed=True) if directed else ba()
+    w = oracle.normalized_weights(g) if kind == "weighted" else None
+    alpha = 2.5 / oracle.delta(g, w, directed)
+    G = gedwalk.Graph.from_host(g, weighted=kind == "weighted", directed=directed)
+    for L in (1, 2, 3, 8, 11):
+        for init in (None, [3, 17, 200]):
+            grp, gains, _, _ = G.maximize(6, precision=prec, alpha=alpha, L=L, init=init)
+            ref, ref_gains, _ = oracle.greedy(g, 6, alpha, L, "lazy", init=init, w=w, directed=directed)
+            if init is None:
+                check_sequence(grp, gains, TOL[prec], ref, ref_gains,
+                               *oracle_greedy_checker(oracle, g, alpha, L, w=w, directed=directed))
+            else:
+                assert np.allclose(gains, ref_gains, rtol=TOL[prec], atol=0), L
+    G.free()
