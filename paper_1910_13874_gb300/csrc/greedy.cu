@@ -190,9 +190,10 @@ gedwalk_status maximize_runs(Graph& g, Workspace& ws, const Resolved& r, const G
   RunOut look{};                // the last run's answers, and
   std::vector<int32_t> look_c;  // its guesses
   // FP64 rows of 8 columns cost more than rows of 4 in every sweep, so they wait for a chain that held
-  // for three steps (on a small graph one winner changes the order of the next ones).
+  // for three steps (on a small graph one winner changes the order of the next ones) and are no use for
+  // three steps or fewer.
   const bool two_widths = r.fp64 && sh.levels == 7;
-  int width = two_widths && g.n_active < 20000 ? 3 : n_spec;
+  int width = two_widths && (g.n_active < 20000 || p.k <= 3) ? 3 : n_spec;
   int held = -1;                // steps the last chain has carried (-1: none yet)
   int lvl = -1;                 // its level that stands under the current S (-1: none)
 
