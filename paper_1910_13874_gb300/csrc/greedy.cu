@@ -207,6 +207,7 @@ gedwalk_status maximize_runs(Graph& g, Workspace& ws, const Resolved& r, const G
       if (small) {
         std::vector<double> got(g.n_active);
         GW_TRY(small_gains(g, ws, r, *S_all, got.data()));
+        eng.sweeps += eng.H;  // of phi^miss; the columns' steps are no sweeps
         for (int32_t v = 0; v < g.n_active; ++v) {
           if (inS[v]) continue;
           const Cand e{got[v], v, g.perm[v]};

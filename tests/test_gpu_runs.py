@@ -233,3 +233,12 @@ def test_alpha_beyond_the_bound(cuda_device, prec, kind):
             else:
                 assert np.allclose(gains, ref_gains, rtol=TOL[prec], atol=0), L
     G.free()
+
+
+def test_sweeps_are_counted_for_gains_from_shared_memory(cuda_device):
+    from paper_1910_13874_gb300 import gedwalk
+
+    G = gedwalk.Graph.from_host(ba())
+    G.maximize(3, precision="fp32", L=7, gains_all=True)
+    assert G.maximize_stats()["sweeps"] == 3 * 4  # phi^miss to half the length, per step
+    G.free()
