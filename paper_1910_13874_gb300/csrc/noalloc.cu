@@ -77,7 +77,8 @@ __device__ __forceinline__ double na_store(const uint32_t* __restrict__ mask, fl
 // eight gathers per lane in flight, and above kNaChunk entries gathered by the whole block into shared
 // memory and added up by one warp, so that no group walks a hub alone. Block b writes its sum of
 // hit'(v) to slots[b]. Barabasi-Albert, n = 10^6, m = 8 (88 MB in and out, 16 M gathers): 135 us; a
-// warp per row, 256 rows in sequence, took 2,230 us, and blocks of consecutive rows 380 us.
+// warp per row, 256 rows in sequence, took 2,230 us, and blocks of consecutive rows 380 us. Entry positions
+// are unsigned: up to 2^31 entries, and what is added to look past a row's end must not wrap.
 __global__ void __launch_bounds__(kThreads) na_step(const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
                                                    int32_t n, int32_t iters, const uint32_t* __restrict__ mask,
                                                    const float2* __restrict__ x, float2* __restrict__ y, float alpha,
@@ -122,8 +123,8 @@ __global__ void __launch_bounds__(kThreads) na_step(const int32_t* __restrict__ 
     for (int k = 0; k < 2; ++k)
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const int32_t j = e0[k] + q * kNaLanes + gl;
-        id[k][q] = j < e1[k] ? __ldg(ci + j) : -1;
+        const uint32_t j = static_cast<uint32_t>(e0[k]) + q * kNaLanes + gl;
+        id[k][q] = j < static_cast<uint32_t>(e1[k]) ? __ldg(ci + j) : -1;
       }
 #pragma unroll
     for (int k = 0; k < 2; ++k)
@@ -132,11 +133,12 @@ __global__ void __launch_bounds__(kThreads) na_step(const int32_t* __restrict__ 
         if (id[k][q] >= 0) p[k].add(q, __ldg(x + id[k][q]));
 #pragma unroll
     for (int k = 0; k < 2; ++k) {  // entries 32.. of rows longer than that
-      for (int32_t j0 = e0[k] + 32; j0 < e1[k]; j0 += 32) {
+      const uint32_t end = static_cast<uint32_t>(e1[k]);
+      for (uint32_t j0 = static_cast<uint32_t>(e0[k]) + 32; j0 < end; j0 += 32) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          const int32_t j = j0 + q * kNaLanes + gl;
-          if (j < e1[k]) p[k].add(q, __ldg(x + __ldg(ci + j)));
+          const uint32_t j = j0 + q * kNaLanes + gl;
+          if (j < end) p[k].add(q, __ldg(x + __ldg(ci + j)));
         }
       }
     }

@@ -399,7 +399,7 @@ __device__ __forceinline__ void short_rows(const SweepArgs& a, const Src& src, c
   for (int it = 0; it < nrows; it += 2 * NG) {
     const int ra = it + g, rb = it + NG + g;
     const bool va = ra < nrows, vb = rb < nrows;
-    int ea0 = 0, ea1 = 0, eb0 = 0, eb1 = 0;
+    unsigned ea0 = 0, ea1 = 0, eb0 = 0, eb1 = 0;  // unsigned: positions past a row's end must not wrap at 2^31
     if (va) {
       ea0 = s_rp[ra];
       ea1 = s_rp[ra + 1];
@@ -409,7 +409,7 @@ __device__ __forceinline__ void short_rows(const SweepArgs& a, const Src& src, c
       eb1 = s_rp[rb + 1];
     }
     // all index loads first, then all gathers
-    const int ja0 = ea0 + gl, ja1 = ea0 + gl + W, jb0 = eb0 + gl, jb1 = eb0 + gl + W;
+    const unsigned ja0 = ea0 + gl, ja1 = ea0 + gl + W, jb0 = eb0 + gl, jb1 = eb0 + gl + W;
     const int va0 = ja0 < ea1 ? ld_idx(ci + ja0, pol) : -1;
     const int va1 = ja1 < ea1 ? ld_idx(ci + ja1, pol) : -1;
     const int vb0 = jb0 < eb1 ? ld_idx(ci + jb0, pol) : -1;
@@ -470,11 +470,11 @@ __device__ __forceinline__ void long_rows(const SweepArgs& a, const Src& src, co
   ColAcc<T, NL> cacc;
   cacc.zero();
   for (int rr = 0; rr < nrows; ++rr) {
-    const int e0 = s_rp[rr], e1 = s_rp[rr + 1];
+    const unsigned e1 = s_rp[rr + 1];
     T acc[C];
 #pragma unroll
     for (int c = 0; c < C; ++c) acc[c] = T(0);
-    int j = e0 + lane;
+    unsigned j = static_cast<unsigned>(s_rp[rr]) + lane;
     for (; j + 96 < e1; j += 128) {
       const int v0 = ld_idx(ci + j, pol), v1 = ld_idx(ci + j + 32, pol), v2 = ld_idx(ci + j + 64, pol),
                 v3 = ld_idx(ci + j + 96, pol);
@@ -511,8 +511,9 @@ __device__ __forceinline__ void heavy_slice(const SweepArgs& a, const Src& src, 
   T acc[C];
 #pragma unroll
   for (int c = 0; c < C; ++c) acc[c] = T(0);
-  int j = u.y + lane;
-  for (; j + 96 < u.z; j += 128) {
+  unsigned j = static_cast<unsigned>(u.y) + lane;
+  const unsigned end = u.z;
+  for (; j + 96 < end; j += 128) {
     const int v0 = ld_idx(ci + j, pol), v1 = ld_idx(ci + j + 32, pol), v2 = ld_idx(ci + j + 64, pol),
               v3 = ld_idx(ci + j + 96, pol);
     src.add(acc, v0);
@@ -520,7 +521,7 @@ __device__ __forceinline__ void heavy_slice(const SweepArgs& a, const Src& src, 
     src.add(acc, v2);
     src.add(acc, v3);
   }
-  for (; j < u.z; j += 32) src.add(acc, ld_idx(ci + j, pol));
+  for (; j < end; j += 32) src.add(acc, ld_idx(ci + j, pol));
   SC::run(acc, lane);
   // this unit's own slot carries nothing: the row's sums go to the heavy row's slot
   if constexpr (NS > 0) {
