@@ -97,8 +97,8 @@ __device__ __forceinline__ Pair to_pair(double x) {
 }
 
 // Per-lane column sums over the rows of one unit. FP64 vectors sum in FP64. FP32 vectors sum with
-// compensated FP32 additions (Kahan: the error is at most 2u * sum |y| + O(m u^2), u = 2^-24, over
-// m <= 128 rows) and convert once per unit to FP64, in which every later sum (over lanes, units and
+// compensated FP32 additions (Kahan: the error is at most 2u * sum |y| + O(m u^2), u = 2^-24, over a
+// unit's m <= 128 rows) and convert once per unit to FP64, in which every later sum (over lanes, units and
 // sweeps) is taken. On a GB300 an FP64 addition costs about 64 FP32 ones, and one conversion and
 // one FP64 addition per row and column cost more than the rest of the epilogue.
 template <typename T, int N>

@@ -3,8 +3,10 @@
 // The gain of c needs the half-length column of walks through c (run.cu). All n columns share one
 // small graph, so a block keeps its columns in shared memory from the first step to the last and no
 // step waits for another block: one launch instead of n / 15 runs of ceil(L/2) sweeps each (Erdos-
-// Renyi, n = 3001, degree 10, FP32: 23.2 ms, 5 us a sweep, nearly all of it launch and latency). A
-// block is bound by its shared-memory gathers: rows of K columns, random.
+// Renyi, n = 3001, degree 10, FP32: 23.2 ms, 5 us a sweep, nearly all of it launch and latency; now
+// 1.32 ms). A block is bound by instructions and latency: an index load and a 4-byte shared load per lane
+// and entry, five loads and some forty operations per row and step, one block of 32 warps per SM (the
+// columns take 192 KB); the shared-memory gathers by themselves would take a quarter of the time.
 #include <algorithm>
 
 #include "run.h"

@@ -191,7 +191,11 @@ gedwalk_status maximize_runs(Graph& g, Workspace& ws, const Resolved& r, const G
   std::vector<int32_t> look_c;  // its guesses
   // FP64 rows of 8 columns cost more than rows of 4 in every sweep, so they wait for a chain that held
   // for three steps (on a small graph one winner changes the order of the next ones) and are no use for
-  // three steps or fewer.
+  // three steps or fewer. k = 20, ms starting with three / seven: Erdos-Renyi 4,000 1.38 / 1.61, 12,000
+  // 1.19 / 1.38, 30,000 1.72 / 2.08, 100,000 3.51 / 2.99, 400,000 9.55 / 8.11; Barabasi-Albert 4,000 0.60 /
+  // 0.49, 30,000 0.76 / 0.64, 400,000 2.73 / 2.33; R-MAT of 2^13 rows 0.85 / 1.10, 2^18 2.87 / 2.43. So the line
+  // could lie anywhere between 12,000 and 100,000, and hubs would have it lower. Waiting for one or two steps
+  // instead of three changes nothing, for five costs up to a half more.
   const bool two_widths = r.fp64 && sh.levels == 7;
   int width = two_widths && (g.n_active < 20000 || p.k <= 3) ? 3 : n_spec;
   int held = -1;                // steps the last chain has carried (-1: none yet)

@@ -166,7 +166,6 @@ struct Workspace {
   uint64_t graph_clock = 0;
   cudaStream_t own_stream = nullptr;  // capturable stream used when the caller passes stream 0
   cudaEvent_t order_ev = nullptr;     // orders own_stream after the caller's stream
-  std::vector<uint8_t> host_small;  // staging
   void* run_io = nullptr;           // pinned block of the runs' copies: one size, kept while captured
                                     // sequences refer to it
   void* pinned = nullptr;           // pinned host staging buffer

@@ -65,9 +65,11 @@ struct RunDev {  // device-side state of the runs of one workspace
 
 // Runs a launch sequence, captured once per configuration and replayed as a CUDA graph; directly on the
 // legacy default stream. The capture comes with the second use, above kLateEntries entries with the
-// fourth: sweeps outlast their launches there, and a new graph's short maximisation (two runs on R-MAT
-// scale 20) spent 0.3 of its 1.9 ms on capturing and instantiating. `issue` gets the two timing events of a
-// capture (or null).
+// fourth: sweeps outlast their launches there, so a new graph's short maximisation gains nothing from it.
+// First call of k = 10 on a new handle, capture with the second / fourth use, ms: R-MAT scale 20 (31 M
+// entries) 1.86 / 1.57, scale 18 (7.6 M) 1.11 / 0.73; Barabasi-Albert 4 to 16 M 1.03 / 0.96 to 1.42 / 1.40;
+// below the line 0.52 / 0.64 (R-MAT scale 16) to 0.74 / 0.45 (Barabasi-Albert 1.6 M), within the runs' spread.
+// `issue` gets the two timing events of a capture (or null).
 constexpr int64_t kLateEntries = int64_t(4) << 20;
 struct Sequence {
   uint64_t key;

@@ -356,8 +356,10 @@ gedwalk_status score_one(Graph& g, Workspace& ws, const std::vector<int32_t>& S_
 
 // Picks the column-block width with the lowest sweep time per column (timed on this graph). A
 // gather fetches whole 32-byte sectors, so widths below 8 FP32 columns waste part of each; above
-// 32 the walk vectors of a 10^6-vertex graph (n * C * 4 bytes, twice) outgrow the L2 and the
-// per-column time rises (the tuning log records it).
+// 32 a sweep's pair of vectors of a 10^6-vertex graph outgrows the L2 and the per-column time rises (the
+// tuning log records it). Only the dense sweep is timed: the meeting pass and a block's launches, a quarter
+// of its time, favour wider blocks (Barabasi-Albert 10^6, 512 groups: 20.7 ms at the 16 columns it picks, 19.8
+// at 32, 21.6 at 64).
 gedwalk_status autotune_batch(Graph& g, Workspace& ws, const Resolved& r) {
   if (g.batch_cols > 0) return GEDWALK_OK;
   cudaStream_t s = r.stream;
