@@ -171,8 +171,8 @@ __device__ __forceinline__ void join_set(const int32_t* __restrict__ list, int32
 
 // The same for a whole group, which may be half of the graph. With blockIdx.y = 0 a warp takes a member at a
 // time and up to kJoinRow entries of its row; the other slices of the grid (where rows are longer than that)
-// look through 32 members at a time for the rest of hubs' rows, which they share. A block per member took
-// 30 ms for half of R-MAT scale 20, the sweeps 0.35. count: list[-1] when negative (a captured launch).
+// look through up to 32 members at a time for the rest of hubs' rows, which they share. A block per member
+// took 30 ms for half of R-MAT scale 20, the sweeps 0.35. count: list[-1] when negative (a captured launch).
 constexpr int kJoinRow = 256;
 __global__ void join_kernel(const int32_t* __restrict__ list, int32_t count, const Rows g, uint32_t* __restrict__ mask) {
   if (count < 0) count = list[-1];
@@ -191,8 +191,9 @@ __global__ void join_kernel(const int32_t* __restrict__ list, int32_t count, con
     return;
   }
   const int slice = static_cast<int>(blockIdx.y) - 1, slices = static_cast<int>(gridDim.y) - 1;
-  for (int64_t i0 = 32 * static_cast<int64_t>(warp); i0 < count; i0 += 32 * static_cast<int64_t>(warps)) {
-    const int32_t mine = i0 + lane < count ? list[i0 + lane] : -1;
+  const int per = max(1, min(32, (count + warps - 1) / warps));  // few members: each its own warps
+  for (int64_t i0 = per * static_cast<int64_t>(warp); i0 < count; i0 += per * static_cast<int64_t>(warps)) {
+    const int32_t mine = lane < per && i0 + lane < count ? list[i0 + lane] : -1;
     for (int o = 0; o <= g.directed; ++o) {
       const int r = g.directed ? 1 - o : 0;
       const bool hub = mine >= 0 && g.rp[r][mine + 1] - g.rp[r][mine] > kJoinRow;

@@ -110,7 +110,7 @@ __global__ void batch_totals(const double* __restrict__ T, int64_t n, int32_t n_
 // batch_count_scale makes them h_1 = alpha |N(v) cap S_j|, rounded once (adding alpha up in FP32 drifts with
 // the count: 2.7e-4 of the score on a star of 100,000 leaves). With blockIdx.y = 0 a warp takes a member and
 // up to kScatterRow entries of its row; the other slices of the grid (where rows are longer) look through
-// 32 members at a time for the rest of hubs' rows, which they share.
+// up to 32 members at a time for the rest of hubs' rows, which they share.
 constexpr int kScatterRow = 256;
 __global__ void batch_scatter(int32_t* __restrict__ X, int32_t cols, const int32_t* __restrict__ mrow,
                               const int32_t* __restrict__ mcol, int32_t count, const int32_t* __restrict__ rp,
@@ -132,8 +132,10 @@ __global__ void batch_scatter(int32_t* __restrict__ X, int32_t cols, const int32
     return;
   }
   const int slice = static_cast<int>(blockIdx.y) - 1, slices = static_cast<int>(gridDim.y) - 1;
-  for (int64_t i0 = 32 * static_cast<int64_t>(warp); i0 < count; i0 += 32 * static_cast<int64_t>(warps)) {
-    const int32_t mine = i0 + lane < count ? mrow[i0 + lane] : -1, col = i0 + lane < count ? mcol[i0 + lane] : 0;
+  const int per = max(1, min(32, (count + warps - 1) / warps));  // few members: each its own warps
+  for (int64_t i0 = per * static_cast<int64_t>(warp); i0 < count; i0 += per * static_cast<int64_t>(warps)) {
+    const bool some = lane < per && i0 + lane < count;
+    const int32_t mine = some ? mrow[i0 + lane] : -1, col = some ? mcol[i0 + lane] : 0;
     const bool hub = mine >= 0 && rp[mine + 1] - rp[mine] > kScatterRow;
     for (unsigned m = __ballot_sync(kFullMask, hub); m; m &= m - 1) {
       const int32_t s = __shfl_sync(kFullMask, mine, __ffs(m) - 1), c = __shfl_sync(kFullMask, col, __ffs(m) - 1);
