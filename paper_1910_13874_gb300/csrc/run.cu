@@ -32,11 +32,11 @@
 // grows), from the walk-total tables. (Directed: F sums psi, U phi; the returns are not counted.)
 //
 // Measured on a GB300 (one maximisation, before: full-length sweeps that store every level's phi, a
-// bound pass per step and the visits-times-continuations bound): R-MAT scale 22, k = 100, FP32 144.3
-// -> 34.5 ms (60 to 64 sweeps of 493 us instead of 135 of 587 and 54 of 498); Erdos-Renyi n = 100,003,
-// degree 16, k = 27 18.1 -> 2.0 ms (the sharper bound leaves one or two candidate batches);
-// Barabasi-Albert n = 10^6, k = 25, FP64 38.2 -> 7.4 ms; Algorithm 2 on R-MAT scale 20, k = 50 93.6 ->
-// 9.9 ms.
+// bound pass per step and the visits-times-continuations bound): R-MAT scale 22, k = 100, FP32 126 to 144
+// -> 33.6 to 38 ms, by the graph's seed (60 to 68 sweeps of 494 us instead of 135 of 587 and 54 of 498); Erdos-Renyi
+// n = 100,003, degree 16, k = 27 18.1 -> 2.1 ms (the sharper bound leaves one or two candidate batches);
+// Barabasi-Albert n = 10^6, k = 25, FP64 39.2 -> 7.5 ms (10.2 where a chain breaks); Algorithm 2 on R-MAT
+// scale 20, k = 50 96.5 -> 10.1 ms.
 #include <algorithm>
 #include <cmath>
 
@@ -504,9 +504,10 @@ __device__ __forceinline__ void block_levels(WarpList (&w)[NL], float* sv, int* 
 // correction, against the lowest last entry of the lists, decides. The rows come by decreasing
 // degree, so after a warp's first iteration few pass. A bound of exactly 0 matters only when every
 // bound is 0, so its vertex is recorded only while the warp's list is empty, and by one atomic per block
-// (one per row, all to one address, serialise: k = 1 on a star of 100,000 leaves, 0.44 ms). 279 -> 123 us (418 MB
-// of traffic at 3.4 TB/s, 37% of the warps resident: a row's vectors and sums take the registers); on 10^5
-// rows, where a warp has one iteration, the lists cost most (device_util.cuh): 97 -> 63 us.
+// (one per row, all to one address, serialise: k = 1 on a star of 100,000 leaves, 0.44 ms). R-MAT scale 22:
+// 279 -> 123 us with FP32 gain terms, 180 us with pairs (97 M warp instructions instead of 42 M bound it, at 37% of
+// the warps: a row's vectors, their low parts and the sums take the registers; 417 MB of traffic). On 10^5
+// rows, where a warp has one iteration, the lists cost most (device_util.cuh): 97 -> 77 us.
 template <typename T, int C, bool CHAIN, bool SEL, bool DIR>
 __global__ void __launch_bounds__(kThreads, DIR || sizeof(T) * C > 32 ? 2 : kMeetPerSM) meet_kernel(const MeetArgs a) {
   constexpr int D = C - 1;
