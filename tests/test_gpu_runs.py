@@ -175,7 +175,7 @@ def test_fp64_chain_widths(cuda_device):
 
 @pytest.mark.parametrize("kw", [{}, dict(lookahead=1)])
 def test_long_walks_are_certified(cuda_device, kw):
-    # 30 sweeps a run: the rounding a certification allows for grows with them (2.5e-7 each, so 1e-5)
+    # 30 sweeps a run: the rounding a certification allows for grows with the root of their number
     from paper_1910_13874_gb300 import gedwalk
 
     g = gg.erdos_renyi(2000, 8, 5)
